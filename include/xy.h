@@ -125,9 +125,10 @@ typedef struct {
                              tile kernel per SM (at most 80 registers a thread), 4 (at
                              most 64: more warps per SM), 2 (at most 128: more
                              independent work in flight per warp, fewer warps), or 0
-                             for the library's default: 3 for the persistent sweep,
-                             4 for one fused launch per sweep (the faster plans at
-                             L = 4096 and at L = 8192, 16384).  Results do not
+                             for the library's default: 2 for the persistent sweep
+                             where that holds all of a sweep's tiles, else 3; 4 for
+                             one fused launch per sweep (the faster plans at L <= 1024,
+                             L = 4096 and L = 8192, 16384).  Results do not
                              depend on it; tuning callers time the plans
                              (autotune.py). */
 } xy_params;

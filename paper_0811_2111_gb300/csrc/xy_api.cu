@@ -58,11 +58,19 @@ void set_thread_msg(const char* fmt, ...) {
 // every sweep; beyond it (L = 8192: 36 waves) the per-sweep launch is faster.
 constexpr int kAutoPersistentMaxL = 4096;
 
+// Default work plan of the persistent sweep: 2 CTAs per SM (128 registers a
+// thread) where that many hold all of a sweep's tiles (L <= 1024 on 152 SMs:
+// a sweep is then one tile's latency, and more registers shorten it: 5.8
+// against 6.4 us per sweep at L = 512, 8.9 against 9.3 at 1024), else 3 (L =
+// 2048: 19.2 against 19.5 us).
+constexpr int kFewTilesPerSm = 2;
+
 struct xy_ctx {
   uint32_t magic;
   xy_params p;
   cudaStream_t stream;
   int device;
+  int sms;                 // multiprocessors of the device
   float* d_theta;          // [2][L][L/2]: the state between calls
   bool owns_theta;
   float* d_pong;           // second buffer of the fused kernel (library-owned)
@@ -358,6 +366,8 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
   snprintf(c->msg, sizeof(c->msg), "no error");
   const size_t N = (size_t)p->L * (size_t)p->L;
   cudaError_t e = cudaGetDevice(&c->device);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   if (e == cudaSuccess) {
     if (d_angles) {
       c->d_theta = static_cast<float*>(d_angles);
@@ -487,7 +497,8 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
     a.error = c->d_wait;
     a.spin_limit = xyk::fused_persistent_spin_limit();
     a.skip_items = 0;
-    a.minb = c->p.ctas_per_sm ? c->p.ctas_per_sm : 3;
+    a.minb = c->p.ctas_per_sm ? c->p.ctas_per_sm
+             : xyk::fused_tiles(c->p.L) <= kFewTilesPerSm * c->sms ? 2 : 3;
     // one launch per at most fused_persistent_max_sweeps sweeps (the kernel's
     // work items are counted in 32 bits)
     const int64_t chunk = xyk::fused_persistent_max_sweeps(c->p.L);

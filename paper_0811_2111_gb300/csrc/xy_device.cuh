@@ -232,6 +232,141 @@ __device__ __forceinline__ SiteResult metropolis_step(float t, float c0, float s
   return r;
 }
 
+// ---- two sites at a time ----
+// The kernels' inner loops update the two sites of a Philox pair together, on
+// packed FP32 instructions (fma / add / mul .rn.f32x2): two independent IEEE
+// operations in one issue slot, so every lane gets the bits of the scalar
+// functions above.  A packed instruction holds both FMA pipes for two cycles
+// (measured 64 per SM and clock: the scalar FP32 rate, in half the issue
+// slots), and the tile kernels were bound by issue slots (74-76 % used) with
+// the FMA pipes half idle.  The fused sweep: 140.4 -> 117 issued instructions
+// per update; persistent at L = 4096 79.1 -> 73.7 us per sweep, one launch per
+// sweep at L = 16384 1205 -> 1106 us (SFU 912 -> 858).  What bounds them now is
+// the heavy FMA pipe (68 %: the packed instructions and, four cycles each, the
+// Philox products), whose bursts the warps' phases do not quite even out.
+// Measured and not kept: the quadrant step packed too (112.7 instructions, 74.8
+// and 1108 us) or on the ALU pipe (75.1 and 1130 us), and the accept test on
+// ex2.approx with expf only within rounding of the threshold (six FMA-pipe
+// instructions fewer, the branch as many more: 73.6 and 1116 us).
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+// a - b as one FMA (-b + a: the same single rounding).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, dup2(-1.f), a); }
+
+// sincos_poly of two angles: the same operations in the same order.
+__device__ __forceinline__ void sincos_poly2(float2 t, float2* s_out, float2* c_out) {
+  const float2 qt = fma2(t, dup2(kTwoOverPi), dup2(kRoundMagic));
+  const float2 qf = add2(qt, dup2(-kRoundMagic));
+  float2 r = fma2(qf, dup2(-kPio2Hi), t);
+  r = fma2(qf, dup2(-kPio2Lo), r);
+  const float2 r2 = mul2(r, r);
+  float2 ps = fma2(r2, dup2(-0.000194956359337084f), dup2(0.00833197869360447f));
+  ps = fma2(r2, ps, dup2(-0.16666650772094727f));
+  const float2 sr = fma2(mul2(r, r2), ps, r);
+  float2 pc = fma2(r2, dup2(2.4390450562350452e-05f), dup2(-0.0013886763481423259f));
+  pc = fma2(r2, pc, dup2(0.04166662320494652f));
+  pc = fma2(r2, pc, dup2(-0.5f));
+  const float2 cr = fma2(r2, pc, dup2(1.0f));
+  // the quadrant step in scalar FMAs: they run on either FMA pipe, so beside
+  // the Philox products, which hold only the heavy one
+  const float px = __fsub_rn(qf.x, 2.0f), py = __fsub_rn(qf.y, 2.0f);
+  const float ax = __fsub_rn(1.0f, fabsf(px)), ay = __fsub_rn(1.0f, fabsf(py));
+  const float bx = __fmul_rn(px, __fsub_rn(2.0f, fabsf(px)));
+  const float by = __fmul_rn(py, __fsub_rn(2.0f, fabsf(py)));
+  *s_out = make_float2(__fmaf_rn(-ax, sr.x, __fmul_rn(-bx, cr.x)),
+                       __fmaf_rn(-ay, sr.y, __fmul_rn(-by, cr.y)));
+  *c_out = make_float2(__fmaf_rn(bx, sr.x, __fmul_rn(-ax, cr.x)),
+                       __fmaf_rn(by, sr.y, __fmul_rn(-ay, cr.y)));
+}
+
+template <int MODE>
+__device__ __forceinline__ void unit_vector2(float2 t, float2* s, float2* c) {
+  if (MODE == 0) {
+    sincos_poly2(t, s, c);
+  } else {
+    unit_vector<MODE>(t.x, &s->x, &c->x);
+    unit_vector<MODE>(t.y, &s->y, &c->y);
+  }
+}
+
+// A pair's Metropolis words with the top bits of the two proposal words (x and
+// z) flipped, for metropolis_pair: (w0 >> 8) - 2^23 is then one arithmetic
+// shift.  The flip rides on the last round's keys, which are uniform.
+__device__ __forceinline__ uint4 philox_pair_words(uint32_t counter, uint32_t sweep,
+                                                   uint32_t lattice_id, const RoundKeys& rk) {
+  uint4 x = make_uint4(counter, sweep, lattice_id, 1u);
+#pragma unroll
+  for (int round = 0; round < 10; ++round) {
+    const uint32_t flip = round == 9 ? 0x80000000u : 0u;
+    uint32_t hi_a, lo_a, hi_b, lo_b;
+    mul_wide(kMulA, x.x, &hi_a, &lo_a);
+    mul_wide(kMulB, x.z, &hi_b, &lo_b);
+    x = make_uint4(hi_b ^ x.y ^ (rk.k0[round] ^ flip), lo_b, hi_a ^ x.w ^ (rk.k1[round] ^ flip),
+                   lo_a);
+  }
+  return x;
+}
+
+struct PairResult {
+  float2 th, c, s;
+  bool acc0, acc1;
+};
+
+// metropolis_step of the two sites of a Philox pair (angles t, unit vectors
+// (c0, s0), neighbour sums (Sc, Ss), words w of philox_pair_words): the same
+// decisions and results, bit for bit.  The wrap's two candidates compare as
+// unsigned bit patterns: of raw + 2 pi, raw and raw - 2 pi exactly the wanted
+// one has the smallest pattern (negative floats compare above positive ones;
+// raw is never -0, being a rounded sum with t >= 0).
+template <int MODE>
+__device__ __forceinline__ PairResult metropolis_pair(float2 t, float2 c0, float2 s0, float2 Sc,
+                                                      float2 Ss, const uint4& w, float K,
+                                                      float delta) {
+  const float2 step = make_float2((float)((int32_t)w.x >> 8), (float)((int32_t)w.z >> 8));
+  const float2 raw = fma2(dup2(delta * kR23), step, t);
+  const float2 up = add2(raw, dup2(kTwoPi)), down = add2(raw, dup2(-kTwoPi));
+  float2 tp;
+  tp.x = __uint_as_float(__vimin3_u32(__float_as_uint(up.x), __float_as_uint(raw.x),
+                                      __float_as_uint(down.x)));
+  tp.y = __uint_as_float(__vimin3_u32(__float_as_uint(up.y), __float_as_uint(raw.y),
+                                      __float_as_uint(down.y)));
+  float2 s1, c1;
+  unit_vector2<MODE>(tp, &s1, &c1);
+  const float2 X = fma2(sub2(c1, c0), Sc, mul2(sub2(s1, s0), Ss));
+  PairResult r;
+  const float2 y = mul2(X, dup2(K));
+  r.acc0 = u24(w.y) < boltzmann<MODE>(y.x);
+  r.acc1 = u24(w.w) < boltzmann<MODE>(y.y);
+  r.th = make_float2(r.acc0 ? tp.x : t.x, r.acc1 ? tp.y : t.y);
+  r.c = make_float2(r.acc0 ? c1.x : c0.x, r.acc1 ? c1.y : c0.y);
+  r.s = make_float2(r.acc0 ? s1.x : s0.x, r.acc1 ? s1.y : s0.y);
+  return r;
+}
+
+// The four neighbours (left, right, down, up) of two sites of one row, as the
+// pairs' cosines and sines, and their sums (xyd::nb_sum's order).
+struct PairNeighbours {
+  float2 lc, ls, rc, rs, dc, ds, uc, us;
+  float2 Sc, Ss;
+  __device__ __forceinline__ void sum() {
+    Sc = add2(add2(lc, rc), add2(dc, uc));
+    Ss = add2(add2(ls, rs), add2(ds, us));
+  }
+};
+
+// measure_terms of two black sites (unit vectors (cb, sb)) whose rows' red
+// sites with the same (y, k) have the unit vectors (cm, sm).
+__device__ __forceinline__ void measure_terms2(float2 cb, float2 sb, const PairNeighbours& n,
+                                               float2 cm, float2 sm, float2 v[5]) {
+  v[0] = fma2(cb, n.Sc, mul2(sb, n.Ss));
+  v[1] = fma2(sb, sub2(n.rc, n.lc), mul2(cb, sub2(n.ls, n.rs)));
+  v[2] = fma2(sb, sub2(n.uc, n.dc), mul2(cb, sub2(n.ds, n.us)));
+  v[3] = add2(cb, cm);
+  v[4] = add2(sb, sm);
+}
+
 }  // namespace xyd
 
 namespace xyd {
@@ -279,6 +414,16 @@ __device__ __forceinline__ void fx_add2(FxSums& f, const float a[5], const float
   f.s[0] += fx_bits(a[0], kFxScaleC) + fx_bits(b[0], kFxScaleC);
 #pragma unroll
   for (int i = 1; i < 5; ++i) f.s[i] += fx_bits(a[i], kFxScale) + fx_bits(b[i], kFxScale);
+  f.n += 2u;
+}
+
+// The same from packed terms (.x and .y: the two sites).
+__device__ __forceinline__ void fx_add2(FxSums& f, const float2 v[5]) {
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const float2 b = fma2(v[i], dup2(i == 0 ? kFxScaleC : kFxScale), dup2(kRoundMagic));
+    f.s[i] += __float_as_uint(b.x) + __float_as_uint(b.y);
+  }
   f.n += 2u;
 }
 
@@ -392,6 +537,17 @@ struct SweepSums {
       for (int i = 0; i < 5; ++i) {
         neumaier_add(acc[i], cmp[i], a[i]);
         neumaier_add(acc[i], cmp[i], b[i]);
+      }
+    }
+  }
+  __device__ __forceinline__ void add2(const float2 v[5]) {
+    if (RED == 0) {
+      fx_add2(fx, v);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        neumaier_add(acc[i], cmp[i], v[i].x);
+        neumaier_add(acc[i], cmp[i], v[i].y);
       }
     }
   }

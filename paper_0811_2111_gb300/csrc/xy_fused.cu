@@ -46,17 +46,18 @@ constexpr int kRedRows = kSRows - 2;         // the red plane's stage rows 1 .. 
 //         stage rows 0..35 as rows 0..35, red stage rows 1..34 as rows
 //         36..69 (the layout TMA writes; 128-byte aligned)
 //   angs  red angles of the halo columns k0-1 and k0+64, stage rows 1..34
-//   csr   red unit vectors (cos, sin) of stage rows 1..34, plane cols k0-2 ..
-//         k0+65 (column k - k0 + kCsOff: lane l's pair at 2l + 2 is 16-byte
-//         aligned; k0-1 .. k0+64 used)
+//   csr   red unit vectors of stage rows 1..34, plane cols k0-2 .. k0+65
+//         (column k - k0 + kCsOff; k0-1 .. k0+64 used), two columns per
+//         float4 as (cos, cos, sin, sin), the operands of the packed FP32
+//         instructions: lane l's pair is float4 l + 1
 //   csb   black unit vectors of stage rows 0..35, same columns
 // then the commit's per-warp partial sums and counters.  The persistent
 // kernel keeps NANG = 2 ang buffers: the next tile's rows arrive in the other.
 constexpr int kCsOff = 2;
-constexpr int kCsCols = kTileK + 4;
+constexpr int kCsPairs = kTileK / 2 + 2;
 constexpr int kRawRows = kSRows + kRedRows;
 constexpr int kRedRaw0 = kSRows - 1;        // ang row of red stage row r: kRedRaw0 + r
-typedef float2 CsRow[kCsCols];
+typedef float4 CsRow[kCsPairs];
 typedef float AngRow[kTileK];
 constexpr size_t kRawRowBytes = sizeof(AngRow);
 constexpr size_t kAngBytes = kRawRowBytes * kRawRows;
@@ -92,53 +93,56 @@ __device__ __forceinline__ int wrap_once(int v, int n) {
   return v;
 }
 
-// The four neighbour unit vectors of the two sites at columns c0, c0+1 (c0
-// even) of row i of the other colour's unit vectors `nb`, where a site at
-// column c has its same-row neighbours at c+q-1 and c+q.  The three same-row
-// columns c0+q-1 .. c0+q+1 are the aligned pair (c0, c0+1) and one edge
-// column, c0-1 (q = 0) or c0+2 (q = 1); q is a compile-time constant where the
-// row loops are unrolled (rows alternate q), so no selects are issued.  Rows
-// i-1 and i of the pair's columns come in as D and P (a warp walks its rows
-// downwards, so they are the previous row's P and U); row i+1 is loaded and
-// returned in U.
-struct PairNeighbours {
-  float Sc[2], Ss[2];
-  float2 l[2], r[2], d[2], u[2];
-};
+// The cosine and sine pairs of a float4 of unit vectors.
+__device__ __forceinline__ float2 cosines(const float4& v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 sines(const float4& v) { return make_float2(v.z, v.w); }
 
-__device__ __forceinline__ void pair_neighbours(const CsRow* nb, int i, int c0, int q,
+__device__ __forceinline__ void put_pair(float4* at, const float2& c, const float2& s) {
+  *at = make_float4(c.x, c.y, s.x, s.y);
+}
+
+// The unit vector (cos, sin) at unit-vector column c of a row.
+__device__ __forceinline__ float2 get_one(const CsRow& row, int c) {
+  const float* p = reinterpret_cast<const float*>(&row[c >> 1]) + (c & 1);
+  return make_float2(p[0], p[2]);
+}
+
+__device__ __forceinline__ void put_one(CsRow& row, int c, float cv, float sv) {
+  float* p = reinterpret_cast<float*>(&row[c >> 1]) + (c & 1);
+  p[0] = cv;
+  p[2] = sv;
+}
+
+// The four neighbour unit vectors of the two sites of pair j of row i of the
+// other colour's unit vectors `nb`, where a site at column c has its same-row
+// neighbours at c+q-1 and c+q.  The three same-row columns are the pair's own
+// and one of the pair before (q = 0) or after (q = 1); q is a compile-time
+// constant where the row loops are unrolled (rows alternate q), so no selects
+// are issued.  Rows i-1 and i of the pair's columns come in as D and P (a warp
+// walks its rows downwards, so they are the previous row's P and U); row i+1
+// is loaded and returned in U.
+__device__ __forceinline__ void pair_neighbours(const CsRow* nb, int i, int j, int q,
                                                 const float4 D, const float4 P, float4& U,
-                                                PairNeighbours& n) {
-  const float2 e = nb[i][q ? c0 + 2 : c0 - 1];
-  const float2 p0 = make_float2(P.x, P.y), p1 = make_float2(P.z, P.w);
-  U = *reinterpret_cast<const float4*>(&nb[i + 1][c0]);
+                                                xyd::PairNeighbours& n) {
+  const float4 E = nb[i][q ? j + 1 : j - 1];
+  U = nb[i + 1][j];
   if (q) {
-    n.l[0] = p0;
-    n.r[0] = p1;
-    n.l[1] = p1;
-    n.r[1] = e;
+    n.lc = cosines(P);
+    n.ls = sines(P);
+    n.rc = make_float2(P.y, E.x);
+    n.rs = make_float2(P.w, E.z);
   } else {
-    n.l[0] = e;
-    n.r[0] = p0;
-    n.l[1] = p0;
-    n.r[1] = p1;
+    n.lc = make_float2(E.y, P.x);
+    n.ls = make_float2(E.w, P.z);
+    n.rc = cosines(P);
+    n.rs = sines(P);
   }
-  n.d[0] = make_float2(D.x, D.y);
-  n.d[1] = make_float2(D.z, D.w);
-  n.u[0] = make_float2(U.x, U.y);
-  n.u[1] = make_float2(U.z, U.w);
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    n.Sc[j] = xyd::nb_sum(n.l[j].x, n.r[j].x, n.d[j].x, n.u[j].x);
-    n.Ss[j] = xyd::nb_sum(n.l[j].y, n.r[j].y, n.d[j].y, n.u[j].y);
-  }
+  n.dc = cosines(D);
+  n.ds = sines(D);
+  n.uc = cosines(U);
+  n.us = sines(U);
+  n.sum();
 }
-
-__device__ __forceinline__ float4 ld4(const float2* p) {
-  return *reinterpret_cast<const float4*>(p);
-}
-
-__device__ __forceinline__ void st4(float2* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 
 // The scalars of one fused sweep; the Philox round keys are passed separately
 // (by reference, so a kernel can leave them in its parameter space).
@@ -161,17 +165,17 @@ template <int MODE, class Args>
 __device__ __forceinline__ void red_ring_site(float th, CsRow* csr, const CsRow* csb, int r,
                                               int c, int q, uint32_t site, uint32_t x,
                                               const Args& a, const xyd::RoundKeys& rk) {
-  const float2 l = csb[r][c + q - 1], rt = csb[r][c + q];
-  const float2 d = csb[r - 1][c], u = csb[r + 1][c];
+  const float2 l = get_one(csb[r], c + q - 1), rt = get_one(csb[r], c + q);
+  const float2 d = get_one(csb[r - 1], c), u = get_one(csb[r + 1], c);
   const float Sc = xyd::nb_sum(l.x, rt.x, d.x, u.x);
   const float Ss = xyd::nb_sum(l.y, rt.y, d.y, u.y);
   const uint4 w = xyd::philox4x32_10(
       make_uint4(xyd::metropolis_counter(site, x), a.sweep, a.lattice_id, 1u), rk);
   const uint2 uw = xyd::metropolis_words(w, x);
-  const float2 own = csr[r - 1][c];
+  const float2 own = get_one(csr[r - 1], c);
   const xyd::SiteResult res =
       xyd::metropolis_step<MODE>(th, own.x, own.y, Sc, Ss, uw.x, uw.y, a.K, a.delta);
-  csr[r - 1][c] = make_float2(res.c, res.s);   // the black half reads the unit vector only
+  put_one(csr[r - 1], c, res.c, res.s);        // the black half reads the unit vector only
 }
 
 // One sweep of the tile (bx, by) of one lattice.  Args is FusedArgs (the
@@ -189,6 +193,10 @@ __device__ __forceinline__ void red_ring_site(float th, CsRow* csr, const CsRow*
 // before the barrier that ends the staging, `mid` before the barrier between
 // the red and the black half, `post` right after that barrier, `end` after the
 // tile's last store to dst and before the CTA's closing barrier.
+// AHEAD: see the row loops; on where the rows are loaded per thread (the
+// batch's tiles: 11.65 against 11.89 ms per 1000 sweeps of 41 lattices of
+// L = 256), off where TMA feeds them (one launch per sweep at L = 16384: 1106
+// against 1136 us; persistent a tie).
 struct NoHook {
   __device__ __forceinline__ void operator()() const {}
 };
@@ -209,6 +217,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
                                                  const PostHook& post = PostHook(),
                                                  const RawWait& raw_wait = RawWait()) {
   using Lay = Layout<NANG>;
+  constexpr bool AHEAD = !TMA;
   extern __shared__ __align__(128) unsigned char smem[];
   AngRow* ang = reinterpret_cast<AngRow*>(smem + (size_t)ang_sel * kAngBytes);
   float* angs = reinterpret_cast<float*>(smem + Lay::kAngsAt);     // [34][2]
@@ -290,38 +299,38 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
       const int rr = (t >> 4) + 16 * i;
       const int p = rr < kSRows ? 1 : 0;
       const int r = rr < kSRows ? rr : rr - kSRows + 1;
-      float s0, c0, s1, c1, s2, c2, s3, c3;
-      xyd::unit_vector<MODE>(v[i].x, &s0, &c0);
-      xyd::unit_vector<MODE>(v[i].y, &s1, &c1);
-      xyd::unit_vector<MODE>(v[i].z, &s2, &c2);
-      xyd::unit_vector<MODE>(v[i].w, &s3, &c3);
+      float2 s01, c01, s23, c23;
+      xyd::unit_vector2<MODE>(make_float2(v[i].x, v[i].y), &s01, &c01);
+      xyd::unit_vector2<MODE>(make_float2(v[i].z, v[i].w), &s23, &c23);
       // the group's angles go to its ang row (staged row rr) unless TMA put
       // them there; only the red rows and the black tile rows 2..33 are read
       // (uniform over each half warp)
       if (!TMA && (p == 0 || (r >= 2 && r < kSRows - 2)))
         *reinterpret_cast<float4*>(&ang[rr][4 * cg]) = v[i];
-      float2* u = p ? &csb[r][kCsOff + 4 * cg] : &csr[r - 1][kCsOff + 4 * cg];
-      st4(u, make_float4(c0, s0, c1, s1));
-      st4(u + 2, make_float4(c2, s2, c3, s3));
+      float4* u = p ? &csb[r][1 + 2 * cg] : &csr[r - 1][1 + 2 * cg];
+      put_pair(u, c01, s01);
+      put_pair(u + 1, c23, s23);
     }
     if (has_tail) {
-      float s0, c0, s1, c1;
-      xyd::unit_vector<MODE>(vt.x, &s0, &c0);
-      xyd::unit_vector<MODE>(vt.y, &s1, &c1);
+      float2 s01, c01;
+      xyd::unit_vector2<MODE>(vt, &s01, &c01);
       if (!TMA) *reinterpret_cast<float2*>(&ang[64 + (t >> 5)][2 * tail_c]) = vt;
-      st4(&csr[tail_r - 1][kCsOff + 2 * tail_c], make_float4(c0, s0, c1, s1));
+      put_pair(&csr[tail_r - 1][1 + tail_c], c01, s01);
     }
+    if (nh > 0) {
+      float2 sv, cv;
+      xyd::unit_vector2<MODE>(make_float2(vh[0], vh[1]), &sv, &cv);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      if (j < nh) {
-        float sv, cv;
-        xyd::unit_vector<MODE>(vh[j], &sv, &cv);
-        const int hcol = hside[j] ? kCsOff + kTileK : kCsOff - 1;
-        if (hp[j] == 0) {                                  // red side-ring angles
-          angs[2 * (hr[j] - 1) + hside[j]] = vh[j];
-          csr[hr[j] - 1][hcol] = make_float2(cv, sv);
-        } else {
-          csb[hr[j]][hcol] = make_float2(cv, sv);
+      for (int j = 0; j < 2; ++j) {
+        if (j < nh) {
+          const float cj = j ? cv.y : cv.x, sj = j ? sv.y : sv.x;
+          const int hcol = hside[j] ? kCsOff + kTileK : kCsOff - 1;
+          if (hp[j] == 0) {                                  // red side-ring angles
+            angs[2 * (hr[j] - 1) + hside[j]] = vh[j];
+            put_one(csr[hr[j] - 1], hcol, cj, sj);
+          } else {
+            put_one(csb[hr[j]], hcol, cj, sj);
+          }
         }
       }
     }
@@ -331,36 +340,43 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
 
   const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
   const uint32_t uL = (uint32_t)L;
-  const int c0 = 2 * lane + kCsOff;                        // unit-vector column of the lane's pair
+  const int pj = lane + 1;                                 // the lane's pair in a row
   const int kp = k0 + 2 * lane;                            // plane column of the pair
   unsigned int n_acc = 0;
 
   // ---- red half: the tile (counted, written to dst) ----
-  float4 nbD = ld4(&csb[warp * 4 + 1][c0]);
-  float4 nbP = ld4(&csb[warp * 4 + 2][c0]);
+  float4 nbD = csb[warp * 4 + 1][pj];
+  float4 nbP = csb[warp * 4 + 2][pj];
+  // AHEAD: each row's Philox words are drawn one row ahead, beside the row
+  // before it (plane row c of the next row: q = (y + c) & 1)
+  uint4 w_next = make_uint4(0u, 0u, 0u, 0u);
+  auto words = [&](int rr, int c) {
+    const uint32_t y = (uint32_t)(y0 + warp * 4 + rr);
+    // sites x and x + 2 of the pair (kp even, so x & 2 == 0): one block
+    return xyd::philox_pair_words(y * uL + 2u * (uint32_t)kp + ((y + (uint32_t)c) & 1u), a.sweep,
+                                  a.lattice_id, rk);
+  };
+  if (AHEAD) w_next = words(0, 0);
 #pragma unroll
   for (int rr = 0; rr < 4; ++rr) {
     const int ty = warp * 4 + rr;
     const int y = y0 + ty;
     const int r = ty + 2;
     const int q = y & 1;                                   // red: x = 2k + (y & 1)
-    PairNeighbours n;
+    xyd::PairNeighbours n;
     float4 nbU;
-    pair_neighbours(csb, r, c0, q, nbD, nbP, nbU, n);
+    pair_neighbours(csb, r, pj, q, nbD, nbP, nbU, n);
     nbD = nbP;
     nbP = nbU;
-    const uint32_t site0 = (uint32_t)y * uL + 2u * (uint32_t)kp + (uint32_t)q;
-    // sites x and x + 2 of the pair (kp even, so x & 2 == 0): one block
-    const uint4 w = xyd::philox4x32_10(make_uint4(site0, a.sweep, a.lattice_id, 1u), rk);
+    const uint4 w = AHEAD ? w_next : words(rr, 0);
+    if (AHEAD) w_next = rr < 3 ? words(rr + 1, 0) : words(0, 1);
     const float2 t = *reinterpret_cast<const float2*>(&ang[kRedRaw0 + r][2 * lane]);
-    const float4 o = ld4(&csr[r - 1][c0]);
-    const xyd::SiteResult r0 =
-        xyd::metropolis_step<MODE>(t.x, o.x, o.y, n.Sc[0], n.Ss[0], w.x, w.y, a.K, a.delta);
-    const xyd::SiteResult r1 =
-        xyd::metropolis_step<MODE>(t.y, o.z, o.w, n.Sc[1], n.Ss[1], w.z, w.w, a.K, a.delta);
-    n_acc += (r0.accept ? 1u : 0u) + (r1.accept ? 1u : 0u);
-    st4(&csr[r - 1][c0], make_float4(r0.c, r0.s, r1.c, r1.s));
-    *reinterpret_cast<float2*>(a.dst + (size_t)y * W + kp) = make_float2(r0.th, r1.th);
+    const float4 o = csr[r - 1][pj];
+    const xyd::PairResult p =
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
+    n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
+    put_pair(&csr[r - 1][pj], p.c, p.s);
+    *reinterpret_cast<float2*>(a.dst + (size_t)y * W + kp) = p.th;
   }
   // ---- red half: the ring at distance one (recomputed, not counted) ----
   // The ring rows above and below the tile are 32 pairs each (sites x and
@@ -373,18 +389,16 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const int y = wrap_once(y0 + ty, L);
     const int r = ty + 2;
     const int q = y & 1;
-    PairNeighbours n;
+    xyd::PairNeighbours n;
     float4 U;
-    pair_neighbours(csb, r, c0, q, ld4(&csb[r - 1][c0]), ld4(&csb[r][c0]), U, n);
+    pair_neighbours(csb, r, pj, q, csb[r - 1][pj], csb[r][pj], U, n);
     const uint32_t site0 = (uint32_t)y * uL + 2u * (uint32_t)kp + (uint32_t)q;
-    const uint4 w = xyd::philox4x32_10(make_uint4(site0, a.sweep, a.lattice_id, 1u), rk);
+    const uint4 w = xyd::philox_pair_words(site0, a.sweep, a.lattice_id, rk);
     const float2 t = *reinterpret_cast<const float2*>(&ang[kRedRaw0 + r][2 * lane]);
-    const float4 o = ld4(&csr[r - 1][c0]);
-    const xyd::SiteResult r0 =
-        xyd::metropolis_step<MODE>(t.x, o.x, o.y, n.Sc[0], n.Ss[0], w.x, w.y, a.K, a.delta);
-    const xyd::SiteResult r1 =
-        xyd::metropolis_step<MODE>(t.y, o.z, o.w, n.Sc[1], n.Ss[1], w.z, w.w, a.K, a.delta);
-    st4(&csr[r - 1][c0], make_float4(r0.c, r0.s, r1.c, r1.s));
+    const float4 o = csr[r - 1][pj];
+    const xyd::PairResult p =
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
+    put_pair(&csr[r - 1][pj], p.c, p.s);
   } else if (warp == 2) {
     const int ty = lane;
     const int tk = ((y0 + ty) & 1) ? -1 : kTileK;          // left ring on odd rows, right on even
@@ -403,39 +417,33 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
   xyd::SweepSums<RED> sums;
   sums.init();
   float* dst_blk = a.dst + plane;
-  nbD = ld4(&csr[warp * 4][c0]);                           // red stage rows r - 1, r
-  nbP = ld4(&csr[warp * 4 + 1][c0]);
+  nbD = csr[warp * 4][pj];                                 // red stage rows r - 1, r
+  nbP = csr[warp * 4 + 1][pj];
 #pragma unroll
   for (int rr = 0; rr < 4; ++rr) {
     const int ty = warp * 4 + rr;
     const int y = y0 + ty;
     const int r = ty + 2;
     const int q = (y + 1) & 1;                             // black: x = 2k + ((y + 1) & 1)
-    PairNeighbours n;
+    xyd::PairNeighbours n;
     float4 nbU;
-    pair_neighbours(csr, r - 1, c0, q, nbD, nbP, nbU, n);
+    pair_neighbours(csr, r - 1, pj, q, nbD, nbP, nbU, n);
     const float4 m = nbP;                                  // the red pair of the same row
     nbD = nbP;
     nbP = nbU;
-    const uint32_t site0 = (uint32_t)y * uL + 2u * (uint32_t)kp + (uint32_t)q;
-    // sites x and x + 2 of the pair (kp even, so x & 2 == 0): one block
-    const uint4 w = xyd::philox4x32_10(make_uint4(site0, a.sweep, a.lattice_id, 1u), rk);
+    const uint4 w = AHEAD ? w_next : words(rr, 1);
+    if (AHEAD && rr < 3) w_next = words(rr + 1, 1);
     const float2 t = *reinterpret_cast<const float2*>(&ang[r][2 * lane]);
-    const float4 o = ld4(&csb[r][c0]);
-    const xyd::SiteResult r0 =
-        xyd::metropolis_step<MODE>(t.x, o.x, o.y, n.Sc[0], n.Ss[0], w.x, w.y, a.K, a.delta);
-    const xyd::SiteResult r1 =
-        xyd::metropolis_step<MODE>(t.y, o.z, o.w, n.Sc[1], n.Ss[1], w.z, w.w, a.K, a.delta);
-    n_acc += (r0.accept ? 1u : 0u) + (r1.accept ? 1u : 0u);
-    *reinterpret_cast<float2*>(dst_blk + (size_t)y * W + kp) = make_float2(r0.th, r1.th);
+    const float4 o = csb[r][pj];
+    const xyd::PairResult p =
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
+    n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
+    *reinterpret_cast<float2*>(dst_blk + (size_t)y * W + kp) = p.th;
 
     // red sites with the same (y, k): their spins enter M once each
-    float v0[5], v1[5];
-    xyd::measure_terms(r0.c, r0.s, n.l[0].x, n.l[0].y, n.r[0].x, n.r[0].y, n.d[0].x, n.d[0].y,
-                       n.u[0].x, n.u[0].y, n.Sc[0], n.Ss[0], m.x, m.y, v0);
-    xyd::measure_terms(r1.c, r1.s, n.l[1].x, n.l[1].y, n.r[1].x, n.r[1].y, n.d[1].x, n.d[1].y,
-                       n.u[1].x, n.u[1].y, n.Sc[1], n.Ss[1], m.z, m.w, v1);
-    sums.add2(v0, v1);
+    float2 v[5];
+    xyd::measure_terms2(p.c, p.s, n, cosines(m), sines(m), v);
+    sums.add2(v);
   }
 
   end();
