@@ -75,6 +75,7 @@ struct xy_ctx {
   bool owns_theta;
   float* d_pong;           // second buffer of the fused kernel (library-owned)
   bool fused;              // sweeps use the fused kernel
+  bool resident;           // XY_ALGO_AUTO: the lattice fits on the chip (xy_resident.cu)
   bool persistent;         // ... all sweeps of an xy_sweep call in one cooperative launch
   bool auto_persistent;    // chosen by XY_ALGO_AUTO: per-sweep launches if it does not fit
   unsigned int* d_tiles;   // the persistent launch's per-tile sweep counters
@@ -286,6 +287,20 @@ cudaError_t timed_persistent(xy_ctx* c, const xyk::FusedPersistArgs& a) {
   return e;
 }
 
+// At most this many sweeps in one resident launch (a fraction of a second).
+constexpr int64_t kResidentSweeps = 1 << 16;
+
+cudaError_t timed_resident(xy_ctx* c, const xyk::ResidentArgs& a) {
+  if (c->timing_every <= 0)
+    return xyk::launch_resident(c->p.sincos_mode, a, c->stream);
+  cudaEvent_t e0, e1;
+  cudaError_t e = next_events(c, 0, &e0, &e1);
+  if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
+  if (e == cudaSuccess) e = xyk::launch_resident(c->p.sincos_mode, a, c->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
+  return e;
+}
+
 void release(xy_ctx* c) {
   for (int k = 0; k < 2; ++k) {
     for (cudaEvent_t e : c->ev[k]) cudaEventDestroy(e);
@@ -391,6 +406,13 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
     if (e == cudaSuccess && !xyk::encode_fused_maps(&c->maps, c->d_theta, c->d_pong, p->L))
       e = cudaErrorNotSupported;
   }
+  if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->ctas_per_sm == 0 &&
+      p->reduce_mode == XY_REDUCE_EXACT && xyk::resident_supported(p->L)) {
+    if (xyk::prepare_resident(p->sincos_mode, p->L, &c->resident) != cudaSuccess) {
+      (void)cudaGetLastError();       // the tile kernels take the lattice
+      c->resident = false;
+    }
+  }
   if (e == cudaSuccess && c->persistent)
     e = xyk::dev_malloc(&c->d_tiles, sizeof(unsigned int) * ((size_t)xyk::fused_tiles(p->L) + 1));
   if (e != cudaSuccess) {
@@ -480,7 +502,27 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
   st = grow_records(c, c->rec_count + n);
   if (st != XY_OK) return st;
   const xyd::RoundKeys rk = xyd::make_round_keys(c->p.seed);
-  if (c->persistent) {
+  // the two half-sweep kernels are timed one by one, so with timing on a
+  // lattice reported as XY_ALGO_TWO_PASS runs them
+  if (c->resident && (c->persistent || c->timing_every <= 0)) {
+    xyk::ResidentArgs a;
+    a.theta = c->d_theta;
+    a.L = c->p.L;
+    a.K = (float)(c->p.beta * c->p.J);
+    a.delta = (float)c->p.delta;
+    a.rk = rk;
+    a.lattice_id = c->p.lattice_id;
+    a.beta = c->p.beta;
+    for (int64_t done = 0; done < n;) {
+      const int64_t m = std::min<int64_t>(n - done, kResidentSweeps);
+      a.sweep0 = (uint32_t)(c->next_sweep + (uint64_t)done);
+      a.n_sweeps = (int)m;
+      a.rec = c->d_rec + c->rec_count + done;
+      const cudaError_t e = timed_resident(c, a);
+      if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: resident launch");
+      done += m;
+    }
+  } else if (c->persistent) {
     xyk::FusedPersistArgs a;
     a.buf[0] = c->d_theta;
     a.buf[1] = c->d_pong;

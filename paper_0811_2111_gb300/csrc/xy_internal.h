@@ -163,6 +163,28 @@ int fused_persistent_max_sweeps(int L);
 cudaError_t launch_fused_persistent(int sincos_mode, int reduce_mode, const FusedPersistArgs& a,
                                     cudaStream_t stream);
 
+// All sweeps of a call of a small lattice in one cluster launch, in place, the
+// lattice held on the chip, exact sums (xy_resident.cu).
+struct ResidentArgs {
+  float* theta;          // [2][L][W]: the state, read and rewritten
+  int L;
+  float K;
+  float delta;
+  xyd::RoundKeys rk;
+  uint32_t lattice_id;
+  uint32_t sweep0;       // Philox sweep word of the first sweep
+  int n_sweeps;
+  xy_record* rec;        // records of the n sweeps, zeroed
+  double beta;
+  int ctas;              // set by the launcher
+};
+constexpr size_t kResidentSmem = 96 * 1024;   // dynamic shared memory of a strip, at most
+// Whether side L is held resident, and (prepare; outside any capture) whether
+// the device can run its cluster.
+bool resident_supported(int L);
+cudaError_t prepare_resident(int sincos_mode, int L, bool* fits);
+cudaError_t launch_resident(int sincos_mode, const ResidentArgs& a, cudaStream_t stream);
+
 // All sweeps of a call of the four-replica fused sweep in one cooperative
 // launch (tiles ordered by per-tile sweep counters, bounded waits).
 struct QuadPersistArgs {

@@ -1,0 +1,371 @@
+// xy_resident.cu -- all sweeps of a call of a small lattice in one launch, the
+// lattice never leaving the chip: one thread-block cluster holds it, a strip of
+// full rows per CTA.
+//
+// A sweep of a small lattice is two dependent half-sweeps of a few hundred
+// cycles; with one launch per half-sweep (L = 32: 22 us per sweep) or one tile
+// of 32 x 128 sites after the other through global memory (L = 128: 4.9 us) it
+// is all latency.  Here every thread owns the same pairs of sites (plane
+// columns 2m, 2m + 1 of a row: one Philox block) of both colours for the whole
+// launch: their angles and unit vectors stay in its registers, and shared
+// memory holds only what neighbours read, the unit vectors of both colours as
+// (cos, cos, sin, sin) per pair, with the strip's two halo rows and the two
+// halo columns as copies.  A half-sweep reads the other colour's unit vectors,
+// updates its pairs (xyd::metropolis_pair, so every decision is bit for bit
+// that of the other kernels), and stores the new unit vectors to its own
+// strip, to the halo columns, and, from a strip's first and last row, to the
+// neighbouring CTAs' halo rows through distributed shared memory; one cluster
+// barrier (release / acquire) ends it.  The next half-sweep's Philox words
+// depend on no state and are drawn between the barrier's arrive and wait.
+//
+// Why one barrier per half-sweep is enough: a half-sweep of colour c reads
+// unit vectors of colour 1 - c only (its own pairs are in registers; the red
+// spins of the magnetisation are read in the black half) and writes those of
+// colour c only, here and in the neighbours' halo rows.
+//
+// Exact sums only: they do not depend on who adds what, while the compensated
+// sums round by thread and warp and keep the kernels that define them.
+// Any even side whose strips fit (L odd multiples of 2 included): rows have
+// (W + 1) / 2 pairs, and where W = L / 2 is odd the last pair's second column
+// is column W, the halo copy of column 0; its lane's results are dropped.
+//
+// What bounds it is the latency of a half-sweep's dependent chain (about a
+// thousand cycles with its barrier), at 256 the SM's FMA pipes as well;
+// resident_ctas has the times.
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "xy_device.cuh"
+#include "xy_internal.h"
+
+namespace cg = cooperative_groups;
+
+namespace xyk {
+
+namespace {
+
+constexpr int kRThreads = 512;               // at most; the launch takes what the pairs need
+constexpr int kRWarps = kRThreads / 32;
+constexpr int kRMaxPairs = 2;                // pairs per thread and colour
+
+__host__ __device__ inline int strip_rows(int L, int C, int rank) {
+  return L / C + (rank < L % C ? 1 : 0);
+}
+__host__ __device__ inline int strip_first(int L, int C, int rank) {
+  return rank * (L / C) + (rank < L % C ? rank : L % C);
+}
+
+// Unit vectors of one colour: (rows + 2) x (pairs + 2) float4, row r + 1 the
+// strip's row r, float4 m + 1 the pair m.
+__host__ __device__ inline int plane_vec4(int max_rows, int W) {
+  return (max_rows + 2) * ((W + 1) / 2 + 2);
+}
+
+// NP: pairs of each colour a thread owns, at most.  (Blocks of 1024 threads leave
+// 64 registers a thread and spill the state: L = 256 4.6 against 3.5 us per
+// sweep with 512 threads of two pairs.)
+template <int MODE, int NP>
+__global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ uint32_t s_part[kRWarps][5];
+  __shared__ uint32_t s_cnt[kRWarps];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = a.ctas, rank = (int)cluster.block_rank();
+  const int L = a.L, W = L / 2, Wp = (W + 1) / 2, Wq = Wp + 2;
+  const int max_rows = strip_rows(L, C, 0);
+  const int rows = strip_rows(L, C, rank), y0 = strip_first(L, C, rank);
+  const int npairs = rows * Wp;
+  const int nthreads = blockDim.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = nthreads >> 5;
+  const size_t plane = (size_t)L * (size_t)W;
+  float4* cs = reinterpret_cast<float4*>(smem);            // [2][max_rows + 2][Wq]
+  const int pvec = plane_vec4(max_rows, W);
+  // the neighbouring strips: their halo row next to this strip's first / last row
+  const int up_rank = rank + 1 == C ? 0 : rank + 1, dn_rank = rank == 0 ? C - 1 : rank - 1;
+  float4* up_halo = cluster.map_shared_rank(cs, up_rank);                      // row 0
+  float4* dn_halo = cluster.map_shared_rank(cs, dn_rank) +
+                    (strip_rows(L, C, dn_rank) + 1) * Wq;                      // row rows + 1
+
+  // this thread's pairs
+  int at[NP];            // float4 of the pair in a plane
+  int yy[NP], kk[NP];    // row and first plane column
+  bool on[NP], two[NP];  // owned; its second column exists
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int i = threadIdx.x + p * nthreads;
+    on[p] = i < npairs;
+    const int r = on[p] ? i / Wp : 0, m = on[p] ? i - r * Wp : 0;
+    at[p] = (r + 1) * Wq + m + 1;
+    yy[p] = y0 + r;
+    kk[p] = 2 * m;
+    two[p] = 2 * m + 1 < W;
+  }
+  // stores of a pair's unit vectors of colour c: the strip, its halo columns
+  // (column 0's copy behind the last column, the last column's before column
+  // 0) and the neighbours' halo rows
+  auto put = [&](int p, int c, float2 cv, float2 sv) {
+    float4* own = cs + c * pvec;
+    const float4 v = make_float4(cv.x, cv.y, sv.x, sv.y);
+    const int r = yy[p] - y0;
+    if (two[p]) {
+      own[at[p]] = v;
+    } else {                               // the halo copy in the second column stays
+      float* f = reinterpret_cast<float*>(&own[at[p]]);
+      f[0] = v.x;
+      f[2] = v.z;
+    }
+    float* row = reinterpret_cast<float*>(&own[(r + 1) * Wq]);
+    if (kk[p] == 0) {                      // column 0 -> column W
+      float* f = row + 4 * ((W + 2) >> 1) + (W & 1);
+      f[0] = v.x;
+      f[2] = v.z;
+    }
+    if (kk[p] + 2 >= W) {                  // column W - 1 -> column -1
+      row[1] = two[p] ? v.y : v.x;
+      row[3] = two[p] ? v.w : v.z;
+    }
+    const int m = (kk[p] >> 1) + 1;
+    if (r == 0) dn_halo[c * pvec + m] = v;
+    if (r == rows - 1) up_halo[c * pvec + m] = v;
+  };
+
+  float2 th[2][NP], cv[2][NP], sv[2][NP];
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      th[c][p] = make_float2(0.f, 0.f);
+      if (on[p]) {
+        const float* g = a.theta + c * plane + (size_t)yy[p] * W + kk[p];
+        th[c][p].x = g[0];
+        if (two[p]) th[c][p].y = g[1];
+      }
+      xyd::unit_vector2<MODE>(th[c][p], &sv[c][p], &cv[c][p]);
+    }
+  auto words = [&](int p, int c, uint32_t sweep) {
+    const uint32_t y = (uint32_t)yy[p];
+    return xyd::philox_pair_words(
+        y * (uint32_t)L + 2u * (uint32_t)kk[p] + ((y + (uint32_t)c) & 1u), sweep, a.lattice_id,
+        a.rk);
+  };
+  uint4 w[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) w[p] = words(p, 0, a.sweep0);
+  cluster.sync();                          // every CTA has started: its memory may be written
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int p = 0; p < NP; ++p)
+      if (on[p]) put(p, c, cv[c][p], sv[c][p]);
+  cluster.sync();
+
+  // The previous sweep's sums, left in s_part / s_cnt before the barrier: one
+  // warp per sum adds the warps' values (16-bit halves, one lane per warp) and
+  // issues the record's atomic.
+  auto commit = [&](xy_record* rec) {
+    for (int task = warp; task < 6; task += nwarps) {
+      const bool has = lane < nwarps;
+      if (task == 5) {
+        const uint32_t n = has ? s_cnt[lane] : 0u;
+        const uint32_t total = __reduce_add_sync(0xffffffffu, n & 0x7fffffffu);
+        const bool bad = __any_sync(0xffffffffu, (n & 0x80000000u) != 0u);
+        if (lane == 0) {
+          atomicAdd(reinterpret_cast<unsigned long long*>(&rec->accepted),
+                    (unsigned long long)total);
+          if (bad) atomicOr(reinterpret_cast<unsigned long long*>(&rec->flags), 1ull);
+          if (rank == 0) rec->beta = a.beta;
+        }
+      } else {
+        const int32_t v = has ? (int32_t)s_part[lane][task] : 0;
+        const uint32_t lo = __reduce_add_sync(0xffffffffu, (uint32_t)v & 0xffffu);
+        const int32_t hi = (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(v >> 16));
+        if (lane == 0)
+          atomicAdd(reinterpret_cast<unsigned long long*>(&rec->sum[task]),
+                    (unsigned long long)((long long)hi * 65536ll + (long long)lo)
+                        << (XY_FX_SHIFT - xyd::fx_term_shift(task)));
+      }
+    }
+  };
+
+  for (int s = 0; s < a.n_sweeps; ++s) {
+    const uint32_t sweep = a.sweep0 + (uint32_t)s;
+    unsigned int n_acc = 0;
+    xyd::SweepSums<0> sums;                // at most 2 NP black sites per thread
+    sums.init();
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float4* nb = cs + (1 - c) * pvec;
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        if (!on[p]) continue;
+        const int q = (yy[p] + c) & 1;     // x = 2k + q
+        const float4 P = nb[at[p]], D = nb[at[p] - Wq], U = nb[at[p] + Wq];
+        const float4 E = nb[q ? at[p] + 1 : at[p] - 1];
+        xyd::PairNeighbours n;
+        n.lc = q ? make_float2(P.x, P.y) : make_float2(E.y, P.x);
+        n.ls = q ? make_float2(P.z, P.w) : make_float2(E.w, P.z);
+        n.rc = q ? make_float2(P.y, E.x) : make_float2(P.x, P.y);
+        n.rs = q ? make_float2(P.w, E.z) : make_float2(P.z, P.w);
+        n.dc = make_float2(D.x, D.y);
+        n.ds = make_float2(D.z, D.w);
+        n.uc = make_float2(U.x, U.y);
+        n.us = make_float2(U.z, U.w);
+        n.sum();
+        const xyd::PairResult r = xyd::metropolis_pair<MODE>(th[c][p], cv[c][p], sv[c][p], n.Sc,
+                                                             n.Ss, w[p], a.K, a.delta);
+        th[c][p] = r.th;
+        cv[c][p] = r.c;
+        sv[c][p] = r.s;
+        put(p, c, r.c, r.s);
+        n_acc += (r.acc0 ? 1u : 0u) + (r.acc1 && two[p] ? 1u : 0u);
+        if (c == 1) {
+          // red sites with the same (y, k): their spins enter M once each
+          float2 v[5];
+          xyd::measure_terms2(r.c, r.s, n, make_float2(P.x, P.y), make_float2(P.z, P.w), v);
+          if (two[p]) {
+            sums.add2(v);
+          } else {
+            const float v0[5] = {v[0].x, v[1].x, v[2].x, v[3].x, v[4].x};
+            sums.add(v0);
+          }
+        }
+      }
+      if (c == 0 && s > 0) commit(a.rec + (s - 1));
+      if (c == 1) {
+        const unsigned int acc = __reduce_add_sync(0xffffffffu, n_acc);
+        const bool bad = __any_sync(0xffffffffu, xyd::fx_nonfinite(sums.fx));
+        uint32_t t[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+          t[i] = __reduce_add_sync(0xffffffffu, (uint32_t)xyd::fx_value(sums.fx, i));
+        if (lane == 0) {
+          s_cnt[warp] = acc | (bad ? 0x80000000u : 0u);
+#pragma unroll
+          for (int i = 0; i < 5; ++i) s_part[warp][i] = t[i];
+        }
+      }
+      __syncwarp();
+      if (C > 1) cluster.barrier_arrive();
+      // drawn for a sweep past the last too (never used)
+#pragma unroll
+      for (int p = 0; p < NP; ++p) w[p] = words(p, 1 - c, sweep + (c == 1 ? 1u : 0u));
+      if (C > 1) {
+        cluster.barrier_wait();
+      } else {
+        __syncthreads();
+      }
+    }
+  }
+  commit(a.rec + (a.n_sweeps - 1));
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int p = 0; p < NP; ++p)
+      if (on[p]) {
+        float* g = a.theta + c * plane + (size_t)yy[p] * W + kk[p];
+        g[0] = th[c][p].x;
+        if (two[p]) g[1] = th[c][p].y;
+      }
+}
+
+// CTAs of the cluster for side L (0: not resident).  One CTA while a thread
+// per pair keeps its barrier cheap, then enough of them that a strip is a
+// pair or two per thread; the cluster barrier costs about 0.2 us a half-sweep,
+// whatever the cluster's size.  Measured, us per sweep by cluster size:
+//   L = 32   1: 1.00   4: 1.49   8: 1.82  16: 1.84   (two launches a sweep: 22)
+//   L = 48   1: 2.16   4: 1.56   8: 1.39  16: 1.51
+//   L = 64   1: 2.75   4: 1.49   8: 1.45  16: 1.50
+//   L = 80             4: 1.93   8: 1.53  16: 1.45
+//   L = 128            4: 3.50   8: 1.98  16: 1.52   (persistent tiles: 4.9)
+//   L = 256                      8: 6.55  16: 3.55   (persistent tiles: 5.3)
+// Above 256 a thread would own more pairs than its registers hold (L = 320
+// with four each 5.9) and the tiles are as fast.
+int resident_ctas(int L) {
+  if (L < 4 || L > 256) return 0;
+  return L <= 32 ? 1 : L <= 64 ? 8 : 16;
+}
+
+struct Plan {
+  int ctas, np, threads;
+  size_t smem;
+};
+
+Plan plan_of(int L) {
+  Plan p = {};
+  p.ctas = resident_ctas(L);
+  if (p.ctas == 0 || (L & 1)) return Plan{};
+  const int W = L / 2, rows = strip_rows(L, p.ctas, 0);
+  const int pairs = rows * ((W + 1) / 2);
+  p.np = (pairs + kRThreads - 1) / kRThreads;
+  if (p.np > kRMaxPairs) return Plan{};
+  p.threads = ((pairs + p.np - 1) / p.np + 31) / 32 * 32;
+  p.smem = sizeof(float4) * 2 * (size_t)plane_vec4(rows, W);
+  return p;
+}
+
+cudaLaunchConfig_t config_of(const Plan& p, cudaStream_t stream, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.ctas);
+  cfg.blockDim = dim3(p.threads);
+  cfg.dynamicSmemBytes = p.smem;
+  cfg.stream = stream;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = p.ctas;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// f(kernel) for the instantiation of a plan.
+template <class F>
+cudaError_t with_kernel(int mode, const Plan& p, const F& f) {
+  switch (mode) {
+    case 0: return p.np == 1 ? f(k_sweep_resident<0, 1>) : f(k_sweep_resident<0, 2>);
+    case 1: return p.np == 1 ? f(k_sweep_resident<1, 1>) : f(k_sweep_resident<1, 2>);
+    default: return p.np == 1 ? f(k_sweep_resident<2, 1>) : f(k_sweep_resident<2, 2>);
+  }
+}
+
+}  // namespace
+
+bool resident_supported(int L) {
+  const Plan p = plan_of(L);
+  return p.ctas > 0 && p.smem <= kResidentSmem;
+}
+
+cudaError_t prepare_resident(int sincos_mode, int L, bool* fits) {
+  *fits = false;
+  const Plan p = plan_of(L);
+  if (p.ctas == 0 || p.smem > kResidentSmem) return cudaErrorInvalidValue;
+  return with_kernel(sincos_mode, p, [&](auto* fn) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kResidentSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = config_of(p, nullptr, &attr);
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
+    *fits = e == cudaSuccess && n >= 1;
+    return e;
+  });
+}
+
+cudaError_t launch_resident(int sincos_mode, const ResidentArgs& args,
+                            cudaStream_t stream) {
+  const Plan p = plan_of(args.L);
+  if (p.ctas == 0 || p.smem > kResidentSmem || args.n_sweeps < 1) return cudaErrorInvalidValue;
+  ResidentArgs a = args;
+  a.ctas = p.ctas;
+  return with_kernel(sincos_mode, p, [&](auto* fn) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = config_of(p, stream, &attr);
+    return cudaLaunchKernelEx(&cfg, fn, a);
+  });
+}
+
+}  // namespace xyk
