@@ -76,6 +76,7 @@ struct xy_ctx {
   float* d_pong;           // second buffer of the fused kernel (library-owned)
   bool fused;              // sweeps use the fused kernel
   bool resident;           // XY_ALGO_AUTO: the lattice fits on the chip (xy_resident.cu)
+  bool ragged;             // XY_ALGO_AUTO: persistent sweeps on overlapping tiles
   bool persistent;         // ... all sweeps of an xy_sweep call in one cooperative launch
   bool auto_persistent;    // chosen by XY_ALGO_AUTO: per-sweep launches if it does not fit
   unsigned int* d_tiles;   // the persistent launch's per-tile sweep counters
@@ -312,8 +313,8 @@ void release(xy_ctx* c) {
   if (c->d_pong) cudaFree(c->d_pong);
   if (c->d_scratch) cudaFree(c->d_scratch);
   if (c->d_flag) cudaFree(c->d_flag);
-  if (c->d_tiles) cudaFree(c->d_tiles);
-  if (c->d_wait) cudaFree(c->d_wait);
+  if (c->d_tiles && !c->ragged) cudaFree(c->d_tiles);
+  if (c->d_wait && !c->ragged) cudaFree(c->d_wait);
   c->d_tiles = nullptr;
   c->d_wait = nullptr;
   c->d_theta = nullptr;
@@ -411,6 +412,22 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
     if (xyk::prepare_resident(p->sincos_mode, p->L, &c->resident) != cudaSuccess) {
       (void)cudaGetLastError();       // the tile kernels take the lattice
       c->resident = false;
+    }
+  }
+  if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->ctas_per_sm == 0 &&
+      p->reduce_mode == XY_REDUCE_EXACT && !c->resident && xyk::ragged_supported(p->L)) {
+    // the second buffer, behind it the counters and the wait word: optional
+    // (without them the two-pass kernels run in place) and one allocation
+    const size_t words = (size_t)xyk::fused_tiles(p->L) + 2;
+    cudaError_t r = xyk::dev_malloc(&c->d_pong, N * sizeof(float) + words * sizeof(unsigned int));
+    if (r == cudaSuccess) {
+      c->ragged = true;
+      c->d_tiles = reinterpret_cast<unsigned int*>(c->d_pong + N);
+      c->d_wait = c->d_tiles + words - 1;
+      e = cudaMemsetAsync(c->d_wait, 0, sizeof(unsigned int), c->stream);
+    } else {
+      (void)cudaGetLastError();
+      c->d_pong = nullptr;
     }
   }
   if (e == cudaSuccess && c->persistent)
@@ -522,7 +539,7 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
       if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: resident launch");
       done += m;
     }
-  } else if (c->persistent) {
+  } else if (c->persistent || (c->ragged && c->timing_every <= 0)) {
     xyk::FusedPersistArgs a;
     a.buf[0] = c->d_theta;
     a.buf[1] = c->d_pong;
@@ -550,6 +567,30 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
       a.n_sweeps = (int)m;
       a.rec = c->d_rec + c->rec_count + done;
       cudaError_t e = timed_persistent(c, a);
+      if (e == cudaErrorCooperativeLaunchTooLarge && c->ragged) {
+        // the grid does not fit beside other work: the same sweeps in place by
+        // the two-pass kernels (bit-identical)
+        (void)cudaGetLastError();
+        xyk::HalfSweepArgs h;
+        h.theta = a.buf[0];
+        h.L = a.L;
+        h.W = a.W;
+        h.K = a.K;
+        h.delta = a.delta;
+        h.rk = a.rk;
+        h.lattice_id = a.lattice_id;
+        h.beta = a.beta;
+        e = cudaSuccess;
+        for (int64_t i = 0; i < m && e == cudaSuccess; ++i) {
+          h.sweep = a.sweep0 + (uint32_t)i;
+          h.rec = a.rec + i;
+          e = timed_half_sweep(c, 0, h);
+          if (e == cudaSuccess) e = timed_half_sweep(c, 1, h);
+        }
+        if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: launch");
+        done += m;
+        continue;
+      }
       if (e == cudaErrorCooperativeLaunchTooLarge && c->auto_persistent) {
         // the grid does not fit beside other work on the device: the same
         // sweeps as one fused launch each (bit-identical)

@@ -19,7 +19,8 @@
 // per sweep (8 B per update instead of 12 B) and each site's unit vector is
 // computed once per sweep instead of once per half-sweep.
 //
-// Requires W = L/2 to be a multiple of 64 and L a multiple of 32 (L % 128 == 0).
+// Requires W = L/2 to be a multiple of 64 and L a multiple of 32 (L % 128 == 0);
+// the persistent sweep takes any other even L >= 130 on overlapping tiles.
 // Decisions are bit-identical to the two-pass kernels: both call the same
 // xyd::unit_vector / xyd::nb_sum / xyd::metropolis_step with pinned rounding.
 #include <cuda_runtime.h>
@@ -84,8 +85,11 @@ static_assert(4 * (kSmemBytes + 1024 + 128) <= 228 * 1024,
 static_assert(3 * (kPersistSmemBytes + 1024 + 512) <= 228 * 1024,
               "three persistent tiles (and their static shared memory) must fit one SM");
 
-// Tiles of one sweep of side L (L % 128 == 0).
-inline int fused_tiles_of(int L) { return (L / 2 / kTileK) * (L / kTileRows); }
+// Tiles of one sweep of side L (the last row and column of tiles overlap their
+// neighbours unless L % 128 == 0).
+__host__ __device__ inline int tile_cols(int W) { return (W + kTileK - 1) / kTileK; }
+__host__ __device__ inline int tile_rows(int L) { return (L + kTileRows - 1) / kTileRows; }
+inline int fused_tiles_of(int L) { return tile_cols(L / 2) * tile_rows(L); }
 
 __device__ __forceinline__ int wrap_once(int v, int n) {
   v += (v < 0) ? n : 0;
@@ -206,8 +210,16 @@ __device__ __forceinline__ unsigned char* smem_base() {
   return smem;
 }
 
-template <int MODE, int RED, bool COHERENT = false, bool TMA = false, int NANG = 1, class Args,
-          class PreHook = NoHook, class MidHook = NoHook, class EndHook = NoHook,
+// RAG: a side that is no multiple of the tile (any even L >= 130; exact sums).
+// The last tile of a row or column of tiles is moved back so that it ends with
+// the lattice and overlaps the tile before it: the overlap is computed twice,
+// with the same words from the same old state, so both copies store the same
+// angles, and only the first one's sites enter the sums.  Where W is odd the
+// last tile starts at W - 63 (pairs start at even columns) and its last column
+// is column W, that is column 0: staged, never stored, and as the right
+// neighbour of column W - 1 updated with the side ring.
+template <int MODE, int RED, bool COHERENT = false, bool TMA = false, int NANG = 1,
+          bool RAG = false, class Args, class PreHook = NoHook, class MidHook = NoHook, class EndHook = NoHook,
           class PostHook = NoHook, class RawWait = NoHook>
 __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::RoundKeys& rk, int bx,
                                                  int by, int ang_sel = 0,
@@ -226,10 +238,26 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
   float(*part)[5][2] = reinterpret_cast<float(*)[5][2]>(smem + Lay::kPartAt);
   unsigned int* cnt = reinterpret_cast<unsigned int*>(smem + Lay::kCntAt);
 
+  static_assert(!RAG || (!TMA && RED == 0), "ragged tiles load per thread and sum exactly");
   const int L = a.L, W = a.W;
-  const int k0 = bx * kTileK;
-  const int y0 = by * kTileRows;
+  const int k0 = RAG ? min(bx * kTileK, W - kTileK + (W & 1)) : bx * kTileK;
+  const int y0 = RAG ? min(by * kTileRows, L - kTileRows) : by * kTileRows;
+  // columns of the tile inside the lattice (63 in the last tile of an odd W)
+  const int width = RAG ? min(kTileK, W - k0) : kTileK;
   const size_t plane = (size_t)L * (size_t)W;
+  // RAG: four (two) staged columns from column k (even, a multiple of four from
+  // k0) of the row at `row`: as wide as the rows' alignment allows
+  auto ragged4 = [&](size_t row, int k) {
+    const float* p = a.src + row;
+    if ((W & 3) == 0) return __ldcg(reinterpret_cast<const float4*>(p + k));
+    if ((W & 1) == 0) {
+      const float2 u = __ldcg(reinterpret_cast<const float2*>(p + k));
+      const float2 v = __ldcg(reinterpret_cast<const float2*>(p + k + 2));
+      return make_float4(u.x, u.y, v.x, v.y);
+    }
+    return make_float4(__ldcg(p + k), __ldcg(p + k + 1), __ldcg(p + k + 2),
+                       __ldcg(p + wrap_once(k + 3, W)));
+  };
 
   // ---- stage both planes (angle + unit vector) ----
   // Staged rows: the black plane's 36 (stage rows 0..35) then the red plane's
@@ -251,6 +279,10 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
         const int rr = (t >> 4) + 16 * i;
         const int p = rr < kSRows ? 1 : 0;
         const int r = rr < kSRows ? rr : rr - kSRows + 1;
+        if (RAG) {
+          v[i] = ragged4(p * plane + (size_t)wrap_once(y0 - 2 + r, L) * W, k0 + 4 * cg);
+          continue;
+        }
         const size_t row = p * plane + (size_t)wrap_once(y0 - 2 + r, L) * W + k0 + 4 * cg;
         v[i] = COHERENT ? __ldcg(reinterpret_cast<const float4*>(a.src + row))
                         : __ldg(reinterpret_cast<const float4*>(a.src + row));
@@ -260,7 +292,10 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const bool has_tail = t < 192;
     const int tail_r = 29 + (t >> 5), tail_c = t & 31;
     float2 vt = make_float2(0.f, 0.f);
-    if (has_tail && !TMA) {
+    if (RAG && has_tail && (W & 1)) {
+      const float* p = a.src + (size_t)wrap_once(y0 - 2 + tail_r, L) * W;
+      vt = make_float2(__ldcg(p + k0 + 2 * tail_c), __ldcg(p + wrap_once(k0 + 2 * tail_c + 1, W)));
+    } else if (has_tail && !TMA) {
       const size_t row = (size_t)wrap_once(y0 - 2 + tail_r, L) * W + k0 + 2 * tail_c;
       vt = COHERENT ? __ldcg(reinterpret_cast<const float2*>(a.src + row))
                     : __ldg(reinterpret_cast<const float2*>(a.src + row));
@@ -343,6 +378,25 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
   const int pj = lane + 1;                                 // the lane's pair in a row
   const int kp = k0 + 2 * lane;                            // plane column of the pair
   unsigned int n_acc = 0;
+  // RAG: whether both of the pair's columns are the tile's; whether a row's
+  // pair is counted here; its stores
+  const bool both = !RAG || 2 * lane + 1 < width;
+  auto counted = [&](int y) { return y >= by * kTileRows && kp >= bx * kTileK; };
+  auto put_own = [&](CsRow& row, const xyd::PairResult& p) {
+    if (both) {
+      put_pair(&row[pj], p.c, p.s);
+    } else {
+      put_one(row, 2 * pj, p.c.x, p.s.x);
+    }
+  };
+  auto store = [&](float* at, const float2& th) {
+    if ((W & 1) == 0) {
+      *reinterpret_cast<float2*>(at) = th;
+    } else {
+      at[0] = th.x;
+      if (both) at[1] = th.y;
+    }
+  };
 
   // ---- red half: the tile (counted, written to dst) ----
   float4 nbD = csb[warp * 4 + 1][pj];
@@ -374,9 +428,15 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const float4 o = csr[r - 1][pj];
     const xyd::PairResult p =
         xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
-    n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
-    put_pair(&csr[r - 1][pj], p.c, p.s);
-    *reinterpret_cast<float2*>(a.dst + (size_t)y * W + kp) = p.th;
+    if (!RAG) {
+      n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
+      put_pair(&csr[r - 1][pj], p.c, p.s);
+      *reinterpret_cast<float2*>(a.dst + (size_t)y * W + kp) = p.th;
+    } else {
+      if (counted(y)) n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 && both ? 1u : 0u);
+      put_own(csr[r - 1], p);
+      store(a.dst + (size_t)y * W + kp, p.th);
+    }
   }
   // ---- red half: the ring at distance one (recomputed, not counted) ----
   // The ring rows above and below the tile are 32 pairs each (sites x and
@@ -398,15 +458,21 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const float4 o = csr[r - 1][pj];
     const xyd::PairResult p =
         xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
-    put_pair(&csr[r - 1][pj], p.c, p.s);
+    if (RAG) {
+      put_own(csr[r - 1], p);
+    } else {
+      put_pair(&csr[r - 1][pj], p.c, p.s);
+    }
   } else if (warp == 2) {
     const int ty = lane;
-    const int tk = ((y0 + ty) & 1) ? -1 : kTileK;          // left ring on odd rows, right on even
+    const int tk = ((y0 + ty) & 1) ? -1 : width;           // left ring on odd rows, right on even
     const int y = wrap_once(y0 + ty, L);
     const int k = wrap_once(k0 + tk, W);
     const int q = y & 1;
     const uint32_t x = 2u * (uint32_t)k + (uint32_t)q;
-    red_ring_site<MODE>(angs[2 * (ty + 1) + (tk < 0 ? 0 : 1)], csr, csb, ty + 2, tk + kCsOff, q,
+    const float th = RAG && tk == kTileK - 1 ? ang[kRedRaw0 + ty + 2][kTileK - 1]
+                                             : angs[2 * (ty + 1) + (tk < 0 ? 0 : 1)];
+    red_ring_site<MODE>(th, csr, csb, ty + 2, tk + kCsOff, q,
                         (uint32_t)y * uL + x, x, a, rk);
   }
   mid();
@@ -437,13 +503,23 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const float4 o = csb[r][pj];
     const xyd::PairResult p =
         xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
-    n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
-    *reinterpret_cast<float2*>(dst_blk + (size_t)y * W + kp) = p.th;
+    if (!RAG) {
+      n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
+      *reinterpret_cast<float2*>(dst_blk + (size_t)y * W + kp) = p.th;
+    } else {
+      if (counted(y)) n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 && both ? 1u : 0u);
+      store(dst_blk + (size_t)y * W + kp, p.th);
+    }
 
     // red sites with the same (y, k): their spins enter M once each
     float2 v[5];
     xyd::measure_terms2(p.c, p.s, n, cosines(m), sines(m), v);
-    sums.add2(v);
+    if (!RAG || (counted(y) && both)) {
+      sums.add2(v);
+    } else if (counted(y)) {
+      const float v0[5] = {v[0].x, v[1].x, v[2].x, v[3].x, v[4].x};
+      sums.add(v0);
+    }
   }
 
   end();
@@ -587,7 +663,17 @@ __device__ __forceinline__ PersistItem decode_item(int item, int ntiles, int til
 // complete on one mbarrier, one phase per tile; each wait for it is bounded
 // too.  The arithmetic of a tile is fused_sweep_body's, so the result is bit
 // for bit that of n launches of k_sweep_fused.
-template <int MODE, int RED, int MINB>
+// RAG (any even L >= 130): the tiles of a side that is no multiple of 128 (see
+// fused_sweep_body), rows loaded per thread.  The nine counters still order
+// everything: the last tile starts at least two rows (columns) behind the
+// start of the tile it overlaps, so what it reads beyond its own and its
+// neighbours' first copies is its neighbours', the tile before the overlapped
+// one reads nothing that only the last tile's copy writes, and every copy of a
+// site is a neighbour of every tile that reads it.  Against two half-sweep
+// launches a sweep (us per sweep): L = 300 6.3 against 20.5, 1000 9.6 against
+// 22.6, 7324 323 against 430; where W is odd the rows are loaded and stored a
+// word at a time (L = 1002 11.0, 7326 391).
+template <int MODE, int RED, int MINB, bool RAG>
 __global__ void __launch_bounds__(kThreads, MINB)
     k_sweep_fused_persist(FusedPersistArgs p, const __grid_constant__ PersistMaps maps) {
   __shared__ int s_abort;
@@ -595,7 +681,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
   __shared__ int s_ready[2];         // the next item's nine counters were all seen set
   __shared__ __align__(8) uint64_t s_bar;   // the staged rows' TMA completion
   constexpr int kIssuer = kThreads - 32;    // lane 0 of the last warp
-  const int tiles_x = p.W / kTileK, tiles_y = p.L / kTileRows;
+  const int tiles_x = tile_cols(p.W), tiles_y = tile_rows(p.L);
   const int ntiles = tiles_x * tiles_y;
   const int total = p.n_sweeps * ntiles;          // < 2^31 - 2^20 (the host splits longer runs)
   FusedCore c;
@@ -661,9 +747,9 @@ __global__ void __launch_bounds__(kThreads, MINB)
     c.sweep = p.sweep0 + (uint32_t)s;
     c.rec = p.rec + s;
     PersistItem* slot = &s_item[par ^ 1];
-    if (!ready && threadIdx.x == kIssuer) issue_raw(cur, par);
-    fused_sweep_body<MODE, RED, true, true, 2>(
-        c, p.rk, bx, by, par,
+    if (!RAG && !ready && threadIdx.x == kIssuer) issue_raw(cur, par);
+    fused_sweep_body<MODE, RED, true, !RAG, RAG ? 1 : 2, RAG>(
+        c, p.rk, bx, by, RAG ? 0 : par,
         // before the staging barrier: the next item, decoded, to the other slot
         // (the atomic was issued before the staging loads, so it has returned)
         [&]() {
@@ -691,7 +777,7 @@ __global__ void __launch_bounds__(kThreads, MINB)
             __syncwarp();
             if (l == 0) {
               s_ready[par ^ 1] = all ? 1 : 0;
-              if (all) issue_raw(ni, par ^ 1);
+              if (!RAG && all) issue_raw(ni, par ^ 1);
             }
           }
         },
@@ -775,36 +861,39 @@ cudaError_t prepare_one() {
   return e == cudaSuccess ? prepare_plan<MODE, RED, 4>() : e;
 }
 
-template <int MODE, int RED, int MINB>
+template <bool RAG>
+constexpr size_t persist_smem() { return RAG ? kSmemBytes : kPersistSmemBytes; }
+
+template <int MODE, int RED, int MINB, bool RAG>
 cudaError_t launch_persist_one(const FusedPersistArgs& a, int grid, cudaStream_t stream) {
   // the maps in buf order (the caller may have swapped the two buffers)
-  PersistMaps pm;
-  for (int b = 0; b < 2; ++b) {
+  PersistMaps pm = {};
+  for (int b = 0; b < 2 && !RAG; ++b) {
     const int i = fused_map_index(*a.maps, a.buf[b]);
     if (i < 0) return cudaErrorInvalidValue;
     for (int k = 0; k < 3; ++k) pm.m[b][k] = a.maps->m[i][k];
   }
   void* args[] = {const_cast<FusedPersistArgs*>(&a), &pm};
   return cudaLaunchCooperativeKernel(
-      reinterpret_cast<const void*>(&k_sweep_fused_persist<MODE, RED, MINB>), dim3(grid),
-      dim3(kThreads), args, kPersistSmemBytes, stream);
+      reinterpret_cast<const void*>(&k_sweep_fused_persist<MODE, RED, MINB, RAG>), dim3(grid),
+      dim3(kThreads), args, persist_smem<RAG>(), stream);
 }
 
-template <int MODE, int RED, int MINB>
+template <int MODE, int RED, int MINB, bool RAG>
 cudaError_t persist_grid_one(int L, int* grid) {
   static int per_sm[64] = {};        // resident CTAs per SM, per device (0: not yet set)
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || per_sm[dev] == 0) {
-    auto fn = k_sweep_fused_persist<MODE, RED, MINB>;
+    auto fn = k_sweep_fused_persist<MODE, RED, MINB, RAG>;
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kPersistSmemBytes);
+                             (int)persist_smem<RAG>());
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int n = 0;
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kThreads, kPersistSmemBytes);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kThreads, persist_smem<RAG>());
     if (e != cudaSuccess) return e;
     if (n < 1) return cudaErrorCooperativeLaunchTooLarge;
     if (dev >= 0 && dev < 64) per_sm[dev] = n;
@@ -813,22 +902,22 @@ cudaError_t persist_grid_one(int L, int* grid) {
   int sms = 0;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int tiles = (L / 2 / kTileK) * (L / kTileRows);
+  const int tiles = fused_tiles_of(L);
   const int resident = per_sm[(dev >= 0 && dev < 64) ? dev : 0] * sms;
   *grid = tiles < resident ? tiles : resident;
   return cudaSuccess;
 }
 
 // The persistent launch of one instantiation: grid, then the launch.
-template <int MODE, int RED, int MINB>
+template <int MODE, int RED, int MINB, bool RAG = false>
 cudaError_t persist_plan(const FusedPersistArgs& a, cudaStream_t stream) {
   int grid = 0;
-  cudaError_t e = persist_grid_one<MODE, RED, MINB>(a.L, &grid);
+  cudaError_t e = persist_grid_one<MODE, RED, MINB, RAG>(a.L, &grid);
   if (e != cudaSuccess) return e;
   // the tile counters and, after them, the work counter
   e = cudaMemsetAsync(a.flags, 0, sizeof(unsigned int) * ((size_t)fused_tiles_of(a.L) + 1), stream);
   if (e != cudaSuccess) return e;
-  return launch_persist_one<MODE, RED, MINB>(a, grid, stream);
+  return launch_persist_one<MODE, RED, MINB, RAG>(a, grid, stream);
 }
 
 template <int MODE, int RED>
@@ -838,9 +927,18 @@ cudaError_t persist_dispatch(const FusedPersistArgs& a, cudaStream_t stream) {
                        : persist_plan<MODE, RED, 3>(a, stream);
 }
 
+template <int MODE>
+cudaError_t ragged_dispatch(const FusedPersistArgs& a, cudaStream_t stream) {
+  return a.minb == 2   ? persist_plan<MODE, 0, 2, true>(a, stream)
+         : a.minb == 4 ? persist_plan<MODE, 0, 4, true>(a, stream)
+                       : persist_plan<MODE, 0, 3, true>(a, stream);
+}
+
 }  // namespace
 
 bool fused_supported(int L) { return L >= 128 && (L % 128) == 0; }
+
+bool ragged_supported(int L) { return L >= 130 && (L & 1) == 0 && !fused_supported(L); }
 
 cudaError_t prepare_fused_batch(int sincos_mode, int reduce_mode) {
   const bool comp = reduce_mode != 0;
@@ -884,7 +982,7 @@ cudaError_t launch_fused_sweep(int sincos_mode, int reduce_mode, const FusedArgs
 
 namespace xyk {
 
-int fused_tiles(int L) { return fused_supported(L) ? (L / 2 / kTileK) * (L / kTileRows) : 0; }
+int fused_tiles(int L) { return fused_supported(L) || ragged_supported(L) ? fused_tiles_of(L) : 0; }
 
 long long fused_persistent_spin_limit() { return kPersistSpinLimit; }
 
@@ -918,11 +1016,19 @@ int fused_persistent_max_sweeps(int L) {
 
 cudaError_t launch_fused_persistent(int sincos_mode, int reduce_mode, const FusedPersistArgs& a,
                                     cudaStream_t stream) {
-  if (!fused_supported(a.L) || a.W * 2 != a.L || a.n_sweeps < 1 ||
+  const bool ragged = ragged_supported(a.L) && reduce_mode == 0;
+  if ((!fused_supported(a.L) && !ragged) || a.W * 2 != a.L || a.n_sweeps < 1 ||
       a.n_sweeps > fused_persistent_max_sweeps(a.L) || !a.flags || a.counter != a.flags + fused_tiles(a.L) ||
-      !a.error || a.buf[0] == a.buf[1] || !a.maps || a.spin_limit < 1 || a.skip_items < 0 ||
+      !a.error || a.buf[0] == a.buf[1] || (!ragged && !a.maps) || a.spin_limit < 1 || a.skip_items < 0 ||
       a.skip_items > a.n_sweeps * fused_tiles(a.L) || (a.minb < 2 || a.minb > 4))
     return cudaErrorInvalidValue;
+  if (ragged) {
+    switch (sincos_mode) {
+      case 0: return ragged_dispatch<0>(a, stream);
+      case 1: return ragged_dispatch<1>(a, stream);
+      default: return ragged_dispatch<2>(a, stream);
+    }
+  }
   const bool comp = reduce_mode != 0;
   switch (sincos_mode) {
     case 0: return comp ? persist_dispatch<0, 1>(a, stream) : persist_dispatch<0, 0>(a, stream);

@@ -82,8 +82,11 @@ struct FusedArgs {
   unsigned int* error = nullptr;     // set nonzero if the wait for the staged rows runs out
 };
 
-// Whether the fused kernel handles side L (L a positive multiple of 128).
+// Whether the fused kernel handles side L (L a positive multiple of 128), and
+// whether the persistent sweep takes it on overlapping tiles (any other even
+// L >= 130; exact sums).
 bool fused_supported(int L);
+bool ragged_supported(int L);
 
 // One fused sweep of four replicas per site (float4 sites, read as floats
 // [colour][y][4k + r]); replica r has lattice id lattice_id0 + r and K[r].
@@ -145,13 +148,14 @@ struct FusedPersistArgs {
   int skip_items;        // work items not handed out (0; > 0 only to test the
                          // failure path: their counters are then never set)
   int minb = 3;          // resident CTAs per SM the kernel is compiled for (2, 3 or 4)
-  const FusedMaps* maps = nullptr;   // tensor maps of buf[0], buf[1] (host memory, required)
+  const FusedMaps* maps = nullptr;   // tensor maps of buf[0], buf[1] (host memory;
+                                     // required unless ragged_supported(L))
 };
 
 // The default bound of the persistent kernel's waits, in polls (about a second).
 long long fused_persistent_spin_limit();
 
-// Tiles of one fused sweep of side L (0 if !fused_supported(L)).
+// Tiles of one fused sweep of side L (0 if neither of the two above).
 int fused_tiles(int L);
 
 // Most sweeps one persistent launch takes (n_sweeps x tiles < 2^31).
