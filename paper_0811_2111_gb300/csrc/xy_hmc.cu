@@ -829,6 +829,67 @@ __device__ __forceinline__ void hmc_site_step(float c, float s, float Sc, float 
   t = hmc_wrap(__fmaf_rn(eps, p, t));
 }
 
+// The unit vectors of four adjacent sites as pairs of the even and of the odd
+// ones, (c0, c2), (c1, c3): then an even pair's right neighbours are the odd
+// pair and an odd pair's left neighbours the even one, as they stand in the
+// registers, and of the packed sums' operands only (left lane's c3, c1) and
+// (c2, right lane's c0) have to be put together.  The frame keeps its groups of
+// four in the same order, frame_col(q) the place of column q.  46.7 issued
+// instructions per site-step against 57.7 with scalar arithmetic; per unit
+// trajectory L = 512 75.2 against 77.5 us, 1024 139 against 145, 2048 572
+// against 610-648, 4096 3.20 against 3.21 ms (SFU sincos 2.67 against 2.84):
+// the two CTAs of an SM wait on each other's barriers and on dependent packed
+// instructions, not for issue slots or memory.  Measured and not kept: the
+// wrap packed too (4096 3.25 ms), three CTAs per SM (140 bytes spilled, 512
+// 94 us), consecutive launches walking the tiles in opposite orders (a tie),
+// and the second step's stores after the band instead of row by row (4096
+// 3.46 ms: the stores burst and stall the warp).
+struct Quad4 {
+  float2 cE, cO, sE, sO;
+};
+
+__device__ __forceinline__ int frame_col(int q) {
+  return (q & ~3) | ((q & 1) << 1) | ((q >> 1) & 1);
+}
+
+template <int MODE>
+__device__ __forceinline__ Quad4 quad_vectors(const float4& t) {
+  float2 s01, c01, s23, c23;
+  xyd::unit_vector2<MODE>(make_float2(t.x, t.y), &s01, &c01);
+  xyd::unit_vector2<MODE>(make_float2(t.z, t.w), &s23, &c23);
+  return Quad4{make_float2(c01.x, c23.x), make_float2(c01.y, c23.y), make_float2(s01.x, s23.x),
+               make_float2(s01.y, s23.y)};
+}
+
+__device__ __forceinline__ void put_quad(float* c, float* s, const Quad4& v) {
+  *reinterpret_cast<float4*>(c) = make_float4(v.cE.x, v.cE.y, v.cO.x, v.cO.y);
+  *reinterpret_cast<float4*>(s) = make_float4(v.sE.x, v.sE.y, v.sO.x, v.sO.y);
+}
+
+__device__ __forceinline__ Quad4 get_quad(const float* c, const float* s) {
+  const float4 a = *reinterpret_cast<const float4*>(c), b = *reinterpret_cast<const float4*>(s);
+  return Quad4{make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
+               make_float2(b.z, b.w)};
+}
+
+// One leap-frog step of four adjacent sites `o` (angles t, momenta p) with the
+// rows below and above and the neighbouring lanes' sites (cl, sl), (cr, sr).
+__device__ __forceinline__ void quad_step(const Quad4& o, const Quad4& dn, const Quad4& up,
+                                          float cl, float sl, float cr, float sr, float K, float a,
+                                          float eps, float4& p, float4& t) {
+  using xyd::add2;
+  const float2 ScE = add2(add2(make_float2(cl, o.cO.x), o.cO), add2(dn.cE, up.cE));
+  const float2 SsE = add2(add2(make_float2(sl, o.sO.x), o.sO), add2(dn.sE, up.sE));
+  const float2 ScO = add2(add2(o.cE, make_float2(o.cE.y, cr)), add2(dn.cO, up.cO));
+  const float2 SsO = add2(add2(o.sE, make_float2(o.sE.y, sr)), add2(dn.sO, up.sO));
+  const float2 FE = hmc_force2(o.cE, o.sE, ScE, SsE, K);
+  const float2 FO = hmc_force2(o.cO, o.sO, ScO, SsO, K);
+  p = make_float4(__fmaf_rn(a, FE.x, p.x), __fmaf_rn(a, FO.x, p.y), __fmaf_rn(a, FE.y, p.z),
+                  __fmaf_rn(a, FO.y, p.w));
+  t = make_float4(hmc_wrap(__fmaf_rn(eps, p.x, t.x)), hmc_wrap(__fmaf_rn(eps, p.y, t.y)),
+                  hmc_wrap(__fmaf_rn(eps, p.z, t.z)), hmc_wrap(__fmaf_rn(eps, p.w, t.w)));
+}
+
 // PREF = false: one tile per CTA (grid = the tile columns x rows), its loads straight into
 // registers.  PREF = true: a grid of resident CTAs walks the tiles blockIdx.x,
 // + gridDim.x, ... (the tiles of a launch are independent: it reads one angle
@@ -970,47 +1031,37 @@ __global__ void __launch_bounds__(kP2Threads, 2)
   }
 
   // ---- unit vectors of the old state; what crosses a warp goes to the frame
-  float c[kP2Band][4], s[kP2Band][4];
+  Quad4 v[kP2Band];
 #pragma unroll
-  for (int r = 0; r < kP2Band; ++r) {
-    xyd::unit_vector<MODE>(t4[r].x, &s[r][0], &c[r][0]);
-    xyd::unit_vector<MODE>(t4[r].y, &s[r][1], &c[r][1]);
-    xyd::unit_vector<MODE>(t4[r].z, &s[r][2], &c[r][2]);
-    xyd::unit_vector<MODE>(t4[r].w, &s[r][3], &c[r][3]);
-  }
+  for (int r = 0; r < kP2Band; ++r) v[r] = quad_vectors<MODE>(t4[r]);
+  // ring site A and halo-two site H, then ring site B or halo-two site G
+  const int aq = frame_col(ax + 4), bq = frame_col(bx + 4), gq = frame_col(gx + 4);
   float ca, sa, cb = 0.f, sb = 0.f;
-  xyd::unit_vector<MODE>(ta, &sa, &ca);
-  if (hasb) xyd::unit_vector<MODE>(tb, &sb, &cb);
   {
-    float hs, hc;
-    xyd::unit_vector<MODE>(th_h, &hs, &hc);
-    fc[hy + 2][ax + 4] = hc;
-    fs[hy + 2][ax + 4] = hs;
-    if (hasg) {
-      xyd::unit_vector<MODE>(th_g, &hs, &hc);
-      fc[gy + 2][gx + 4] = hc;
-      fs[gy + 2][gx + 4] = hs;
+    float2 s2, c2;
+    xyd::unit_vector2<MODE>(make_float2(ta, th_h), &s2, &c2);
+    ca = c2.x;
+    sa = s2.x;
+    fc[ay + 2][aq] = ca;
+    fs[ay + 2][aq] = sa;
+    fc[hy + 2][aq] = c2.y;
+    fs[hy + 2][aq] = s2.y;
+    if (hasb || hasg) {
+      xyd::unit_vector<MODE>(hasb ? tb : th_g, &sb, &cb);
+      fc[(hasb ? by : gy) + 2][hasb ? bq : gq] = cb;
+      fs[(hasb ? by : gy) + 2][hasb ? bq : gq] = sb;
     }
   }
-  fc[ay + 2][ax + 4] = ca;
-  fs[ay + 2][ax + 4] = sa;
-  if (hasb) {
-    fc[by + 2][bx + 4] = cb;
-    fs[by + 2][bx + 4] = sb;
-  }
   // the band's first and last row, and the tile's first and last column
-  *reinterpret_cast<float4*>(&fc[rb + 2][4 * lane + 4]) = make_float4(c[0][0], c[0][1], c[0][2], c[0][3]);
-  *reinterpret_cast<float4*>(&fs[rb + 2][4 * lane + 4]) = make_float4(s[0][0], s[0][1], s[0][2], s[0][3]);
-  *reinterpret_cast<float4*>(&fc[rb + kP2Band + 1][4 * lane + 4]) =
-      make_float4(c[kP2Band - 1][0], c[kP2Band - 1][1], c[kP2Band - 1][2], c[kP2Band - 1][3]);
-  *reinterpret_cast<float4*>(&fs[rb + kP2Band + 1][4 * lane + 4]) =
-      make_float4(s[kP2Band - 1][0], s[kP2Band - 1][1], s[kP2Band - 1][2], s[kP2Band - 1][3]);
+  put_quad(&fc[rb + 2][4 * lane + 4], &fs[rb + 2][4 * lane + 4], v[0]);
+  put_quad(&fc[rb + kP2Band + 1][4 * lane + 4], &fs[rb + kP2Band + 1][4 * lane + 4],
+           v[kP2Band - 1]);
   if (lane == 0 || lane == 31) {
     const int q = lane == 0 ? 4 : kP2Cols + 3;             // tile column 0 or 127
 #pragma unroll
     for (int r = 1; r < kP2Band - 1; ++r) {
-      fc[rb + r + 2][q] = lane == 0 ? c[r][0] : c[r][3];
-      fs[rb + r + 2][q] = lane == 0 ? s[r][0] : s[r][3];
+      fc[rb + r + 2][q] = lane == 0 ? v[r].cE.x : v[r].cO.y;
+      fs[rb + r + 2][q] = lane == 0 ? v[r].sE.x : v[r].sO.y;
     }
   }
   __syncthreads();
@@ -1021,123 +1072,72 @@ __global__ void __launch_bounds__(kP2Threads, 2)
 
   // ---- first step: the ring sites (from the frame), then the tile --------
   const float K = a.K, ka = a.a, eps = a.eps;
-  {
-    const int r = ay + 2, q = ax + 4;
-    const float Sc = xyd::nb_sum(fc[r][q - 1], fc[r][q + 1], fc[r - 1][q], fc[r + 1][q]);
-    const float Ss = xyd::nb_sum(fs[r][q - 1], fs[r][q + 1], fs[r - 1][q], fs[r + 1][q]);
-    hmc_site_step(ca, sa, Sc, Ss, K, ka, eps, pa, ta);
-  }
-  if (hasb) {
-    const int r = by + 2, q = bx + 4;
-    const float Sc = xyd::nb_sum(fc[r][q - 1], fc[r][q + 1], fc[r - 1][q], fc[r + 1][q]);
-    const float Ss = xyd::nb_sum(fs[r][q - 1], fs[r][q + 1], fs[r - 1][q], fs[r + 1][q]);
-    hmc_site_step(cb, sb, Sc, Ss, K, ka, eps, pb, tb);
-  }
+  auto ring_step = [&](int r, int q, float c0, float s0, float& p, float& t) {
+    const int l = frame_col(q - 1), m = frame_col(q), n = frame_col(q + 1);
+    const float Sc = xyd::nb_sum(fc[r][l], fc[r][n], fc[r - 1][m], fc[r + 1][m]);
+    const float Ss = xyd::nb_sum(fs[r][l], fs[r][n], fs[r - 1][m], fs[r + 1][m]);
+    hmc_site_step(c0, s0, Sc, Ss, K, ka, eps, p, t);
+  };
+  ring_step(ay + 2, ax + 4, ca, sa, pa, ta);
+  if (hasb) ring_step(by + 2, bx + 4, cb, sb, pb, tb);
   // the ring's new unit vectors (its momenta and angles are not needed again)
-  xyd::unit_vector<MODE>(ta, &sa, &ca);
-  if (hasb) xyd::unit_vector<MODE>(tb, &sb, &cb);
-  // vertical neighbours of the band: the row below its first and above its last
-  float4 cdn = *reinterpret_cast<const float4*>(&fc[rb + 1][4 * lane + 4]);
-  float4 sdn = *reinterpret_cast<const float4*>(&fs[rb + 1][4 * lane + 4]);
-  float4 cup = *reinterpret_cast<const float4*>(&fc[rb + kP2Band + 2][4 * lane + 4]);
-  float4 sup = *reinterpret_cast<const float4*>(&fs[rb + kP2Band + 2][4 * lane + 4]);
-#pragma unroll
-  for (int r = 0; r < kP2Band; ++r) {
-    float cl = __shfl_up_sync(0xffffffffu, c[r][3], 1);
-    float sl = __shfl_up_sync(0xffffffffu, s[r][3], 1);
-    float cr = __shfl_down_sync(0xffffffffu, c[r][0], 1);
-    float sr = __shfl_down_sync(0xffffffffu, s[r][0], 1);
-    if (lane == 0) {
-      cl = fc[rb + r + 2][3];
-      sl = fs[rb + r + 2][3];
-    }
-    if (lane == 31) {
-      cr = fc[rb + r + 2][kP2Cols + 4];
-      sr = fs[rb + r + 2][kP2Cols + 4];
-    }
-    const float pr[4] = {p4[r].x, p4[r].y, p4[r].z, p4[r].w};
-    const float tr[4] = {t4[r].x, t4[r].y, t4[r].z, t4[r].w};
-    const float cd[4] = {cdn.x, cdn.y, cdn.z, cdn.w}, sd[4] = {sdn.x, sdn.y, sdn.z, sdn.w};
-    const float cu[4] = {cup.x, cup.y, cup.z, cup.w}, su[4] = {sup.x, sup.y, sup.z, sup.w};
-    float po[4], to[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float nlc = j == 0 ? cl : c[r][j - 1], nls = j == 0 ? sl : s[r][j - 1];
-      const float nrc = j == 3 ? cr : c[r][j + 1], nrs = j == 3 ? sr : s[r][j + 1];
-      const float ndc = r == 0 ? cd[j] : c[r - 1][j], nds = r == 0 ? sd[j] : s[r - 1][j];
-      const float nuc = r == kP2Band - 1 ? cu[j] : c[r + 1][j];
-      const float nus = r == kP2Band - 1 ? su[j] : s[r + 1][j];
-      float p = pr[j], t = tr[j];
-      hmc_site_step(c[r][j], s[r][j], xyd::nb_sum(nlc, nrc, ndc, nuc),
-                    xyd::nb_sum(nls, nrs, nds, nus), K, ka, eps, p, t);
-      po[j] = p;
-      to[j] = t;
-    }
-    p4[r] = make_float4(po[0], po[1], po[2], po[3]);
-    t4[r] = make_float4(to[0], to[1], to[2], to[3]);
+  {
+    float2 s2, c2;
+    xyd::unit_vector2<MODE>(make_float2(ta, tb), &s2, &c2);
+    ca = c2.x;
+    sa = s2.x;
+    cb = c2.y;
+    sb = s2.y;
   }
+  // a step of the band: vertical neighbours from its own rows or the frame's
+  // rows below and above, horizontal ones from the neighbouring lanes (the
+  // warp's edge lanes: the frame's ring columns)
+  auto band_step = [&](auto&& done) {
+    Quad4 dn = get_quad(&fc[rb + 1][4 * lane + 4], &fs[rb + 1][4 * lane + 4]);
+    const Quad4 top = get_quad(&fc[rb + kP2Band + 2][4 * lane + 4], &fs[rb + kP2Band + 2][4 * lane + 4]);
+#pragma unroll
+    for (int r = 0; r < kP2Band; ++r) {
+      float cl = __shfl_up_sync(0xffffffffu, v[r].cO.y, 1);
+      float sl = __shfl_up_sync(0xffffffffu, v[r].sO.y, 1);
+      float cr = __shfl_down_sync(0xffffffffu, v[r].cE.x, 1);
+      float sr = __shfl_down_sync(0xffffffffu, v[r].sE.x, 1);
+      if (lane == 0) {
+        cl = fc[rb + r + 2][3];
+        sl = fs[rb + r + 2][3];
+      }
+      if (lane == 31) {
+        cr = fc[rb + r + 2][kP2Cols + 4];
+        sr = fs[rb + r + 2][kP2Cols + 4];
+      }
+      quad_step(v[r], dn, r == kP2Band - 1 ? top : v[r == kP2Band - 1 ? r : r + 1], cl, sl, cr, sr,
+                K, ka, eps, p4[r], t4[r]);
+      dn = v[r];
+      done(r);
+    }
+  };
+  band_step([](int) {});
   // new unit vectors (the old ones are no longer read by this thread)
 #pragma unroll
-  for (int r = 0; r < kP2Band; ++r) {
-    xyd::unit_vector<MODE>(t4[r].x, &s[r][0], &c[r][0]);
-    xyd::unit_vector<MODE>(t4[r].y, &s[r][1], &c[r][1]);
-    xyd::unit_vector<MODE>(t4[r].z, &s[r][2], &c[r][2]);
-    xyd::unit_vector<MODE>(t4[r].w, &s[r][3], &c[r][3]);
-  }
+  for (int r = 0; r < kP2Band; ++r) v[r] = quad_vectors<MODE>(t4[r]);
   __syncthreads();   // every old frame value has been read
-  fc[ay + 2][ax + 4] = ca;
-  fs[ay + 2][ax + 4] = sa;
+  fc[ay + 2][aq] = ca;
+  fs[ay + 2][aq] = sa;
   if (hasb) {
-    fc[by + 2][bx + 4] = cb;
-    fs[by + 2][bx + 4] = sb;
+    fc[by + 2][bq] = cb;
+    fs[by + 2][bq] = sb;
   }
-  *reinterpret_cast<float4*>(&fc[rb + 2][4 * lane + 4]) = make_float4(c[0][0], c[0][1], c[0][2], c[0][3]);
-  *reinterpret_cast<float4*>(&fs[rb + 2][4 * lane + 4]) = make_float4(s[0][0], s[0][1], s[0][2], s[0][3]);
-  *reinterpret_cast<float4*>(&fc[rb + kP2Band + 1][4 * lane + 4]) =
-      make_float4(c[kP2Band - 1][0], c[kP2Band - 1][1], c[kP2Band - 1][2], c[kP2Band - 1][3]);
-  *reinterpret_cast<float4*>(&fs[rb + kP2Band + 1][4 * lane + 4]) =
-      make_float4(s[kP2Band - 1][0], s[kP2Band - 1][1], s[kP2Band - 1][2], s[kP2Band - 1][3]);
+  put_quad(&fc[rb + 2][4 * lane + 4], &fs[rb + 2][4 * lane + 4], v[0]);
+  put_quad(&fc[rb + kP2Band + 1][4 * lane + 4], &fs[rb + kP2Band + 1][4 * lane + 4],
+           v[kP2Band - 1]);
   __syncthreads();
 
   // ---- second step: the tile, written out ----------------------------------
-  cdn = *reinterpret_cast<const float4*>(&fc[rb + 1][4 * lane + 4]);
-  sdn = *reinterpret_cast<const float4*>(&fs[rb + 1][4 * lane + 4]);
-  cup = *reinterpret_cast<const float4*>(&fc[rb + kP2Band + 2][4 * lane + 4]);
-  sup = *reinterpret_cast<const float4*>(&fs[rb + kP2Band + 2][4 * lane + 4]);
   float* __restrict__ th_dst = hmc_buf(a, dst);
-#pragma unroll
-  for (int r = 0; r < kP2Band; ++r) {
-    float cl = __shfl_up_sync(0xffffffffu, c[r][3], 1);
-    float sl = __shfl_up_sync(0xffffffffu, s[r][3], 1);
-    float cr = __shfl_down_sync(0xffffffffu, c[r][0], 1);
-    float sr = __shfl_down_sync(0xffffffffu, s[r][0], 1);
-    if (lane == 0) {
-      cl = fc[rb + r + 2][3];
-      sl = fs[rb + r + 2][3];
-    }
-    if (lane == 31) {
-      cr = fc[rb + r + 2][kP2Cols + 4];
-      sr = fs[rb + r + 2][kP2Cols + 4];
-    }
-    const float cd[4] = {cdn.x, cdn.y, cdn.z, cdn.w}, sd[4] = {sdn.x, sdn.y, sdn.z, sdn.w};
-    const float cu[4] = {cup.x, cup.y, cup.z, cup.w}, su[4] = {sup.x, sup.y, sup.z, sup.w};
-    float po[4], to[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float nlc = j == 0 ? cl : c[r][j - 1], nls = j == 0 ? sl : s[r][j - 1];
-      const float nrc = j == 3 ? cr : c[r][j + 1], nrs = j == 3 ? sr : s[r][j + 1];
-      const float ndc = r == 0 ? cd[j] : c[r - 1][j], nds = r == 0 ? sd[j] : s[r - 1][j];
-      const float nuc = r == kP2Band - 1 ? cu[j] : c[r + 1][j];
-      const float nus = r == kP2Band - 1 ? su[j] : s[r + 1][j];
-      po[j] = (&p4[r].x)[j];
-      to[j] = (&t4[r].x)[j];
-      hmc_site_step(c[r][j], s[r][j], xyd::nb_sum(nlc, nrc, ndc, nuc),
-                    xyd::nb_sum(nls, nrs, nds, nus), K, ka, eps, po[j], to[j]);
-    }
+  band_step([&](int r) {
     const size_t g = (size_t)(y0 + rb + r) * L + xb;
-    *reinterpret_cast<float4*>(a.p_out + g) = make_float4(po[0], po[1], po[2], po[3]);
-    *reinterpret_cast<float4*>(th_dst + g) = make_float4(to[0], to[1], to[2], to[3]);
-  }
+    *reinterpret_cast<float4*>(a.p_out + g) = p4[r];
+    *reinterpret_cast<float4*>(th_dst + g) = t4[r];
+  });
   if (PREF) __syncthreads();   // the next tile's staging rewrites the frame
   }
 }

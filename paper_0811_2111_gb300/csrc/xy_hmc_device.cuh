@@ -57,6 +57,13 @@ __device__ __forceinline__ float hmc_force(float c, float s, float Sc, float Ss,
   return __fmul_rn(K, __fmaf_rn(c, Ss, -__fmul_rn(s, Sc)));
 }
 
+// The forces on two sites.
+__device__ __forceinline__ float2 hmc_force2(float2 c, float2 s, float2 Sc, float2 Ss, float K) {
+  const float2 m = xyd::mul2(s, Sc);
+  return xyd::mul2(xyd::dup2(K),
+                   make_float2(__fmaf_rn(c.x, Ss.x, -m.x), __fmaf_rn(c.y, Ss.y, -m.y)));
+}
+
 // Fixed-point rounding with FP32 operations only (GB300 runs float -> int64
 // conversions on its narrow FP64 pipe).  Adding 1.5 * 2^23 rounds any |x| <
 // 2^22 to the nearest integer (ties to even), which the low bits of the sum
