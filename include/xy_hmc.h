@@ -86,11 +86,13 @@ typedef struct {
  * have finished the previous step (per-tile counters in device memory, bounded
  * waits reported as XY_ETIMEOUT; needs what TILED_TMA needs and every CTA of
  * the grid resident; bit-identical, but measured slower than TILED_TMA on
- * GB300: 256 against 331 G site-steps/s at L = 4096).  AUTO takes CLUSTER for L = 128
- * and 256, else TILED_TMA when L % 128 == 0 and the encoder is available
- * (TILED if not), else SITE (the choices measured fastest on GB300: e.g.
- * TILED_TMA 51.4 us per step at L = 4096 against 57.0 for TILED and 58.3 for
- * TILED2; CLUSTER 2.8 us per step at L = 128 against 4.0 for TILED_TMA).  All
+ * GB300: 256 against 331 G site-steps/s at L = 4096).  AUTO holds
+ * lattices of 4 <= L <= 176 on the chip and runs many trajectories per cluster
+ * launch (where the device can run the cluster), takes SITE up to L = 351, and
+ * from there TILED2's two steps per launch, on overlapping tiles where L is no
+ * multiple of 128 (the begin, final and odd step then by SITE); the choices
+ * measured fastest on GB300 (us per unit trajectory: L = 128 17.6 against 29.6
+ * SITE, 39.3 CLUSTER and 43.3 TILED2; 512 75 against 104 SITE).  All
  * give bit-identical angles, momenta and sums. */
 enum { XY_HMC_KERNEL_AUTO = 0, XY_HMC_KERNEL_TILED = 1, XY_HMC_KERNEL_SITE = 2,
        XY_HMC_KERNEL_TILED2 = 3, XY_HMC_KERNEL_TILED_TMA = 4, XY_HMC_KERNEL_CLUSTER = 5,

@@ -906,7 +906,36 @@ struct Tile2Maps {
   CUtensorMap p;
 };
 
-template <int MODE, bool PREF>
+// RAG (PREF = false; any L >= 130): the last tiles of a side that is no multiple
+// of the tile move back to end with the lattice and overlap the tiles before
+// them.  A launch reads one angle and one momentum buffer and writes others,
+// so the sites of an overlap are computed twice from the same inputs and
+// stored twice with the same bits.  Rows are loaded and stored as wide as
+// their alignment allows (16, 8 or 4 bytes for L % 4 = 0, 2, odd).
+__device__ __forceinline__ float4 load_row4(const float* p, int L) {
+  if ((L & 3) == 0) return *reinterpret_cast<const float4*>(p);
+  if ((L & 1) == 0) {
+    const float2 u = *reinterpret_cast<const float2*>(p), v = *reinterpret_cast<const float2*>(p + 2);
+    return make_float4(u.x, u.y, v.x, v.y);
+  }
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+
+__device__ __forceinline__ void store_row4(float* p, const float4& v, int L) {
+  if ((L & 3) == 0) {
+    *reinterpret_cast<float4*>(p) = v;
+  } else if ((L & 1) == 0) {
+    *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y);
+    *reinterpret_cast<float2*>(p + 2) = make_float2(v.z, v.w);
+  } else {
+    p[0] = v.x;
+    p[1] = v.y;
+    p[2] = v.z;
+    p[3] = v.w;
+  }
+}
+
+template <int MODE, bool PREF, bool RAG = false>
 __global__ void __launch_bounds__(kP2Threads, 2)
     k_hmc_tile2(HmcArgs a, const __grid_constant__ Tile2Maps maps) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -972,8 +1001,10 @@ __global__ void __launch_bounds__(kP2Threads, 2)
   if (PREF && (int)blockIdx.x < n_tiles) prefetch(blockIdx.x);
   for (int tile = PREF ? (int)blockIdx.x : 0; tile < (PREF ? n_tiles : 1);
        tile += PREF ? (int)gridDim.x : 1) {
-  const int x0 = PREF ? (tile % tiles_x) * kP2Cols : (int)blockIdx.x * kP2Cols;
-  const int y0 = PREF ? (tile / tiles_x) * kP2Rows : (int)blockIdx.y * kP2Rows;
+  const int x0 = PREF ? (tile % tiles_x) * kP2Cols
+                 : RAG ? min((int)blockIdx.x * kP2Cols, L - kP2Cols) : (int)blockIdx.x * kP2Cols;
+  const int y0 = PREF ? (tile / tiles_x) * kP2Rows
+                 : RAG ? min((int)blockIdx.y * kP2Rows, L - kP2Rows) : (int)blockIdx.y * kP2Rows;
 
   // ---- loads: own 4 x 4 block (angles and momenta), one site of the ring's
   // top or bottom row (threads 0..255), one of its side columns (0..63), one
@@ -993,9 +1024,9 @@ __global__ void __launch_bounds__(kP2Threads, 2)
     // the boxes: rows of 128 floats, the thread's 4 x 4 block at row rb + r,
     // columns 4 lane .. 4 lane + 3
     t4[r] = PREF ? pre_rows[(rb + r) * (kP2Cols / 4) + lane]
-                 : *reinterpret_cast<const float4*>(th_src + g);
+                 : RAG ? load_row4(th_src + g, L) : *reinterpret_cast<const float4*>(th_src + g);
     p4[r] = PREF ? pre_rows[(kP2Rows + rb + r) * (kP2Cols / 4) + lane]
-                 : *reinterpret_cast<const float4*>(a.p_in + g);
+                 : RAG ? load_row4(a.p_in + g, L) : *reinterpret_cast<const float4*>(a.p_in + g);
   }
   // ring site A: row -1 (tid < 128) or 32, column tid & 127
   const int ay = tid < kP2Cols ? -1 : kP2Rows, ax = tid & (kP2Cols - 1);
@@ -1135,8 +1166,13 @@ __global__ void __launch_bounds__(kP2Threads, 2)
   float* __restrict__ th_dst = hmc_buf(a, dst);
   band_step([&](int r) {
     const size_t g = (size_t)(y0 + rb + r) * L + xb;
-    *reinterpret_cast<float4*>(a.p_out + g) = p4[r];
-    *reinterpret_cast<float4*>(th_dst + g) = t4[r];
+    if (RAG) {
+      store_row4(a.p_out + g, p4[r], L);
+      store_row4(th_dst + g, t4[r], L);
+    } else {
+      *reinterpret_cast<float4*>(a.p_out + g) = p4[r];
+      *reinterpret_cast<float4*>(th_dst + g) = t4[r];
+    }
   });
   if (PREF) __syncthreads();   // the next tile's staging rewrites the frame
   }
@@ -1240,10 +1276,27 @@ __global__ void k_hmc_canon_reset(HmcCtl* ctl) {
 // Two full steps per launch: two CTAs per SM (the registers' limit); the
 // tile-walking form when each would get at least kP2PrefMinTilesPerCta tiles
 // and the tensor maps are given, else one tile per CTA.
+}  // namespace
+
+bool hmc_tiled_ok(int L) { return L >= kTileCols && L % kTileCols == 0; }
+
+bool hmc_ragged_ok(int L) { return L > kTileCols && L % kTileCols != 0; }
+
+namespace {
+
 template <int MODE>
 cudaError_t launch_step2(const HmcArgs& a, const CUtensorMap* th_maps, const CUtensorMap* p_map,
                          cudaStream_t stream) {
-  if (!a.tiled || !a.pairs || a.p_in == a.p_out) return cudaErrorInvalidValue;
+  if (!a.pairs || a.p_in == a.p_out) return cudaErrorInvalidValue;
+  if (!hmc_tiled_ok(a.L)) {
+    if (!hmc_ragged_ok(a.L)) return cudaErrorInvalidValue;
+    Tile2Maps none;
+    memset(&none, 0, sizeof(none));
+    const dim3 grid((a.L + kP2Cols - 1) / kP2Cols, (a.L + kP2Rows - 1) / kP2Rows);
+    k_hmc_tile2<MODE, false, true><<<grid, kP2Threads, kP2Smem, stream>>>(a, none);
+    return cudaGetLastError();
+  }
+  if (!a.tiled) return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1288,8 +1341,6 @@ cudaError_t launch_mode(int kind, const HmcArgs& a, cudaStream_t stream) {
 
 }  // namespace
 
-bool hmc_tiled_ok(int L) { return L >= kTileCols && L % kTileCols == 0; }
-
 cudaError_t hmc_prepare(int sincos_mode) {
   static bool done[3][64] = {};
   int dev = 0;
@@ -1310,6 +1361,13 @@ cudaError_t hmc_prepare(int sincos_mode) {
     e = cudaFuncSetAttribute(fp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2SmemPref);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(fp, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  const void* fr = m == 0 ? (const void*)k_hmc_tile2<0, false, true>
+                          : (m == 1 ? (const void*)k_hmc_tile2<1, false, true>
+                                    : (const void*)k_hmc_tile2<2, false, true>);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2Smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fr, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   const void* g4 = m == 0 ? (const void*)k_hmc_step_tma<0, 4>
                           : (m == 1 ? (const void*)k_hmc_step_tma<1, 4> : (const void*)k_hmc_step_tma<2, 4>);
   if (e == cudaSuccess)

@@ -10,6 +10,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <new>
 #include <unordered_set>
@@ -23,6 +24,14 @@ namespace {
 
 constexpr uint32_t kMagicLive = 0x484D434Cu;   // "HMCL"
 constexpr uint32_t kMagicDead = 0xDEADBEEFu;
+
+// AUTO: from this side on the full steps run two per launch on 32 x 128 tiles
+// (overlapping ones where L is no multiple of 128), below it one launch per
+// step of one thread per site, which fills the GPU with fewer sites (us per
+// unit trajectory, two per launch / per site: L = 256 57.6 / 45.3, 320 62.4 /
+// 56.9, 384 66.0 / 68.7, 500 82.9 / 103, 1000 171 / 375, 1001 193 / 376, 2000
+// 704 / 1768).
+constexpr int kAutoPairsMinL = 352;
 
 thread_local char g_msg[512] = "no error";
 
@@ -59,6 +68,7 @@ struct xy_hmc {
   bool use_persist;                  // a trajectory's steps in one cooperative TMA launch
   unsigned int* d_tiles;             // its per-tile step counters
   bool use_cluster;                  // whole trajectories in one cluster launch
+  bool use_resident;                 // AUTO: many trajectories per cluster launch
   bool use_pairs;                    // full steps two per launch (k_hmc_tile2)
   int tma_rows;                      // tile (and box) rows of the TMA step kernel: 32 or 16
   int tma_ctas;                      // persistent grid of the TMA step kernel
@@ -226,7 +236,7 @@ xyk::HmcArgs args_of(const xy_hmc* h) {
   a.lattice_id = h->p.lattice_id;
   a.tiled = h->p.kernel == XY_HMC_KERNEL_TILED || h->p.kernel == XY_HMC_KERNEL_TILED2 ||
             h->p.kernel == XY_HMC_KERNEL_TILED_TMA || h->p.kernel == XY_HMC_KERNEL_PERSISTENT ||
-            (h->p.kernel == XY_HMC_KERNEL_AUTO && xyk::hmc_tiled_ok(h->p.L));
+            (h->p.kernel == XY_HMC_KERNEL_AUTO && h->use_pairs && xyk::hmc_tiled_ok(h->p.L));
   a.pairs = h->use_pairs ? 1 : 0;
   return a;
 }
@@ -239,6 +249,9 @@ xyk::HmcArgs args_of(const xy_hmc* h) {
 cudaError_t enqueue_trajectory(const xy_hmc* h, int begin, int n, int mode, cudaStream_t s) {
   xyk::HmcArgs a = args_of(h);
   const int m = h->p.sincos_mode;
+  if (h->use_resident)
+    return xyk::launch_hmc_resident(m, a, n, 1, begin == xyk::kHmcBeginDraw ? 1 : 0, mode,
+                                    h->p.beta, h->p.J, s);
   if (h->use_cluster)
     return xyk::launch_hmc_cluster(m, a, n, begin == xyk::kHmcBeginDraw ? 1 : 0, mode, h->p.beta,
                                    h->p.J, s);
@@ -422,19 +435,22 @@ xy_status xy_hmc_create(const xy_hmc_params* p, void* cuda_stream, void* d_angle
     step = "control block";
     e = xyk::dev_malloc(&h->d_ctl, sizeof(xyk::HmcCtl));
   }
-  // AUTO: the cluster kernel where it measured faster than the others (L =
-  // 128, 256); below that the per-launch cost of any kernel dominates
-  h->use_cluster = p->kernel == XY_HMC_KERNEL_CLUSTER ||
-                   (p->kernel == XY_HMC_KERNEL_AUTO && (p->L == 128 || p->L == 256));
-  // AUTO: full steps two per launch wherever the tiled kernels run (measured
-  // faster than one TMA-fed step per launch at L = 512 ... 4096); the odd
-  // step of a trajectory runs on the TMA kernel
-  h->use_pairs = p->kernel == XY_HMC_KERNEL_TILED2 ||
-                 (p->kernel == XY_HMC_KERNEL_AUTO && !h->use_cluster && xyk::hmc_tiled_ok(p->L));
+  // AUTO: lattices the chip can hold
+  if (e == cudaSuccess && p->kernel == XY_HMC_KERNEL_AUTO &&
+      xyk::prepare_hmc_resident(p->sincos_mode, p->L, &h->use_resident) != cudaSuccess) {
+    (void)cudaGetLastError();
+    h->use_resident = false;
+  }
+  h->use_cluster = p->kernel == XY_HMC_KERNEL_CLUSTER;
+  // AUTO: full steps two per launch (measured faster than one TMA-fed step per
+  // launch at L = 512 ... 4096); the odd step of a trajectory runs on the TMA
+  // kernel where the tiles divide the side, else one thread per site
+  const bool auto_pairs =
+      p->kernel == XY_HMC_KERNEL_AUTO && !h->use_resident && p->L >= kAutoPairsMinL;
+  h->use_pairs = p->kernel == XY_HMC_KERNEL_TILED2 || auto_pairs;
   const bool want_tma = p->kernel == XY_HMC_KERNEL_TILED_TMA || p->kernel == XY_HMC_KERNEL_PERSISTENT ||
                         p->kernel == XY_HMC_KERNEL_TILED2 ||
-                        (p->kernel == XY_HMC_KERNEL_AUTO && !h->use_cluster &&
-                         xyk::hmc_tiled_ok(p->L));
+                        (auto_pairs && xyk::hmc_tiled_ok(p->L));
   if (e == cudaSuccess && want_tma) {
     step = "tensor maps";
     int n_sm = 0;
@@ -495,7 +511,17 @@ xy_status xy_hmc_run(xy_hmc* h, int64_t n_traj) {
     return fail(h, XY_EINVAL, "xy_hmc_run: trajectory counter would pass 2^32 - 1");
   st = grow_records(h, h->rec_count + n_traj);
   if (st != XY_OK) return st;
-  if (h->use_persist) {
+  if (h->use_resident) {
+    // at most this many leap-frog steps in one launch (a fraction of a second)
+    const int64_t chunk = std::max<int64_t>(1, (1 << 17) / h->p.n_md);
+    for (int64_t done = 0; done < n_traj;) {
+      const int64_t m = std::min<int64_t>(n_traj - done, chunk);
+      H_CUDA(h, xyk::launch_hmc_resident(h->p.sincos_mode, args_of(h), h->p.n_md, (int)m, 1, 0,
+                                         h->p.beta, h->p.J, h->stream),
+             "xy_hmc_run: resident launch");
+      done += m;
+    }
+  } else if (h->use_persist) {
     // a trajectory is five launches here (begin, the counters' memset, the
     // steps, final, accept): launched directly, no graph
     H_CUDA(h, xyk::hmc_prepare(h->p.sincos_mode), "xy_hmc_run: kernel attributes");

@@ -166,6 +166,11 @@ __device__ __forceinline__ void hmc_buffers(const HmcArgs& a, uint32_t cur, int*
   *dst = (int)((cur + (uint32_t)a.dst_off) % 3u);
 }
 
+// dH in FP64 from the exact integer differences of K (2^-24) and C (2^-30).
+__device__ __forceinline__ double hmc_dH(long long dK, long long dC, double beta, double J) {
+  return (double)dK * 0x1p-24 - beta * J * ((double)dC * 0x1p-30);
+}
+
 // The test (mode 0: u < exp(-dH) with u = u24 of Philox counter (0, traj,
 // lattice id, 4), writes a record and advances the counters) or the commit of
 // a plain integration (mode 1).  dH is formed in FP64 from the exact integer
@@ -175,7 +180,7 @@ __device__ __forceinline__ bool hmc_decide(HmcCtl* c, uint32_t lattice_id, const
                                            int mode, double beta, double J) {
   const long long dK = (long long)(c->acc[1][0] - c->acc[0][0]);
   const long long dC = (long long)(c->acc[1][1] - c->acc[0][1]);
-  const double dH = (double)dK * 0x1p-24 - beta * J * ((double)dC * 0x1p-30);
+  const double dH = hmc_dH(dK, dC, beta, J);
   bool take = true;
   if (mode == 0) {
     const uint4 w = xyd::philox4x32_10(make_uint4(0u, (uint32_t)c->traj, lattice_id, 4u), rk);

@@ -435,13 +435,15 @@ struct HmcArgs {
   xyd::RoundKeys rk;
   uint32_t lattice_id;
   int tiled;             // 1: tiled kernels (needs hmc_tiled_ok(L)), 0: one thread per site
-  int pairs;             // 1: full steps two per launch (kHmcStep2; tiled only)
+  int pairs;             // 1: full steps two per launch (kHmcStep2)
 };
 
 // One leap-frog launch of `kind` with the tiled or the per-site kernel (both
 // give bit-identical results).
 cudaError_t launch_hmc(int kind, int sincos_mode, const HmcArgs& a, cudaStream_t stream);
 bool hmc_tiled_ok(int L);
+// Whether the two-step kernel takes L on overlapping tiles (kHmcStep2 only).
+bool hmc_ragged_ok(int L);
 // The test (mode 0: Metropolis on dH, writes a record) or, mode 1, the plain
 // commit of an integration; both move acc to last and clear acc.
 cudaError_t launch_hmc_accept(int mode, const HmcArgs& a, double beta, double J,
@@ -491,5 +493,12 @@ bool hmc_cluster_ok(int L);
 cudaError_t hmc_cluster_prepare(int sincos_mode);
 cudaError_t launch_hmc_cluster(int sincos_mode, const HmcArgs& a, int n_md, int draw, int mode,
                                double beta, double J, cudaStream_t stream);
+
+// n_traj trajectories in one cluster launch (xy_hmc_resident.cu), 4 <= L <= 176:
+// draw and mode as launch_hmc_cluster (mode 1: n_traj = 1).  prepare, outside
+// any capture: whether the side is held and the device can run its cluster.
+cudaError_t prepare_hmc_resident(int sincos_mode, int L, bool* fits);
+cudaError_t launch_hmc_resident(int sincos_mode, const HmcArgs& a, int n_md, int n_traj, int draw,
+                                int mode, double beta, double J, cudaStream_t stream);
 
 }  // namespace xyk

@@ -38,6 +38,7 @@
 
 #include "xy_device.cuh"
 #include "xy_internal.h"
+#include "xy_strip.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -49,18 +50,8 @@ constexpr int kRThreads = 512;               // at most; the launch takes what t
 constexpr int kRWarps = kRThreads / 32;
 constexpr int kRMaxPairs = 2;                // pairs per thread and colour
 
-__host__ __device__ inline int strip_rows(int L, int C, int rank) {
-  return L / C + (rank < L % C ? 1 : 0);
-}
-__host__ __device__ inline int strip_first(int L, int C, int rank) {
-  return rank * (L / C) + (rank < L % C ? rank : L % C);
-}
-
-// Unit vectors of one colour: (rows + 2) x (pairs + 2) float4, row r + 1 the
-// strip's row r, float4 m + 1 the pair m.
-__host__ __device__ inline int plane_vec4(int max_rows, int W) {
-  return (max_rows + 2) * ((W + 1) / 2 + 2);
-}
+using xys::plane_vec4;
+using xys::strip_rows;
 
 // NP: pairs of each colour a thread owns, at most.  (Blocks of 1024 threads leave
 // 64 registers a thread and spill the state: L = 256 4.6 against 3.5 us per
@@ -72,62 +63,20 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
   __shared__ uint32_t s_cnt[kRWarps];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = a.ctas, rank = (int)cluster.block_rank();
-  const int L = a.L, W = L / 2, Wp = (W + 1) / 2, Wq = Wp + 2;
-  const int max_rows = strip_rows(L, C, 0);
-  const int rows = strip_rows(L, C, rank), y0 = strip_first(L, C, rank);
-  const int npairs = rows * Wp;
+  const int L = a.L, W = L / 2;
+  const xys::Strip st(L, W, C, rank);
   const int nthreads = blockDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = nthreads >> 5;
   const size_t plane = (size_t)L * (size_t)W;
-  float4* cs = reinterpret_cast<float4*>(smem);            // [2][max_rows + 2][Wq]
-  const int pvec = plane_vec4(max_rows, W);
-  // the neighbouring strips: their halo row next to this strip's first / last row
-  const int up_rank = rank + 1 == C ? 0 : rank + 1, dn_rank = rank == 0 ? C - 1 : rank - 1;
-  float4* up_halo = cluster.map_shared_rank(cs, up_rank);                      // row 0
-  float4* dn_halo = cluster.map_shared_rank(cs, dn_rank) +
-                    (strip_rows(L, C, dn_rank) + 1) * Wq;                      // row rows + 1
-
-  // this thread's pairs
-  int at[NP];            // float4 of the pair in a plane
-  int yy[NP], kk[NP];    // row and first plane column
-  bool on[NP], two[NP];  // owned; its second column exists
+  float4* cs = reinterpret_cast<float4*>(smem);            // [2] planes
+  const int pvec = plane_vec4(strip_rows(L, C, 0), W);
+  float4* up_cs = cluster.map_shared_rank(cs, st.up_rank);
+  float4* dn_cs = cluster.map_shared_rank(cs, st.dn_rank);
+  xys::Pair pr[NP];                                        // this thread's pairs
 #pragma unroll
-  for (int p = 0; p < NP; ++p) {
-    const int i = threadIdx.x + p * nthreads;
-    on[p] = i < npairs;
-    const int r = on[p] ? i / Wp : 0, m = on[p] ? i - r * Wp : 0;
-    at[p] = (r + 1) * Wq + m + 1;
-    yy[p] = y0 + r;
-    kk[p] = 2 * m;
-    two[p] = 2 * m + 1 < W;
-  }
-  // stores of a pair's unit vectors of colour c: the strip, its halo columns
-  // (column 0's copy behind the last column, the last column's before column
-  // 0) and the neighbours' halo rows
+  for (int p = 0; p < NP; ++p) pr[p].set(st, threadIdx.x + p * nthreads);
   auto put = [&](int p, int c, float2 cv, float2 sv) {
-    float4* own = cs + c * pvec;
-    const float4 v = make_float4(cv.x, cv.y, sv.x, sv.y);
-    const int r = yy[p] - y0;
-    if (two[p]) {
-      own[at[p]] = v;
-    } else {                               // the halo copy in the second column stays
-      float* f = reinterpret_cast<float*>(&own[at[p]]);
-      f[0] = v.x;
-      f[2] = v.z;
-    }
-    float* row = reinterpret_cast<float*>(&own[(r + 1) * Wq]);
-    if (kk[p] == 0) {                      // column 0 -> column W
-      float* f = row + 4 * ((W + 2) >> 1) + (W & 1);
-      f[0] = v.x;
-      f[2] = v.z;
-    }
-    if (kk[p] + 2 >= W) {                  // column W - 1 -> column -1
-      row[1] = two[p] ? v.y : v.x;
-      row[3] = two[p] ? v.w : v.z;
-    }
-    const int m = (kk[p] >> 1) + 1;
-    if (r == 0) dn_halo[c * pvec + m] = v;
-    if (r == rows - 1) up_halo[c * pvec + m] = v;
+    xys::put(st, pr[p], cs + c * pvec, up_cs + c * pvec, dn_cs + c * pvec, cv, sv);
   };
 
   float2 th[2][NP], cv[2][NP], sv[2][NP];
@@ -136,17 +85,17 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       th[c][p] = make_float2(0.f, 0.f);
-      if (on[p]) {
-        const float* g = a.theta + c * plane + (size_t)yy[p] * W + kk[p];
+      if (pr[p].on) {
+        const float* g = a.theta + c * plane + (size_t)(st.y0 + pr[p].r) * W + pr[p].k;
         th[c][p].x = g[0];
-        if (two[p]) th[c][p].y = g[1];
+        if (pr[p].two) th[c][p].y = g[1];
       }
       xyd::unit_vector2<MODE>(th[c][p], &sv[c][p], &cv[c][p]);
     }
   auto words = [&](int p, int c, uint32_t sweep) {
-    const uint32_t y = (uint32_t)yy[p];
+    const uint32_t y = (uint32_t)(st.y0 + pr[p].r);
     return xyd::philox_pair_words(
-        y * (uint32_t)L + 2u * (uint32_t)kk[p] + ((y + (uint32_t)c) & 1u), sweep, a.lattice_id,
+        y * (uint32_t)L + 2u * (uint32_t)pr[p].k + ((y + (uint32_t)c) & 1u), sweep, a.lattice_id,
         a.rk);
   };
   uint4 w[NP];
@@ -157,7 +106,7 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
   for (int c = 0; c < 2; ++c)
 #pragma unroll
     for (int p = 0; p < NP; ++p)
-      if (on[p]) put(p, c, cv[c][p], sv[c][p]);
+      if (pr[p].on) put(p, c, cv[c][p], sv[c][p]);
   cluster.sync();
 
   // The previous sweep's sums, left in s_part / s_cnt before the barrier: one
@@ -198,10 +147,10 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
       const float4* nb = cs + (1 - c) * pvec;
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
-        if (!on[p]) continue;
-        const int q = (yy[p] + c) & 1;     // x = 2k + q
-        const float4 P = nb[at[p]], D = nb[at[p] - Wq], U = nb[at[p] + Wq];
-        const float4 E = nb[q ? at[p] + 1 : at[p] - 1];
+        if (!pr[p].on) continue;
+        const int q = (st.y0 + pr[p].r + c) & 1;     // x = 2k + q
+        const float4 P = nb[pr[p].at], D = nb[pr[p].at - st.pitch], U = nb[pr[p].at + st.pitch];
+        const float4 E = nb[q ? pr[p].at + 1 : pr[p].at - 1];
         xyd::PairNeighbours n;
         n.lc = q ? make_float2(P.x, P.y) : make_float2(E.y, P.x);
         n.ls = q ? make_float2(P.z, P.w) : make_float2(E.w, P.z);
@@ -218,12 +167,12 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
         cv[c][p] = r.c;
         sv[c][p] = r.s;
         put(p, c, r.c, r.s);
-        n_acc += (r.acc0 ? 1u : 0u) + (r.acc1 && two[p] ? 1u : 0u);
+        n_acc += (r.acc0 ? 1u : 0u) + (r.acc1 && pr[p].two ? 1u : 0u);
         if (c == 1) {
           // red sites with the same (y, k): their spins enter M once each
           float2 v[5];
           xyd::measure_terms2(r.c, r.s, n, make_float2(P.x, P.y), make_float2(P.z, P.w), v);
-          if (two[p]) {
+          if (pr[p].two) {
             sums.add2(v);
           } else {
             const float v0[5] = {v[0].x, v[1].x, v[2].x, v[3].x, v[4].x};
@@ -262,10 +211,10 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
   for (int c = 0; c < 2; ++c)
 #pragma unroll
     for (int p = 0; p < NP; ++p)
-      if (on[p]) {
-        float* g = a.theta + c * plane + (size_t)yy[p] * W + kk[p];
+      if (pr[p].on) {
+        float* g = a.theta + c * plane + (size_t)(st.y0 + pr[p].r) * W + pr[p].k;
         g[0] = th[c][p].x;
-        if (two[p]) g[1] = th[c][p].y;
+        if (pr[p].two) g[1] = th[c][p].y;
       }
 }
 
