@@ -8,6 +8,8 @@ there is no fallback path.
 import ctypes as C
 import os
 
+import numpy as np
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 # The library this process uses: libxy.so, or the debug build (libxy_debug.so)
 # when XY_GB300_LIB names it (the debug-build test runs in a child process).
@@ -46,6 +48,18 @@ class xy_obs(C.Structure):
     _fields_ = [("e", C.c_double), ("abs_m", C.c_double), ("upsilon", C.c_double),
                 ("C", C.c_double), ("Ix", C.c_double), ("Iy", C.c_double), ("Mx", C.c_double),
                 ("My", C.c_double), ("accepted", C.c_uint64), ("beta", C.c_double)]
+
+
+# xy_obs as a numpy record, and the order of the front ends' result dicts.
+OBS_DTYPE = np.dtype([(n, np.uint64 if n == "accepted" else np.float64) for n, _ in xy_obs._fields_])
+OBS_NAMES = ("e", "abs_m", "upsilon", "C", "Ix", "Iy", "Mx", "My", "beta", "accepted")
+
+
+def obs_arrays(obs):
+    """{name: array} of a ctypes array of xy_obs: one strided copy per field (reading 1000
+    records field by field took 1.6 ms of Python, more than the 1000 sweeps of L = 32)."""
+    a = np.frombuffer(obs, OBS_DTYPE) if len(obs) else np.empty(0, OBS_DTYPE)
+    return {n: a[n].copy() for n in OBS_NAMES}
 
 
 class xy_batch_params(C.Structure):

@@ -75,9 +75,7 @@ class HMC:
         count = n - first if count is None else count
         dH = np.zeros(max(count, 1), np.float64)
         obs = X.xy_hmc_measure(self.h, first, count, dH.ctypes.data_as(C.c_void_p))
-        names = ["e", "abs_m", "upsilon", "C", "Ix", "Iy", "Mx", "My", "beta"]
-        out = {k: np.array([getattr(o, k) for o in obs], np.float64) for k in names}
-        out["accepted"] = np.array([o.accepted for o in obs], np.uint64)
+        out = X.obs_arrays(obs)
         out["dH"] = dH[:count]
         return out
 

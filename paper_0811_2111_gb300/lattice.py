@@ -79,10 +79,7 @@ class Lattice:
         n, _ = X.xy_info(self.ctx)
         count = n - first if count is None else count
         obs = X.xy_measure(self.ctx, first, count)
-        names = ["e", "abs_m", "upsilon", "C", "Ix", "Iy", "Mx", "My", "beta"]
-        out = {k: np.array([getattr(o, k) for o in obs], np.float64) for k in names}
-        out["accepted"] = np.array([o.accepted for o in obs], np.uint64)
-        return out
+        return X.obs_arrays(obs)
 
     def state(self):
         buf = np.empty(self.L * self.L, np.float32)
@@ -214,10 +211,7 @@ class Batch:
         _, nrec, _, _ = X.xy_batch_info(self.b)
         count = nrec - first if count is None else count
         obs = X.xy_batch_measure(self.b, lattice, first, count)
-        names = ["e", "abs_m", "upsilon", "C", "Ix", "Iy", "Mx", "My", "beta"]
-        out = {k: np.array([getattr(o, k) for o in obs], np.float64) for k in names}
-        out["accepted"] = np.array([o.accepted for o in obs], np.uint64)
-        return out
+        return X.obs_arrays(obs)
 
     def betas(self):
         out = np.empty(self.n, np.float64)
@@ -318,10 +312,7 @@ class Quad:
         n, _ = X.xy_quad_info(self.q)
         count = n - first if count is None else count
         obs = X.xy_quad_measure(self.q, replica, first, count)
-        names = ["e", "abs_m", "upsilon", "C", "Ix", "Iy", "Mx", "My", "beta"]
-        out = {k: np.array([getattr(o, k) for o in obs], np.float64) for k in names}
-        out["accepted"] = np.array([o.accepted for o in obs], np.uint64)
-        return out
+        return X.obs_arrays(obs)
 
     def state(self, replica):
         buf = np.empty(self.L * self.L, np.float32)

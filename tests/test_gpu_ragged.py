@@ -71,3 +71,15 @@ def test_captured_sweeps_replay(L):
             g.replay()
             ref.sweep(4)
             assert np.array_equal(lat.state()[0], ref.state()[0])
+
+
+def test_a_large_state_lands_whole_in_a_fresh_array():
+    """State read into an array whose pages do not exist yet (touched in parallel first)."""
+    from paper_0811_2111_gb300.lattice import Lattice
+    with Lattice(1536, 1.0, 3) as lat:
+        a = lat.state()[0]
+        b = np.full((1536, 1536), 7.0, np.float32)
+        import ctypes as C
+        from paper_0811_2111_gb300 import _lib as X
+        X.xy_get_state(lat.ctx, b.ctypes.data_as(C.c_void_p))
+        assert np.array_equal(a, b)
