@@ -315,14 +315,14 @@ struct PairResult {
 };
 
 // metropolis_step of the two sites of a Philox pair (angles t, unit vectors
-// (c0, s0), neighbour sums (Sc, Ss), words w of philox_pair_words): the same
-// decisions and results, bit for bit.  The wrap's two candidates compare as
+// (c0, s0), neighbour sums (Sc, Ss), words w of philox_pair_words, each site's
+// K): the same decisions and results, bit for bit.  The wrap's two candidates compare as
 // unsigned bit patterns: of raw + 2 pi, raw and raw - 2 pi exactly the wanted
 // one has the smallest pattern (negative floats compare above positive ones;
 // raw is never -0, being a rounded sum with t >= 0).
 template <int MODE>
 __device__ __forceinline__ PairResult metropolis_pair(float2 t, float2 c0, float2 s0, float2 Sc,
-                                                      float2 Ss, const uint4& w, float K,
+                                                      float2 Ss, const uint4& w, float2 K,
                                                       float delta) {
   const float2 step = make_float2((float)((int32_t)w.x >> 8), (float)((int32_t)w.z >> 8));
   const float2 raw = fma2(dup2(delta * kR23), step, t);
@@ -336,7 +336,7 @@ __device__ __forceinline__ PairResult metropolis_pair(float2 t, float2 c0, float
   unit_vector2<MODE>(tp, &s1, &c1);
   const float2 X = fma2(sub2(c1, c0), Sc, mul2(sub2(s1, s0), Ss));
   PairResult r;
-  const float2 y = mul2(X, dup2(K));
+  const float2 y = mul2(X, K);
   r.acc0 = u24(w.y) < boltzmann<MODE>(y.x);
   r.acc1 = u24(w.w) < boltzmann<MODE>(y.y);
   r.th = make_float2(r.acc0 ? tp.x : t.x, r.acc1 ? tp.y : t.y);

@@ -427,7 +427,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const float2 t = *reinterpret_cast<const float2*>(&ang[kRedRaw0 + r][2 * lane]);
     const float4 o = csr[r - 1][pj];
     const xyd::PairResult p =
-        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, xyd::dup2(a.K), a.delta);
     if (!RAG) {
       n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
       put_pair(&csr[r - 1][pj], p.c, p.s);
@@ -457,7 +457,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const float2 t = *reinterpret_cast<const float2*>(&ang[kRedRaw0 + r][2 * lane]);
     const float4 o = csr[r - 1][pj];
     const xyd::PairResult p =
-        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, xyd::dup2(a.K), a.delta);
     if (RAG) {
       put_own(csr[r - 1], p);
     } else {
@@ -502,7 +502,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const float2 t = *reinterpret_cast<const float2*>(&ang[r][2 * lane]);
     const float4 o = csb[r][pj];
     const xyd::PairResult p =
-        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, a.K, a.delta);
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, xyd::dup2(a.K), a.delta);
     if (!RAG) {
       n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 ? 1u : 0u);
       *reinterpret_cast<float2*>(dst_blk + (size_t)y * W + kp) = p.th;

@@ -20,8 +20,12 @@
 // words under lattice id lattice_id0 + r, and K_r = beta_r J), so replica r is
 // bit for bit the single lattice with lattice id lattice_id0 + r.
 //
-// A lane updates two adjacent elements -- two replicas of one site -- so its
-// same-row neighbours are two aligned float4 loads of (cos, sin) pairs.
+// A lane updates two adjacent elements -- two replicas of one site -- together
+// on packed FP32 instructions; unit vectors are stored as (cos, cos, sin, sin)
+// of two elements, so its same-row neighbours are whole float4s.  Scalar / packed,
+// us per sweep: L = 256 8.1 / 6.8, 512 11.4 / 10.0, 1024 26.9 / 23.1, 4096 371 /
+// 335 (SFU sincos 289 / 281; CUDA's sincosf, which does not pack, 9.9 / 8.9 at
+// 256, 31.1 / 32.0 at 1024 and a tie at 2048).
 // Requires L % 32 == 0 (then 4W = 2L is a multiple of 64).
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -40,11 +44,12 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kSRows = kTileRows + 4;        // rows y0-2 .. y0+33
 constexpr int kSCols = kTileF + 8;           // elements f0-4 .. f0+67 (one halo site per side)
+constexpr int kSPairs = kSCols / 2;          // two adjacent elements per float4 of unit vectors
 constexpr int kRing = 2 * kTileF + kTileRows * kR;   // 256 ring elements, one per thread
 constexpr int kStageRowsTotal = kSRows + (kSRows - 2);
 
 constexpr size_t kThBytes = sizeof(float) * 2 * kSRows * kSCols;
-constexpr size_t kCsBytes = sizeof(float2) * 2 * kSRows * kSCols;
+constexpr size_t kCsBytes = sizeof(float4) * 2 * kSRows * kSPairs;
 constexpr size_t kPartBytes = sizeof(float) * kWarps * kR * 5 * 2;
 constexpr size_t kCntBytes = sizeof(unsigned int) * kWarps * kR;
 constexpr size_t kSmemBytes = kThBytes + kCsBytes + kPartBytes + kCntBytes;
@@ -52,7 +57,24 @@ constexpr size_t kSmemBytes = kThBytes + kCsBytes + kPartBytes + kCntBytes;
 static_assert(kRing == kThreads, "one ring element per thread");
 
 typedef float ThArr[kSRows][kSCols];
-typedef float2 CsArr[kSRows][kSCols];
+// (cos, cos, sin, sin) of stage columns 2j, 2j + 1: the packed instructions'
+// operands
+typedef float4 CsArr[kSRows][kSPairs];
+
+__device__ __forceinline__ float2 cosines(const float4& v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 sines(const float4& v) { return make_float2(v.z, v.w); }
+
+// The unit vector (cos, sin) at stage column c of a row.
+__device__ __forceinline__ float2 get_one(const float4* row, int c) {
+  const float* p = reinterpret_cast<const float*>(&row[c >> 1]) + (c & 1);
+  return make_float2(p[0], p[2]);
+}
+
+__device__ __forceinline__ void put_one(float4* row, int c, float cv, float sv) {
+  float* p = reinterpret_cast<float*>(&row[c >> 1]) + (c & 1);
+  p[0] = cv;
+  p[2] = sv;
+}
 
 __device__ __forceinline__ int wrap_once(int v, int n) {
   v += (v < 0) ? n : 0;
@@ -67,10 +89,11 @@ __device__ __forceinline__ float parity_sum(float v) {
   for (int o = 16; o > 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// (integers: one redux.sync per parity instead of four shuffles and adds)
 __device__ __forceinline__ unsigned int parity_sum(unsigned int v) {
-#pragma unroll
-  for (int o = 16; o > 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  const unsigned int even = __reduce_add_sync(0xffffffffu, (threadIdx.x & 1) ? 0u : v);
+  const unsigned int odd = __reduce_add_sync(0xffffffffu, (threadIdx.x & 1) ? v : 0u);
+  return (threadIdx.x & 1) ? odd : even;
 }
 
 // Per-thread sums of the two replicas a lane holds: exact fixed point
@@ -90,15 +113,23 @@ struct QuadSums {
       }
     }
   }
-  __device__ __forceinline__ void add(const float v0[5], const float v1[5]) {
+  // v: the terms of the lane's two replicas
+  __device__ __forceinline__ void add(const float2 v[5]) {
     if (RED == 0) {
-      xyd::fx_add(fx[0], v0);
-      xyd::fx_add(fx[1], v1);
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        const float2 b = xyd::fma2(v[i], xyd::dup2(i == 0 ? xyd::kFxScaleC : xyd::kFxScale),
+                                   xyd::dup2(xyd::kRoundMagic));
+        fx[0].s[i] += __float_as_uint(b.x);
+        fx[1].s[i] += __float_as_uint(b.y);
+      }
+      fx[0].n += 1u;
+      fx[1].n += 1u;
     } else {
 #pragma unroll
       for (int i = 0; i < 5; ++i) {
-        xyd::neumaier_add(acc[0][i], cmp[0][i], v0[i]);
-        xyd::neumaier_add(acc[1][i], cmp[1][i], v1[i]);
+        xyd::neumaier_add(acc[0][i], cmp[0][i], v[i].x);
+        xyd::neumaier_add(acc[1][i], cmp[1][i], v[i].y);
       }
     }
   }
@@ -194,35 +225,6 @@ __device__ __forceinline__ float replica_k(const QuadFusedArgs& a, int j) {
   return (j & 2) ? k23 : k01;
 }
 
-// Two adjacent elements (replicas j0, j0 + 1 of one site) of row r at stage
-// columns c0, c0 + 1 of colour `own`, against the other colour's plane `nb`:
-// same-row neighbours of the site at k + q - 1 (columns c0 + 4q - 4, +1) and
-// k + q (c0 + 4q, +1).
-struct PairNb {
-  float Sc[2], Ss[2];
-  float2 l[2], r[2], d[2], u[2];
-};
-
-__device__ __forceinline__ void pair_nb(const CsArr& nb, int r, int c0, int q, PairNb& n) {
-  const float4 Lf = *reinterpret_cast<const float4*>(&nb[r][c0 + 4 * q - 4]);
-  const float4 Rt = *reinterpret_cast<const float4*>(&nb[r][c0 + 4 * q]);
-  const float4 D = *reinterpret_cast<const float4*>(&nb[r - 1][c0]);
-  const float4 U = *reinterpret_cast<const float4*>(&nb[r + 1][c0]);
-  n.l[0] = make_float2(Lf.x, Lf.y);
-  n.l[1] = make_float2(Lf.z, Lf.w);
-  n.r[0] = make_float2(Rt.x, Rt.y);
-  n.r[1] = make_float2(Rt.z, Rt.w);
-  n.d[0] = make_float2(D.x, D.y);
-  n.d[1] = make_float2(D.z, D.w);
-  n.u[0] = make_float2(U.x, U.y);
-  n.u[1] = make_float2(U.z, U.w);
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    n.Sc[j] = xyd::nb_sum(n.l[j].x, n.r[j].x, n.d[j].x, n.u[j].x);
-    n.Ss[j] = xyd::nb_sum(n.l[j].y, n.r[j].y, n.d[j].y, n.u[j].y);
-  }
-}
-
 // Stage both planes of the tile (bx, by) as (angle, cos, sin): the black
 // plane's 36 rows (stage rows 0..35), then the red plane's 34 (stage rows
 // 1..34), 16 float4 (one site, four replicas) per row, plus the halo site on
@@ -264,14 +266,12 @@ __device__ __forceinline__ void quad_stage(const float* src, ThArr* th, CsArr* c
     vh = ld(hp * plane + (size_t)wrap_once(y0 - 2 + hr, L) * F + 4 * (size_t)ks);
   }
   auto put = [&](int p, int r, int col, float4 a, bool keep_angles) {
-    float s0, c0, s1, c1, s2, c2, s3, c3;
-    xyd::unit_vector<MODE>(a.x, &s0, &c0);
-    xyd::unit_vector<MODE>(a.y, &s1, &c1);
-    xyd::unit_vector<MODE>(a.z, &s2, &c2);
-    xyd::unit_vector<MODE>(a.w, &s3, &c3);
+    float2 s01, c01, s23, c23;
+    xyd::unit_vector2<MODE>(make_float2(a.x, a.y), &s01, &c01);
+    xyd::unit_vector2<MODE>(make_float2(a.z, a.w), &s23, &c23);
     if (keep_angles) *reinterpret_cast<float4*>(&th[p][r][col]) = a;
-    *reinterpret_cast<float4*>(&cs[p][r][col]) = make_float4(c0, s0, c1, s1);
-    *reinterpret_cast<float4*>(&cs[p][r][col + 2]) = make_float4(c2, s2, c3, s3);
+    cs[p][r][col >> 1] = make_float4(c01.x, c01.y, s01.x, s01.y);
+    cs[p][r][(col >> 1) + 1] = make_float4(c23.x, c23.y, s23.x, s23.y);
   };
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -284,28 +284,27 @@ __device__ __forceinline__ void quad_stage(const float* src, ThArr* th, CsArr* c
   if (has_halo) put(hp, hr, hside ? kTileF + 4 : 0, vh, hp == 0);
 }
 
-// pair_nb with the other colour's rows r - 1 and r of the pair's columns in
-// registers (D, P: the previous row's P and U, as a warp walks its rows
-// downwards): loads the same-row edge element and row r + 1 (returned in U).
-__device__ __forceinline__ void pair_nb_rolled(const CsArr& nb, int r, int c0, int q,
+// The neighbours of the two replicas of stage pair j (one site) of row r
+// against the other colour's plane `nb`: the site's same-row neighbours lie two
+// pairs to either side, one of them in the pair's own column (q = 1 left, q = 0
+// right).  The other colour's rows r - 1 and r of the pair come in registers
+// (D, P: the previous row's P and U, as a warp walks its rows downwards); row
+// r + 1 is loaded and returned in U.
+__device__ __forceinline__ void pair_nb_rolled(const CsArr& nb, int r, int j, int q,
                                                const float4 D, const float4 P, float4& U,
-                                               PairNb& n) {
-  const float4 E = *reinterpret_cast<const float4*>(&nb[r][q ? c0 + 4 : c0 - 4]);
-  U = *reinterpret_cast<const float4*>(&nb[r + 1][c0]);
+                                               xyd::PairNeighbours& n) {
+  const float4 E = nb[r][q ? j + 2 : j - 2];
+  U = nb[r + 1][j];
   const float4 Lf = q ? P : E, Rt = q ? E : P;
-  n.l[0] = make_float2(Lf.x, Lf.y);
-  n.l[1] = make_float2(Lf.z, Lf.w);
-  n.r[0] = make_float2(Rt.x, Rt.y);
-  n.r[1] = make_float2(Rt.z, Rt.w);
-  n.d[0] = make_float2(D.x, D.y);
-  n.d[1] = make_float2(D.z, D.w);
-  n.u[0] = make_float2(U.x, U.y);
-  n.u[1] = make_float2(U.z, U.w);
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    n.Sc[j] = xyd::nb_sum(n.l[j].x, n.r[j].x, n.d[j].x, n.u[j].x);
-    n.Ss[j] = xyd::nb_sum(n.l[j].y, n.r[j].y, n.d[j].y, n.u[j].y);
-  }
+  n.lc = cosines(Lf);
+  n.ls = sines(Lf);
+  n.rc = cosines(Rt);
+  n.rs = sines(Rt);
+  n.dc = cosines(D);
+  n.ds = sines(D);
+  n.uc = cosines(U);
+  n.us = sines(U);
+  n.sum();
 }
 
 struct NoHook {
@@ -348,7 +347,7 @@ __device__ __forceinline__ void quad_sweep_body(const Args& item, int bx, int by
 
   const int L = a.L, W = a.W;
   const int F = 4 * W;                                     // elements per plane row
-  const int f0 = bx * kTileF;                      // first element of the tile
+  const int f0 = bx * kTileF;                              // first element of the tile
   const int ks0 = f0 >> 2;                                 // its first site column
   const int y0 = by * kTileRows;
   const size_t plane = (size_t)L * (size_t)F;
@@ -360,49 +359,53 @@ __device__ __forceinline__ void quad_sweep_body(const Args& item, int bx, int by
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t uL = (uint32_t)L;
   const int c0 = 2 * lane + 4;                             // stage column of the lane's pair
+  const int pj = lane + 2;                                 // its float4 of unit vectors
   const int fp = f0 + 2 * lane;                            // element of the pair
   const int j0 = fp & 3;                                   // its replicas j0, j0 + 1
   const uint32_t kq = (uint32_t)(fp >> 2);                 // its site column
   const uint32_t id0 = a.lattice_id0 + (uint32_t)j0, id1 = id0 + 1u;
-  const float K0 = (lane & 1) ? a.K[2] : a.K[0];
-  const float K1 = (lane & 1) ? a.K[3] : a.K[1];
+  const float2 K = (lane & 1) ? make_float2(a.K[2], a.K[3]) : make_float2(a.K[0], a.K[1]);
   unsigned int n_acc[2] = {0u, 0u};
+  // (the persistent kernel with CUDA's sincosf: two rows unrolled, the code is
+  // long enough)
+  constexpr int kUnroll = COHERENT && MODE == 2 ? 2 : 4;
+  // The words of the lane's two replicas at its site of row y, colour c: lanes l
+  // and l ^ 2 hold replicas j0, j0 + 1 of a Philox pair's two sites (x & 2 ==
+  // lane & 2); each draws one replica's block, keeps its own half and passes
+  // the other half across.
+  auto words = [&](int y, int c) {
+    const uint32_t x = 2u * kq + (uint32_t)((y + c) & 1);
+    const bool up = (x & 2u) != 0u;
+    const uint4 wb = xyd::philox_pair_words(
+        xyd::metropolis_counter((uint32_t)y * uL + x, x), item.sweep, up ? id1 : id0, a.rk);
+    const uint32_t g0 = __shfl_xor_sync(0xffffffffu, up ? wb.x : wb.z, 2);
+    const uint32_t g1 = __shfl_xor_sync(0xffffffffu, up ? wb.y : wb.w, 2);
+    return up ? make_uint4(g0, g1, wb.z, wb.w) : make_uint4(wb.x, wb.y, g0, g1);
+  };
 
   // ---- red half: the tile (counted, written to dst) ----
-  float4 nbD = *reinterpret_cast<const float4*>(&cs[1][warp * 4 + 1][c0]);
-  float4 nbP = *reinterpret_cast<const float4*>(&cs[1][warp * 4 + 2][c0]);
-#pragma unroll 2
+  float4 nbD = cs[1][warp * 4 + 1][pj];
+  float4 nbP = cs[1][warp * 4 + 2][pj];
+#pragma unroll kUnroll
   for (int rr = 0; rr < 4; ++rr) {
     const int ty = warp * 4 + rr;
     const int y = y0 + ty;
     const int r = ty + 2;
     const int q = y & 1;                                   // red: x = 2k + (y & 1)
-    PairNb n;
+    xyd::PairNeighbours n;
     float4 nbU;
-    pair_nb_rolled(cs[1], r, c0, q, nbD, nbP, nbU, n);
+    pair_nb_rolled(cs[1], r, pj, q, nbD, nbP, nbU, n);
     nbD = nbP;
     nbP = nbU;
-    const uint32_t x = 2u * kq + (uint32_t)q;
-    const uint32_t ctr = xyd::metropolis_counter((uint32_t)y * uL + x, x);
-    // lanes l and l ^ 2 hold replicas j0, j0 + 1 of the pair's two sites
-    // (x & 2 == lane & 2): each draws one replica's block, keeps its own
-    // half and passes the other half across
-    const bool up = (x & 2u) != 0u;
-    const uint4 wb = xyd::philox4x32_10(make_uint4(ctr, item.sweep, up ? id1 : id0, 1u), a.rk);
-    const uint32_t g0 = __shfl_xor_sync(0xffffffffu, up ? wb.x : wb.z, 2);
-    const uint32_t g1 = __shfl_xor_sync(0xffffffffu, up ? wb.y : wb.w, 2);
-    const uint2 w0 = up ? make_uint2(g0, g1) : make_uint2(wb.x, wb.y);
-    const uint2 w1 = up ? make_uint2(wb.z, wb.w) : make_uint2(g0, g1);
+    const uint4 w = words(y, 0);
     const float2 t = *reinterpret_cast<const float2*>(&th[0][r][c0]);
-    const float4 o = *reinterpret_cast<const float4*>(&cs[0][r][c0]);
-    const xyd::SiteResult r0 =
-        xyd::metropolis_step<MODE>(t.x, o.x, o.y, n.Sc[0], n.Ss[0], w0.x, w0.y, K0, a.delta);
-    const xyd::SiteResult r1 =
-        xyd::metropolis_step<MODE>(t.y, o.z, o.w, n.Sc[1], n.Ss[1], w1.x, w1.y, K1, a.delta);
-    n_acc[0] += r0.accept ? 1u : 0u;
-    n_acc[1] += r1.accept ? 1u : 0u;
-    *reinterpret_cast<float4*>(&cs[0][r][c0]) = make_float4(r0.c, r0.s, r1.c, r1.s);
-    *reinterpret_cast<float2*>(item.dst + (size_t)y * F + fp) = make_float2(r0.th, r1.th);
+    const float4 o = cs[0][r][pj];
+    const xyd::PairResult p =
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, K, a.delta);
+    n_acc[0] += p.acc0 ? 1u : 0u;
+    n_acc[1] += p.acc1 ? 1u : 0u;
+    cs[0][r][pj] = make_float4(p.c.x, p.c.y, p.s.x, p.s.y);
+    *reinterpret_cast<float2*>(item.dst + (size_t)y * F + fp) = p.th;
   }
   // ---- red half: the ring at distance one (recomputed, not counted) ----
   // rows -1 and 32 (64 elements each): one lane per pair of sites (sites 2j
@@ -419,21 +422,23 @@ __device__ __forceinline__ void quad_sweep_body(const Args& item, int bx, int by
     const int y = wrap_once(y0 + ty, L);
     const int q = y & 1;
     const uint32_t x = 2u * (uint32_t)(ks0 + 2 * (j >> 2)) + (uint32_t)q;   // x & 2 == 0
-    const uint4 w = xyd::philox4x32_10(
-        make_uint4((uint32_t)y * uL + x, item.sweep, a.lattice_id0 + (uint32_t)rep, 1u), a.rk);
-    const float K = replica_k(a, rep);
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int c = sc + 4 * e;
-      const float2 l = cs[1][r][c + 4 * q - 4], rt = cs[1][r][c + 4 * q];
-      const float2 d = cs[1][r - 1][c], u = cs[1][r + 1][c];
-      const float Sc = xyd::nb_sum(l.x, rt.x, d.x, u.x);
-      const float Ss = xyd::nb_sum(l.y, rt.y, d.y, u.y);
-      const float2 own = cs[0][r][c];
-      const xyd::SiteResult res = xyd::metropolis_step<MODE>(
-          th[0][r][c], own.x, own.y, Sc, Ss, e ? w.z : w.x, e ? w.w : w.y, K, a.delta);
-      cs[0][r][c] = make_float2(res.c, res.s);
-    }
+    const uint4 w = xyd::philox_pair_words((uint32_t)y * uL + x, item.sweep,
+                                           a.lattice_id0 + (uint32_t)rep, a.rk);
+    // the two sites, sc and sc + 4; their same-row neighbours sc + 4q - 4,
+    // sc + 4q and sc + 4q, sc + 4q + 4
+    const float4* row = cs[1][r];
+    const float2 l = get_one(row, sc + 4 * q - 4), m = get_one(row, sc + 4 * q),
+                 e = get_one(row, sc + 4 * q + 4);
+    const float2 d0 = get_one(cs[1][r - 1], sc), d1 = get_one(cs[1][r - 1], sc + 4);
+    const float2 u0 = get_one(cs[1][r + 1], sc), u1 = get_one(cs[1][r + 1], sc + 4);
+    const float2 Sc = make_float2(xyd::nb_sum(l.x, m.x, d0.x, u0.x), xyd::nb_sum(m.x, e.x, d1.x, u1.x));
+    const float2 Ss = make_float2(xyd::nb_sum(l.y, m.y, d0.y, u0.y), xyd::nb_sum(m.y, e.y, d1.y, u1.y));
+    const float2 o0 = get_one(cs[0][r], sc), o1 = get_one(cs[0][r], sc + 4);
+    const xyd::PairResult p = xyd::metropolis_pair<MODE>(
+        make_float2(th[0][r][sc], th[0][r][sc + 4]), make_float2(o0.x, o1.x),
+        make_float2(o0.y, o1.y), Sc, Ss, w, xyd::dup2(replica_k(a, rep)), a.delta);
+    put_one(cs[0][r], sc, p.c.x, p.s.x);
+    put_one(cs[0][r], sc + 4, p.c.y, p.s.y);
   } else if (threadIdx.x < 64 + kTileRows * kR) {
     const int e = threadIdx.x - 64;
     const int ty = e >> 2;
@@ -445,17 +450,17 @@ __device__ __forceinline__ void quad_sweep_body(const Args& item, int bx, int by
     const int j = sc & 3;
     const uint32_t x = 2u * (uint32_t)ks + (uint32_t)q;
     const uint32_t site = (uint32_t)y * uL + x;
-    const float2 l = cs[1][r][sc + 4 * q - 4], rt = cs[1][r][sc + 4 * q];
-    const float2 d = cs[1][r - 1][sc], u = cs[1][r + 1][sc];
+    const float2 l = get_one(cs[1][r], sc + 4 * q - 4), rt = get_one(cs[1][r], sc + 4 * q);
+    const float2 d = get_one(cs[1][r - 1], sc), u = get_one(cs[1][r + 1], sc);
     const float Sc = xyd::nb_sum(l.x, rt.x, d.x, u.x);
     const float Ss = xyd::nb_sum(l.y, rt.y, d.y, u.y);
     const uint4 w = xyd::philox4x32_10(
         make_uint4(xyd::metropolis_counter(site, x), item.sweep, a.lattice_id0 + (uint32_t)j, 1u), a.rk);
     const uint2 uw = xyd::metropolis_words(w, x);
-    const float2 own = cs[0][r][sc];
+    const float2 own = get_one(cs[0][r], sc);
     const xyd::SiteResult res = xyd::metropolis_step<MODE>(th[0][r][sc], own.x, own.y, Sc, Ss,
                                                            uw.x, uw.y, replica_k(a, j), a.delta);
-    cs[0][r][sc] = make_float2(res.c, res.s);
+    put_one(cs[0][r], sc, res.c, res.s);
   }
   mid();
   __syncthreads();
@@ -464,48 +469,33 @@ __device__ __forceinline__ void quad_sweep_body(const Args& item, int bx, int by
   QuadSums<RED> sums;
   sums.init();
   float* dst_blk = item.dst + plane;
-  nbD = *reinterpret_cast<const float4*>(&cs[0][warp * 4 + 1][c0]);
-  nbP = *reinterpret_cast<const float4*>(&cs[0][warp * 4 + 2][c0]);
-#pragma unroll 2
+  nbD = cs[0][warp * 4 + 1][pj];
+  nbP = cs[0][warp * 4 + 2][pj];
+#pragma unroll kUnroll
   for (int rr = 0; rr < 4; ++rr) {
     const int ty = warp * 4 + rr;
     const int y = y0 + ty;
     const int r = ty + 2;
     const int q = (y + 1) & 1;                             // black: x = 2k + ((y + 1) & 1)
-    PairNb n;
+    xyd::PairNeighbours n;
     float4 nbU;
-    pair_nb_rolled(cs[0], r, c0, q, nbD, nbP, nbU, n);
+    pair_nb_rolled(cs[0], r, pj, q, nbD, nbP, nbU, n);
     const float4 m = nbP;                                  // the red pair of the same row
     nbD = nbP;
     nbP = nbU;
-    const uint32_t x = 2u * kq + (uint32_t)q;
-    const uint32_t ctr = xyd::metropolis_counter((uint32_t)y * uL + x, x);
-    // lanes l and l ^ 2 hold replicas j0, j0 + 1 of the pair's two sites
-    // (x & 2 == lane & 2): each draws one replica's block, keeps its own
-    // half and passes the other half across
-    const bool up = (x & 2u) != 0u;
-    const uint4 wb = xyd::philox4x32_10(make_uint4(ctr, item.sweep, up ? id1 : id0, 1u), a.rk);
-    const uint32_t g0 = __shfl_xor_sync(0xffffffffu, up ? wb.x : wb.z, 2);
-    const uint32_t g1 = __shfl_xor_sync(0xffffffffu, up ? wb.y : wb.w, 2);
-    const uint2 w0 = up ? make_uint2(g0, g1) : make_uint2(wb.x, wb.y);
-    const uint2 w1 = up ? make_uint2(wb.z, wb.w) : make_uint2(g0, g1);
+    const uint4 w = words(y, 1);
     const float2 t = *reinterpret_cast<const float2*>(&th[1][r][c0]);
-    const float4 o = *reinterpret_cast<const float4*>(&cs[1][r][c0]);
-    const xyd::SiteResult r0 =
-        xyd::metropolis_step<MODE>(t.x, o.x, o.y, n.Sc[0], n.Ss[0], w0.x, w0.y, K0, a.delta);
-    const xyd::SiteResult r1 =
-        xyd::metropolis_step<MODE>(t.y, o.z, o.w, n.Sc[1], n.Ss[1], w1.x, w1.y, K1, a.delta);
-    n_acc[0] += r0.accept ? 1u : 0u;
-    n_acc[1] += r1.accept ? 1u : 0u;
-    *reinterpret_cast<float2*>(dst_blk + (size_t)y * F + fp) = make_float2(r0.th, r1.th);
+    const float4 o = cs[1][r][pj];
+    const xyd::PairResult p =
+        xyd::metropolis_pair<MODE>(t, cosines(o), sines(o), n.Sc, n.Ss, w, K, a.delta);
+    n_acc[0] += p.acc0 ? 1u : 0u;
+    n_acc[1] += p.acc1 ? 1u : 0u;
+    *reinterpret_cast<float2*>(dst_blk + (size_t)y * F + fp) = p.th;
 
     // red elements with the same (y, k, replica): their spins enter M once each
-    float v0[5], v1[5];
-    xyd::measure_terms(r0.c, r0.s, n.l[0].x, n.l[0].y, n.r[0].x, n.r[0].y, n.d[0].x, n.d[0].y,
-                       n.u[0].x, n.u[0].y, n.Sc[0], n.Ss[0], m.x, m.y, v0);
-    xyd::measure_terms(r1.c, r1.s, n.l[1].x, n.l[1].y, n.r[1].x, n.r[1].y, n.d[1].x, n.d[1].y,
-                       n.u[1].x, n.u[1].y, n.Sc[1], n.Ss[1], m.z, m.w, v1);
-    sums.add(v0, v1);
+    float2 v[5];
+    xyd::measure_terms2(p.c, p.s, n, cosines(m), sines(m), v);
+    sums.add(v);
   }
 
   end();
@@ -513,184 +503,9 @@ __device__ __forceinline__ void quad_sweep_body(const Args& item, int bx, int by
   quad_commit<RED>(sums, n_acc, part, cnt, item.rec, a.beta, bx == 0 && by == 0, j0);
 }
 
-// The per-sweep kernel keeps its own copy of the tile arithmetic of
-// quad_sweep_body (identical statements; the two are tested bit for bit
-// against each other): compiled through the shared template body it issued
-// 2.5 % more instructions (363.7 M against 354.6 M warp instructions per
-// L = 4096 launch) and took 4 % longer.
 template <int MODE, int RED>
 __global__ void __launch_bounds__(kThreads, 3) k_quad_fused(QuadFusedArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  ThArr* th = reinterpret_cast<ThArr*>(smem);
-  CsArr* cs = reinterpret_cast<CsArr*>(smem + kThBytes);
-  float(*part)[kR][5][2] = reinterpret_cast<float(*)[kR][5][2]>(smem + kThBytes + kCsBytes);
-  unsigned int(*cnt)[kR] =
-      reinterpret_cast<unsigned int(*)[kR]>(smem + kThBytes + kCsBytes + kPartBytes);
-
-  const int L = a.L, W = a.W;
-  const int F = 4 * W;                                     // elements per plane row
-  const int f0 = blockIdx.x * kTileF;                      // first element of the tile
-  const int ks0 = f0 >> 2;                                 // its first site column
-  const int y0 = blockIdx.y * kTileRows;
-  const size_t plane = (size_t)L * (size_t)F;
-
-  // ---- stage both planes (angle + unit vector) ----
-  quad_stage<MODE, false>(a.src, th, cs, y0, f0, ks0, L, W, F, plane);
-  __syncthreads();
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t uL = (uint32_t)L;
-  const int c0 = 2 * lane + 4;                             // stage column of the lane's pair
-  const int fp = f0 + 2 * lane;                            // element of the pair
-  const int j0 = fp & 3;                                   // its replicas j0, j0 + 1
-  const uint32_t kq = (uint32_t)(fp >> 2);                 // its site column
-  const uint32_t id0 = a.lattice_id0 + (uint32_t)j0, id1 = id0 + 1u;
-  const float K0 = (lane & 1) ? a.K[2] : a.K[0];
-  const float K1 = (lane & 1) ? a.K[3] : a.K[1];
-  unsigned int n_acc[2] = {0u, 0u};
-
-  // ---- red half: the tile (counted, written to dst) ----
-  float4 nbD = *reinterpret_cast<const float4*>(&cs[1][warp * 4 + 1][c0]);
-  float4 nbP = *reinterpret_cast<const float4*>(&cs[1][warp * 4 + 2][c0]);
-#pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int ty = warp * 4 + rr;
-    const int y = y0 + ty;
-    const int r = ty + 2;
-    const int q = y & 1;                                   // red: x = 2k + (y & 1)
-    PairNb n;
-    float4 nbU;
-    pair_nb_rolled(cs[1], r, c0, q, nbD, nbP, nbU, n);
-    nbD = nbP;
-    nbP = nbU;
-    const uint32_t x = 2u * kq + (uint32_t)q;
-    const uint32_t ctr = xyd::metropolis_counter((uint32_t)y * uL + x, x);
-    // lanes l and l ^ 2 hold replicas j0, j0 + 1 of the pair's two sites
-    // (x & 2 == lane & 2): each draws one replica's block, keeps its own
-    // half and passes the other half across
-    const bool up = (x & 2u) != 0u;
-    const uint4 wb = xyd::philox4x32_10(make_uint4(ctr, a.sweep, up ? id1 : id0, 1u), a.rk);
-    const uint32_t g0 = __shfl_xor_sync(0xffffffffu, up ? wb.x : wb.z, 2);
-    const uint32_t g1 = __shfl_xor_sync(0xffffffffu, up ? wb.y : wb.w, 2);
-    const uint2 w0 = up ? make_uint2(g0, g1) : make_uint2(wb.x, wb.y);
-    const uint2 w1 = up ? make_uint2(wb.z, wb.w) : make_uint2(g0, g1);
-    const float2 t = *reinterpret_cast<const float2*>(&th[0][r][c0]);
-    const float4 o = *reinterpret_cast<const float4*>(&cs[0][r][c0]);
-    const xyd::SiteResult r0 =
-        xyd::metropolis_step<MODE>(t.x, o.x, o.y, n.Sc[0], n.Ss[0], w0.x, w0.y, K0, a.delta);
-    const xyd::SiteResult r1 =
-        xyd::metropolis_step<MODE>(t.y, o.z, o.w, n.Sc[1], n.Ss[1], w1.x, w1.y, K1, a.delta);
-    n_acc[0] += r0.accept ? 1u : 0u;
-    n_acc[1] += r1.accept ? 1u : 0u;
-    *reinterpret_cast<float4*>(&cs[0][r][c0]) = make_float4(r0.c, r0.s, r1.c, r1.s);
-    *reinterpret_cast<float2*>(a.dst + (size_t)y * F + fp) = make_float2(r0.th, r1.th);
-  }
-  // ---- red half: the ring at distance one (recomputed, not counted) ----
-  // rows -1 and 32 (64 elements each): one lane per pair of sites (sites 2j
-  // and 2j + 1 of the tile row share a Philox block, as in the tile) and
-  // replica, warps 0 and 1; the halo site of rows 0..31 on the side the black
-  // tile reaches (left on odd rows, right on even; 128 elements), one per lane
-  // of warps 2..5.  Warps 6 and 7 wait at the barrier.
-  if (threadIdx.x < 64) {
-    const int ty = threadIdx.x < 32 ? -1 : kTileRows;
-    const int j = threadIdx.x & 31;
-    const int rep = j & 3;                                 // replica
-    const int sc = 4 + 8 * (j >> 2) + rep;                 // element of site 2 (j >> 2)
-    const int r = ty + 2;
-    const int y = wrap_once(y0 + ty, L);
-    const int q = y & 1;
-    const uint32_t x = 2u * (uint32_t)(ks0 + 2 * (j >> 2)) + (uint32_t)q;   // x & 2 == 0
-    const uint4 w = xyd::philox4x32_10(
-        make_uint4((uint32_t)y * uL + x, a.sweep, a.lattice_id0 + (uint32_t)rep, 1u), a.rk);
-    const float K = replica_k(a, rep);
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int c = sc + 4 * e;
-      const float2 l = cs[1][r][c + 4 * q - 4], rt = cs[1][r][c + 4 * q];
-      const float2 d = cs[1][r - 1][c], u = cs[1][r + 1][c];
-      const float Sc = xyd::nb_sum(l.x, rt.x, d.x, u.x);
-      const float Ss = xyd::nb_sum(l.y, rt.y, d.y, u.y);
-      const float2 own = cs[0][r][c];
-      const xyd::SiteResult res = xyd::metropolis_step<MODE>(
-          th[0][r][c], own.x, own.y, Sc, Ss, e ? w.z : w.x, e ? w.w : w.y, K, a.delta);
-      cs[0][r][c] = make_float2(res.c, res.s);
-    }
-  } else if (threadIdx.x < 64 + kTileRows * kR) {
-    const int e = threadIdx.x - 64;
-    const int ty = e >> 2;
-    const int sc = (((y0 + ty) & 1) ? 0 : kTileF + 4) + (e & 3);
-    const int r = ty + 2;
-    const int y = y0 + ty;
-    const int q = y & 1;
-    const int ks = wrap_once(ks0 + ((sc - 4) >> 2), W);   // floor: stage columns 0..3 -> ks0 - 1
-    const int j = sc & 3;
-    const uint32_t x = 2u * (uint32_t)ks + (uint32_t)q;
-    const uint32_t site = (uint32_t)y * uL + x;
-    const float2 l = cs[1][r][sc + 4 * q - 4], rt = cs[1][r][sc + 4 * q];
-    const float2 d = cs[1][r - 1][sc], u = cs[1][r + 1][sc];
-    const float Sc = xyd::nb_sum(l.x, rt.x, d.x, u.x);
-    const float Ss = xyd::nb_sum(l.y, rt.y, d.y, u.y);
-    const uint4 w = xyd::philox4x32_10(
-        make_uint4(xyd::metropolis_counter(site, x), a.sweep, a.lattice_id0 + (uint32_t)j, 1u), a.rk);
-    const uint2 uw = xyd::metropolis_words(w, x);
-    const float2 own = cs[0][r][sc];
-    const xyd::SiteResult res = xyd::metropolis_step<MODE>(th[0][r][sc], own.x, own.y, Sc, Ss,
-                                                           uw.x, uw.y, replica_k(a, j), a.delta);
-    cs[0][r][sc] = make_float2(res.c, res.s);
-  }
-  __syncthreads();
-
-  // ---- black half of the tile, with the sweep sums ----
-  QuadSums<RED> sums;
-  sums.init();
-  float* dst_blk = a.dst + plane;
-  nbD = *reinterpret_cast<const float4*>(&cs[0][warp * 4 + 1][c0]);
-  nbP = *reinterpret_cast<const float4*>(&cs[0][warp * 4 + 2][c0]);
-#pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int ty = warp * 4 + rr;
-    const int y = y0 + ty;
-    const int r = ty + 2;
-    const int q = (y + 1) & 1;                             // black: x = 2k + ((y + 1) & 1)
-    PairNb n;
-    float4 nbU;
-    pair_nb_rolled(cs[0], r, c0, q, nbD, nbP, nbU, n);
-    const float4 m = nbP;                                  // the red pair of the same row
-    nbD = nbP;
-    nbP = nbU;
-    const uint32_t x = 2u * kq + (uint32_t)q;
-    const uint32_t ctr = xyd::metropolis_counter((uint32_t)y * uL + x, x);
-    // lanes l and l ^ 2 hold replicas j0, j0 + 1 of the pair's two sites
-    // (x & 2 == lane & 2): each draws one replica's block, keeps its own
-    // half and passes the other half across
-    const bool up = (x & 2u) != 0u;
-    const uint4 wb = xyd::philox4x32_10(make_uint4(ctr, a.sweep, up ? id1 : id0, 1u), a.rk);
-    const uint32_t g0 = __shfl_xor_sync(0xffffffffu, up ? wb.x : wb.z, 2);
-    const uint32_t g1 = __shfl_xor_sync(0xffffffffu, up ? wb.y : wb.w, 2);
-    const uint2 w0 = up ? make_uint2(g0, g1) : make_uint2(wb.x, wb.y);
-    const uint2 w1 = up ? make_uint2(wb.z, wb.w) : make_uint2(g0, g1);
-    const float2 t = *reinterpret_cast<const float2*>(&th[1][r][c0]);
-    const float4 o = *reinterpret_cast<const float4*>(&cs[1][r][c0]);
-    const xyd::SiteResult r0 =
-        xyd::metropolis_step<MODE>(t.x, o.x, o.y, n.Sc[0], n.Ss[0], w0.x, w0.y, K0, a.delta);
-    const xyd::SiteResult r1 =
-        xyd::metropolis_step<MODE>(t.y, o.z, o.w, n.Sc[1], n.Ss[1], w1.x, w1.y, K1, a.delta);
-    n_acc[0] += r0.accept ? 1u : 0u;
-    n_acc[1] += r1.accept ? 1u : 0u;
-    *reinterpret_cast<float2*>(dst_blk + (size_t)y * F + fp) = make_float2(r0.th, r1.th);
-
-    // red elements with the same (y, k, replica): their spins enter M once each
-    float v0[5], v1[5];
-    xyd::measure_terms(r0.c, r0.s, n.l[0].x, n.l[0].y, n.r[0].x, n.r[0].y, n.d[0].x, n.d[0].y,
-                       n.u[0].x, n.u[0].y, n.Sc[0], n.Ss[0], m.x, m.y, v0);
-    xyd::measure_terms(r1.c, r1.s, n.l[1].x, n.l[1].y, n.r[1].x, n.r[1].y, n.d[1].x, n.d[1].y,
-                       n.u[1].x, n.u[1].y, n.Sc[1], n.Ss[1], m.z, m.w, v1);
-    sums.add(v0, v1);
-  }
-
-  // ---- per-replica sums -> records ----
-  quad_commit<RED>(sums, n_acc, part, cnt, a.rec, a.beta,
-                   blockIdx.x == 0 && blockIdx.y == 0, j0);
+  quad_sweep_body<MODE, RED, false>(a, blockIdx.x, blockIdx.y);
 }
 
 // Polls of a tile counter before a wait gives up (with a short sleep between
@@ -720,8 +535,8 @@ __device__ __forceinline__ void q_store_release(unsigned int* p, unsigned int v)
 // one that runs out sets *error and ends the CTA, and waiting CTAs that see
 // *error end too.  The tile arithmetic is quad_sweep_body's, so the result is
 // bit for bit that of one k_quad_fused launch per sweep.
-template <int MODE, int RED>
-__global__ void __launch_bounds__(kThreads, 3) k_quad_fused_persist(QuadPersistArgs p) {
+template <int MODE, int RED, int MINB>
+__global__ void __launch_bounds__(kThreads, MINB) k_quad_fused_persist(QuadPersistArgs p) {
   __shared__ int s_abort;
   __shared__ int s_item[2];
   __shared__ int s_ready[2];
@@ -805,9 +620,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_quad_fused_persist(QuadPersistA
   }
 }
 
-template <int MODE, int RED>
-cudaError_t launch_persist_one(const QuadPersistArgs& p, cudaStream_t stream) {
-  auto fn = k_quad_fused_persist<MODE, RED>;
+template <int MODE, int RED, int MINB>
+cudaError_t launch_persist_plan(const QuadPersistArgs& p, cudaStream_t stream) {
+  auto fn = k_quad_fused_persist<MODE, RED, MINB>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int per_sm = 0, dev = 0, sms = 0;
@@ -824,6 +639,20 @@ cudaError_t launch_persist_one(const QuadPersistArgs& p, cudaStream_t stream) {
   void* args[] = {const_cast<QuadPersistArgs*>(&p)};
   return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fn), dim3(grid), dim3(kThreads),
                                      args, kSmemBytes, stream);
+}
+
+template <int MODE, int RED>
+cudaError_t launch_persist_one(const QuadPersistArgs& p, cudaStream_t stream) {
+  // where two CTAs per SM hold all of a sweep's tiles a sweep is one tile's
+  // latency and 128 registers a thread shorten it (L = 256 6.8 against 7.3 us
+  // per sweep, 512 10.1 against 10.5); else three hide it better (1024 23.0
+  // against 23.8)
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  return quad_persistent_tiles(p.a.L) <= 2 * sms ? launch_persist_plan<MODE, RED, 2>(p, stream)
+                                                 : launch_persist_plan<MODE, RED, 3>(p, stream);
 }
 
 template <int MODE, int RED>

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
         n.us = make_float2(U.z, U.w);
         n.sum();
         const xyd::PairResult r = xyd::metropolis_pair<MODE>(th[c][p], cv[c][p], sv[c][p], n.Sc,
-                                                             n.Ss, w[p], a.K, a.delta);
+                                                             n.Ss, w[p], xyd::dup2(a.K), a.delta);
         th[c][p] = r.th;
         cv[c][p] = r.c;
         sv[c][p] = r.s;
