@@ -324,6 +324,10 @@ cudaError_t launch_narrow_batch_sweep(int sincos_mode, int reduce_mode, const Fu
 // one), which is exactly what recomputing it from the stored angle would give,
 // so every site update -- and each lattice's state -- is bit for bit that of
 // the single-lattice kernels, at one sincos per update instead of two.
+// With L / 2 even a pair's two sites run together on packed FP32 instructions
+// (200 lattices of L = 96: 11.6 -> 11.3 us per sweep of all, compensated sums
+// 13.1 -> 12.5; SFU sincos 9.2 -> 9.4): a dependent chain per pair at 16 warps an
+// SM bounds it.
 // ---------------------------------------------------------------------------
 namespace xyk {
 
@@ -383,12 +387,23 @@ __global__ void __launch_bounds__(kSThreads, 2) k_batch_small(SmallBatchArgs a) 
     }
   };
 
-  for (int i = threadIdx.x; i < 2 * half; i += kSThreads) {
-    const float t = __ldg(src + i);
-    float s, c;
-    xyd::unit_vector<MODE>(t, &s, &c);
-    th[i] = t;
-    cs[i] = make_float2(c, s);
+  float4* vec = reinterpret_cast<float4*>(cs);
+  if (paired) {
+    for (int i = threadIdx.x; i < half; i += kSThreads) {   // both colours' pairs
+      const float2 t = __ldg(reinterpret_cast<const float2*>(src) + i);
+      float2 s, c;
+      xyd::unit_vector2<MODE>(t, &s, &c);
+      reinterpret_cast<float2*>(th)[i] = t;
+      vec[i] = make_float4(c.x, c.y, s.x, s.y);
+    }
+  } else {
+    for (int i = threadIdx.x; i < 2 * half; i += kSThreads) {
+      const float t = __ldg(src + i);
+      float s, c;
+      xyd::unit_vector<MODE>(t, &s, &c);
+      th[i] = t;
+      cs[i] = make_float2(c, s);
+    }
   }
   __syncthreads();
 
@@ -400,88 +415,54 @@ __global__ void __launch_bounds__(kSThreads, 2) k_batch_small(SmallBatchArgs a) 
     sums.init();
     auto add_terms = [&](const float* v) { sums.add(v); };
     if (paired) {
-      // ---- red half, a pair per step: sites k = 2m and k + 1 of row y
-      // (flat index o = 2P); left/right neighbours k+q-1, k+q for the first,
-      // k+q, k+q+1 for the second ----
-      for (int P = threadIdx.x, y = py0, m = pm0; P < npairs; P += kSThreads) {
-        // debug build: the carried (y, m) is the pair's position, in range
-        if (!XY_DCHECK(y >= 0 && y < L && m >= 0 && m < Wp && y * Wp + m == P, 0)) {
+      // A pair's unit vectors are one float4 (cos, cos, sin, sin): pair P of
+      // colour c is vec[c * npairs + P].
+      auto half_sweep = [&](int c) {
+        const float4* nb = vec + (1 - c) * npairs;
+        for (int P = threadIdx.x, y = py0, m = pm0; P < npairs; P += kSThreads) {
+          // debug build: the carried (y, m) is the pair's position, in range
+          if (!XY_DCHECK(y >= 0 && y < L && m >= 0 && m < Wp && y * Wp + m == P, 0)) {
+            step_pair(y, m);
+            continue;
+          }
+          const int q = (y + c) & 1;                                 // x = 2k + q
+          const int yd = y == 0 ? L - 1 : y - 1, yu = y == L - 1 ? 0 : y + 1;
+          // same-row neighbours: the pair's own columns and one of the pair
+          // before (q = 0) or after (q = 1)
+          const int me = q ? (m + 1 == Wp ? 0 : m + 1) : (m == 0 ? Wp - 1 : m - 1);
+          const float4 C = nb[P], E = nb[y * Wp + me], D = nb[yd * Wp + m], U = nb[yu * Wp + m];
+          xyd::PairNeighbours n;
+          n.lc = q ? make_float2(C.x, C.y) : make_float2(E.y, C.x);
+          n.ls = q ? make_float2(C.z, C.w) : make_float2(E.w, C.z);
+          n.rc = q ? make_float2(C.y, E.x) : make_float2(C.x, C.y);
+          n.rs = q ? make_float2(C.w, E.z) : make_float2(C.z, C.w);
+          n.dc = make_float2(D.x, D.y);
+          n.ds = make_float2(D.z, D.w);
+          n.uc = make_float2(U.x, U.y);
+          n.us = make_float2(U.z, U.w);
+          n.sum();
+          const uint4 w = xyd::philox_pair_words(
+              (uint32_t)y * uL + 4u * (uint32_t)m + (uint32_t)q, sweep, lid, a.rk);
+          float2* angle = reinterpret_cast<float2*>(th + c * half) + P;
+          const float4 o = vec[c * npairs + P];
+          const xyd::PairResult r = xyd::metropolis_pair<MODE>(
+              *angle, make_float2(o.x, o.y), make_float2(o.z, o.w), n.Sc, n.Ss, w, xyd::dup2(K),
+              a.delta);
+          *angle = r.th;
+          vec[c * npairs + P] = make_float4(r.c.x, r.c.y, r.s.x, r.s.y);
+          n_acc += (r.acc0 ? 1u : 0u) + (r.acc1 ? 1u : 0u);
+          if (c == 1) {
+            // the red sites with the same (y, k) and (y, k + 1) enter M once each
+            float2 v[5];
+            xyd::measure_terms2(r.c, r.s, n, make_float2(C.x, C.y), make_float2(C.z, C.w), v);
+            sums.add2(v);
+          }
           step_pair(y, m);
-          continue;
         }
-        const int k = 2 * m, o = 2 * P;
-        const int q = y & 1;
-        const int yd = y == 0 ? L - 1 : y - 1, yu = y == L - 1 ? 0 : y + 1;
-        int kl = k + q - 1, kr = k + q + 1;
-        kl += kl < 0 ? W : 0;
-        kr -= kr >= W ? W : 0;
-        const float2* row = cs + half + y * W;
-        const float2 lf = row[kl], md = row[k + q], rg = row[kr];
-        const float4 dn = *reinterpret_cast<const float4*>(cs + half + yd * W + k);
-        const float4 up = *reinterpret_cast<const float4*>(cs + half + yu * W + k);
-        const float Sc0 = xyd::nb_sum(lf.x, md.x, dn.x, up.x);
-        const float Ss0 = xyd::nb_sum(lf.y, md.y, dn.y, up.y);
-        const float Sc1 = xyd::nb_sum(md.x, rg.x, dn.z, up.z);
-        const float Ss1 = xyd::nb_sum(md.y, rg.y, dn.w, up.w);
-        const uint32_t x0 = 2u * (uint32_t)k + (uint32_t)q;          // x0 & 2 == 0
-        const uint4 w =
-            xyd::philox4x32_10(make_uint4((uint32_t)y * uL + x0, sweep, lid, 1u), a.rk);
-        const float2 t = *reinterpret_cast<const float2*>(th + o);
-        const float4 own = *reinterpret_cast<const float4*>(cs + o);
-        const xyd::SiteResult r0 =
-            xyd::metropolis_step<MODE>(t.x, own.x, own.y, Sc0, Ss0, w.x, w.y, K, a.delta);
-        const xyd::SiteResult r1 =
-            xyd::metropolis_step<MODE>(t.y, own.z, own.w, Sc1, Ss1, w.z, w.w, K, a.delta);
-        *reinterpret_cast<float2*>(th + o) = make_float2(r0.th, r1.th);
-        *reinterpret_cast<float4*>(cs + o) = make_float4(r0.c, r0.s, r1.c, r1.s);
-        n_acc += (r0.accept ? 1u : 0u) + (r1.accept ? 1u : 0u);
-        step_pair(y, m);
-      }
+      };
+      half_sweep(0);
       __syncthreads();
-      // ---- black half, a pair per step, with the sweep sums ----
-      for (int P = threadIdx.x, y = py0, m = pm0; P < npairs; P += kSThreads) {
-        // debug build: the carried (y, m) is the pair's position, in range
-        if (!XY_DCHECK(y >= 0 && y < L && m >= 0 && m < Wp && y * Wp + m == P, 0)) {
-          step_pair(y, m);
-          continue;
-        }
-        const int k = 2 * m, o = half + 2 * P;
-        const int q = (y + 1) & 1;
-        const int yd = y == 0 ? L - 1 : y - 1, yu = y == L - 1 ? 0 : y + 1;
-        int kl = k + q - 1, kr = k + q + 1;
-        kl += kl < 0 ? W : 0;
-        kr -= kr >= W ? W : 0;
-        const float2* row = cs + y * W;
-        const float2 lf = row[kl], md = row[k + q], rg = row[kr];
-        const float4 dn = *reinterpret_cast<const float4*>(cs + yd * W + k);
-        const float4 up = *reinterpret_cast<const float4*>(cs + yu * W + k);
-        const float Sc0 = xyd::nb_sum(lf.x, md.x, dn.x, up.x);
-        const float Ss0 = xyd::nb_sum(lf.y, md.y, dn.y, up.y);
-        const float Sc1 = xyd::nb_sum(md.x, rg.x, dn.z, up.z);
-        const float Ss1 = xyd::nb_sum(md.y, rg.y, dn.w, up.w);
-        const uint32_t x0 = 2u * (uint32_t)k + (uint32_t)q;          // x0 & 2 == 0
-        const uint4 w =
-            xyd::philox4x32_10(make_uint4((uint32_t)y * uL + x0, sweep, lid, 1u), a.rk);
-        const float2 t = *reinterpret_cast<const float2*>(th + o);
-        const float4 own = *reinterpret_cast<const float4*>(cs + o);
-        const xyd::SiteResult r0 =
-            xyd::metropolis_step<MODE>(t.x, own.x, own.y, Sc0, Ss0, w.x, w.y, K, a.delta);
-        const xyd::SiteResult r1 =
-            xyd::metropolis_step<MODE>(t.y, own.z, own.w, Sc1, Ss1, w.z, w.w, K, a.delta);
-        *reinterpret_cast<float2*>(th + o) = make_float2(r0.th, r1.th);
-        *reinterpret_cast<float4*>(cs + o) = make_float4(r0.c, r0.s, r1.c, r1.s);
-        n_acc += (r0.accept ? 1u : 0u) + (r1.accept ? 1u : 0u);
-        // the red sites with the same (y, k) and (y, k + 1) enter M once each
-        const float4 mr = *reinterpret_cast<const float4*>(cs + 2 * P);
-        float v[5];
-        xyd::measure_terms(r0.c, r0.s, lf.x, lf.y, md.x, md.y, dn.x, dn.y, up.x, up.y, Sc0, Ss0,
-                           mr.x, mr.y, v);
-        add_terms(v);
-        xyd::measure_terms(r1.c, r1.s, md.x, md.y, rg.x, rg.y, dn.z, dn.w, up.z, up.w, Sc1, Ss1,
-                           mr.z, mr.w, v);
-        add_terms(v);
-        step_pair(y, m);
-      }
+      half_sweep(1);      // black, with the sweep sums
     } else {
       // ---- red half: red site (y, k) is x = 2k + (y & 1); its black
       // neighbours (y, k+q-1), (y, k+q), (y-1, k), (y+1, k) ----
