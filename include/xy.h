@@ -313,7 +313,10 @@ typedef struct {
     int32_t reduce_mode;        /* as in xy_params                                   */
     uint32_t lattice_id0;       /* lattice i uses lattice id lattice_id0 + i         */
     int32_t sweeps_per_round;   /* sweeps per launch (and between exchanges), >= 1   */
-    int32_t target_band_sites;  /* sites per CTA band of the work plan (0: 8192)     */
+    int32_t target_band_sites;  /* sites per CTA band of the work plan (0: 8192; with
+                                   AUTO and exact sums the lattices that would be banded
+                                   are held on the chip instead, one cluster each, as are
+                                   the others of a one-side batch where that is faster) */
     int32_t algorithm;          /* XY_ALGO_AUTO / _FUSED: state ping-ponged between two
                                    buffers; lattices with L % 128 == 0 run the fused
                                    sweep kernel's tiles and other multiples of 32 its

@@ -11,12 +11,14 @@ Single lattices (``tune_lattice``; xy_params): the algorithm (all sweeps of
 a call in one persistent launch, one launch per sweep, or two sweeps per
 launch with temporal blocking) and the tile kernel's CTAs per SM (3 at up to
 80 registers a thread, 4 at up to 64: more warps, or 2 at up to 128: more
-independent work in flight per warp, fewer warps).
+independent work in flight per warp, fewer warps); the library's default plan
+("auto", which holds sides up to 256 on the chip) is a candidate too.
 
 Batches (``tune_batch``; xy_batch_params): the CTAs per grouped tile launch
 (lattices of one side are launched in groups, one graph branch each, so
 that the groups' sweeps overlap), the grouped tile kernel's CTAs per SM, and
-(only where banded lattices exist) the band size of the cluster kernel.
+(only where banded lattices exist) the band size of the cluster kernel (0: those
+lattices held on the chip).
 
 Cache file: $XY_GB300_AUTOTUNE_CACHE, else ~/.cache/xy_gb300/autotune.json.
 """
@@ -25,10 +27,10 @@ import json
 import os
 
 LATTICE_CANDIDATES = (("persistent", 3), ("persistent", 4), ("persistent", 2), ("fused", 3),
-                      ("fused", 4), ("fused", 2), ("fused2", 3))
+                      ("fused", 4), ("fused", 2), ("fused2", 3), ("auto", 0))
 GROUP_CTAS = (64, 128, 256, 512)
 BATCH_CTAS_PER_SM = (3, 4, 2)
-BAND_TARGETS = (2048, 8192)
+BAND_TARGETS = (0, 2048, 8192)
 
 
 def cache_path():

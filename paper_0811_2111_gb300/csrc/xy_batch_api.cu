@@ -103,7 +103,10 @@ struct xy_batch {
   std::vector<int32_t> small_lattices;
   int32_t* d_small = nullptr;
   size_t small_smem = 0;
-  std::vector<cudaStream_t> branch_streams;
+  // lattices held on the chip (xy_resident.cu), by side: a whole round per
+  // launch of one cluster each, every side on its own branch
+  std::vector<int> res_L, res_start, res_size, res_ctas;   // res_start: into group_lattices
+  std::vector<cudaStream_t> branch_streams;   // groups, then resident sides
   std::vector<cudaEvent_t> ev_joins;
   cudaEvent_t ev_fork = nullptr;
   cudaGraphExec_t graph = nullptr;
@@ -197,13 +200,45 @@ void make_plan(xy_batch* b, int target_sites) {
   // 0) go to groups; lattices that fit one CTA's shared memory run whole
   // rounds in one launch; the other multiples of 32 go to groups on the narrow
   // tiles; the rest to the cluster-launched bands
-  std::map<int, std::vector<int>> groups;
+  std::map<int, std::vector<int>> groups, by_side, resident;
   std::vector<int> banded;
+  // AUTO with exact sums and no band size given: lattices that would be banded
+  // are held on the chip (us per sweep of all: 41 of L = 98 8.5 -> 5.8, 27 of
+  // 138 10.6 -> 5.8, 41 of 250 34 -> 20, two of 250 12.5 -> 3.4).  With the
+  // default plan throughout and one side in the whole batch so are the others
+  // where that is estimated faster than their own path (measured: tiles 230 G
+  // updates/s and no less than 5 us a sweep, narrow tiles 155 and 4.5, whole
+  // lattices 0.5 us + 0.8 ns a site): ten of L = 64 3.0 -> 1.65, ten of 96 6.25
+  // -> 1.95, four of 128 5.0 -> 1.6, two of 256 5.0 -> 3.3.  Beside lattices of
+  // other sides those paths share the GPU better.
+  std::map<int, int> res_ctas;
+  if (b->p.algorithm == XY_ALGO_AUTO && b->p.reduce_mode == XY_REDUCE_EXACT &&
+      b->p.target_band_sites == 0) {
+    const bool default_plan = b->p.group_ctas == 0 && b->p.ctas_per_sm == 0;
+    for (int i = 0; i < b->n; ++i) by_side[b->L[i]].push_back(i);
+    for (auto& kv : by_side) {
+      const int L = kv.first, n = (int)kv.second.size();
+      const double sites = (double)n * L * L;
+      const double other = xyk::fused_supported(L) ? std::max(5.0, sites / 230e3)
+                           : xyk::small_supported(L) ? (0.5 + 0.8e-3 * L * L) * ((n + 303) / 304)
+                           : xyk::narrow_supported(L) ? std::max(4.5, sites / 155e3) : 1e30;
+      if (other < 1e30 && (by_side.size() > 1 || !default_plan)) continue;
+      int ctas = 0;
+      double us = 0.0;
+      if (xyk::prepare_resident_batch(b->p.sincos_mode, L, n, &ctas, &us) != cudaSuccess) {
+        (void)cudaGetLastError();
+        continue;
+      }
+      if (ctas > 0 && us < other) res_ctas[L] = ctas;
+    }
+  }
   b->small_lattices.clear();
   b->small_smem = 0;
   for (int i = 0; i < b->n; ++i) {
     const int Li = b->L[i];
-    if (b->fused && xyk::fused_supported(Li)) {
+    if (res_ctas.count(Li)) {
+      resident[Li].push_back(i);
+    } else if (b->fused && xyk::fused_supported(Li)) {
       groups[Li].push_back(i);
     } else if (b->fused && xyk::small_supported(Li)) {
       b->small_lattices.push_back(i);
@@ -238,6 +273,17 @@ void make_plan(xy_batch* b, int target_sites) {
       for (int j = 0; j < n; ++j) b->group_lattices.push_back(kv.second[k + j]);
       k += n;
     }
+  }
+  b->res_L.clear();
+  b->res_start.clear();
+  b->res_size.clear();
+  b->res_ctas.clear();
+  for (auto& kv : resident) {
+    b->res_L.push_back(kv.first);
+    b->res_ctas.push_back(res_ctas[kv.first]);
+    b->res_start.push_back((int)b->group_lattices.size());
+    b->res_size.push_back((int)kv.second.size());
+    for (int i : kv.second) b->group_lattices.push_back(i);
   }
   std::vector<int> order;
   std::vector<int> nbands(b->n, 0), rows(b->n, 0);
@@ -382,14 +428,45 @@ xyk::FusedBatchArgs group_args(const xy_batch* b, size_t g, int s) {
   return f;
 }
 
+xyk::ResidentArgs resident_args(const xy_batch* b, size_t g) {
+  xyk::ResidentArgs a;
+  a.theta = b->d_theta;
+  a.theta2 = b->d_theta2;
+  a.L = b->res_L[g];
+  a.K = 0.f;
+  a.delta = (float)b->p.delta;
+  a.rk = xyd::make_round_keys(b->p.seed);
+  a.lattice_id = b->p.lattice_id0;
+  a.sweep0 = 0;
+  a.n_sweeps = b->p.sweeps_per_round;
+  a.rec = b->d_rec;
+  a.rec_stride = b->rec_cap;
+  a.beta = 0.0;
+  a.ctas = b->res_ctas[g];
+  a.lattices = b->d_groups + b->res_start[g];
+  a.offset = b->d_offset;
+  a.betas = b->d_beta;
+  a.counters = b->d_counters;
+  a.J = b->p.J;
+  return a;
+}
+
 // One round: the banded cluster kernel (all of its sweeps in one launch) on
 // the main branch and, on one parallel branch per group, the grouped fused
 // sweeps (one launch per sweep); then, after all branches, the exchange
 // kernel, which also advances the counters.
 cudaError_t enqueue_round(const xy_batch* b, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  const size_t ng = b->group_L.size();
-  if (ng > 0) e = cudaEventRecord(b->ev_fork, s);
+  const size_t ng = b->group_L.size(), nb = ng + b->res_L.size();
+  if (nb > 0) e = cudaEventRecord(b->ev_fork, s);
+  for (size_t g = ng; g < nb && e == cudaSuccess; ++g) {
+    cudaStream_t gs = b->branch_streams[g];
+    e = cudaStreamWaitEvent(gs, b->ev_fork, 0);
+    if (e == cudaSuccess)
+      e = xyk::launch_resident_batch(b->p.sincos_mode, resident_args(b, g - ng),
+                                     b->res_size[g - ng], gs);
+    if (e == cudaSuccess) e = cudaEventRecord(b->ev_joins[g], gs);
+  }
   for (size_t g = 0; g < ng && e == cudaSuccess; ++g) {
     cudaStream_t gs = b->branch_streams[g];
     e = cudaStreamWaitEvent(gs, b->ev_fork, 0);
@@ -426,7 +503,7 @@ cudaError_t enqueue_round(const xy_batch* b, cudaStream_t s) {
                                            b->n_ctas, s)
                  : xyk::launch_batch_round(b->p.sincos_mode, b->p.reduce_mode, round_args(b),
                                            b->n_ctas, s);
-  for (size_t g = 0; g < ng && e == cudaSuccess; ++g) e = cudaStreamWaitEvent(s, b->ev_joins[g], 0);
+  for (size_t g = 0; g < nb && e == cudaSuccess; ++g) e = cudaStreamWaitEvent(s, b->ev_joins[g], 0);
   if (e == cudaSuccess) e = xyk::launch_exchange(exchange_args(b), s);
   return e;
 }
@@ -602,10 +679,10 @@ xy_status xy_batch_create(const xy_batch_params* p, void* cuda_stream, xy_batch*
   alloc((void**)&b->d_partials, sizeof(double) * (size_t)b->n * xyk::kMaxSegments * xyk::kPartials);
   alloc((void**)&b->d_groups, sizeof(int32_t) * b->group_lattices.size());
   alloc((void**)&b->d_small, sizeof(int32_t) * b->small_lattices.size());
-  if (e == cudaSuccess && !b->group_L.empty()) {
+  if (e == cudaSuccess && b->group_L.size() + b->res_L.size() > 0) {
     step = "branch streams";
     e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
-    for (size_t g = 0; g < b->group_L.size() && e == cudaSuccess; ++g) {
+    for (size_t g = 0; g < b->group_L.size() + b->res_L.size() && e == cudaSuccess; ++g) {
       cudaStream_t st = nullptr;
       cudaEvent_t ev = nullptr;
       e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
@@ -705,7 +782,10 @@ xy_status xy_batch_info(const xy_batch* b, int32_t* n_lattices, int64_t* n_recor
   if (n_lattices) *n_lattices = b->n;
   if (n_records) *n_records = b->rec_count;
   if (next_sweep) *next_sweep = b->next_sweep;
-  if (n_ctas) *n_ctas = b->n_ctas;
+  if (n_ctas) {
+    *n_ctas = b->n_ctas;
+    for (size_t g = 0; g < b->res_L.size(); ++g) *n_ctas += b->res_size[g] * b->res_ctas[g];
+  }
   return XY_OK;
 }
 
@@ -716,8 +796,8 @@ xy_status xy_batch_launches_per_round(const xy_batch* b, int32_t* launches) {
     bmsg("xy_batch_launches_per_round: NULL output");
     return XY_EINVAL;
   }
-  *launches = (int32_t)b->group_L.size() * b->p.sweeps_per_round + (b->n_ctas > 0 ? 1 : 0) +
-              (b->small_lattices.empty() ? 0 : 1) + 1;
+  *launches = (int32_t)b->group_L.size() * b->p.sweeps_per_round + (int32_t)b->res_L.size() +
+              (b->n_ctas > 0 ? 1 : 0) + (b->small_lattices.empty() ? 0 : 1) + 1;
   return XY_OK;
 }
 

@@ -184,7 +184,17 @@ struct ResidentArgs {
   int n_sweeps;
   xy_record* rec;        // records of the n sweeps, zeroed
   double beta;
-  int ctas;              // set by the launcher
+  int ctas;              // CTAs per cluster; set by launch_resident
+  // a batch's lattices of side L (null lattices: the single one above): the
+  // state ping-pongs between theta and theta2 by sweep parity, counters[0] is
+  // the first sweep, rec the batch's records, lattice_id that of lattice 0
+  const int32_t* lattices = nullptr;   // [clusters]
+  float* theta2 = nullptr;
+  const int64_t* offset = nullptr;
+  const double* betas = nullptr;
+  const uint32_t* counters = nullptr;
+  int64_t rec_stride = 0;
+  double J = 0.0;
 };
 constexpr size_t kResidentSmem = 96 * 1024;   // dynamic shared memory of a strip, at most
 // Whether side L is held resident, and (prepare; outside any capture) whether
@@ -192,6 +202,11 @@ constexpr size_t kResidentSmem = 96 * 1024;   // dynamic shared memory of a stri
 bool resident_supported(int L);
 cudaError_t prepare_resident(int sincos_mode, int L, bool* fits);
 cudaError_t launch_resident(int sincos_mode, const ResidentArgs& a, cudaStream_t stream);
+// The same for n lattices of side L of a batch, one cluster each: the cluster
+// size to take (0: none fits) and the estimated time of a sweep of all of them.
+cudaError_t prepare_resident_batch(int sincos_mode, int L, int n, int* ctas, double* us);
+cudaError_t launch_resident_batch(int sincos_mode, const ResidentArgs& a, int n,
+                                  cudaStream_t stream);
 
 // All sweeps of a call of the four-replica fused sweep in one cooperative
 // launch (tiles ordered by per-tile sweep counters, bounded waits).

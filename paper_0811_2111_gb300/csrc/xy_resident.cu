@@ -64,6 +64,25 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
   cg::cluster_group cluster = cg::this_cluster();
   const int C = a.ctas, rank = (int)cluster.block_rank();
   const int L = a.L, W = L / 2;
+  // the cluster's lattice: the only one, in place, or one of a batch, from the
+  // buffer of the first sweep's parity to that behind the last's
+  const float* src = a.theta;
+  float* dst = a.theta;
+  float K = a.K;
+  double beta = a.beta;
+  uint32_t lattice_id = a.lattice_id, sweep0 = a.sweep0;
+  xy_record* rec = a.rec;
+  if (a.lattices) {
+    const int li = a.lattices[blockIdx.x / C];
+    sweep0 = a.counters[0];
+    const uint32_t last = sweep0 + (uint32_t)a.n_sweeps - 1u;
+    src = ((sweep0 & 1u) ? a.theta2 : a.theta) + a.offset[li];
+    dst = ((last & 1u) ? a.theta : a.theta2) + a.offset[li];
+    beta = a.betas[li];
+    K = (float)(beta * a.J);
+    lattice_id = a.lattice_id + (uint32_t)li;
+    rec = a.rec + (size_t)li * a.rec_stride + sweep0;
+  }
   const xys::Strip st(L, W, C, rank);
   const int nthreads = blockDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = nthreads >> 5;
@@ -86,7 +105,7 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
     for (int p = 0; p < NP; ++p) {
       th[c][p] = make_float2(0.f, 0.f);
       if (pr[p].on) {
-        const float* g = a.theta + c * plane + (size_t)(st.y0 + pr[p].r) * W + pr[p].k;
+        const float* g = src + c * plane + (size_t)(st.y0 + pr[p].r) * W + pr[p].k;
         th[c][p].x = g[0];
         if (pr[p].two) th[c][p].y = g[1];
       }
@@ -95,12 +114,12 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
   auto words = [&](int p, int c, uint32_t sweep) {
     const uint32_t y = (uint32_t)(st.y0 + pr[p].r);
     return xyd::philox_pair_words(
-        y * (uint32_t)L + 2u * (uint32_t)pr[p].k + ((y + (uint32_t)c) & 1u), sweep, a.lattice_id,
+        y * (uint32_t)L + 2u * (uint32_t)pr[p].k + ((y + (uint32_t)c) & 1u), sweep, lattice_id,
         a.rk);
   };
   uint4 w[NP];
 #pragma unroll
-  for (int p = 0; p < NP; ++p) w[p] = words(p, 0, a.sweep0);
+  for (int p = 0; p < NP; ++p) w[p] = words(p, 0, sweep0);
   cluster.sync();                          // every CTA has started: its memory may be written
 #pragma unroll
   for (int c = 0; c < 2; ++c)
@@ -112,7 +131,7 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
   // The previous sweep's sums, left in s_part / s_cnt before the barrier: one
   // warp per sum adds the warps' values (16-bit halves, one lane per warp) and
   // issues the record's atomic.
-  auto commit = [&](xy_record* rec) {
+  auto commit = [&](xy_record* r) {
     for (int task = warp; task < 6; task += nwarps) {
       const bool has = lane < nwarps;
       if (task == 5) {
@@ -120,17 +139,17 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
         const uint32_t total = __reduce_add_sync(0xffffffffu, n & 0x7fffffffu);
         const bool bad = __any_sync(0xffffffffu, (n & 0x80000000u) != 0u);
         if (lane == 0) {
-          atomicAdd(reinterpret_cast<unsigned long long*>(&rec->accepted),
+          atomicAdd(reinterpret_cast<unsigned long long*>(&r->accepted),
                     (unsigned long long)total);
-          if (bad) atomicOr(reinterpret_cast<unsigned long long*>(&rec->flags), 1ull);
-          if (rank == 0) rec->beta = a.beta;
+          if (bad) atomicOr(reinterpret_cast<unsigned long long*>(&r->flags), 1ull);
+          if (rank == 0) r->beta = beta;
         }
       } else {
         const int32_t v = has ? (int32_t)s_part[lane][task] : 0;
         const uint32_t lo = __reduce_add_sync(0xffffffffu, (uint32_t)v & 0xffffu);
         const int32_t hi = (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)(v >> 16));
         if (lane == 0)
-          atomicAdd(reinterpret_cast<unsigned long long*>(&rec->sum[task]),
+          atomicAdd(reinterpret_cast<unsigned long long*>(&r->sum[task]),
                     (unsigned long long)((long long)hi * 65536ll + (long long)lo)
                         << (XY_FX_SHIFT - xyd::fx_term_shift(task)));
       }
@@ -138,7 +157,7 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
   };
 
   for (int s = 0; s < a.n_sweeps; ++s) {
-    const uint32_t sweep = a.sweep0 + (uint32_t)s;
+    const uint32_t sweep = sweep0 + (uint32_t)s;
     unsigned int n_acc = 0;
     xyd::SweepSums<0> sums;                // at most 2 NP black sites per thread
     sums.init();
@@ -162,7 +181,7 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
         n.us = make_float2(U.z, U.w);
         n.sum();
         const xyd::PairResult r = xyd::metropolis_pair<MODE>(th[c][p], cv[c][p], sv[c][p], n.Sc,
-                                                             n.Ss, w[p], xyd::dup2(a.K), a.delta);
+                                                             n.Ss, w[p], xyd::dup2(K), a.delta);
         th[c][p] = r.th;
         cv[c][p] = r.c;
         sv[c][p] = r.s;
@@ -180,7 +199,7 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
           }
         }
       }
-      if (c == 0 && s > 0) commit(a.rec + (s - 1));
+      if (c == 0 && s > 0) commit(rec + (s - 1));
       if (c == 1) {
         const unsigned int acc = __reduce_add_sync(0xffffffffu, n_acc);
         const bool bad = __any_sync(0xffffffffu, xyd::fx_nonfinite(sums.fx));
@@ -206,13 +225,13 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
       }
     }
   }
-  commit(a.rec + (a.n_sweeps - 1));
+  commit(rec + (a.n_sweeps - 1));
 #pragma unroll
   for (int c = 0; c < 2; ++c)
 #pragma unroll
     for (int p = 0; p < NP; ++p)
       if (pr[p].on) {
-        float* g = a.theta + c * plane + (size_t)(st.y0 + pr[p].r) * W + pr[p].k;
+        float* g = dst + c * plane + (size_t)(st.y0 + pr[p].r) * W + pr[p].k;
         g[0] = th[c][p].x;
         if (pr[p].two) g[1] = th[c][p].y;
       }
@@ -240,22 +259,25 @@ struct Plan {
   size_t smem;
 };
 
-Plan plan_of(int L) {
+Plan plan_of(int L, int ctas) {
   Plan p = {};
-  p.ctas = resident_ctas(L);
-  if (p.ctas == 0 || (L & 1)) return Plan{};
+  p.ctas = ctas;
+  if (p.ctas == 0 || p.ctas > L || (L & 1)) return Plan{};
   const int W = L / 2, rows = strip_rows(L, p.ctas, 0);
   const int pairs = rows * ((W + 1) / 2);
   p.np = (pairs + kRThreads - 1) / kRThreads;
   if (p.np > kRMaxPairs) return Plan{};
   p.threads = ((pairs + p.np - 1) / p.np + 31) / 32 * 32;
   p.smem = sizeof(float4) * 2 * (size_t)plane_vec4(rows, W);
-  return p;
+  return p.smem <= kResidentSmem ? p : Plan{};
 }
 
-cudaLaunchConfig_t config_of(const Plan& p, cudaStream_t stream, cudaLaunchAttribute* attr) {
+Plan plan_of(int L) { return plan_of(L, resident_ctas(L)); }
+
+cudaLaunchConfig_t config_of(const Plan& p, int n_lattices, cudaStream_t stream,
+                             cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.ctas);
+  cfg.gridDim = dim3(p.ctas * n_lattices);
   cfg.blockDim = dim3(p.threads);
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = stream;
@@ -280,39 +302,84 @@ cudaError_t with_kernel(int mode, const Plan& p, const F& f) {
 
 }  // namespace
 
-bool resident_supported(int L) {
-  const Plan p = plan_of(L);
-  return p.ctas > 0 && p.smem <= kResidentSmem;
-}
+namespace {
 
-cudaError_t prepare_resident(int sincos_mode, int L, bool* fits) {
-  *fits = false;
-  const Plan p = plan_of(L);
-  if (p.ctas == 0 || p.smem > kResidentSmem) return cudaErrorInvalidValue;
-  return with_kernel(sincos_mode, p, [&](auto* fn) {
+// Sets the kernel's attributes and reports how many clusters of plan p the
+// device runs at a time.
+cudaError_t clusters_of(int mode, const Plan& p, int* n) {
+  *n = 0;
+  return with_kernel(mode, p, [&](auto* fn) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kResidentSmem);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = config_of(p, nullptr, &attr);
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
-    *fits = e == cudaSuccess && n >= 1;
-    return e;
+    const cudaLaunchConfig_t cfg = config_of(p, 1, nullptr, &attr);
+    return cudaOccupancyMaxActiveClusters(n, fn, &cfg);
   });
 }
 
-cudaError_t launch_resident(int sincos_mode, const ResidentArgs& args,
-                            cudaStream_t stream) {
+}  // namespace
+
+bool resident_supported(int L) { return plan_of(L).ctas > 0; }
+
+cudaError_t prepare_resident(int sincos_mode, int L, bool* fits) {
+  *fits = false;
+  const Plan p = plan_of(L);
+  if (p.ctas == 0) return cudaErrorInvalidValue;
+  int n = 0;
+  const cudaError_t e = clusters_of(sincos_mode, p, &n);
+  *fits = e == cudaSuccess && n >= 1;
+  return e;
+}
+
+// Time of a sweep of n lattices of side L by cluster size: a strip's latency
+// (1.45 us for up to 128 pairs of a colour per CTA, 1.5 for 256, 2.0 for 512,
+// 3.5 for 1024, single lattices of L = 64 ... 256), once per wave of the
+// clusters that run at a time.
+cudaError_t prepare_resident_batch(int sincos_mode, int L, int n, int* ctas, double* us) {
+  *ctas = 0;
+  *us = 0.0;
+  for (int c = 1; c <= 16; c *= 2) {
+    const Plan p = plan_of(L, c);
+    if (p.ctas == 0) continue;
+    int at_a_time = 0;
+    const cudaError_t e = clusters_of(sincos_mode, p, &at_a_time);
+    if (e != cudaSuccess) return e;
+    if (at_a_time < 1) continue;
+    const int pairs = strip_rows(L, c, 0) * ((L / 2 + 1) / 2);
+    const double strip = pairs <= 256 ? 1.4 + 0.0004 * pairs : 1.0 + 0.002 * pairs +
+                         (p.np > 1 ? 0.5 : 0.0);
+    const double t = strip * (double)((n + at_a_time - 1) / at_a_time);
+    if (*ctas == 0 || t < *us) {
+      *ctas = c;
+      *us = t;
+    }
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_resident(int sincos_mode, const ResidentArgs& args, cudaStream_t stream) {
   const Plan p = plan_of(args.L);
-  if (p.ctas == 0 || p.smem > kResidentSmem || args.n_sweeps < 1) return cudaErrorInvalidValue;
+  if (p.ctas == 0 || args.n_sweeps < 1) return cudaErrorInvalidValue;
   ResidentArgs a = args;
   a.ctas = p.ctas;
+  a.lattices = nullptr;
   return with_kernel(sincos_mode, p, [&](auto* fn) {
     cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = config_of(p, stream, &attr);
+    const cudaLaunchConfig_t cfg = config_of(p, 1, stream, &attr);
+    return cudaLaunchKernelEx(&cfg, fn, a);
+  });
+}
+
+cudaError_t launch_resident_batch(int sincos_mode, const ResidentArgs& a, int n,
+                                  cudaStream_t stream) {
+  const Plan p = plan_of(a.L, a.ctas);
+  if (p.ctas == 0 || a.n_sweeps < 1 || n < 1 || !a.lattices) return cudaErrorInvalidValue;
+  return with_kernel(sincos_mode, p, [&](auto* fn) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = config_of(p, n, stream, &attr);
     return cudaLaunchKernelEx(&cfg, fn, a);
   });
 }
