@@ -239,13 +239,14 @@ __device__ __forceinline__ SiteResult metropolis_step(float t, float c0, float s
 // functions above.  A packed instruction holds both FMA pipes for two cycles
 // (measured 64 per SM and clock: the scalar FP32 rate, in half the issue
 // slots), and the tile kernels were bound by issue slots (74-76 % used) with
-// the FMA pipes half idle.  The fused sweep: 140.4 -> 117 issued instructions
-// per update; persistent at L = 4096 79.1 -> 73.7 us per sweep, one launch per
-// sweep at L = 16384 1205 -> 1106 us (SFU 912 -> 858).  What bounds them now is
-// the heavy FMA pipe (68 %: the packed instructions and, four cycles each, the
+// the FMA pipes half idle.  The fused sweep: 140.4 -> 111 issued instructions
+// per update; persistent at L = 4096 79.1 -> 73.5 us per sweep, one launch per
+// sweep at L = 16384 1205 -> 1097 us (SFU 912 -> 858).  What bounds them now is
+// the heavy FMA pipe (67 %: the packed instructions and, four cycles each, the
 // Philox products), whose bursts the warps' phases do not quite even out.
-// Measured and not kept: the quadrant step packed too (112.7 instructions, 74.8
-// and 1108 us) or on the ALU pipe (75.1 and 1130 us), and the accept test on
+// Measured and not kept: the quadrant step scalar (117.7 instructions, 74.0 and
+// 1110 us), wholly packed with one more product for the sign (112, 74.5 and
+// 1105 us) or on the ALU pipe (75.1 and 1130 us), and the accept test on
 // ex2.approx with expf only within rounding of the threshold (six FMA-pipe
 // instructions fewer, the branch as many more: 73.6 and 1116 us).
 __device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
@@ -269,16 +270,15 @@ __device__ __forceinline__ void sincos_poly2(float2 t, float2* s_out, float2* c_
   pc = fma2(r2, pc, dup2(0.04166662320494652f));
   pc = fma2(r2, pc, dup2(-0.5f));
   const float2 cr = fma2(r2, pc, dup2(1.0f));
-  // the quadrant step in scalar FMAs: they run on either FMA pipe, so beside
-  // the Philox products, which hold only the heavy one
-  const float px = __fsub_rn(qf.x, 2.0f), py = __fsub_rn(qf.y, 2.0f);
-  const float ax = __fsub_rn(1.0f, fabsf(px)), ay = __fsub_rn(1.0f, fabsf(py));
-  const float bx = __fmul_rn(px, __fsub_rn(2.0f, fabsf(px)));
-  const float by = __fmul_rn(py, __fsub_rn(2.0f, fabsf(py)));
-  *s_out = make_float2(__fmaf_rn(-ax, sr.x, __fmul_rn(-bx, cr.x)),
-                       __fmaf_rn(-ay, sr.y, __fmul_rn(-by, cr.y)));
-  *c_out = make_float2(__fmaf_rn(bx, sr.x, __fmul_rn(-ax, cr.x)),
-                       __fmaf_rn(by, sr.y, __fmul_rn(-ay, cr.y)));
+  // the quadrant step with the opposite factors, na = |p| - 1 and
+  // nb = p (|p| - 2), so that the sine needs no negation and packs; the
+  // cosine's last FMA negates nb, which a packed operand cannot
+  const float2 p = add2(qf, dup2(-2.0f));
+  const float2 na = make_float2(__fsub_rn(fabsf(p.x), 1.0f), __fsub_rn(fabsf(p.y), 1.0f));
+  const float2 nb = mul2(p, add2(na, dup2(-1.0f)));
+  *s_out = fma2(na, sr, mul2(nb, cr));
+  const float2 m = mul2(na, cr);
+  *c_out = make_float2(__fmaf_rn(-nb.x, sr.x, m.x), __fmaf_rn(-nb.y, sr.y, m.y));
 }
 
 template <int MODE>
