@@ -77,6 +77,8 @@ struct xy_ctx {
   bool fused;              // sweeps use the fused kernel
   bool resident;           // XY_ALGO_AUTO: the lattice fits on the chip (xy_resident.cu)
   bool ragged;             // XY_ALGO_AUTO: persistent sweeps on overlapping tiles
+  bool grid;               // XY_ALGO_AUTO: every tile stays with its CTA (xy_grid.cu)
+  unsigned long long* d_words;   // its exchange words, then ctl[2] and the wait word
   bool persistent;         // ... all sweeps of an xy_sweep call in one cooperative launch
   bool auto_persistent;    // chosen by XY_ALGO_AUTO: per-sweep launches if it does not fit
   unsigned int* d_tiles;   // the persistent launch's per-tile sweep counters
@@ -302,6 +304,40 @@ cudaError_t timed_resident(xy_ctx* c, const xyk::ResidentArgs& a) {
   return e;
 }
 
+cudaError_t timed_grid(xy_ctx* c, const xyk::GridArgs& a) {
+  if (c->timing_every <= 0)
+    return xyk::launch_grid(c->p.sincos_mode, a, c->sms, c->stream);
+  cudaEvent_t e0, e1;
+  cudaError_t e = next_events(c, 0, &e0, &e1);
+  if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
+  if (e == cudaSuccess) e = xyk::launch_grid(c->p.sincos_mode, a, c->sms, c->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
+  return e;
+}
+
+// m sweeps of the state at theta, in place, by the two-pass kernels: the same
+// bits where a cooperative launch found no room.
+cudaError_t two_pass_sweeps(xy_ctx* c, float* theta, uint32_t sweep0, int64_t m, xy_record* rec,
+                            const xyd::RoundKeys& rk) {
+  xyk::HalfSweepArgs h;
+  h.theta = theta;
+  h.L = c->p.L;
+  h.W = c->p.L / 2;
+  h.K = (float)(c->p.beta * c->p.J);
+  h.delta = (float)c->p.delta;
+  h.rk = rk;
+  h.lattice_id = c->p.lattice_id;
+  h.beta = c->p.beta;
+  cudaError_t e = cudaSuccess;
+  for (int64_t i = 0; i < m && e == cudaSuccess; ++i) {
+    h.sweep = sweep0 + (uint32_t)i;
+    h.rec = rec + i;
+    e = timed_half_sweep(c, 0, h);
+    if (e == cudaSuccess) e = timed_half_sweep(c, 1, h);
+  }
+  return e;
+}
+
 void release(xy_ctx* c) {
   for (int k = 0; k < 2; ++k) {
     for (cudaEvent_t e : c->ev[k]) cudaEventDestroy(e);
@@ -314,7 +350,9 @@ void release(xy_ctx* c) {
   if (c->d_scratch) cudaFree(c->d_scratch);
   if (c->d_flag) cudaFree(c->d_flag);
   if (c->d_tiles && !c->ragged) cudaFree(c->d_tiles);
-  if (c->d_wait && !c->ragged) cudaFree(c->d_wait);
+  if (c->d_wait && !c->ragged && !c->d_words) cudaFree(c->d_wait);
+  if (c->d_words) cudaFree(c->d_words);
+  c->d_words = nullptr;
   c->d_tiles = nullptr;
   c->d_wait = nullptr;
   c->d_theta = nullptr;
@@ -400,7 +438,28 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
   c->auto_persistent = c->persistent && p->algorithm == XY_ALGO_AUTO;
   c->fused = p->algorithm == XY_ALGO_FUSED || p->algorithm == XY_ALGO_FUSED2 ||
              c->persistent || (p->algorithm == XY_ALGO_AUTO && xyk::fused_supported(p->L));
-  if (e == cudaSuccess && c->fused) {
+  if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->ctas_per_sm == 0 &&
+      p->reduce_mode == XY_REDUCE_EXACT && xyk::grid_supported(p->L)) {
+    bool fits = false;
+    if (xyk::prepare_grid(p->sincos_mode, p->L, c->sms, &fits) != cudaSuccess)
+      (void)cudaGetLastError();       // the other kernels take the lattice
+    if (fits) {
+      // optional, and one allocation: the words, the two of ctl, the wait word
+      const size_t bytes = xyk::grid_words(p->L) * sizeof(unsigned long long);
+      if (xyk::dev_malloc(&c->d_words, bytes + 4 * sizeof(unsigned int)) == cudaSuccess) {
+        unsigned int* ctl = reinterpret_cast<unsigned int*>(c->d_words) + bytes / sizeof(unsigned int);
+        c->d_wait = ctl + 2;
+        e = cudaMemsetAsync(c->d_words, 0, bytes + 4 * sizeof(unsigned int), c->stream);
+        // ctl[0] = 1 (the low byte)
+        if (e == cudaSuccess) e = cudaMemsetAsync(ctl, 1, 1, c->stream);
+      } else {
+        (void)cudaGetLastError();
+        c->d_words = nullptr;
+      }
+    }
+  }
+  c->grid = c->d_words != nullptr;
+  if (e == cudaSuccess && c->fused && !c->grid) {
     e = xyk::dev_malloc(&c->d_pong, N * sizeof(float));
     if (e == cudaSuccess) e = xyk::dev_malloc(&c->d_wait, sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_wait, 0, sizeof(unsigned int), c->stream);
@@ -408,14 +467,16 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
       e = cudaErrorNotSupported;
   }
   if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->ctas_per_sm == 0 &&
-      p->reduce_mode == XY_REDUCE_EXACT && xyk::resident_supported(p->L)) {
+      p->reduce_mode == XY_REDUCE_EXACT && !c->grid &&
+      xyk::resident_supported(p->L)) {
     if (xyk::prepare_resident(p->sincos_mode, p->L, &c->resident) != cudaSuccess) {
       (void)cudaGetLastError();       // the tile kernels take the lattice
       c->resident = false;
     }
   }
   if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->ctas_per_sm == 0 &&
-      p->reduce_mode == XY_REDUCE_EXACT && !c->resident && xyk::ragged_supported(p->L)) {
+      p->reduce_mode == XY_REDUCE_EXACT && !c->resident && !c->grid &&
+      xyk::ragged_supported(p->L)) {
     // the second buffer, behind it the counters and the wait word: optional
     // (without them the two-pass kernels run in place) and one allocation
     const size_t words = (size_t)xyk::fused_tiles(p->L) + 2;
@@ -430,7 +491,7 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
       c->d_pong = nullptr;
     }
   }
-  if (e == cudaSuccess && c->persistent)
+  if (e == cudaSuccess && c->persistent && !c->grid)
     e = xyk::dev_malloc(&c->d_tiles, sizeof(unsigned int) * ((size_t)xyk::fused_tiles(p->L) + 1));
   if (e != cudaSuccess) {
     st = (e == cudaErrorMemoryAllocation) ? XY_ENOMEM : XY_ECUDA;
@@ -539,6 +600,33 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
       if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: resident launch");
       done += m;
     }
+  } else if (c->grid && (c->persistent || c->timing_every <= 0)) {
+    xyk::GridArgs a;
+    a.theta = c->d_theta;
+    a.words = c->d_words;
+    a.error = c->d_wait;
+    a.ctl = c->d_wait - 2;
+    a.L = c->p.L;
+    a.K = (float)(c->p.beta * c->p.J);
+    a.delta = (float)c->p.delta;
+    a.rk = rk;
+    a.lattice_id = c->p.lattice_id;
+    a.beta = c->p.beta;
+    a.spin_limit = xyk::fused_persistent_spin_limit();
+    for (int64_t done = 0; done < n;) {
+      const int64_t m = std::min<int64_t>(n - done, kResidentSweeps);
+      a.sweep0 = (uint32_t)(c->next_sweep + (uint64_t)done);
+      a.n_sweeps = (int)m;
+      a.rec = c->d_rec + c->rec_count + done;
+      cudaError_t e = timed_grid(c, a);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {
+        // the grid does not fit beside other work
+        (void)cudaGetLastError();
+        e = two_pass_sweeps(c, c->d_theta, a.sweep0, m, a.rec, rk);
+      }
+      if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: grid launch");
+      done += m;
+    }
   } else if (c->persistent || (c->ragged && c->timing_every <= 0)) {
     xyk::FusedPersistArgs a;
     a.buf[0] = c->d_theta;
@@ -568,25 +656,9 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
       a.rec = c->d_rec + c->rec_count + done;
       cudaError_t e = timed_persistent(c, a);
       if (e == cudaErrorCooperativeLaunchTooLarge && c->ragged) {
-        // the grid does not fit beside other work: the same sweeps in place by
-        // the two-pass kernels (bit-identical)
+        // the grid does not fit beside other work (the state is in a.buf[0])
         (void)cudaGetLastError();
-        xyk::HalfSweepArgs h;
-        h.theta = a.buf[0];
-        h.L = a.L;
-        h.W = a.W;
-        h.K = a.K;
-        h.delta = a.delta;
-        h.rk = a.rk;
-        h.lattice_id = a.lattice_id;
-        h.beta = a.beta;
-        e = cudaSuccess;
-        for (int64_t i = 0; i < m && e == cudaSuccess; ++i) {
-          h.sweep = a.sweep0 + (uint32_t)i;
-          h.rec = a.rec + i;
-          e = timed_half_sweep(c, 0, h);
-          if (e == cudaSuccess) e = timed_half_sweep(c, 1, h);
-        }
+        e = two_pass_sweeps(c, a.buf[0], a.sweep0, m, a.rec, rk);
         if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: launch");
         done += m;
         continue;

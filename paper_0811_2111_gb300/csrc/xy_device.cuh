@@ -314,35 +314,57 @@ struct PairResult {
   bool acc0, acc1;
 };
 
-// metropolis_step of the two sites of a Philox pair (angles t, unit vectors
-// (c0, s0), neighbour sums (Sc, Ss), words w of philox_pair_words, each site's
-// K): the same decisions and results, bit for bit.  The wrap's two candidates compare as
-// unsigned bit patterns: of raw + 2 pi, raw and raw - 2 pi exactly the wanted
-// one has the smallest pattern (negative floats compare above positive ones;
-// raw is never -0, being a rounded sum with t >= 0).
+// The two sites' proposals: the angles, their unit vectors and the words of the
+// accept tests.  They depend on no neighbour, so a kernel may draw them early.
+struct PairProposal {
+  float2 th, c, s;
+  uint32_t u0, u1;
+};
+
+// The proposals of the two sites of a Philox pair (angles t, words w of
+// philox_pair_words).  The wrap's two candidates compare as unsigned bit
+// patterns: of raw + 2 pi, raw and raw - 2 pi exactly the wanted one has the
+// smallest pattern (negative floats compare above positive ones; raw is never
+// -0, being a rounded sum with t >= 0).
+template <int MODE>
+__device__ __forceinline__ PairProposal propose_pair(float2 t, const uint4& w, float delta) {
+  const float2 step = make_float2((float)((int32_t)w.x >> 8), (float)((int32_t)w.z >> 8));
+  const float2 raw = fma2(dup2(delta * kR23), step, t);
+  const float2 up = add2(raw, dup2(kTwoPi)), down = add2(raw, dup2(-kTwoPi));
+  PairProposal p;
+  p.th.x = __uint_as_float(__vimin3_u32(__float_as_uint(up.x), __float_as_uint(raw.x),
+                                        __float_as_uint(down.x)));
+  p.th.y = __uint_as_float(__vimin3_u32(__float_as_uint(up.y), __float_as_uint(raw.y),
+                                        __float_as_uint(down.y)));
+  unit_vector2<MODE>(p.th, &p.s, &p.c);
+  p.u0 = w.y;
+  p.u1 = w.w;
+  return p;
+}
+
+// Their accept tests against the neighbour sums (Sc, Ss), from the angles t and
+// unit vectors (c0, s0), each site's K.
+template <int MODE>
+__device__ __forceinline__ PairResult accept_pair(const PairProposal& p, float2 t, float2 c0,
+                                                  float2 s0, float2 Sc, float2 Ss, float2 K) {
+  const float2 X = fma2(sub2(p.c, c0), Sc, mul2(sub2(p.s, s0), Ss));
+  const float2 y = mul2(X, K);
+  PairResult r;
+  r.acc0 = u24(p.u0) < boltzmann<MODE>(y.x);
+  r.acc1 = u24(p.u1) < boltzmann<MODE>(y.y);
+  r.th = make_float2(r.acc0 ? p.th.x : t.x, r.acc1 ? p.th.y : t.y);
+  r.c = make_float2(r.acc0 ? p.c.x : c0.x, r.acc1 ? p.c.y : c0.y);
+  r.s = make_float2(r.acc0 ? p.s.x : s0.x, r.acc1 ? p.s.y : s0.y);
+  return r;
+}
+
+// metropolis_step of the two sites of a Philox pair: the same decisions and
+// results, bit for bit.
 template <int MODE>
 __device__ __forceinline__ PairResult metropolis_pair(float2 t, float2 c0, float2 s0, float2 Sc,
                                                       float2 Ss, const uint4& w, float2 K,
                                                       float delta) {
-  const float2 step = make_float2((float)((int32_t)w.x >> 8), (float)((int32_t)w.z >> 8));
-  const float2 raw = fma2(dup2(delta * kR23), step, t);
-  const float2 up = add2(raw, dup2(kTwoPi)), down = add2(raw, dup2(-kTwoPi));
-  float2 tp;
-  tp.x = __uint_as_float(__vimin3_u32(__float_as_uint(up.x), __float_as_uint(raw.x),
-                                      __float_as_uint(down.x)));
-  tp.y = __uint_as_float(__vimin3_u32(__float_as_uint(up.y), __float_as_uint(raw.y),
-                                      __float_as_uint(down.y)));
-  float2 s1, c1;
-  unit_vector2<MODE>(tp, &s1, &c1);
-  const float2 X = fma2(sub2(c1, c0), Sc, mul2(sub2(s1, s0), Ss));
-  PairResult r;
-  const float2 y = mul2(X, K);
-  r.acc0 = u24(w.y) < boltzmann<MODE>(y.x);
-  r.acc1 = u24(w.w) < boltzmann<MODE>(y.y);
-  r.th = make_float2(r.acc0 ? tp.x : t.x, r.acc1 ? tp.y : t.y);
-  r.c = make_float2(r.acc0 ? c1.x : c0.x, r.acc1 ? c1.y : c0.y);
-  r.s = make_float2(r.acc0 ? s1.x : s0.x, r.acc1 ? s1.y : s0.y);
-  return r;
+  return accept_pair<MODE>(propose_pair<MODE>(t, w, delta), t, c0, s0, Sc, Ss, K);
 }
 
 // The four neighbours (left, right, down, up) of two sites of one row, as the

@@ -28,6 +28,7 @@
 
 #include "xy_device.cuh"
 #include "xy_internal.h"
+#include "xy_tile.cuh"
 #include "xy_tma.cuh"
 
 namespace xyk {
@@ -35,7 +36,6 @@ namespace xyk {
 namespace {
 
 constexpr int kTileRows = 32;
-constexpr int kTileK = 64;                   // plane columns (2 per lane)
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kSRows = kTileRows + 4;        // stage rows: global rows y0-2 .. y0+33
@@ -54,11 +54,8 @@ constexpr int kRedRows = kSRows - 2;         // the red plane's stage rows 1 .. 
 //   csb   black unit vectors of stage rows 0..35, same columns
 // then the commit's per-warp partial sums and counters.  The persistent
 // kernel keeps NANG = 2 ang buffers: the next tile's rows arrive in the other.
-constexpr int kCsOff = 2;
-constexpr int kCsPairs = kTileK / 2 + 2;
 constexpr int kRawRows = kSRows + kRedRows;
 constexpr int kRedRaw0 = kSRows - 1;        // ang row of red stage row r: kRedRaw0 + r
-typedef float4 CsRow[kCsPairs];
 typedef float AngRow[kTileK];
 constexpr size_t kRawRowBytes = sizeof(AngRow);
 constexpr size_t kAngBytes = kRawRowBytes * kRawRows;
@@ -90,63 +87,6 @@ static_assert(3 * (kPersistSmemBytes + 1024 + 512) <= 228 * 1024,
 __host__ __device__ inline int tile_cols(int W) { return (W + kTileK - 1) / kTileK; }
 __host__ __device__ inline int tile_rows(int L) { return (L + kTileRows - 1) / kTileRows; }
 inline int fused_tiles_of(int L) { return tile_cols(L / 2) * tile_rows(L); }
-
-__device__ __forceinline__ int wrap_once(int v, int n) {
-  v += (v < 0) ? n : 0;
-  v -= (v >= n) ? n : 0;
-  return v;
-}
-
-// The cosine and sine pairs of a float4 of unit vectors.
-__device__ __forceinline__ float2 cosines(const float4& v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 sines(const float4& v) { return make_float2(v.z, v.w); }
-
-__device__ __forceinline__ void put_pair(float4* at, const float2& c, const float2& s) {
-  *at = make_float4(c.x, c.y, s.x, s.y);
-}
-
-// The unit vector (cos, sin) at unit-vector column c of a row.
-__device__ __forceinline__ float2 get_one(const CsRow& row, int c) {
-  const float* p = reinterpret_cast<const float*>(&row[c >> 1]) + (c & 1);
-  return make_float2(p[0], p[2]);
-}
-
-__device__ __forceinline__ void put_one(CsRow& row, int c, float cv, float sv) {
-  float* p = reinterpret_cast<float*>(&row[c >> 1]) + (c & 1);
-  p[0] = cv;
-  p[2] = sv;
-}
-
-// The four neighbour unit vectors of the two sites of pair j of row i of the
-// other colour's unit vectors `nb`, where a site at column c has its same-row
-// neighbours at c+q-1 and c+q.  The three same-row columns are the pair's own
-// and one of the pair before (q = 0) or after (q = 1); q is a compile-time
-// constant where the row loops are unrolled (rows alternate q), so no selects
-// are issued.  Rows i-1 and i of the pair's columns come in as D and P (a warp
-// walks its rows downwards, so they are the previous row's P and U); row i+1
-// is loaded and returned in U.
-__device__ __forceinline__ void pair_neighbours(const CsRow* nb, int i, int j, int q,
-                                                const float4 D, const float4 P, float4& U,
-                                                xyd::PairNeighbours& n) {
-  const float4 E = nb[i][q ? j + 1 : j - 1];
-  U = nb[i + 1][j];
-  if (q) {
-    n.lc = cosines(P);
-    n.ls = sines(P);
-    n.rc = make_float2(P.y, E.x);
-    n.rs = make_float2(P.w, E.z);
-  } else {
-    n.lc = make_float2(E.y, P.x);
-    n.ls = make_float2(E.w, P.z);
-    n.rc = cosines(P);
-    n.rs = sines(P);
-  }
-  n.dc = cosines(D);
-  n.ds = sines(D);
-  n.uc = cosines(U);
-  n.us = sines(U);
-  n.sum();
-}
 
 // The scalars of one fused sweep; the Philox round keys are passed separately
 // (by reference, so a kernel can leave them in its parameter space).

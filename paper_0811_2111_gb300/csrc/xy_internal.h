@@ -171,6 +171,36 @@ int fused_persistent_max_sweeps(int L);
 cudaError_t launch_fused_persistent(int sincos_mode, int reduce_mode, const FusedPersistArgs& a,
                                     cudaStream_t stream);
 
+// All sweeps of a call of a middling lattice in one cooperative launch, in
+// place, every tile staying with its CTA, exact sums (xy_grid.cu).
+struct GridArgs {
+  float* theta;          // [2][L][W]: the state, read and rewritten
+  unsigned long long* words;   // grid_words(L) exchange words, zeroed once
+  unsigned int* ctl;     // [2]: the next tag (1 at first), CTAs that have finished (0)
+  unsigned int* error;   // set nonzero when a bounded wait runs out
+  int L;
+  float K;
+  float delta;
+  xyd::RoundKeys rk;
+  uint32_t lattice_id;
+  uint32_t sweep0;       // Philox sweep word of the first sweep
+  int n_sweeps;
+  xy_record* rec;        // records of the n sweeps, zeroed
+  double beta;
+  long long spin_limit;  // polls before a wait gives up
+  int nx, ny, tile_warps;      // set by launch_grid
+};
+// Largest single lattice held by one cluster (xy_resident.cu); larger ones go
+// to one tile per SM where they fit: us per sweep, cluster and tiles, L = 128
+// 1.52 and 1.59, 160 1.94 and 1.68, 256 3.1 and 1.51.
+constexpr int kClusterMaxL = 128;
+bool grid_supported(int L);
+// Exchange words of side L.
+size_t grid_words(int L);
+// Whether side L fits a device of `sms` multiprocessors (outside any capture).
+cudaError_t prepare_grid(int sincos_mode, int L, int sms, bool* fits);
+cudaError_t launch_grid(int sincos_mode, const GridArgs& a, int sms, cudaStream_t stream);
+
 // All sweeps of a call of a small lattice in one cluster launch, in place, the
 // lattice held on the chip, exact sums (xy_resident.cu).
 struct ResidentArgs {

@@ -246,9 +246,11 @@ __global__ void __launch_bounds__(kRThreads) k_sweep_resident(ResidentArgs a) {
 //   L = 64   1: 2.75   4: 1.49   8: 1.45  16: 1.50
 //   L = 80             4: 1.93   8: 1.53  16: 1.45
 //   L = 128            4: 3.50   8: 1.98  16: 1.52   (persistent tiles: 4.9)
-//   L = 256                      8: 6.55  16: 3.55   (persistent tiles: 5.3)
-// Above 256 a thread would own more pairs than its registers hold (L = 320
-// with four each 5.9) and the tiles are as fast.
+//   L = 256                      8: 6.55  16: 3.1    (persistent tiles: 5.3)
+// A single lattice above kClusterMaxL is spread over the whole chip instead
+// (xy_grid.cu, L = 256 1.51); where it does not find room there, and in a batch,
+// the clusters take sides up to 256, above which a thread would own more pairs
+// than its registers hold (L = 320 with four each 5.9).
 int resident_ctas(int L) {
   if (L < 4 || L > 256) return 0;
   return L <= 32 ? 1 : L <= 64 ? 8 : 16;
