@@ -795,30 +795,6 @@ constexpr int kP2Band = kP2Rows / kP2Warps;                  // 4 rows per warp
 constexpr int kFrRows = kP2Rows + 4;                         // tile rows -2 .. 33
 constexpr int kFrCols = kP2Cols + 8;                         // tile columns -4 .. 131
 constexpr size_t kP2Smem = sizeof(float) * 2 * kFrRows * kFrCols;
-// The tile-walking form (PREF) adds the next tile's loads, brought in while the
-// current tile runs: its angle and momentum rows as two TMA boxes of 32 x 128
-// floats, then each thread's six scalars by cp.async (ring site A's angle and
-// momentum, ring site B's, the halo-two sites H and G).
-constexpr size_t kP2PreRowsAt = kP2Smem;
-constexpr size_t kP2PreScalarsAt = kP2PreRowsAt + sizeof(float4) * 2 * kP2Band * kP2Threads;
-constexpr size_t kP2SmemPref = kP2PreScalarsAt + sizeof(float) * 6 * kP2Threads;
-static_assert(2 * (kP2SmemPref + 1024) <= 228 * 1024, "two tile-walking CTAs must fit one SM");
-static_assert(kP2PreRowsAt % 128 == 0 && 2 * kP2Band * kP2Threads * 4 == 2 * kP2Rows * kP2Cols,
-              "the TMA boxes (two of 32 x 128 floats) fill the 128-byte aligned row slots");
-// The tile-walking form runs when every resident CTA gets at least this many
-// tiles of a launch (measured per unit trajectory with the rows by per-thread
-// cp.async: 3.44 against 3.56 ms at L = 4096, 17.8 against 18.9 at 8192; a tie
-// at 2048, about 3.4 tiles per CTA; with a tile per CTA only the extra
-// shared-memory round trip is left).
-constexpr int kP2PrefMinTilesPerCta = 4;
-
-__device__ __forceinline__ void hmc_cp4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-
 __device__ __forceinline__ int wrap_near(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
 // One leap-frog step of a site: kick by a F(unit vector, neighbour sums),
@@ -890,23 +866,7 @@ __device__ __forceinline__ void quad_step(const Quad4& o, const Quad4& dn, const
                   hmc_wrap(__fmaf_rn(eps, p.z, t.z)), hmc_wrap(__fmaf_rn(eps, p.w, t.w)));
 }
 
-// PREF = false: one tile per CTA (grid = the tile columns x rows), its loads straight into
-// registers.  PREF = true: a grid of resident CTAs walks the tiles blockIdx.x,
-// + gridDim.x, ... (the tiles of a launch are independent: it reads one angle
-// and one momentum buffer and writes two others); right after the current
-// tile's staging barrier thread 0 has TMA copy the next tile's rows and every
-// thread copies its ring and halo sites into its own shared-memory slots by
-// cp.async, so they arrive while the two steps run.  Both forms run the same
-// arithmetic on the same values: bit-identical.
-// The tile-walking form's tensor maps (boxes of 32 rows x 128 columns): the
-// three angle buffers (the launch reads the one the control block names) and
-// the momenta it reads; a kernel parameter.
-struct Tile2Maps {
-  CUtensorMap th[3];
-  CUtensorMap p;
-};
-
-// RAG (PREF = false; any L >= 130): the last tiles of a side that is no multiple
+// RAG (any L >= 130): the last tiles of a side that is no multiple
 // of the tile move back to end with the lattice and overlap the tiles before
 // them.  A launch reads one angle and one momentum buffer and writes others,
 // so the sites of an overlap are computed twice from the same inputs and
@@ -935,117 +895,51 @@ __device__ __forceinline__ void store_row4(float* p, const float4& v, int L) {
   }
 }
 
-template <int MODE, bool PREF, bool RAG = false>
-__global__ void __launch_bounds__(kP2Threads, 2)
-    k_hmc_tile2(HmcArgs a, const __grid_constant__ Tile2Maps maps) {
+template <int MODE, bool RAG>
+__global__ void __launch_bounds__(kP2Threads, 2) k_hmc_tile2(HmcArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   float (*fc)[kFrCols] = reinterpret_cast<float (*)[kFrCols]>(smem);
   float (*fs)[kFrCols] = reinterpret_cast<float (*)[kFrCols]>(smem + sizeof(float) * kFrRows * kFrCols);
-  float4* pre_rows = reinterpret_cast<float4*>(smem + kP2PreRowsAt);   // [2 * kP2Band][threads]
-  float* pre_sc = reinterpret_cast<float*>(smem + kP2PreScalarsAt);     // [6][threads]
 
   const int L = a.L;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tiles_x = L / kP2Cols, n_tiles = tiles_x * (L / kP2Rows);
   int src, dst;
   hmc_buffers(a, a.ctl->cur, &src, &dst);
   const float* __restrict__ th_src = hmc_buf(a, src);
 
   const int rb = kP2Band * warp;                             // first tile row of the band
-  // the loads of tile t (PREF): the tile's angle and momentum rows as two
-  // TMA boxes of 32 x 128 (thread 0, completing on s_bar), and this thread's
-  // ring and halo sites by cp.async into its own slots: the same sites as the
-  // loads in the tile loop below
-  __shared__ __align__(8) uint64_t s_bar;
-  uint32_t phase = 0;
-  if (PREF) {
-    if (tid == 0) {
-      xyt::mbar_init(&s_bar, 1);
-      xyt::fence_mbarrier_init();
-    }
-    __syncthreads();
-  }
-  auto prefetch = [&](int t) {
-    const int px0 = (t % tiles_x) * kP2Cols, py0 = (t / tiles_x) * kP2Rows;
-    if (tid == 0) {
-      xyt::mbar_arrive_expect_tx(&s_bar, (uint32_t)(2 * sizeof(float) * kP2Rows * kP2Cols));
-      xyt::tma_load_2d(pre_rows, &maps.th[src], px0, py0, &s_bar);
-      xyt::tma_load_2d(pre_rows + kP2Rows * kP2Cols / 4, &maps.p, px0, py0, &s_bar);
-    }
-    const int ay = tid < kP2Cols ? -1 : kP2Rows, ax = tid & (kP2Cols - 1);
-    const size_t ga = (size_t)wrap_near(py0 + ay, L) * L + (px0 + ax);
-    hmc_cp4(&pre_sc[0 * kP2Threads + tid], th_src + ga);
-    hmc_cp4(&pre_sc[1 * kP2Threads + tid], a.p_in + ga);
-    if (tid < 2 * kP2Rows) {
-      const int bx = tid < kP2Rows ? -1 : kP2Cols, by = tid & (kP2Rows - 1);
-      const size_t gb = (size_t)(py0 + by) * L + wrap_near(px0 + bx, L);
-      hmc_cp4(&pre_sc[2 * kP2Threads + tid], th_src + gb);
-      hmc_cp4(&pre_sc[3 * kP2Threads + tid], a.p_in + gb);
-    }
-    const int hy = tid < kP2Cols ? -2 : kP2Rows + 1;
-    hmc_cp4(&pre_sc[4 * kP2Threads + tid], th_src + (size_t)wrap_near(py0 + hy, L) * L + (px0 + ax));
-    if (tid >= 64 && tid < 132) {
-      int gy, gx;
-      if (tid < 128) {
-        gx = (tid - 64) < kP2Rows ? -2 : kP2Cols + 1;
-        gy = (tid - 64) & (kP2Rows - 1);
-      } else {
-        gy = (tid & 2) ? kP2Rows : -1;
-        gx = (tid & 1) ? kP2Cols : -1;
-      }
-      hmc_cp4(&pre_sc[5 * kP2Threads + tid],
-              th_src + (size_t)wrap_near(py0 + gy, L) * L + wrap_near(px0 + gx, L));
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  if (PREF && (int)blockIdx.x < n_tiles) prefetch(blockIdx.x);
-  for (int tile = PREF ? (int)blockIdx.x : 0; tile < (PREF ? n_tiles : 1);
-       tile += PREF ? (int)gridDim.x : 1) {
-  const int x0 = PREF ? (tile % tiles_x) * kP2Cols
-                 : RAG ? min((int)blockIdx.x * kP2Cols, L - kP2Cols) : (int)blockIdx.x * kP2Cols;
-  const int y0 = PREF ? (tile / tiles_x) * kP2Rows
-                 : RAG ? min((int)blockIdx.y * kP2Rows, L - kP2Rows) : (int)blockIdx.y * kP2Rows;
+  const int x0 = RAG ? min((int)blockIdx.x * kP2Cols, L - kP2Cols) : (int)blockIdx.x * kP2Cols;
+  const int y0 = RAG ? min((int)blockIdx.y * kP2Rows, L - kP2Rows) : (int)blockIdx.y * kP2Rows;
 
   // ---- loads: own 4 x 4 block (angles and momenta), one site of the ring's
   // top or bottom row (threads 0..255), one of its side columns (0..63), one
   // halo-two site of rows -2 / 33 (0..255), of columns -2 / 129 (64..127) or a
-  // ring corner (128..131); from this thread's slots (PREF) or from global
-  // memory
+  // ring corner (128..131); 
   const int xb = x0 + 4 * lane;
   float4 t4[kP2Band], p4[kP2Band];
-  if (PREF) {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (!xyt::mbar_wait_bounded(&s_bar, phase, kSpinLimit)) atomicOr(&a.ctl->error, 1u);
-    phase ^= 1u;
-  }
 #pragma unroll
   for (int r = 0; r < kP2Band; ++r) {
     const size_t g = (size_t)(y0 + rb + r) * L + xb;
-    // the boxes: rows of 128 floats, the thread's 4 x 4 block at row rb + r,
-    // columns 4 lane .. 4 lane + 3
-    t4[r] = PREF ? pre_rows[(rb + r) * (kP2Cols / 4) + lane]
-                 : RAG ? load_row4(th_src + g, L) : *reinterpret_cast<const float4*>(th_src + g);
-    p4[r] = PREF ? pre_rows[(kP2Rows + rb + r) * (kP2Cols / 4) + lane]
-                 : RAG ? load_row4(a.p_in + g, L) : *reinterpret_cast<const float4*>(a.p_in + g);
+    t4[r] = RAG ? load_row4(th_src + g, L) : *reinterpret_cast<const float4*>(th_src + g);
+    p4[r] = RAG ? load_row4(a.p_in + g, L) : *reinterpret_cast<const float4*>(a.p_in + g);
   }
   // ring site A: row -1 (tid < 128) or 32, column tid & 127
   const int ay = tid < kP2Cols ? -1 : kP2Rows, ax = tid & (kP2Cols - 1);
   const size_t ga = (size_t)wrap_near(y0 + ay, L) * L + (x0 + ax);
-  float ta = PREF ? pre_sc[0 * kP2Threads + tid] : th_src[ga];
-  float pa = PREF ? pre_sc[1 * kP2Threads + tid] : a.p_in[ga];
+  float ta = th_src[ga];
+  float pa = a.p_in[ga];
   // ring site B: column -1 (tid < 32) or 128, row tid & 31
   const bool hasb = tid < 2 * kP2Rows;
   const int bx = tid < kP2Rows ? -1 : kP2Cols, by = tid & (kP2Rows - 1);
   float tb = 0.f, pb = 0.f;
   if (hasb) {
     const size_t gb = (size_t)(y0 + by) * L + wrap_near(x0 + bx, L);
-    tb = PREF ? pre_sc[2 * kP2Threads + tid] : th_src[gb];
-    pb = PREF ? pre_sc[3 * kP2Threads + tid] : a.p_in[gb];
+    tb = th_src[gb];
+    pb = a.p_in[gb];
   }
   // halo-two site H: rows -2 / 33; G: columns -2 / 129 or a corner
   const int hy = tid < kP2Cols ? -2 : kP2Rows + 1;
-  const float th_h =
-      PREF ? pre_sc[4 * kP2Threads + tid] : th_src[(size_t)wrap_near(y0 + hy, L) * L + (x0 + ax)];
+  const float th_h = th_src[(size_t)wrap_near(y0 + hy, L) * L + (x0 + ax)];
   const bool hasg = tid >= 64 && tid < 132;
   int gy = 0, gx = 0;
   float th_g = 0.f;
@@ -1057,8 +951,7 @@ __global__ void __launch_bounds__(kP2Threads, 2)
       gy = (tid & 2) ? kP2Rows : -1;
       gx = (tid & 1) ? kP2Cols : -1;
     }
-    th_g = PREF ? pre_sc[5 * kP2Threads + tid]
-                : th_src[(size_t)wrap_near(y0 + gy, L) * L + wrap_near(x0 + gx, L)];
+    th_g = th_src[(size_t)wrap_near(y0 + gy, L) * L + wrap_near(x0 + gx, L)];
   }
 
   // ---- unit vectors of the old state; what crosses a warp goes to the frame
@@ -1096,10 +989,6 @@ __global__ void __launch_bounds__(kP2Threads, 2)
     }
   }
   __syncthreads();
-
-  // every thread has read its slots before the barrier above: the next tile's
-  // copies land there while this one runs
-  if (PREF && tile + (int)gridDim.x < n_tiles) prefetch(tile + (int)gridDim.x);
 
   // ---- first step: the ring sites (from the frame), then the tile --------
   const float K = a.K, ka = a.a, eps = a.eps;
@@ -1174,8 +1063,154 @@ __global__ void __launch_bounds__(kP2Threads, 2)
       *reinterpret_cast<float4*>(th_dst + g) = t4[r];
     }
   });
-  if (PREF) __syncthreads();   // the next tile's staging rewrites the frame
+}
+
+// ---------------------------------------------------------------------------
+// Two full kick-drift steps per launch, each warp on its own.  A warp walks down
+// the rows of a strip of 128 columns, four per lane, of which the outer lanes'
+// are halo (the strips advance by 120 columns), and the unit vectors of both
+// steps pass through its registers: with row r read it takes row r - 1 through
+// the first step and row r - 2 through the second.  Horizontal neighbours come
+// by shuffle; the rows arrive in the lane's own places in shared memory by
+// cp.async, kRowsAhead rows ahead.  A warp's segment of rows starts two rows
+// early and ends two rows late.  So there is no ring, no frame and no barrier:
+// the tiles of k_hmc_tile2 spend a third of their time on those (their two CTAs
+// per SM wait for each other and for dependent instructions, 51 % of the issue
+// slots used).  The price is 128 columns computed for 120 and (rows + 3) rows for
+// rows.  Here the FMA pipes are 64 % busy and 63 % of the issue slots used, DRAM
+// at 4 TB/s; what is left is the tail of a launch (one wave: warps end at
+// different times, 78 % resident on average) and the 16 warps per SM that the
+// registers allow.
+//
+// us per unit trajectory, tiles and this: L = 1792 460 and 434, 2048 580 and 575
+// (SFU sincos 520 and 413), 2560 1038 and 889, 3072 1740 and 1332, 4096 3343 and
+// 2575, 8192 17360 and 12930; where the side is no multiple of 128 1500 384 and
+// 367, 2000 706 and 612, 3000 2032 and 1438.  Below, a segment has too few rows
+// for its early and late ones (1536 306 and 325, 1000 174 and 194).  With the
+// next row's loads in registers instead of three rows ahead in shared memory
+// 4096 2735; strips advancing by 124 with 8-byte accesses 2638; loops unrolled
+// once 3449 (the rows' registers then move), twice 2916.
+//
+// VEC: columns that one access may take (the rows' alignment): 4, 2 or 1 where L
+// is a multiple of 4, even or odd.
+// ---------------------------------------------------------------------------
+constexpr int kRowsThreads = 128;
+constexpr int kRowsWarps = kRowsThreads / 32;
+constexpr int kRowsPerSm = 4;              // CTAs per SM: 16 warps, 128 registers a thread
+constexpr int kRowsAhead = 3;              // rows on their way to shared memory
+constexpr int kRowsUnroll = 3;             // the rows' registers rotate with period three
+constexpr int kStripCols = 120;
+constexpr int kRowsMinTiled = 1792, kRowsMinRagged = 1500;
+
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+
+template <int VEC>
+__device__ __forceinline__ void hmc_cp_async(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if (VEC == 4) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  } else {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(4 * VEC) : "memory");
   }
+}
+
+template <int MODE, int VEC>
+__global__ void __launch_bounds__(kRowsThreads, kRowsPerSm)
+    k_hmc_rows2(HmcArgs a, int strips, int rows) {
+  __shared__ float4 s_rows[kRowsWarps][kRowsAhead][2][32];   // a lane reads its own places only
+  constexpr int NV = 4 / VEC;
+  const int L = a.L;
+  const int lane = threadIdx.x & 31;
+  const int w = blockIdx.x * kRowsWarps + (threadIdx.x >> 5);
+  const int strip = w % strips, ys = (w / strips) * rows;
+  if (ys >= L) return;
+  const int ye = min(ys + rows, L);
+  int src, dst;
+  hmc_buffers(a, a.ctl->cur, &src, &dst);
+  const float* __restrict__ th_src = hmc_buf(a, src);
+  float* __restrict__ th_dst = hmc_buf(a, dst);
+  const int xs = strip * kStripCols - 4 + 4 * lane;
+  const bool inner = lane > 0 && lane < 31;
+  uint32_t x[NV];                          // the lane's columns (a side may wrap between accesses)
+#pragma unroll
+  for (int i = 0; i < NV; ++i) x[i] = (uint32_t)wrap_near(xs + i * VEC, L);
+  const float K = a.K, ka = a.a, eps = a.eps;
+  float4 (*ahead)[2][32] = s_rows[threadIdx.x >> 5];
+  auto fetch = [&](int r, int slot) {
+    const uint32_t g = (uint32_t)wrap_near(min(r, ye + 1), L) * (uint32_t)L;
+    float* t = reinterpret_cast<float*>(&ahead[slot][0][lane]);
+    float* p = reinterpret_cast<float*>(&ahead[slot][1][lane]);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      hmc_cp_async<VEC>(t + i * VEC, th_src + (g + x[i]));
+      hmc_cp_async<VEC>(p + i * VEC, a.p_in + (g + x[i]));
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto step = [&](const Quad4& o, const Quad4& dn, const Quad4& up, float4& p, float4& t) {
+    const float cl = __shfl_up_sync(0xffffffffu, o.cO.y, 1);
+    const float sl = __shfl_up_sync(0xffffffffu, o.sO.y, 1);
+    const float cr = __shfl_down_sync(0xffffffffu, o.cE.x, 1);
+    const float sr = __shfl_down_sync(0xffffffffu, o.sE.x, 1);
+    quad_step(o, dn, up, cl, sl, cr, sr, K, ka, eps, p, t);
+  };
+  auto store = [&](float* at, const float4& v, int i) {
+    if (VEC == 4) {
+      *reinterpret_cast<float4*>(at) = v;
+    } else if (VEC == 2) {
+      *reinterpret_cast<float2*>(at) = i ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+    } else {
+      *at = i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
+    }
+  };
+  int slot = 0;
+#pragma unroll
+  for (int i = 0; i < kRowsAhead; ++i) fetch(ys - 2 + i, i);
+  float4 t0, p0, t1, p1;                   // row r - 1 as read, row r - 2 after one step
+  Quad4 a0, a1;                            // rows r - 2 and r - 1 as read
+  Quad4 w0, w1;                            // rows r - 3 and r - 2 after one step
+  // row r: its unit vectors; STAGE >= 1: row r - 1's first step; 2: row r - 2's
+  // second step, written out
+  auto row = [&](auto stage, int r) {
+    constexpr int STAGE = decltype(stage)::value;
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRowsAhead - 1) : "memory");
+    const float4 tc = ahead[slot][0][lane], pc = ahead[slot][1][lane];
+    fetch(r + kRowsAhead, slot);
+    slot = slot + 1 == kRowsAhead ? 0 : slot + 1;
+    const Quad4 n = quad_vectors<MODE>(tc);
+    if (STAGE >= 1) {
+      step(a1, a0, n, p0, t0);
+      const Quad4 wn = quad_vectors<MODE>(t0);
+      if (STAGE >= 2) {
+        step(w1, w0, wn, p1, t1);
+        const uint32_t g = (uint32_t)(r - 2) * (uint32_t)L;
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+          if (inner && xs + i * VEC < L) {
+            store(a.p_out + (g + x[i]), p1, i);
+            store(th_dst + (g + x[i]), t1, i);
+          }
+      }
+      w0 = w1;
+      w1 = wn;
+      t1 = t0;
+      p1 = p0;
+    }
+    a0 = a1;
+    a1 = n;
+    t0 = tc;
+    p0 = pc;
+  };
+  row(IntC<0>(), ys - 2);
+  row(IntC<0>(), ys - 1);
+  row(IntC<1>(), ys);
+  row(IntC<1>(), ys + 1);
+#pragma unroll kRowsUnroll
+  for (int r = ys + 2; r < ye + 2; ++r) row(IntC<2>(), r);
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -1273,9 +1308,6 @@ __global__ void k_hmc_canon_reset(HmcCtl* ctl) {
   if (threadIdx.x == 0 && blockIdx.x == 0) ctl->cur = 0u;
 }
 
-// Two full steps per launch: two CTAs per SM (the registers' limit); the
-// tile-walking form when each would get at least kP2PrefMinTilesPerCta tiles
-// and the tensor maps are given, else one tile per CTA.
 }  // namespace
 
 bool hmc_tiled_ok(int L) { return L >= kTileCols && L % kTileCols == 0; }
@@ -1284,40 +1316,42 @@ bool hmc_ragged_ok(int L) { return L > kTileCols && L % kTileCols != 0; }
 
 namespace {
 
+// Two full steps per launch: by rows where the segments are long enough (one
+// wave of warps, so the longest that keep every SM full), else by tiles.
 template <int MODE>
-cudaError_t launch_step2(const HmcArgs& a, const CUtensorMap* th_maps, const CUtensorMap* p_map,
-                         cudaStream_t stream) {
+cudaError_t launch_step2(const HmcArgs& a, cudaStream_t stream) {
   if (!a.pairs || a.p_in == a.p_out) return cudaErrorInvalidValue;
-  if (!hmc_tiled_ok(a.L)) {
-    if (!hmc_ragged_ok(a.L)) return cudaErrorInvalidValue;
-    Tile2Maps none;
-    memset(&none, 0, sizeof(none));
-    const dim3 grid((a.L + kP2Cols - 1) / kP2Cols, (a.L + kP2Rows - 1) / kP2Rows);
-    k_hmc_tile2<MODE, false, true><<<grid, kP2Threads, kP2Smem, stream>>>(a, none);
-    return cudaGetLastError();
-  }
-  if (!a.tiled) return cudaErrorInvalidValue;
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  const int n_tiles = (a.L / kP2Cols) * (a.L / kP2Rows);
-  Tile2Maps m;
-  if (th_maps && p_map && n_tiles >= kP2PrefMinTilesPerCta * 2 * sms) {
-    for (int i = 0; i < 3; ++i) m.th[i] = th_maps[i];
-    m.p = *p_map;
-    k_hmc_tile2<MODE, true><<<2 * sms, kP2Threads, kP2SmemPref, stream>>>(a, m);
-  } else {
-    memset(&m, 0, sizeof(m));
+  const bool tiled = hmc_tiled_ok(a.L);
+  if (!tiled && !hmc_ragged_ok(a.L)) return cudaErrorInvalidValue;
+  if (tiled && !a.tiled) return cudaErrorInvalidValue;
+  if (a.L >= (tiled ? kRowsMinTiled : kRowsMinRagged)) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int strips = (a.L + kStripCols - 1) / kStripCols;
+    const int fit = sms * kRowsPerSm * kRowsWarps / strips, segs = fit > 1 ? fit : 1;
+    const int rows = (a.L + segs - 1) / segs;
+    const int warps = strips * ((a.L + rows - 1) / rows);
+    const int grid = (warps + kRowsWarps - 1) / kRowsWarps;
+    switch (a.L % 4) {
+      case 0: k_hmc_rows2<MODE, 4><<<grid, kRowsThreads, 0, stream>>>(a, strips, rows); break;
+      case 2: k_hmc_rows2<MODE, 2><<<grid, kRowsThreads, 0, stream>>>(a, strips, rows); break;
+      default: k_hmc_rows2<MODE, 1><<<grid, kRowsThreads, 0, stream>>>(a, strips, rows);
+    }
+  } else if (tiled) {
     k_hmc_tile2<MODE, false>
-        <<<dim3(a.L / kP2Cols, a.L / kP2Rows), kP2Threads, kP2Smem, stream>>>(a, m);
+        <<<dim3(a.L / kP2Cols, a.L / kP2Rows), kP2Threads, kP2Smem, stream>>>(a);
+  } else {
+    const dim3 grid((a.L + kP2Cols - 1) / kP2Cols, (a.L + kP2Rows - 1) / kP2Rows);
+    k_hmc_tile2<MODE, true><<<grid, kP2Threads, kP2Smem, stream>>>(a);
   }
   return cudaGetLastError();
 }
 
 template <int MODE>
 cudaError_t launch_mode(int kind, const HmcArgs& a, cudaStream_t stream) {
-  if (kind == kHmcStep2) return launch_step2<MODE>(a, nullptr, nullptr, stream);
+  if (kind == kHmcStep2) return launch_step2<MODE>(a, stream);
   if (a.tiled) {
     const dim3 grid(a.L / kTileCols, a.L / kTileRows);
     switch (kind) {
@@ -1354,16 +1388,9 @@ cudaError_t hmc_prepare(int sincos_mode) {
   e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2Smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  const void* fp = m == 0 ? (const void*)k_hmc_tile2<0, true>
+  const void* fr = m == 0 ? (const void*)k_hmc_tile2<0, true>
                           : (m == 1 ? (const void*)k_hmc_tile2<1, true>
                                     : (const void*)k_hmc_tile2<2, true>);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2SmemPref);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fp, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  const void* fr = m == 0 ? (const void*)k_hmc_tile2<0, false, true>
-                          : (m == 1 ? (const void*)k_hmc_tile2<1, false, true>
-                                    : (const void*)k_hmc_tile2<2, false, true>);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(fr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2Smem);
   if (e == cudaSuccess)
@@ -1377,18 +1404,6 @@ cudaError_t hmc_prepare(int sincos_mode) {
 
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[m][dev] = true;
   return e;
-}
-
-cudaError_t launch_hmc_step2(int sincos_mode, const HmcArgs& a, const void* th_maps3,
-                             const void* p_map, cudaStream_t stream) {
-  if (!hmc_tiled_ok(a.L)) return cudaErrorInvalidValue;
-  const CUtensorMap* tm = static_cast<const CUtensorMap*>(th_maps3);
-  const CUtensorMap* pm = static_cast<const CUtensorMap*>(p_map);
-  switch (sincos_mode) {
-    case 0: return launch_step2<0>(a, tm, pm, stream);
-    case 1: return launch_step2<1>(a, tm, pm, stream);
-    default: return launch_step2<2>(a, tm, pm, stream);
-  }
 }
 
 cudaError_t launch_hmc(int kind, int sincos_mode, const HmcArgs& a, cudaStream_t stream) {

@@ -63,7 +63,7 @@ void tmsg(const char* fmt, ...) {
 }  // namespace
 
 struct xy_hmc {
-  CUtensorMap maps[5];               // TMA maps (32 x 128 boxes): angle buffers 0..2, d_p, d_p2
+  CUtensorMap maps[4];               // TMA maps (32 x 128 boxes): angle buffers 0..2, d_p
   bool use_tma;
   bool use_persist;                  // a trajectory's steps in one cooperative TMA launch
   unsigned int* d_tiles;             // its per-tile step counters
@@ -270,10 +270,7 @@ cudaError_t enqueue_trajectory(const xy_hmc* h, int begin, int n, int mode, cuda
     if (a.pairs && left >= 2) {
       a.p_in = pcur;
       a.p_out = pother;
-      // the tile-walking form reads its rows by TMA: the angle buffers' maps
-      // and that of the momenta it reads
-      e = h->use_tma ? xyk::launch_hmc_step2(m, a, h->maps, pcur == h->d_p ? &h->maps[3] : &h->maps[4], s)
-                     : xyk::launch_hmc(xyk::kHmcStep2, m, a, s);
+      e = xyk::launch_hmc(xyk::kHmcStep2, m, a, s);
       float* t = pcur;
       pcur = pother;
       pother = t;
@@ -459,7 +456,6 @@ xy_status xy_hmc_create(const xy_hmc_params* p, void* cuda_stream, void* d_angle
     h->tma_rows = 32;   // 32 x 128 tiles measured faster than 16 x 128 (54.1 vs 57.4 us per step)
     for (int i = 0; i < 3 && ok; ++i) ok = encode_map(&h->maps[i], h->th[i], p->L, h->tma_rows);
     if (ok) ok = encode_map(&h->maps[3], h->d_p, p->L, h->tma_rows);
-    if (ok) ok = encode_map(&h->maps[4], h->d_p2, p->L, h->tma_rows);
     // AUTO falls back to the plain tiled kernel without the encoder
     if (e == cudaSuccess && !ok && p->kernel == XY_HMC_KERNEL_TILED_TMA) e = cudaErrorNotSupported;
     h->use_tma = ok;
