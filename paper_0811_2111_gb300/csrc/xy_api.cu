@@ -439,9 +439,9 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
   c->fused = p->algorithm == XY_ALGO_FUSED || p->algorithm == XY_ALGO_FUSED2 ||
              c->persistent || (p->algorithm == XY_ALGO_AUTO && xyk::fused_supported(p->L));
   if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->ctas_per_sm == 0 &&
-      p->reduce_mode == XY_REDUCE_EXACT && xyk::grid_supported(p->L)) {
+      p->reduce_mode == XY_REDUCE_EXACT && p->L > xyk::kClusterMaxL) {
     bool fits = false;
-    if (xyk::prepare_grid(p->sincos_mode, p->L, c->sms, &fits) != cudaSuccess)
+    if (xyk::prepare_grid(p->sincos_mode, p->L, c->sms, 1, &fits) != cudaSuccess)
       (void)cudaGetLastError();       // the other kernels take the lattice
     if (fits) {
       // optional, and one allocation: the words, the two of ctl, the wait word
@@ -607,11 +607,11 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
     a.error = c->d_wait;
     a.ctl = c->d_wait - 2;
     a.L = c->p.L;
-    a.K = (float)(c->p.beta * c->p.J);
+    a.K[0] = (float)(c->p.beta * c->p.J);
     a.delta = (float)c->p.delta;
     a.rk = rk;
     a.lattice_id = c->p.lattice_id;
-    a.beta = c->p.beta;
+    a.beta[0] = c->p.beta;
     a.spin_limit = xyk::fused_persistent_spin_limit();
     for (int64_t done = 0; done < n;) {
       const int64_t m = std::min<int64_t>(n - done, kResidentSweeps);

@@ -36,6 +36,9 @@
 // wait is bounded; one that runs out sets *error and ends the CTA, and those
 // that wait for it see *error and end too.
 //
+// Up to four lattices run side by side in one launch: the replicas of a quad,
+// whose angles lie `step` floats apart, each on its share of the SMs.
+//
 // Exact sums only: they do not depend on who adds what, while the compensated
 // sums round by thread and warp and keep the kernels that define them.  Any even
 // side: rows have (W + 1) / 2 pairs, and where W = L / 2 is odd (ODD) the last
@@ -98,7 +101,9 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
   __shared__ uint32_t s_cnt[32];
   __shared__ int s_abort;
   const int L = a.L, W = L / 2, pitch = (W + 1) & ~1;
-  const int bx = blockIdx.x % a.nx, by = blockIdx.x / a.nx;
+  const int tiles = a.nx * a.ny;
+  const int rep = blockIdx.x / tiles, tile = blockIdx.x - rep * tiles;
+  const int bx = tile % a.nx, by = tile / a.nx;
   const int np = part_size((W + 1) / 2, a.nx, bx), k0 = 2 * part_first((W + 1) / 2, a.nx, bx);
   const int H = 2 * part_size(L / 2, a.ny, by), y0 = 2 * part_first(L / 2, a.ny, by);
   const int width = min(2 * np, W - k0);
@@ -110,11 +115,16 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
   // the pair is the tile's; so is its second site (not the last of an odd W)
   const bool on = lane < np, both = ODD ? 2 * lane + 1 < width : on;
   const size_t plane = (size_t)L * (size_t)W;
-  const uint32_t base = __ldcg(a.ctl);
+  unsigned int* ctl = a.ctl + 2 * rep;
+  const uint32_t base = __ldcg(ctl);
+  const uint32_t lattice_id = a.lattice_id + (uint32_t)rep;
+  xy_record* rec = a.rec + rep;
   if (threadIdx.x == 0) s_abort = 0;
   // where the lane's pair of row y of colour c is exchanged under tag t
   auto word_at = [&](uint32_t t, int c, int y) {
-    return (((t & 1u) * 2u + (uint32_t)c) * (uint32_t)L + (uint32_t)y) * (uint32_t)pitch + (uint32_t)kp;
+    return ((((uint32_t)rep * 2u + (t & 1u)) * 2u + (uint32_t)c) * (uint32_t)L + (uint32_t)y) *
+               (uint32_t)pitch +
+           (uint32_t)kp;
   };
   // lanes past the tile's pairs (fewer than 32) store to a row's last place,
   // which such a tile does not use; the half pair of an odd W leaves the halo
@@ -131,9 +141,9 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
   auto draw = [&](int y, int c, uint32_t sweep) {
     return xyd::philox_pair_words(
         (uint32_t)y * (uint32_t)L + 2u * (uint32_t)kp + (((uint32_t)y + (uint32_t)c) & 1u), sweep,
-        a.lattice_id, a.rk);
+        lattice_id, a.rk);
   };
-  const float2 K = xyd::dup2(a.K);
+  const float2 K = xyd::dup2(a.K[rep]);
 
   if (warp >= a.tile_warps) {
     // ---- halo warps: 0 the row pairs above the tile, 1 those below, the rest
@@ -221,7 +231,7 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
       for (int s = 0; s < a.n_sweeps; ++s) {
         const uint32_t sweep = a.sweep0 + (uint32_t)s, tag = base + (uint32_t)s;
         const uint4 w = xyd::philox4x32_10(
-            make_uint4(xyd::metropolis_counter(site, x), sweep, a.lattice_id, 1u), a.rk);
+            make_uint4(xyd::metropolis_counter(site, x), sweep, lattice_id, 1u), a.rk);
         const uint2 uw = xyd::metropolis_words(w, x);
         auto wait_word = [&](const u64* p) {
           u64 v;
@@ -266,7 +276,7 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
           const float2 d = get_one(nb[-1], cc), u = get_one(nb[1], cc);
           const xyd::SiteResult res = xyd::metropolis_step<MODE>(
               t, c0, s0, xyd::nb_sum(l.x, r.x, d.x, u.x), xyd::nb_sum(l.y, r.y, d.y, u.y), uw.x,
-              uw.y, a.K, a.delta);
+              uw.y, K.x, a.delta);
           put_one(csr[i + 1], cc, res.c, res.s);
         }
         cta_sync();
@@ -290,9 +300,9 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
         const int row = r0 + rr;
         if (row < H) {
           if (on) {
-            const float* g = a.theta + c * plane + (size_t)(y0 + row) * W + kp;
+            const float* g = a.theta + (c * plane + (size_t)(y0 + row) * W + kp) * a.step + rep;
             th[c][rr].x = g[0];
-            if (both) th[c][rr].y = g[1];
+            if (both) th[c][rr].y = g[a.step];
           }
           publish(c, rr, th[c][rr], word_at(base, c, y0 + r0), base);
           xyd::PairResult p;
@@ -314,7 +324,7 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
           if (lane == 0) {
             atomicAdd(reinterpret_cast<u64*>(&r->accepted), (u64)total);
             if (bad) atomicOr(reinterpret_cast<u64*>(&r->flags), 1ull);
-            if (blockIdx.x == 0) r->beta = a.beta;
+            if (tile == 0) r->beta = a.beta[rep];
           }
         } else {
           const int32_t v = has ? (int32_t)s_part[lane][task] : 0;
@@ -365,7 +375,7 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
         if (!last) publish(0, rr, p.th, at, next);
         n_acc += (p.acc0 ? 1u : 0u) + (p.acc1 && !half ? 1u : 0u);
       }
-      if (s > 0) commit(a.rec + (s - 1));
+      if (s > 0) commit(rec + (size_t)(s - 1) * a.step);
       if (NR == 1) ahead = early;
       cta_sync();
       xyd::SweepSums<0> sums;
@@ -417,23 +427,23 @@ __global__ void __launch_bounds__(MAXT) k_sweep_grid(GridArgs a) {
     if (!aborted) {
       // the tile warps alone: the halo warps have left their loop
       asm volatile("bar.sync 1, %0;" ::"r"(a.tile_warps * 32) : "memory");
-      commit(a.rec + (a.n_sweeps - 1));
+      commit(rec + (size_t)(a.n_sweeps - 1) * a.step);
 #pragma unroll
       for (int c = 0; c < 2; ++c)
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr)
           if (on && r0 + rr < H) {
-            float* g = a.theta + c * plane + (size_t)(y0 + r0 + rr) * W + kp;
+            float* g = a.theta + (c * plane + (size_t)(y0 + r0 + rr) * W + kp) * a.step + rep;
             g[0] = th[c][rr].x;
-            if (both) g[1] = th[c][rr].y;
+            if (both) g[a.step] = th[c][rr].y;
           }
     }
   }
   // the exchanges made: the next launch's tags go on from here.  Every thread of
   // the CTA read ctl[0] before its first barrier.
-  if (threadIdx.x == 0 && atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1) {
-    a.ctl[1] = 0u;
-    a.ctl[0] = base + (uint32_t)a.n_sweeps;
+  if (threadIdx.x == 0 && atomicAdd(ctl + 1, 1u) == (unsigned int)tiles - 1u) {
+    ctl[1] = 0u;
+    ctl[0] = base + (uint32_t)a.n_sweeps;
   }
 }
 
@@ -460,7 +470,7 @@ struct Plan {
   size_t smem;
 };
 
-// The tiles of side L on `sms` multiprocessors (shape < 0: they fit none).  As
+// The tiles of a lattice of side L on `sms` multiprocessors (shape < 0: they fit none).  As
 // many as there are SMs, of four rows at least: us per sweep by rows of a tile
 //   L = 256   4: 1.51   8: 1.69   12: 1.91      (one cluster of 16 CTAs: 3.1)
 //   L = 384   8: 1.70  12: 1.93   16: 2.09
@@ -468,6 +478,7 @@ Plan plan_of(int L, int sms) {
   Plan p = {};
   p.shape = -1;
   const int W = L / 2;
+  if (L & 1) return p;
   p.nx = ((W + 1) / 2 + 31) / 32;
   p.ny = sms / p.nx < L / 4 ? sms / p.nx : L / 4;
   if (p.ny < 3) return p;
@@ -507,16 +518,15 @@ cudaError_t with_kernel(int mode, int L, int shape, const F& f) {
 
 }  // namespace
 
-bool grid_supported(int L) { return L > kClusterMaxL && (L & 1) == 0; }
-
 size_t grid_words(int L) {
   return 4 * (size_t)L * (size_t)((L / 2 + 1) & ~1);
 }
 
-cudaError_t prepare_grid(int sincos_mode, int L, int sms, bool* fits) {
+cudaError_t prepare_grid(int sincos_mode, int L, int sms, int replicas, bool* fits) {
   *fits = false;
-  const Plan p = plan_of(L, sms);
-  if (!grid_supported(L) || p.shape < 0) return cudaSuccess;
+  if (replicas < 1 || replicas > kGridReplicas) return cudaErrorInvalidValue;
+  const Plan p = plan_of(L, sms / replicas);
+  if (p.shape < 0) return cudaSuccess;
   int n = 0;
   const cudaError_t e = with_kernel(sincos_mode, L, p.shape, [&](auto* fn) {
     cudaError_t r = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -526,21 +536,22 @@ cudaError_t prepare_grid(int sincos_mode, int L, int sms, bool* fits) {
     if (r != cudaSuccess) return r;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, p.threads, p.smem);
   });
-  *fits = e == cudaSuccess && n * sms >= p.nx * p.ny;
+  *fits = e == cudaSuccess && n * sms >= replicas * p.nx * p.ny;
   return e;
 }
 
 cudaError_t launch_grid(int sincos_mode, const GridArgs& args, int sms, cudaStream_t stream) {
-  const Plan p = plan_of(args.L, sms);
-  if (!grid_supported(args.L) || p.shape < 0 || args.n_sweeps < 1 || args.spin_limit < 1)
+  if (args.replicas < 1 || args.replicas > kGridReplicas || args.n_sweeps < 1 || args.spin_limit < 1)
     return cudaErrorInvalidValue;
+  const Plan p = plan_of(args.L, sms / args.replicas);
+  if (p.shape < 0) return cudaErrorInvalidValue;
   GridArgs a = args;
   a.nx = p.nx;
   a.ny = p.ny;
   a.tile_warps = p.tile_warps;
   return with_kernel(sincos_mode, args.L, p.shape, [&](auto* fn) {
     void* params[] = {&a};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fn), dim3(p.nx * p.ny),
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fn), dim3(args.replicas * p.nx * p.ny),
                                        dim3(p.threads), params, p.smem, stream);
   });
 }

@@ -171,22 +171,27 @@ int fused_persistent_max_sweeps(int L);
 cudaError_t launch_fused_persistent(int sincos_mode, int reduce_mode, const FusedPersistArgs& a,
                                     cudaStream_t stream);
 
-// All sweeps of a call of a middling lattice in one cooperative launch, in
-// place, every tile staying with its CTA, exact sums (xy_grid.cu).
+// All sweeps of a call of a middling lattice, or of `replicas` such lattices side
+// by side, in one cooperative launch, in place, every tile staying with its CTA,
+// exact sums (xy_grid.cu).
+constexpr int kGridReplicas = 4;
 struct GridArgs {
-  float* theta;          // [2][L][W]: the state, read and rewritten
-  unsigned long long* words;   // grid_words(L) exchange words, zeroed once
-  unsigned int* ctl;     // [2]: the next tag (1 at first), CTAs that have finished (0)
+  float* theta;          // the state, read and rewritten: [2][L][W] places of `step` floats,
+                         // replica r's angle the r-th of a place
+  unsigned long long* words;   // replicas x grid_words(L) exchange words, zeroed once
+  unsigned int* ctl;     // per replica: the next tag (1 at first), CTAs that have finished (0)
   unsigned int* error;   // set nonzero when a bounded wait runs out
   int L;
-  float K;
+  int replicas = 1;
+  int step = 1;
+  float K[kGridReplicas];
+  double beta[kGridReplicas];
   float delta;
   xyd::RoundKeys rk;
-  uint32_t lattice_id;
+  uint32_t lattice_id;   // of replica 0
   uint32_t sweep0;       // Philox sweep word of the first sweep
   int n_sweeps;
-  xy_record* rec;        // records of the n sweeps, zeroed
-  double beta;
+  xy_record* rec;        // records of the n sweeps, zeroed; replica r's the r-th of every `step`
   long long spin_limit;  // polls before a wait gives up
   int nx, ny, tile_warps;      // set by launch_grid
 };
@@ -194,11 +199,11 @@ struct GridArgs {
 // to one tile per SM where they fit: us per sweep, cluster and tiles, L = 128
 // 1.52 and 1.59, 160 1.94 and 1.68, 256 3.1 and 1.51.
 constexpr int kClusterMaxL = 128;
-bool grid_supported(int L);
 // Exchange words of side L.
 size_t grid_words(int L);
-// Whether side L fits a device of `sms` multiprocessors (outside any capture).
-cudaError_t prepare_grid(int sincos_mode, int L, int sms, bool* fits);
+// Whether `replicas` lattices of side L fit a device of `sms` multiprocessors side
+// by side (outside any capture).
+cudaError_t prepare_grid(int sincos_mode, int L, int sms, int replicas, bool* fits);
 cudaError_t launch_grid(int sincos_mode, const GridArgs& a, int sms, cudaStream_t stream);
 
 // All sweeps of a call of a small lattice in one cluster launch, in place, the

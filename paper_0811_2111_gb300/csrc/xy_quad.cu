@@ -1,7 +1,8 @@
 // xy_quad.cu -- four replicas per site (the RGBA packing of Sec. 3.2): the
 // two-pass checkerboard half-sweep over float4 sites (any even L), and the C
 // ABI of include/xy_quad.h around it and around the one-launch sweep of
-// xy_quad_fused.cu (L % 32 == 0).
+// xy_quad_fused.cu (L % 32 == 0).  XY_ALGO_AUTO sweeps up to L = 1280 mostly run the
+// replicas as lattices held on the chip instead (xy_grid.cu, exact sums).
 //
 // Layout: [colour][y][k] of float4, component r = replica r.  A half-sweep of
 // colour c stages the other colour's tile plus a one-site halo as unit vectors
@@ -199,6 +200,22 @@ cudaError_t launch_quad_half(int colour, int mode, int red, const QuadArgs& a, c
 // 136.5)
 constexpr int kAutoPersistentMaxL = 1024;
 
+// Whether AUTO takes the replicas held on the chip where they fit.  us per sweep
+// of the four, this and the kernel it replaces:
+//   L no multiple of 32 (two-pass)     500 5.5, 20.6   1000 21.8, 47.3
+//   up to 672 (four or two at a time)  32 1.4, 5.5   256 2.1, 6.9   512 6.5, 10.0
+//                                      640 8.7, 12.7   672 10.9, 13.1
+// above only where the tiles fill their warps' lanes (L % 128 == 0):
+//   768 13.4, 14.9   896 17.4, 18.5   1024 21.1, 23.2   1280 34.1, 36.9
+//   but 704 13.5, 13.6   800 16.0, 15.6   960 21.2, 20.7
+// and, as the tile's own unit vectors are not computed again each sweep, with
+// libm sincos always (800 18.3, 23.6; 1024 25.0, 32.0) and with the SFU's never
+// (896 15.7, 14.7; 1024 19.2, 18.5).
+bool grid_wins(int L, int sincos_mode) {
+  if (L % 32 != 0 || L <= 672) return true;
+  return sincos_mode == 2 || (sincos_mode == 0 && L % 128 == 0);
+}
+
 constexpr uint32_t kMagicLive = 0x51554144u;   // "QUAD"
 constexpr uint32_t kMagicDead = 0xDEADF00Du;
 
@@ -238,6 +255,9 @@ struct xy_quad {
   bool persistent;         // ... all sweeps of a call in one cooperative launch
   bool auto_persistent;    // chosen by XY_ALGO_AUTO: per-sweep launches if it does not fit
   unsigned int* d_tiles;   // the persistent launch's tile counters, work counter, error word
+  int grid;                // replicas held on the chip side by side (xy_grid.cu); 0: not this way
+  int sms;
+  unsigned long long* d_words;   // their exchange words, then the replicas' ctl[2] and the wait word
   int cur;                 // which buffer holds the state (0: d_theta, 1: d_theta2)
   float4* d_theta;         // [2][L][L/2] float4
   float4* d_theta2;        // the fused sweep's second buffer (NULL for two-pass)
@@ -297,13 +317,19 @@ xy_status check(const xy_quad* q) {
 
 float4* current(const xy_quad* q) { return q->cur ? q->d_theta2 : q->d_theta; }
 
+// The replicas' control words (and, behind them, the wait word).
+unsigned int* grid_ctl(const xy_quad* q) {
+  return reinterpret_cast<unsigned int*>(q->d_words + (size_t)q->grid * xyk::grid_words(q->p.L));
+}
+
 // After a synchronize: whether a persistent launch's bounded wait ran out.
 xy_status check_waits(xy_quad* q, const char* where) {
-  if (!q->persistent || !q->d_tiles) return XY_OK;
+  const unsigned int* word = q->grid ? grid_ctl(q) + 2 * q->grid
+                             : q->persistent && q->d_tiles
+                                 ? q->d_tiles + xyk::quad_persistent_tiles(q->p.L) + 1 : nullptr;
+  if (!word) return XY_OK;
   unsigned int w = 0;
-  const int tiles = xyk::quad_persistent_tiles(q->p.L);
-  Q_CUDA(q, cudaMemcpyAsync(&w, q->d_tiles + tiles + 1, sizeof(w), cudaMemcpyDeviceToHost, q->stream),
-         where);
+  Q_CUDA(q, cudaMemcpyAsync(&w, word, sizeof(w), cudaMemcpyDeviceToHost, q->stream), where);
   Q_CUDA(q, cudaStreamSynchronize(q->stream), where);
   if (w) return fail(q, XY_ETIMEOUT, "%s: a persistent sweep's wait for a neighbouring tile ran out",
                      where);
@@ -314,6 +340,7 @@ void release(xy_quad* q) {
   if (q->d_theta) cudaFree(q->d_theta);
   if (q->d_theta2) cudaFree(q->d_theta2);
   if (q->d_tiles) cudaFree(q->d_tiles);
+  if (q->d_words) cudaFree(q->d_words);
   if (q->d_scratch) cudaFree(q->d_scratch);
   if (q->d_nat) cudaFree(q->d_nat);
   if (q->d_rec) cudaFree(q->d_rec);
@@ -337,6 +364,75 @@ xy_status grow(xy_quad* q, int64_t sweeps) {
   if (q->d_rec) cudaFree(q->d_rec);
   q->d_rec = nr;
   q->rec_cap = cap;
+  return XY_OK;
+}
+
+// Sweeps [done, done + m) of a call by the two-pass kernels, in place.
+xy_status two_pass_sweeps(xy_quad* q, int64_t done, int64_t m) {
+  QuadArgs a;
+  a.theta = current(q);
+  a.L = q->p.L;
+  a.W = q->p.L / 2;
+  for (int j = 0; j < kR; ++j) {
+    a.K[j] = (float)(q->beta[j] * q->p.J);
+    a.beta[j] = q->beta[j];
+  }
+  a.delta = (float)q->p.delta;
+  a.rk = xyd::make_round_keys(q->p.seed);
+  a.lattice_id0 = q->p.lattice_id;
+  for (int64_t i = done; i < done + m; ++i) {
+    a.sweep = (uint32_t)(q->next_sweep + (uint64_t)i);
+    a.rec = q->d_rec + (q->rec_count + i) * kR;
+    Q_CUDA(q, launch_quad_half(0, q->p.sincos_mode, q->p.reduce_mode, a, q->stream),
+           "xy_quad_sweep: red half");
+    Q_CUDA(q, launch_quad_half(1, q->p.sincos_mode, q->p.reduce_mode, a, q->stream),
+           "xy_quad_sweep: black half");
+  }
+  return XY_OK;
+}
+
+// At most this many sweeps in one launch of the replicas held on the chip.
+constexpr int64_t kGridSweeps = 1 << 16;
+
+// The n sweeps of a call, q->grid replicas side by side; a launch that finds no
+// room (beside other work) is made up for by the two-pass kernels, which do all
+// four replicas, so only the first of a group of launches may be refused.
+xy_status grid_sweeps(xy_quad* q, int64_t n) {
+  xyk::GridArgs a;
+  a.words = q->d_words;
+  a.ctl = grid_ctl(q);
+  a.error = a.ctl + 2 * q->grid;
+  a.L = q->p.L;
+  a.replicas = q->grid;
+  a.step = kR;
+  a.delta = (float)q->p.delta;
+  a.rk = xyd::make_round_keys(q->p.seed);
+  a.spin_limit = xyk::fused_persistent_spin_limit();
+  for (int64_t done = 0; done < n;) {
+    const int64_t m = std::min<int64_t>(n - done, kGridSweeps);
+    a.sweep0 = (uint32_t)(q->next_sweep + (uint64_t)done);
+    a.n_sweeps = (int)m;
+    for (int r = 0; r < kR; r += q->grid) {
+      a.theta = reinterpret_cast<float*>(q->d_theta) + r;
+      a.lattice_id = q->p.lattice_id + (uint32_t)r;
+      a.rec = q->d_rec + (q->rec_count + done) * kR + r;
+      for (int j = 0; j < q->grid; ++j) {
+        a.K[j] = (float)(q->beta[r + j] * q->p.J);
+        a.beta[j] = q->beta[r + j];
+      }
+      const cudaError_t e = xyk::launch_grid(q->p.sincos_mode, a, q->sms, q->stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge && r == 0) {
+        (void)cudaGetLastError();
+        const xy_status st = two_pass_sweeps(q, done, m);
+        if (st != XY_OK) return st;
+        break;
+      }
+      Q_CUDA(q, e, "xy_quad_sweep: grid launch");
+    }
+    done += m;
+  }
+  q->next_sweep += (uint64_t)n;
+  q->rec_count += n;
   return XY_OK;
 }
 
@@ -397,8 +493,35 @@ xy_status xy_quad_create(const xy_params* p, const double beta[4], void* cuda_st
   const size_t N = (size_t)p->L * (size_t)p->L;
   const char* step = "angle buffer";
   cudaError_t e = xyk::dev_malloc(&q->d_theta, N * sizeof(float4));
-  if (e == cudaSuccess && q->fused) e = xyk::dev_malloc(&q->d_theta2, N * sizeof(float4));
-  if (e == cudaSuccess && q->persistent) {
+  // AUTO: as many replicas side by side on the chip as fit, the others after them
+  if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->reduce_mode == XY_REDUCE_EXACT &&
+      grid_wins(p->L, p->sincos_mode)) {
+    int dev = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&q->sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int g = kR; e == cudaSuccess && g >= 1 && !q->grid; g /= 2) {
+      bool fits = false;
+      if (xyk::prepare_grid(p->sincos_mode, p->L, q->sms, g, &fits) != cudaSuccess)
+        (void)cudaGetLastError();
+      if (fits) q->grid = g;
+    }
+    if (e == cudaSuccess && q->grid) {
+      // optional, and one allocation
+      const size_t bytes = (size_t)q->grid * xyk::grid_words(p->L) * sizeof(unsigned long long);
+      const size_t tail = (2 * (size_t)q->grid + 2) * sizeof(unsigned int);
+      if (xyk::dev_malloc(&q->d_words, bytes + tail) == cudaSuccess) {
+        e = cudaMemsetAsync(q->d_words, 0, bytes + tail, q->stream);
+        for (int g = 0; e == cudaSuccess && g < q->grid; ++g)      // ctl[0] = 1 (the low byte)
+          e = cudaMemsetAsync(grid_ctl(q) + 2 * g, 1, 1, q->stream);
+      } else {
+        (void)cudaGetLastError();
+        q->d_words = nullptr;
+        q->grid = 0;
+      }
+    }
+  }
+  if (e == cudaSuccess && q->fused && !q->grid) e = xyk::dev_malloc(&q->d_theta2, N * sizeof(float4));
+  if (e == cudaSuccess && q->persistent && !q->grid) {
     const size_t words = (size_t)xyk::quad_persistent_tiles(p->L) + 2;
     e = xyk::dev_malloc(&q->d_tiles, words * sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMemsetAsync(q->d_tiles, 0, words * sizeof(unsigned int), q->stream);
@@ -448,6 +571,7 @@ xy_status xy_quad_sweep(xy_quad* q, int64_t n) {
   Q_CUDA(q, cudaMemsetAsync(q->d_rec + q->rec_count * kR, 0, (size_t)n * kR * sizeof(xy_record),
                             q->stream),
          "xy_quad_sweep: record clear");
+  if (q->grid) return grid_sweeps(q, n);
   if (q->persistent) {
     xyk::QuadPersistArgs pa;
     pa.a.src = nullptr;
@@ -522,25 +646,8 @@ xy_status xy_quad_sweep(xy_quad* q, int64_t n) {
     q->rec_count += n;
     return XY_OK;
   }
-  QuadArgs a;
-  a.theta = current(q);
-  a.L = q->p.L;
-  a.W = q->p.L / 2;
-  for (int j = 0; j < kR; ++j) {
-    a.K[j] = (float)(q->beta[j] * q->p.J);
-    a.beta[j] = q->beta[j];
-  }
-  a.delta = (float)q->p.delta;
-  a.rk = xyd::make_round_keys(q->p.seed);
-  a.lattice_id0 = q->p.lattice_id;
-  for (int64_t i = 0; i < n; ++i) {
-    a.sweep = (uint32_t)(q->next_sweep + (uint64_t)i);
-    a.rec = q->d_rec + (q->rec_count + i) * kR;
-    Q_CUDA(q, launch_quad_half(0, q->p.sincos_mode, q->p.reduce_mode, a, q->stream),
-           "xy_quad_sweep: red half");
-    Q_CUDA(q, launch_quad_half(1, q->p.sincos_mode, q->p.reduce_mode, a, q->stream),
-           "xy_quad_sweep: black half");
-  }
+  st = two_pass_sweeps(q, 0, n);
+  if (st != XY_OK) return st;
   q->next_sweep += (uint64_t)n;
   q->rec_count += n;
   return XY_OK;
