@@ -208,8 +208,8 @@ void make_plan(xy_batch* b, int target_sites) {
   // default plan throughout and one side in the whole batch so are the others
   // where that is estimated faster than their own path (measured: tiles 230 G
   // updates/s and no less than 5 us a sweep, narrow tiles 155 and 4.5, whole
-  // lattices 0.5 us + 0.8 ns a site): ten of L = 64 3.0 -> 1.65, ten of 96 6.25
-  // -> 1.95, four of 128 5.0 -> 1.6, two of 256 5.0 -> 3.3.  Beside lattices of
+  // lattices 1.0 us up to L = 32, 1.4 to 36, 1.7 to 44, 2.05 to 48, 2.9 above): ten of L = 64 3.0 ->
+  // 1.65, ten of 96 6.25 -> 1.95, four of 128 5.0 -> 1.6, two of 256 5.0 -> 3.3.  Beside lattices of
   // other sides those paths share the GPU better.
   std::map<int, int> res_ctas;
   if (b->p.algorithm == XY_ALGO_AUTO && b->p.reduce_mode == XY_REDUCE_EXACT &&
@@ -220,7 +220,8 @@ void make_plan(xy_batch* b, int target_sites) {
       const int L = kv.first, n = (int)kv.second.size();
       const double sites = (double)n * L * L;
       const double other = xyk::fused_supported(L) ? std::max(5.0, sites / 230e3)
-                           : xyk::small_supported(L) ? (0.5 + 0.8e-3 * L * L) * ((n + 303) / 304)
+                           : xyk::small_supported(L)
+                               ? (L <= 32 ? 1.0 : L <= 36 ? 1.4 : L <= 44 ? 1.7 : L <= 48 ? 2.05 : 2.9) * ((n + 303) / 304)
                            : xyk::narrow_supported(L) ? std::max(4.5, sites / 155e3) : 1e30;
       if (other < 1e30 && (by_side.size() > 1 || !default_plan)) continue;
       int ctas = 0;

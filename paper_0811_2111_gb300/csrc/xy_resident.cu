@@ -337,23 +337,31 @@ cudaError_t prepare_resident(int sincos_mode, int L, bool* fits) {
 }
 
 // Time of a sweep of n lattices of side L by cluster size: a strip's latency
-// (1.45 us for up to 128 pairs of a colour per CTA, 1.5 for 256, 2.0 for 512,
-// 3.5 for 1024, single lattices of L = 64 ... 256), once per wave of the
-// clusters that run at a time.
+// (1.9 us for up to 64 pairs of a colour per CTA, whose two warps add up the six
+// sums, 1.45 for 128, 1.5 for 256, 2.0 for 512, 3.5 for 1024, single lattices of
+// L = 32 ... 256), once per wave of the
+// clusters that run at a time, and a quarter more for each further CTA that
+// shares an SM (L = 48 in clusters of 8: two lattices 1.55, 20 1.97, 30 2.04, 41
+// 2.31).
 cudaError_t prepare_resident_batch(int sincos_mode, int L, int n, int* ctas, double* us) {
   *ctas = 0;
   *us = 0.0;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   for (int c = 1; c <= 16; c *= 2) {
     const Plan p = plan_of(L, c);
     if (p.ctas == 0) continue;
     int at_a_time = 0;
-    const cudaError_t e = clusters_of(sincos_mode, p, &at_a_time);
+    e = clusters_of(sincos_mode, p, &at_a_time);
     if (e != cudaSuccess) return e;
     if (at_a_time < 1) continue;
     const int pairs = strip_rows(L, c, 0) * ((L / 2 + 1) / 2);
-    const double strip = pairs <= 256 ? 1.4 + 0.0004 * pairs : 1.0 + 0.002 * pairs +
-                         (p.np > 1 ? 0.5 : 0.0);
-    const double t = strip * (double)((n + at_a_time - 1) / at_a_time);
+    const double strip = pairs <= 64 ? 1.9 : pairs <= 256 ? 1.4 + 0.0004 * pairs
+                         : 1.0 + 0.002 * pairs + (p.np > 1 ? 0.5 : 0.0);
+    const int shared = ((n < at_a_time ? n : at_a_time) * c + sms - 1) / sms;
+    const double t = strip * (1.0 + 0.25 * (shared - 1)) * (double)((n + at_a_time - 1) / at_a_time);
     if (*ctas == 0 || t < *us) {
       *ctas = c;
       *us = t;
