@@ -493,6 +493,12 @@ xy_status xy_quad_create(const xy_params* p, const double beta[4], void* cuda_st
   const size_t N = (size_t)p->L * (size_t)p->L;
   const char* step = "angle buffer";
   cudaError_t e = xyk::dev_malloc(&q->d_theta, N * sizeof(float4));
+  if (e == cudaSuccess) {
+    step = "scratch buffers";
+    e = xyk::dev_malloc(&q->d_scratch, N * sizeof(float));
+    if (e == cudaSuccess) e = xyk::dev_malloc(&q->d_nat, N * sizeof(float));
+  }
+  if (e == cudaSuccess) step = "sweep buffers";
   // AUTO: as many replicas side by side on the chip as fit, the others after them
   if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->reduce_mode == XY_REDUCE_EXACT &&
       grid_wins(p->L, p->sincos_mode)) {
@@ -525,11 +531,6 @@ xy_status xy_quad_create(const xy_params* p, const double beta[4], void* cuda_st
     const size_t words = (size_t)xyk::quad_persistent_tiles(p->L) + 2;
     e = xyk::dev_malloc(&q->d_tiles, words * sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMemsetAsync(q->d_tiles, 0, words * sizeof(unsigned int), q->stream);
-  }
-  if (e == cudaSuccess) {
-    step = "scratch buffers";
-    e = xyk::dev_malloc(&q->d_scratch, N * sizeof(float));
-    if (e == cudaSuccess) e = xyk::dev_malloc(&q->d_nat, N * sizeof(float));
   }
   if (e == cudaSuccess) {
     step = "start kernel";

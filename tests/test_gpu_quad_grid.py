@@ -37,7 +37,7 @@ def test_without_the_exchange_words_the_other_kernels_run(L):
     from paper_0811_2111_gb300 import _lib as X
     from paper_0811_2111_gb300.lattice import Quad
     ref = _run(L, "two_pass", (5,))
-    X.lib().xy_debug_fail_alloc(2)      # the state is the first allocation
+    X.lib().xy_debug_fail_alloc(4)      # after the state and the two scratch buffers
     with Quad(L, BETAS, 17, lattice_id=5) as q:
         X.lib().xy_debug_fail_alloc(0)
         q.sweep(5)
