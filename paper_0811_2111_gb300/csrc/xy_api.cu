@@ -59,11 +59,13 @@ void set_thread_msg(const char* fmt, ...) {
 constexpr int kAutoPersistentMaxL = 4096;
 
 // Default work plan of the persistent sweep: 2 CTAs per SM (128 registers a
-// thread) where that many hold all of a sweep's tiles (L <= 1024 on 152 SMs:
-// a sweep is then one tile's latency, and more registers shorten it: 5.8
-// against 6.4 us per sweep at L = 512, 8.9 against 9.3 at 1024), else 3 (L =
-// 2048: 19.2 against 19.5 us).
-constexpr int kFewTilesPerSm = 2;
+// thread) up to six of a sweep's tiles per SM, else 3: with few tiles a sweep
+// waits for a tile's latency, which more registers shorten.  With SFU sincos and
+// on overlapping tiles up to four.  us per sweep, 2 and 3: L = 512 5.8, 6.4   1408
+// 10.3, 11.7   1536 11.8, 12.7 (libm 17.4, 23.8; SFU 9.7, 10.7)   1792 15.0, 15.6
+// (libm 20.8, 25.0; SFU 12.8, 12.1)   2048 19.5, 19.4 (libm 27.4, 25.9);
+// overlapping 1300 10.9, 12.7   1504 12.8, 13.6   2004 22.5, 21.8.
+constexpr int kFewTilesPerSm = 6, kFewTilesPerSmShort = 4;
 
 struct xy_ctx {
   uint32_t magic;
@@ -645,7 +647,9 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
     a.spin_limit = xyk::fused_persistent_spin_limit();
     a.skip_items = 0;
     a.minb = c->p.ctas_per_sm ? c->p.ctas_per_sm
-             : xyk::fused_tiles(c->p.L) <= kFewTilesPerSm * c->sms ? 2 : 3;
+             : xyk::fused_tiles(c->p.L) <=
+                       (c->ragged || c->p.sincos_mode == 1 ? kFewTilesPerSmShort
+                                                           : kFewTilesPerSm) * c->sms ? 2 : 3;
     // one launch per at most fused_persistent_max_sweeps sweeps (the kernel's
     // work items are counted in 32 bits)
     const int64_t chunk = xyk::fused_persistent_max_sweeps(c->p.L);

@@ -150,7 +150,8 @@ __device__ __forceinline__ unsigned char* smem_base() {
   return smem;
 }
 
-// RAG: a side that is no multiple of the tile (any even L >= 130; exact sums).
+// RAG: a side that is no multiple of the tile (any even L >= 130; exact sums; 1
+// where W is even, 2 where it is odd).
 // The last tile of a row or column of tiles is moved back so that it ends with
 // the lattice and overlaps the tile before it: the overlap is computed twice,
 // with the same words from the same old state, so both copies store the same
@@ -159,7 +160,7 @@ __device__ __forceinline__ unsigned char* smem_base() {
 // is column W, that is column 0: staged, never stored, and as the right
 // neighbour of column W - 1 updated with the side ring.
 template <int MODE, int RED, bool COHERENT = false, bool TMA = false, int NANG = 1,
-          bool RAG = false, class Args, class PreHook = NoHook, class MidHook = NoHook, class EndHook = NoHook,
+          int RAG = 0, class Args, class PreHook = NoHook, class MidHook = NoHook, class EndHook = NoHook,
           class PostHook = NoHook, class RawWait = NoHook>
 __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::RoundKeys& rk, int bx,
                                                  int by, int ang_sel = 0,
@@ -180,17 +181,17 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
 
   static_assert(!RAG || (!TMA && RED == 0), "ragged tiles load per thread and sum exactly");
   const int L = a.L, W = a.W;
-  const int k0 = RAG ? min(bx * kTileK, W - kTileK + (W & 1)) : bx * kTileK;
+  const int k0 = RAG ? min(bx * kTileK, W - kTileK + (RAG == 2 ? 1 : 0)) : bx * kTileK;
   const int y0 = RAG ? min(by * kTileRows, L - kTileRows) : by * kTileRows;
   // columns of the tile inside the lattice (63 in the last tile of an odd W)
-  const int width = RAG ? min(kTileK, W - k0) : kTileK;
+  const int width = RAG == 2 ? min(kTileK, W - k0) : kTileK;
   const size_t plane = (size_t)L * (size_t)W;
   // RAG: four (two) staged columns from column k (even, a multiple of four from
   // k0) of the row at `row`: as wide as the rows' alignment allows
   auto ragged4 = [&](size_t row, int k) {
     const float* p = a.src + row;
-    if ((W & 3) == 0) return __ldcg(reinterpret_cast<const float4*>(p + k));
-    if ((W & 1) == 0) {
+    if (RAG == 1) {
+      if ((W & 3) == 0) return __ldcg(reinterpret_cast<const float4*>(p + k));
       const float2 u = __ldcg(reinterpret_cast<const float2*>(p + k));
       const float2 v = __ldcg(reinterpret_cast<const float2*>(p + k + 2));
       return make_float4(u.x, u.y, v.x, v.y);
@@ -232,7 +233,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const bool has_tail = t < 192;
     const int tail_r = 29 + (t >> 5), tail_c = t & 31;
     float2 vt = make_float2(0.f, 0.f);
-    if (RAG && has_tail && (W & 1)) {
+    if (RAG == 2 && has_tail) {
       const float* p = a.src + (size_t)wrap_once(y0 - 2 + tail_r, L) * W;
       vt = make_float2(__ldcg(p + k0 + 2 * tail_c), __ldcg(p + wrap_once(k0 + 2 * tail_c + 1, W)));
     } else if (has_tail && !TMA) {
@@ -320,7 +321,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
   unsigned int n_acc = 0;
   // RAG: whether both of the pair's columns are the tile's; whether a row's
   // pair is counted here; its stores
-  const bool both = !RAG || 2 * lane + 1 < width;
+  const bool both = RAG != 2 || 2 * lane + 1 < width;
   auto counted = [&](int y) { return y >= by * kTileRows && kp >= bx * kTileK; };
   auto put_own = [&](CsRow& row, const xyd::PairResult& p) {
     if (both) {
@@ -330,7 +331,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     }
   };
   auto store = [&](float* at, const float2& th) {
-    if ((W & 1) == 0) {
+    if (RAG != 2) {
       *reinterpret_cast<float2*>(at) = th;
     } else {
       at[0] = th.x;
@@ -410,7 +411,7 @@ __device__ __forceinline__ void fused_sweep_body(const Args& a, const xyd::Round
     const int k = wrap_once(k0 + tk, W);
     const int q = y & 1;
     const uint32_t x = 2u * (uint32_t)k + (uint32_t)q;
-    const float th = RAG && tk == kTileK - 1 ? ang[kRedRaw0 + ty + 2][kTileK - 1]
+    const float th = RAG == 2 && tk == kTileK - 1 ? ang[kRedRaw0 + ty + 2][kTileK - 1]
                                              : angs[2 * (ty + 1) + (tk < 0 ? 0 : 1)];
     red_ring_site<MODE>(th, csr, csb, ty + 2, tk + kCsOff, q,
                         (uint32_t)y * uL + x, x, a, rk);
@@ -610,10 +611,12 @@ __device__ __forceinline__ PersistItem decode_item(int item, int ntiles, int til
 // neighbours' first copies is its neighbours', the tile before the overlapped
 // one reads nothing that only the last tile's copy writes, and every copy of a
 // site is a neighbour of every tile that reads it.  Against two half-sweep
-// launches a sweep (us per sweep): L = 300 6.3 against 20.5, 1000 9.6 against
-// 22.6, 7324 323 against 430; where W is odd the rows are loaded and stored a
-// word at a time (L = 1002 11.0, 7326 391).
-template <int MODE, int RED, int MINB, bool RAG>
+// launches a sweep (us per sweep): L = 1300 10.9 against 30.9, 2004 21.8 against
+// 53.8, 7324 308 against 430; where W is odd the rows are loaded and stored a
+// word at a time (L = 1302 12.2, 7326 387).  With one body for even and odd W the
+// even ones took 5-9 % longer (2004 23.2, 7324 325); with the next tile's rows
+// copied ahead by cp.async 2004 24.7, 7326 340.
+template <int MODE, int RED, int MINB, int RAG>
 __global__ void __launch_bounds__(kThreads, MINB)
     k_sweep_fused_persist(FusedPersistArgs p, const __grid_constant__ PersistMaps maps) {
   __shared__ int s_abort;
@@ -801,10 +804,10 @@ cudaError_t prepare_one() {
   return e == cudaSuccess ? prepare_plan<MODE, RED, 4>() : e;
 }
 
-template <bool RAG>
+template <int RAG>
 constexpr size_t persist_smem() { return RAG ? kSmemBytes : kPersistSmemBytes; }
 
-template <int MODE, int RED, int MINB, bool RAG>
+template <int MODE, int RED, int MINB, int RAG>
 cudaError_t launch_persist_one(const FusedPersistArgs& a, int grid, cudaStream_t stream) {
   // the maps in buf order (the caller may have swapped the two buffers)
   PersistMaps pm = {};
@@ -819,7 +822,7 @@ cudaError_t launch_persist_one(const FusedPersistArgs& a, int grid, cudaStream_t
       dim3(kThreads), args, persist_smem<RAG>(), stream);
 }
 
-template <int MODE, int RED, int MINB, bool RAG>
+template <int MODE, int RED, int MINB, int RAG>
 cudaError_t persist_grid_one(int L, int* grid) {
   static int per_sm[64] = {};        // resident CTAs per SM, per device (0: not yet set)
   int dev = 0;
@@ -849,7 +852,7 @@ cudaError_t persist_grid_one(int L, int* grid) {
 }
 
 // The persistent launch of one instantiation: grid, then the launch.
-template <int MODE, int RED, int MINB, bool RAG = false>
+template <int MODE, int RED, int MINB, int RAG = 0>
 cudaError_t persist_plan(const FusedPersistArgs& a, cudaStream_t stream) {
   int grid = 0;
   cudaError_t e = persist_grid_one<MODE, RED, MINB, RAG>(a.L, &grid);
@@ -867,11 +870,15 @@ cudaError_t persist_dispatch(const FusedPersistArgs& a, cudaStream_t stream) {
                        : persist_plan<MODE, RED, 3>(a, stream);
 }
 
+template <int MODE, int RAG>
+cudaError_t ragged_plan(const FusedPersistArgs& a, cudaStream_t stream) {
+  return a.minb == 2 ? persist_plan<MODE, 0, 2, RAG>(a, stream)
+                     : persist_plan<MODE, 0, 3, RAG>(a, stream);
+}
+
 template <int MODE>
 cudaError_t ragged_dispatch(const FusedPersistArgs& a, cudaStream_t stream) {
-  return a.minb == 2   ? persist_plan<MODE, 0, 2, true>(a, stream)
-         : a.minb == 4 ? persist_plan<MODE, 0, 4, true>(a, stream)
-                       : persist_plan<MODE, 0, 3, true>(a, stream);
+  return (a.W & 1) ? ragged_plan<MODE, 2>(a, stream) : ragged_plan<MODE, 1>(a, stream);
 }
 
 }  // namespace
