@@ -35,8 +35,10 @@ METRIC = "XY spin-updates/s on 1 GB300 (L=4096 and batched) and % of roofline"
 UNIT = "spin-updates/s"
 FLUSH_BYTES = 256 << 20
 
-# Algorithmic instruction count per site update (one issue slot each), the
-# work the method itself requires on this GPU:
+# Algorithmic instruction count per site update (scalar operations, one per lane
+# and issue slot; the kernels' packed FP32 instructions do two in one slot and
+# hold the FMA pipes as long as two), the work the method itself requires on this
+# GPU:
 #   Philox4x32-10: 20 wide multiplies + 20 three-input xors, 2 + 2 of them shared
 #     by all sites of a sweep -> 36 per block, and one block serves two updates
 #     (the sites x and x + 2 of a row share it) -> 18;
@@ -530,9 +532,9 @@ HMC_BYTES_PER_SITE_STEP = 8.0
 # neighbour sums 6, the force 3, kick and drift 2, the wrap into [0, 2 pi) 8.
 HMC_ALG_INSTR_PER_SITE_STEP = {"accurate": 44.0, "fast": 22.0, "libm": 46.0}
 # DRAM bytes of one L = 4096 two-step launch (ncu, caches flushed before the
-# capture: 134.4 MB read, 83.9 MB written; profiles/hmc_tile2_L4096_full.md),
+# capture: 143.4 MB read, 89.7 MB written; profiles/current_kernels_GB300.md),
 # per step.
-HMC_DRAM_BYTES_PER_STEP = 218.2e6 / 2
+HMC_DRAM_BYTES_PER_STEP = 233.1e6 / 2
 
 
 def measure_hmc(dev, sincos, trajectories=40, cpu_seconds=2.0, issue_per_sm_clk=None,
