@@ -523,7 +523,7 @@ def measure_table1_sizes(dev, sincos, cpu_seconds=1.0):
 # Hybrid Monte Carlo (the paper's own algorithm)
 # ---------------------------------------------------------------------------
 
-# The full kick-drift steps run two per launch (k_hmc_tile2): each launch reads
+# The full kick-drift steps run two per launch (k_hmc_rows2): each launch reads
 # and writes the angle and the momentum of every site once, 16 B per site for
 # two steps.
 HMC_BYTES_PER_SITE_STEP = 8.0
@@ -607,7 +607,7 @@ def measure_hmc(dev, sincos, trajectories=40, cpu_seconds=2.0, issue_per_sm_clk=
             "trajectories_per_s": trajectories / (ms * 1e-3), "ms_per_trajectory": ms / trajectories,
             "begin_final_accept_ms": t[1], "acceptance": float(o["accepted"].mean()),
             "mean_exp_minus_dH": float(np.exp(-o["dH"]).mean()), "e": float(o["e"].mean()),
-            "roofline": {"kernel": "k_hmc_tile2 (two leap-frog steps per launch)",
+            "roofline": {"kernel": "k_hmc_rows2 (two leap-frog steps per launch, by rows)",
                          "bound": "alu", "achieved": alu_achieved, "peak": alu_peak,
                          "unit": "Tinstr/s", "frac": alu_achieved / alu_peak,
                          "peak_kind": "measured" if issue_per_sm_clk else "nominal",

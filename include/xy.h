@@ -70,13 +70,16 @@ enum { XY_SINCOS_ACCURATE = 0, XY_SINCOS_FAST = 1, XY_SINCOS_LIBM = 2 };
 /* Sweep kernel: AUTO picks PERSISTENT when L is a multiple of 128 up to 4096
  * (falling back to one fused launch per sweep when the cooperative grid does
  * not fit on the device), FUSED for larger multiples of 128, else TWO_PASS.
- * Under AUTO with exact sums (and ctas_per_sm = 0) a lattice of 4 <= L <= 256
- * that the device can hold on the chip runs all sweeps of a call in one
- * cluster launch, in place, and any other side above 128 that is no multiple
- * of 128 runs PERSISTENT's tiles, the last ones overlapping (a second buffer
- * of L*L floats; without memory for it, or room for the cooperative grid, the
- * two-pass kernels run); xy_algorithm reports TWO_PASS for the latter all the
- * same, and with xy_timing on they run the two timed kernels.
+ * Under AUTO with exact sums (and ctas_per_sm = 0) a lattice that the device can
+ * hold on the chip runs all sweeps of a call in one launch, in place: up to
+ * L = 128 one cluster, up to 1280 one tile per SM (with 16 L^2 bytes for the
+ * words that tiles exchange).  Any other even side above 128 runs PERSISTENT's
+ * tiles, the last ones overlapping where L is no multiple of 128 (a second buffer
+ * of L*L floats).  Without memory for the words or the second buffer, or room for
+ * the cooperative launch, a side takes the next of these, at last the two-pass
+ * kernels.  xy_algorithm reports PERSISTENT and TWO_PASS by the side all the
+ * same, and a lattice reported TWO_PASS runs the two timed kernels with xy_timing
+ * on.
  *   XY_ALGO_FUSED      one launch per sweep (both colours + measure), the state
  *                      ping-pongs between the caller's buffer and a library
  *                      buffer of the same size (8 B moved per update);

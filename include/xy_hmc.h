@@ -92,7 +92,9 @@ typedef struct {
  * from there TILED2's two steps per launch, on overlapping tiles where L is no
  * multiple of 128 (the begin, final and odd step then by SITE); the choices
  * measured fastest on GB300 (us per unit trajectory: L = 128 17.6 against 29.6
- * SITE, 39.3 CLUSTER and 43.3 TILED2; 512 75 against 104 SITE).  All
+ * SITE, 39.3 CLUSTER and 43.3 TILED2; 512 75 against 104 SITE).  TILED2 runs its
+ * two steps on 32 x 128 tiles, and from L = 1792 (1500 where L is no multiple of
+ * 128) by rows, each warp on its own.  All
  * give bit-identical angles, momenta and sums. */
 enum { XY_HMC_KERNEL_AUTO = 0, XY_HMC_KERNEL_TILED = 1, XY_HMC_KERNEL_SITE = 2,
        XY_HMC_KERNEL_TILED2 = 3, XY_HMC_KERNEL_TILED_TMA = 4, XY_HMC_KERNEL_CLUSTER = 5,

@@ -50,7 +50,11 @@ typedef struct xy_quad xy_quad;
  *               XY_ALGO_AUTO -- persistent where L % 32 == 0 and L <= 1024
  *               (falling back to one fused launch per sweep when the
  *               cooperative grid does not fit), fused for larger multiples of
- *               32, else two-pass.
+ *               32, else two-pass; with exact sums most sides from 12 to 1280
+ *               instead run the replicas as lattices held on the chip, in
+ *               place (the algorithm reported is the same; 16 L^2 bytes for
+ *               each replica run at a time instead of the second buffer; without
+ *               them the algorithm reported).
  *               All give the same angles, accept counts and (fused and
  *               persistent) records bit for bit.
  *   beta        four inverse temperatures (>= 0, finite), one per replica.

@@ -25,12 +25,12 @@ namespace {
 constexpr uint32_t kMagicLive = 0x484D434Cu;   // "HMCL"
 constexpr uint32_t kMagicDead = 0xDEADBEEFu;
 
-// AUTO: from this side on the full steps run two per launch on 32 x 128 tiles
+// AUTO: from this side on the full steps run two per launch, on 32 x 128 tiles
 // (overlapping ones where L is no multiple of 128), below it one launch per
 // step of one thread per site, which fills the GPU with fewer sites (us per
 // unit trajectory, two per launch / per site: L = 256 57.6 / 45.3, 320 62.4 /
-// 56.9, 384 66.0 / 68.7, 500 82.9 / 103, 1000 171 / 375, 1001 193 / 376, 2000
-// 704 / 1768).
+// 56.9, 384 66.0 / 68.7, 500 82.9 / 103, 1000 171 / 375, 1001 193 / 376; by rows
+// 2000 612 / 1768).
 constexpr int kAutoPairsMinL = 352;
 
 thread_local char g_msg[512] = "no error";
@@ -69,7 +69,7 @@ struct xy_hmc {
   unsigned int* d_tiles;             // its per-tile step counters
   bool use_cluster;                  // whole trajectories in one cluster launch
   bool use_resident;                 // AUTO: many trajectories per cluster launch
-  bool use_pairs;                    // full steps two per launch (k_hmc_tile2)
+  bool use_pairs;                    // full steps two per launch (k_hmc_tile2, k_hmc_rows2)
   int tma_rows;                      // tile (and box) rows of the TMA step kernel: 32 or 16
   int tma_ctas;                      // persistent grid of the TMA step kernel
   uint32_t magic;
