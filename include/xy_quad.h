@@ -47,7 +47,8 @@ typedef struct xy_quad xy_quad;
  *               device memory, bounded waits reported as XY_ETIMEOUT at the
  *               next synchronizing call; needs L % 32 == 0 and every CTA of
  *               the grid resident, XY_ECUDA otherwise);
- *               XY_ALGO_AUTO -- persistent where L % 32 == 0 and L <= 1024
+ *               XY_ALGO_AUTO -- persistent where L % 32 == 0 and L <= 1536
+ *               (libm sincos: 1024)
  *               (falling back to one fused launch per sweep when the
  *               cooperative grid does not fit), fused for larger multiples of
  *               32, else two-pass; with exact sums most sides from 12 to 1280

@@ -194,26 +194,29 @@ cudaError_t launch_quad_half(int colour, int mode, int red, const QuadArgs& a, c
 // ---------------------------------------------------------------------------
 // C ABI
 // ---------------------------------------------------------------------------
-// XY_ALGO_AUTO takes the persistent sweep up to this side (beyond it one
-// launch per sweep has enough waves of tiles to hide its fill and drain:
-// measured at L = 2048 152.7 against 155.9 G updates/s, at 1024 152.4 against
-// 136.5)
-constexpr int kAutoPersistentMaxL = 1024;
+// XY_ALGO_AUTO takes the persistent sweep up to these sides (beyond, one launch
+// per sweep has enough waves of tiles to hide its fill and drain; with libm
+// sincos its spills cost more).  us per sweep, persistent and per sweep: L = 1056
+// 25.3, 29.0 (libm 34.5, 35.1)   1184 31.0, 34.6 (libm 43.1, 41.3)   1312 37.8, 40.7
+// 1600 56.1, 55.7   2048 93.4, 88.3.
+constexpr int kAutoPersistentMaxL = 1536, kAutoPersistentMaxLLibm = 1024;
 
 // Whether AUTO takes the replicas held on the chip where they fit.  us per sweep
 // of the four, this and the kernel it replaces:
 //   L no multiple of 32 (two-pass)     500 5.5, 20.6   1000 21.8, 47.3
 //   up to 672 (four or two at a time)  32 1.4, 5.5   256 2.1, 6.9   512 6.5, 10.0
-//                                      640 8.7, 12.7   672 10.9, 13.1
-// above only where the tiles fill their warps' lanes (L % 128 == 0):
-//   768 13.4, 14.9   896 17.4, 18.5   1024 21.1, 23.2   1280 34.1, 36.9
-//   but 704 13.5, 13.6   800 16.0, 15.6   960 21.2, 20.7
+//                                      640 8.7, 11.1
+// above only where the tiles fill their warps' lanes (L % 128 == 0) and nearly all
+// SMs: 896 17.4, 18.5   1024 21.1, 23.2   1280 34.1, 35.3   but 704 13.5, 12.1
+// 800 16.0, 14.9   960 21.2, 20.7   1152 (144 of 152 SMs) 29.9, 28.7
 // and, as the tile's own unit vectors are not computed again each sweep, with
-// libm sincos always (800 18.3, 23.6; 1024 25.0, 32.0) and with the SFU's never
-// (896 15.7, 14.7; 1024 19.2, 18.5).
-bool grid_wins(int L, int sincos_mode) {
+// libm sincos always (704 15.4, 15.5; 800 18.3, 19.6; 1024 25.0, 32.0) and with the
+// SFU's never (896 15.7, 14.7; 1024 19.2, 18.5).
+bool grid_wins(int L, int sincos_mode, int sms) {
   if (L % 32 != 0 || L <= 672) return true;
-  return sincos_mode == 2 || (sincos_mode == 0 && L % 128 == 0);
+  const int cols = L / 128;
+  return sincos_mode == 2 ||
+         (sincos_mode == 0 && L % 128 == 0 && 20 * cols * (sms / cols) >= 19 * sms);
 }
 
 constexpr uint32_t kMagicLive = 0x51554144u;   // "QUAD"
@@ -487,7 +490,8 @@ xy_status xy_quad_create(const xy_params* p, const double beta[4], void* cuda_st
   q->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   q->fused = p->algorithm != XY_ALGO_TWO_PASS && xyk::quad_fused_supported(p->L);
   q->persistent = p->algorithm == XY_ALGO_PERSISTENT ||
-                  (p->algorithm == XY_ALGO_AUTO && q->fused && p->L <= kAutoPersistentMaxL);
+                  (p->algorithm == XY_ALGO_AUTO && q->fused &&
+                   p->L <= (p->sincos_mode == 2 ? kAutoPersistentMaxLLibm : kAutoPersistentMaxL));
   q->auto_persistent = q->persistent && p->algorithm == XY_ALGO_AUTO;
   q->cur = 0;
   const size_t N = (size_t)p->L * (size_t)p->L;
@@ -500,12 +504,12 @@ xy_status xy_quad_create(const xy_params* p, const double beta[4], void* cuda_st
   }
   if (e == cudaSuccess) step = "sweep buffers";
   // AUTO: as many replicas side by side on the chip as fit, the others after them
-  if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->reduce_mode == XY_REDUCE_EXACT &&
-      grid_wins(p->L, p->sincos_mode)) {
+  if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->reduce_mode == XY_REDUCE_EXACT) {
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&q->sms, cudaDevAttrMultiProcessorCount, dev);
-    for (int g = kR; e == cudaSuccess && g >= 1 && !q->grid; g /= 2) {
+    const bool wins = grid_wins(p->L, p->sincos_mode, q->sms);
+    for (int g = kR; e == cudaSuccess && wins && g >= 1 && !q->grid; g /= 2) {
       bool fits = false;
       if (xyk::prepare_grid(p->sincos_mode, p->L, q->sms, g, &fits) != cudaSuccess)
         (void)cudaGetLastError();

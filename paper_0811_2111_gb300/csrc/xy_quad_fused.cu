@@ -46,7 +46,6 @@ constexpr int kSRows = kTileRows + 4;        // rows y0-2 .. y0+33
 constexpr int kSCols = kTileF + 8;           // elements f0-4 .. f0+67 (one halo site per side)
 constexpr int kSPairs = kSCols / 2;          // two adjacent elements per float4 of unit vectors
 constexpr int kRing = 2 * kTileF + kTileRows * kR;   // 256 ring elements, one per thread
-constexpr int kStageRowsTotal = kSRows + (kSRows - 2);
 
 constexpr size_t kThBytes = sizeof(float) * 2 * kSRows * kSCols;
 constexpr size_t kCsBytes = sizeof(float4) * 2 * kSRows * kSPairs;
@@ -643,15 +642,15 @@ cudaError_t launch_persist_plan(const QuadPersistArgs& p, cudaStream_t stream) {
 
 template <int MODE, int RED>
 cudaError_t launch_persist_one(const QuadPersistArgs& p, cudaStream_t stream) {
-  // where two CTAs per SM hold all of a sweep's tiles a sweep is one tile's
-  // latency and 128 registers a thread shorten it (L = 256 6.8 against 7.3 us
-  // per sweep, 512 10.1 against 10.5); else three hide it better (1024 23.0
-  // against 23.8)
+  // with few tiles per SM a sweep waits for a tile's latency and 128 registers a
+  // thread shorten it; else three CTAs per SM hide it better.  us per sweep, two
+  // and three: L = 256 6.8, 7.3   640 11.1, 12.7   704 12.1, 13.6 (libm 15.5, 18.2)
+  // 800 14.9, 15.8   960 21.1, 20.9 (SFU 17.9, 16.7)   1024 23.9, 23.4
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  return quad_persistent_tiles(p.a.L) <= 2 * sms ? launch_persist_plan<MODE, RED, 2>(p, stream)
+  return 2 * quad_persistent_tiles(p.a.L) <= 9 * sms ? launch_persist_plan<MODE, RED, 2>(p, stream)
                                                  : launch_persist_plan<MODE, RED, 3>(p, stream);
 }
 
