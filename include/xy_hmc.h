@@ -88,7 +88,8 @@ typedef struct {
  * the grid resident; bit-identical, but measured slower than TILED_TMA on
  * GB300: 256 against 331 G site-steps/s at L = 4096).  AUTO holds
  * lattices of 4 <= L <= 176 on the chip and runs many trajectories per cluster
- * launch (where the device can run the cluster), takes SITE up to L = 351, and
+ * launch (where the device can run the cluster), takes SITE up to L = 351
+ * (419 where L is no multiple of 128, 469 there without accurate sincos), and
  * from there TILED2's two steps per launch, on overlapping tiles where L is no
  * multiple of 128 (the begin, final and odd step then by SITE); the choices
  * measured fastest on GB300 (us per unit trajectory: L = 128 17.6 against 29.6

@@ -25,13 +25,20 @@ namespace {
 constexpr uint32_t kMagicLive = 0x484D434Cu;   // "HMCL"
 constexpr uint32_t kMagicDead = 0xDEADBEEFu;
 
-// AUTO: from this side on the full steps run two per launch, on 32 x 128 tiles
-// (overlapping ones where L is no multiple of 128), below it one launch per
-// step of one thread per site, which fills the GPU with fewer sites (us per
-// unit trajectory, two per launch / per site: L = 256 57.6 / 45.3, 320 62.4 /
-// 56.9, 384 66.0 / 68.7, 500 82.9 / 103, 1000 171 / 375, 1001 193 / 376; by rows
-// 2000 612 / 1768).
-constexpr int kAutoPairsMinL = 352;
+// AUTO: from these sides on the full steps run two per launch, on 32 x 128 tiles
+// (overlapping ones where L is no multiple of 128), below them one launch per
+// step of one thread per site, which fills the GPU with fewer sites.  us per unit
+// trajectory, two per launch / per site: L = 256 57.6 / 45.3, 384 67.9 / 68.7;
+// overlapping 360 69.7 / 67.6, 390 74.2 / 70.0, 420 76.1 / 82.0, 500 82.9 / 103, 1000 171 / 375, by
+// rows 2000 612 / 1768; with SFU or libm sincos, whose unit vectors a thread per
+// site hides better, 400 64.4 / 64.1 and 94.5 / 90.4, 450 75.3 / 77.2 and 107.8 /
+// 107.3, 480 69.9 / 78.2 and 102 / 106.
+constexpr int kAutoPairsMinL = 352, kAutoPairsMinRagged = 420, kAutoPairsMinRaggedOther = 470;
+
+int auto_pairs_min(const xy_hmc_params* p) {
+  if (p->L % 128 == 0) return kAutoPairsMinL;
+  return p->sincos_mode == 0 ? kAutoPairsMinRagged : kAutoPairsMinRaggedOther;
+}
 
 thread_local char g_msg[512] = "no error";
 
@@ -443,7 +450,7 @@ xy_status xy_hmc_create(const xy_hmc_params* p, void* cuda_stream, void* d_angle
   // launch at L = 512 ... 4096); the odd step of a trajectory runs on the TMA
   // kernel where the tiles divide the side, else one thread per site
   const bool auto_pairs =
-      p->kernel == XY_HMC_KERNEL_AUTO && !h->use_resident && p->L >= kAutoPairsMinL;
+      p->kernel == XY_HMC_KERNEL_AUTO && !h->use_resident && p->L >= auto_pairs_min(p);
   h->use_pairs = p->kernel == XY_HMC_KERNEL_TILED2 || auto_pairs;
   const bool want_tma = p->kernel == XY_HMC_KERNEL_TILED_TMA || p->kernel == XY_HMC_KERNEL_PERSISTENT ||
                         p->kernel == XY_HMC_KERNEL_TILED2 ||
