@@ -62,6 +62,14 @@ def obs_arrays(obs):
     return {n: a[n].copy() for n in OBS_NAMES}
 
 
+def state_array(n):
+    """n float32 to read a state into, their pages made present where they are fresh: the
+    array is new, so nothing of it can be lost."""
+    a = np.empty(n, np.float32)
+    lib().xy_touch_pages(a.ctypes.data_as(C.c_void_p), a.nbytes)
+    return a
+
+
 class xy_batch_params(C.Structure):
     _fields_ = [("n", C.c_int32), ("L", C.POINTER(C.c_int32)), ("beta", C.POINTER(C.c_double)),
                 ("ladder", C.POINTER(C.c_int32)), ("J", C.c_double), ("delta", C.c_double),
@@ -174,6 +182,7 @@ def lib():
                                  C.POINTER(C.c_double), C.POINTER(C.c_double)]),
         "xy_peak_last_error": (C.c_char_p, []),
         "xy_debug_fail_alloc": (st, [C.c_int32]),
+        "xy_touch_pages": (st, [P, C.c_int64]),
         "xy_debug_build": (C.c_int32, []),
         "xy_debug_checks": (st, [C.POINTER(C.c_uint32)]),
     }

@@ -909,7 +909,6 @@ xy_status xy_get_state(xy_ctx* c, float* host, uint64_t* next_sweep) {
   if (!c->d_scratch) XY_CUDA(c, xyk::dev_malloc(&c->d_scratch, N * sizeof(float)), "xy_get_state: scratch");
   XY_CUDA(c, xyk::launch_split_to_natural(c->d_theta, c->d_scratch, c->p.L, c->stream),
           "xy_get_state: layout kernel");
-  xyk::touch_pages(host, N * sizeof(float));
   XY_CUDA(c, cudaMemcpyAsync(host, c->d_scratch, N * sizeof(float), cudaMemcpyDeviceToHost,
                              c->stream),
           "xy_get_state: copy");

@@ -654,9 +654,6 @@ xy_status xy_hmc_get_state(xy_hmc* h, float* host_angles, float* host_momenta,
   xy_status st = check(h);
   if (st != XY_OK) return st;
   if (!host_angles) return fail(h, XY_EINVAL, "xy_hmc_get_state: NULL angles");
-  const size_t N = (size_t)h->p.L * (size_t)h->p.L;
-  xyk::touch_pages(host_angles, N * sizeof(float));
-  xyk::touch_pages(host_momenta, N * sizeof(float));
   st = sync(h, "xy_hmc_get_state: stream");
   if (st != XY_OK) return st;
   uint32_t cur = 0;
@@ -665,6 +662,7 @@ xy_status xy_hmc_get_state(xy_hmc* h, float* host_angles, float* host_momenta,
   st = sync(h, "xy_hmc_get_state: stream");
   if (st != XY_OK) return st;
   if (cur > 2) return fail(h, XY_ESTATE, "xy_hmc_get_state: corrupt state buffer index");
+  const size_t N = (size_t)h->p.L * (size_t)h->p.L;
   H_CUDA(h, cudaMemcpyAsync(host_angles, h->th[cur], N * sizeof(float), cudaMemcpyDeviceToHost,
                             h->stream),
          "xy_hmc_get_state: angles");

@@ -43,10 +43,6 @@ inline cudaError_t dev_malloc(T** p, size_t bytes) {
   return dev_malloc_raw(reinterpret_cast<void**>(p), bytes);
 }
 
-// Touches the pages of a host array that is about to be overwritten whole, if
-// it is large and fresh (xy_alloc.cu).
-void touch_pages(void* p, size_t bytes);
-
 // The debug build's device-side check words (xy_debug.h) of the instrumented
 // translation units, read and cleared (0 in the release build).
 unsigned int debug_take_sweep();    // xy_sweep.cu: two-pass sweep, layout kernels

@@ -708,7 +708,6 @@ xy_status xy_quad_get_state(xy_quad* q, int32_t replica, float* host, uint64_t* 
   Q_CUDA(q, cudaGetLastError(), "xy_quad_get_state: extract");
   Q_CUDA(q, xyk::launch_split_to_natural(q->d_scratch, q->d_nat, q->p.L, q->stream),
          "xy_quad_get_state: layout");
-  xyk::touch_pages(host, (size_t)N * sizeof(float));
   Q_CUDA(q, cudaMemcpyAsync(host, q->d_nat, (size_t)N * sizeof(float), cudaMemcpyDeviceToHost,
                             q->stream),
          "xy_quad_get_state: copy");

@@ -84,8 +84,7 @@ class HMC:
 
     def state(self):
         """(angles [L, L] float32, momenta [L, L] float32, next trajectory)."""
-        th = np.empty(self.L * self.L, np.float32)
-        p = np.empty(self.L * self.L, np.float32)
+        th, p = X.state_array(self.L * self.L), X.state_array(self.L * self.L)
         t = X.xy_hmc_get_state(self.h, th.ctypes.data_as(C.c_void_p), p.ctypes.data_as(C.c_void_p))
         return th.reshape(self.L, self.L), p.reshape(self.L, self.L), t
 

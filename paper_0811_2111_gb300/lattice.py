@@ -82,7 +82,7 @@ class Lattice:
         return X.obs_arrays(obs)
 
     def state(self):
-        buf = np.empty(self.L * self.L, np.float32)
+        buf = X.state_array(self.L * self.L)
         nxt = X.xy_get_state(self.ctx, buf.ctypes.data_as(C.c_void_p))
         return buf.reshape(self.L, self.L), nxt
 
@@ -315,7 +315,7 @@ class Quad:
         return X.obs_arrays(obs)
 
     def state(self, replica):
-        buf = np.empty(self.L * self.L, np.float32)
+        buf = X.state_array(self.L * self.L)
         nxt = X.xy_quad_get_state(self.q, replica, buf.ctypes.data_as(C.c_void_p))
         return buf.reshape(self.L, self.L), nxt
 
