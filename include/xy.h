@@ -223,6 +223,15 @@ xy_status xy_algorithm(const xy_ctx *ctx, int32_t *algorithm);
  * Exists to test the failure path; the paper has no counterpart. */
 xy_status xy_selftest_persistent_wait(void *cuda_stream, int64_t polls);
 
+/* The same for the sweep that keeps its tiles on the chip (XY_ALGO_AUTO, exact
+ * sums, 128 < L <= 1280): a context of L = 256 sweeps with one tile's CTA not
+ * launched, so that the waits for its edge sites run out after `polls` polls (1
+ * <= polls <= 2^22; a poll is a round trip to L2, 0.17 us) and the call reports
+ * XY_ETIMEOUT as any other would (the expected result).  Other results as
+ * above; XY_ECUDA also where the device does not hold such a lattice.
+ * Synchronizes cuda_stream; allocates and frees about 1.5 MB of device memory. */
+xy_status xy_selftest_grid_wait(void *cuda_stream, int64_t polls);
+
 /* The library's debug build (libxy_debug.so, compiled with -DXY_DEBUG) guards
  * the index arithmetic of its two-pass sweep, layout and whole-lattice batch
  * kernels: a check that fails sets a bit of a device word and skips the

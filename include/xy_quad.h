@@ -90,6 +90,9 @@ xy_status xy_quad_info(const xy_quad *q, int64_t *n_records, uint64_t *next_swee
  * XY_ALGO_PERSISTENT. */
 xy_status xy_quad_algorithm(const xy_quad *q, int32_t *algorithm);
 
+/* xy_selftest_grid_wait (xy.h) with four replicas of L = 64 side by side. */
+xy_status xy_selftest_quad_grid_wait(void *cuda_stream, int64_t polls);
+
 xy_status xy_quad_synchronize(xy_quad *q);
 xy_status xy_quad_destroy(xy_quad *q);            /* NULL-safe */
 const char *xy_quad_last_error(const xy_quad *q); /* thread-local message if q == NULL */

@@ -81,6 +81,8 @@ struct xy_ctx {
   bool ragged;             // XY_ALGO_AUTO: persistent sweeps on overlapping tiles
   bool grid;               // XY_ALGO_AUTO: every tile stays with its CTA (xy_grid.cu)
   unsigned long long* d_words;   // its exchange words, then ctl[2] and the wait word
+  int skip_tiles;          // xy_selftest_grid_wait: GridArgs::skip_tiles, and
+  long long polls;         // its spin_limit (0: the default)
   bool persistent;         // ... all sweeps of an xy_sweep call in one cooperative launch
   bool auto_persistent;    // chosen by XY_ALGO_AUTO: per-sweep launches if it does not fit
   unsigned int* d_tiles;   // the persistent launch's per-tile sweep counters
@@ -614,7 +616,8 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
     a.rk = rk;
     a.lattice_id = c->p.lattice_id;
     a.beta[0] = c->p.beta;
-    a.spin_limit = xyk::fused_persistent_spin_limit();
+    a.spin_limit = c->polls > 0 ? c->polls : xyk::grid_spin_limit();
+    a.skip_tiles = c->skip_tiles;
     for (int64_t done = 0; done < n;) {
       const int64_t m = std::min<int64_t>(n - done, kResidentSweeps);
       a.sweep0 = (uint32_t)(c->next_sweep + (uint64_t)done);
@@ -899,6 +902,37 @@ xy_status xy_selftest_persistent_wait(void* cuda_stream, int64_t polls) {
   }
   set_thread_msg("xy_selftest_persistent_wait: the waits completed, which they cannot");
   return XY_OK;
+}
+
+xy_status xy_selftest_grid_wait(void* cuda_stream, int64_t polls) {
+  if (polls < 1 || polls > (1 << 22)) {
+    set_thread_msg("xy_selftest_grid_wait: polls must be in [1, 2^22]");
+    return XY_EINVAL;
+  }
+  xy_params p = {};
+  p.L = 256;
+  p.beta = 1.0;
+  p.J = 1.0;
+  p.delta = M_PI;
+  p.seed = 1;
+  p.start = XY_START_HOT;
+  p.sincos_mode = XY_SINCOS_ACCURATE;
+  p.reduce_mode = XY_REDUCE_EXACT;
+  p.algorithm = XY_ALGO_AUTO;
+  xy_ctx* c = nullptr;
+  xy_status st = xy_create(&p, cuda_stream, nullptr, &c);
+  if (st != XY_OK) return st;
+  if (c->grid) {
+    c->skip_tiles = 1;
+    c->polls = (long long)polls;
+    st = xy_sweep(c, 3);
+    if (st == XY_OK) st = xy_synchronize(c);
+  } else {
+    st = XY_ECUDA;
+    set_thread_msg("xy_selftest_grid_wait: the device does not hold L = 256 one tile per SM");
+  }
+  (void)xy_destroy(c);
+  return st;
 }
 
 xy_status xy_get_state(xy_ctx* c, float* host, uint64_t* next_sweep) {

@@ -80,6 +80,11 @@ __device__ __forceinline__ bool word_is(u64 w, uint32_t tag) { return (uint32_t)
 
 constexpr size_t kGridSmem = 128 * 1024;    // unit vectors of a tile of 110 rows
 
+// Polls before a wait gives up: about a second (the loops do not sleep, a word
+// being on its way for less than that: a poll is a round trip to L2, 170 ns on an
+// otherwise idle GPU).
+constexpr long long kGridSpinLimit = 6ll << 20;
+
 // Part i of n near-equal parts of `total`.
 __host__ __device__ inline int part_size(int total, int n, int i) {
   return total / n + (i < total % n ? 1 : 0);
@@ -518,6 +523,8 @@ cudaError_t with_kernel(int mode, int L, int shape, const F& f) {
 
 }  // namespace
 
+long long grid_spin_limit() { return kGridSpinLimit; }
+
 size_t grid_words(int L) {
   return 4 * (size_t)L * (size_t)((L / 2 + 1) & ~1);
 }
@@ -544,14 +551,15 @@ cudaError_t launch_grid(int sincos_mode, const GridArgs& args, int sms, cudaStre
   if (args.replicas < 1 || args.replicas > kGridReplicas || args.n_sweeps < 1 || args.spin_limit < 1)
     return cudaErrorInvalidValue;
   const Plan p = plan_of(args.L, sms / args.replicas);
-  if (p.shape < 0) return cudaErrorInvalidValue;
+  if (p.shape < 0 || args.skip_tiles < 0 || args.skip_tiles >= p.nx * p.ny)
+    return cudaErrorInvalidValue;
   GridArgs a = args;
   a.nx = p.nx;
   a.ny = p.ny;
   a.tile_warps = p.tile_warps;
   return with_kernel(sincos_mode, args.L, p.shape, [&](auto* fn) {
     void* params[] = {&a};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fn), dim3(args.replicas * p.nx * p.ny),
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fn), dim3(args.replicas * p.nx * p.ny - args.skip_tiles),
                                        dim3(p.threads), params, p.smem, stream);
   });
 }

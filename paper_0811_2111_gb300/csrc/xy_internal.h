@@ -188,9 +188,13 @@ struct GridArgs {
   uint32_t sweep0;       // Philox sweep word of the first sweep
   int n_sweeps;
   xy_record* rec;        // records of the n sweeps, zeroed; replica r's the r-th of every `step`
-  long long spin_limit;  // polls before a wait gives up
+  long long spin_limit;  // polls before a wait gives up (grid_spin_limit())
+  int skip_tiles = 0;    // CTAs not launched (0; > 0 only to test the failure path: what
+                         // they would send never arrives)
   int nx, ny, tile_warps;      // set by launch_grid
 };
+// The default bound of its waits, in polls.
+long long grid_spin_limit();
 // Largest single lattice held by one cluster (xy_resident.cu); larger ones go
 // to one tile per SM where they fit: us per sweep, cluster and tiles, L = 128
 // 1.52 and 1.59, 160 1.94 and 1.68, 256 3.1 and 1.51.

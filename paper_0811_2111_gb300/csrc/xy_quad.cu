@@ -261,6 +261,8 @@ struct xy_quad {
   int grid;                // replicas held on the chip side by side (xy_grid.cu); 0: not this way
   int sms;
   unsigned long long* d_words;   // their exchange words, then the replicas' ctl[2] and the wait word
+  int skip_tiles;          // xy_selftest_quad_grid_wait: GridArgs::skip_tiles, and
+  long long polls;         // its spin_limit (0: the default)
   int cur;                 // which buffer holds the state (0: d_theta, 1: d_theta2)
   float4* d_theta;         // [2][L][L/2] float4
   float4* d_theta2;        // the fused sweep's second buffer (NULL for two-pass)
@@ -410,7 +412,8 @@ xy_status grid_sweeps(xy_quad* q, int64_t n) {
   a.step = kR;
   a.delta = (float)q->p.delta;
   a.rk = xyd::make_round_keys(q->p.seed);
-  a.spin_limit = xyk::fused_persistent_spin_limit();
+  a.spin_limit = q->polls > 0 ? q->polls : xyk::grid_spin_limit();
+  a.skip_tiles = q->skip_tiles;
   for (int64_t done = 0; done < n;) {
     const int64_t m = std::min<int64_t>(n - done, kGridSweeps);
     a.sweep0 = (uint32_t)(q->next_sweep + (uint64_t)done);
@@ -696,6 +699,37 @@ xy_status xy_quad_measure(xy_quad* q, int32_t replica, int64_t first, int64_t co
     o.beta = rec.beta;
   }
   return XY_OK;
+}
+
+xy_status xy_selftest_quad_grid_wait(void* cuda_stream, int64_t polls) {
+  if (polls < 1 || polls > (1 << 22)) {
+    tmsg("xy_selftest_quad_grid_wait: polls must be in [1, 2^22]");
+    return XY_EINVAL;
+  }
+  xy_params p = {};
+  p.L = 64;
+  p.J = 1.0;
+  p.delta = M_PI;
+  p.seed = 1;
+  p.start = XY_START_HOT;
+  p.sincos_mode = XY_SINCOS_ACCURATE;
+  p.reduce_mode = XY_REDUCE_EXACT;
+  p.algorithm = XY_ALGO_AUTO;
+  const double beta[kR] = {1.0, 1.0, 1.0, 1.0};
+  xy_quad* q = nullptr;
+  xy_status st = xy_quad_create(&p, beta, cuda_stream, &q);
+  if (st != XY_OK) return st;
+  if (q->grid) {
+    q->skip_tiles = 1;
+    q->polls = (long long)polls;
+    st = xy_quad_sweep(q, 3);
+    if (st == XY_OK) st = xy_quad_synchronize(q);
+  } else {
+    st = XY_ECUDA;
+    tmsg("xy_selftest_quad_grid_wait: the device does not hold four replicas of L = 64");
+  }
+  (void)xy_quad_destroy(q);
+  return st;
 }
 
 xy_status xy_quad_get_state(xy_quad* q, int32_t replica, float* host, uint64_t* next_sweep) {
