@@ -209,9 +209,23 @@ xy_status xy_records_device(xy_ctx *ctx, const xy_record **d_records, int64_t *c
 /* Number of records so far and the next sweep index. */
 xy_status xy_info(const xy_ctx *ctx, int64_t *n_records, uint64_t *next_sweep);
 
-/* The sweep algorithm the context runs (what XY_ALGO_AUTO resolved to):
- * XY_ALGO_FUSED, XY_ALGO_TWO_PASS or XY_ALGO_PERSISTENT. */
+/* The sweep algorithm the context runs (what XY_ALGO_AUTO resolved to, by the
+ * side alone): XY_ALGO_FUSED, XY_ALGO_TWO_PASS or XY_ALGO_PERSISTENT.  The
+ * kernel that AUTO launched is xy_sweep_kernel's. */
 xy_status xy_algorithm(const xy_ctx *ctx, int32_t *algorithm);
+
+/* The kernel that the last xy_sweep call launched last:
+ *   XY_KERNEL_NONE        no sweep yet
+ *   XY_KERNEL_TWO_PASS    two half-sweeps per sweep
+ *   XY_KERNEL_FUSED       one launch per sweep, _FUSED2 one per two sweeps
+ *   XY_KERNEL_PERSISTENT  tiles, all sweeps in one launch; _OVERLAP with the last
+ *                         tiles overlapping (L no multiple of 128)
+ *   XY_KERNEL_CLUSTER     the lattice held on the chip by one cluster
+ *   XY_KERNEL_GRID        ... by one tile per SM. */
+enum { XY_KERNEL_NONE = 0, XY_KERNEL_TWO_PASS = 1, XY_KERNEL_FUSED = 2, XY_KERNEL_FUSED2 = 3,
+       XY_KERNEL_PERSISTENT = 4, XY_KERNEL_OVERLAP = 5, XY_KERNEL_CLUSTER = 6,
+       XY_KERNEL_GRID = 7 };
+xy_status xy_sweep_kernel(const xy_ctx *ctx, int32_t *kernel);
 
 /* Self-test of the persistent sweep's failure path (no context involved):
  * one persistent launch at L = 128 whose first sweep is never handed out, so

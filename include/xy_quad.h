@@ -90,6 +90,10 @@ xy_status xy_quad_info(const xy_quad *q, int64_t *n_records, uint64_t *next_swee
  * XY_ALGO_PERSISTENT. */
 xy_status xy_quad_algorithm(const xy_quad *q, int32_t *algorithm);
 
+/* The kernel that the last xy_quad_sweep call launched last (xy_sweep_kernel's
+ * values; XY_KERNEL_GRID: the replicas held on the chip). */
+xy_status xy_quad_sweep_kernel(const xy_quad *q, int32_t *kernel);
+
 /* xy_selftest_grid_wait (xy.h) with four replicas of L = 64 side by side. */
 xy_status xy_selftest_quad_grid_wait(void *cuda_stream, int64_t polls);
 

@@ -22,6 +22,8 @@ XY_START_HOT, XY_START_COLD = 0, 1
 XY_SINCOS_ACCURATE, XY_SINCOS_FAST, XY_SINCOS_LIBM = 0, 1, 2
 XY_ALGO_AUTO, XY_ALGO_FUSED, XY_ALGO_TWO_PASS, XY_ALGO_PERSISTENT, XY_ALGO_FUSED2 = 0, 1, 2, 3, 4
 XY_REDUCE_EXACT, XY_REDUCE_COMPENSATED = 0, 1
+# xy_sweep_kernel's XY_KERNEL_* by value
+KERNEL_NAMES = (None, "two_pass", "fused", "fused2", "persistent", "overlap", "cluster", "grid")
 XY_FX_SHIFT = 30
 XY_MAX_L = 32768
 
@@ -123,6 +125,7 @@ def lib():
         "xy_records_device": (st, [P, C.POINTER(P), C.POINTER(C.c_int64)]),
         "xy_info": (st, [P, C.POINTER(C.c_int64), C.POINTER(C.c_uint64)]),
         "xy_algorithm": (st, [P, C.POINTER(C.c_int32)]),
+        "xy_sweep_kernel": (st, [P, C.POINTER(C.c_int32)]),
         "xy_selftest_persistent_wait": (st, [P, C.c_int64]),
         "xy_selftest_grid_wait": (st, [P, C.c_int64]),
         "xy_selftest_quad_grid_wait": (st, [P, C.c_int64]),
@@ -177,6 +180,7 @@ def lib():
         "xy_quad_get_state": (st, [P, C.c_int32, P, C.POINTER(C.c_uint64)]),
         "xy_quad_info": (st, [P, C.POINTER(C.c_int64), C.POINTER(C.c_uint64)]),
         "xy_quad_algorithm": (st, [P, C.POINTER(C.c_int32)]),
+        "xy_quad_sweep_kernel": (st, [P, C.POINTER(C.c_int32)]),
         "xy_quad_synchronize": (st, [P]),
         "xy_quad_destroy": (st, [P]),
         "xy_quad_last_error": (C.c_char_p, [P]),
@@ -252,6 +256,12 @@ def xy_info(ctx):
     s = C.c_uint64()
     check(lib().xy_info(ctx, C.byref(n), C.byref(s)), ctx)
     return n.value, s.value
+
+
+def xy_sweep_kernel(ctx):
+    k = C.c_int32()
+    check(lib().xy_sweep_kernel(ctx, C.byref(k)), ctx)
+    return KERNEL_NAMES[k.value]
 
 
 def xy_algorithm(ctx):
@@ -527,6 +537,12 @@ def xy_quad_info(q):
     t = C.c_uint64()
     quad_check(lib().xy_quad_info(q, C.byref(r), C.byref(t)), q)
     return r.value, t.value
+
+
+def xy_quad_sweep_kernel(q):
+    k = C.c_int32()
+    quad_check(lib().xy_quad_sweep_kernel(q, C.byref(k)), q)
+    return KERNEL_NAMES[k.value]
 
 
 def xy_quad_algorithm(q):

@@ -83,6 +83,7 @@ struct xy_ctx {
   unsigned long long* d_words;   // its exchange words, then ctl[2] and the wait word
   int skip_tiles;          // xy_selftest_grid_wait: GridArgs::skip_tiles, and
   long long polls;         // its spin_limit (0: the default)
+  int32_t ran;             // XY_KERNEL_*: what the last sweeps were launched as
   bool persistent;         // ... all sweeps of an xy_sweep call in one cooperative launch
   bool auto_persistent;    // chosen by XY_ALGO_AUTO: per-sweep launches if it does not fit
   unsigned int* d_tiles;   // the persistent launch's per-tile sweep counters
@@ -319,8 +320,8 @@ cudaError_t timed_grid(xy_ctx* c, const xyk::GridArgs& a) {
   return e;
 }
 
-// m sweeps of the state at theta, in place, by the two-pass kernels: the same
-// bits where a cooperative launch found no room.
+// m sweeps of the state at theta, in place, by the two-pass kernels (also, with
+// the same bits, where a cooperative launch found no room).
 cudaError_t two_pass_sweeps(xy_ctx* c, float* theta, uint32_t sweep0, int64_t m, xy_record* rec,
                             const xyd::RoundKeys& rk) {
   xyk::HalfSweepArgs h;
@@ -332,6 +333,7 @@ cudaError_t two_pass_sweeps(xy_ctx* c, float* theta, uint32_t sweep0, int64_t m,
   h.rk = rk;
   h.lattice_id = c->p.lattice_id;
   h.beta = c->p.beta;
+  c->ran = XY_KERNEL_TWO_PASS;
   cudaError_t e = cudaSuccess;
   for (int64_t i = 0; i < m && e == cudaSuccess; ++i) {
     h.sweep = sweep0 + (uint32_t)i;
@@ -587,6 +589,7 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
   // the two half-sweep kernels are timed one by one, so with timing on a
   // lattice reported as XY_ALGO_TWO_PASS runs them
   if (c->resident && (c->persistent || c->timing_every <= 0)) {
+    c->ran = XY_KERNEL_CLUSTER;
     xyk::ResidentArgs a;
     a.theta = c->d_theta;
     a.L = c->p.L;
@@ -623,6 +626,7 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
       a.sweep0 = (uint32_t)(c->next_sweep + (uint64_t)done);
       a.n_sweeps = (int)m;
       a.rec = c->d_rec + c->rec_count + done;
+      c->ran = XY_KERNEL_GRID;
       cudaError_t e = timed_grid(c, a);
       if (e == cudaErrorCooperativeLaunchTooLarge) {
         // the grid does not fit beside other work
@@ -661,6 +665,7 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
       a.sweep0 = (uint32_t)(c->next_sweep + (uint64_t)done);
       a.n_sweeps = (int)m;
       a.rec = c->d_rec + c->rec_count + done;
+      c->ran = c->ragged ? XY_KERNEL_OVERLAP : XY_KERNEL_PERSISTENT;
       cudaError_t e = timed_persistent(c, a);
       if (e == cudaErrorCooperativeLaunchTooLarge && c->ragged) {
         // the grid does not fit beside other work (the state is in a.buf[0])
@@ -674,6 +679,7 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
         // the grid does not fit beside other work on the device: the same
         // sweeps as one fused launch each (bit-identical)
         (void)cudaGetLastError();
+        c->ran = XY_KERNEL_FUSED;
         xyk::FusedArgs f;
         f.L = a.L;
         f.W = a.W;
@@ -730,6 +736,7 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
       a.rec = c->d_rec + c->rec_count + i;
       // two sweeps per launch where two are left (XY_ALGO_FUSED2)
       const int step = (two && i + 1 < n) ? 2 : 1;
+      c->ran = step == 2 ? XY_KERNEL_FUSED2 : XY_KERNEL_FUSED;
       cudaError_t e = step == 2 ? timed_fused2(c, a) : timed_fused(c, a);
       if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: fused launch");
       float* t = cur;
@@ -744,22 +751,9 @@ xy_status xy_sweep(xy_ctx* c, int64_t n) {
               "xy_sweep: copy back");
     }
   } else {
-    xyk::HalfSweepArgs a;
-    a.theta = c->d_theta;
-    a.L = c->p.L;
-    a.W = c->p.L / 2;
-    a.K = (float)(c->p.beta * c->p.J);
-    a.delta = (float)c->p.delta;
-    a.rk = rk;
-    a.lattice_id = c->p.lattice_id;
-    a.beta = c->p.beta;
-    for (int64_t i = 0; i < n; ++i) {
-      a.sweep = (uint32_t)(c->next_sweep + (uint64_t)i);
-      a.rec = c->d_rec + c->rec_count + i;
-      cudaError_t e = timed_half_sweep(c, 0, a);
-      if (e == cudaSuccess) e = timed_half_sweep(c, 1, a);
-      if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: launch");
-    }
+    const cudaError_t e =
+        two_pass_sweeps(c, c->d_theta, (uint32_t)c->next_sweep, n, c->d_rec + c->rec_count, rk);
+    if (e != cudaSuccess) return cuda_fail(c, e, "xy_sweep: launch");
   }
   c->next_sweep += (uint64_t)n;
   c->rec_count += n;
@@ -836,6 +830,17 @@ xy_status xy_algorithm(const xy_ctx* c, int32_t* algorithm) {
   *algorithm = c->persistent ? XY_ALGO_PERSISTENT
                 : c->p.algorithm == XY_ALGO_FUSED2 ? XY_ALGO_FUSED2
                 : (c->fused ? XY_ALGO_FUSED : XY_ALGO_TWO_PASS);
+  return XY_OK;
+}
+
+xy_status xy_sweep_kernel(const xy_ctx* c, int32_t* kernel) {
+  xy_status st = check_ctx(c);
+  if (st != XY_OK) return st;
+  if (!kernel) {
+    set_thread_msg("xy_sweep_kernel: NULL output");
+    return XY_EINVAL;
+  }
+  *kernel = c->ran;
   return XY_OK;
 }
 

@@ -263,6 +263,7 @@ struct xy_quad {
   unsigned long long* d_words;   // their exchange words, then the replicas' ctl[2] and the wait word
   int skip_tiles;          // xy_selftest_quad_grid_wait: GridArgs::skip_tiles, and
   long long polls;         // its spin_limit (0: the default)
+  int32_t ran;             // XY_KERNEL_*: what the last sweeps were launched as
   int cur;                 // which buffer holds the state (0: d_theta, 1: d_theta2)
   float4* d_theta;         // [2][L][L/2] float4
   float4* d_theta2;        // the fused sweep's second buffer (NULL for two-pass)
@@ -374,6 +375,7 @@ xy_status grow(xy_quad* q, int64_t sweeps) {
 
 // Sweeps [done, done + m) of a call by the two-pass kernels, in place.
 xy_status two_pass_sweeps(xy_quad* q, int64_t done, int64_t m) {
+  q->ran = XY_KERNEL_TWO_PASS;
   QuadArgs a;
   a.theta = current(q);
   a.L = q->p.L;
@@ -426,6 +428,7 @@ xy_status grid_sweeps(xy_quad* q, int64_t n) {
         a.K[j] = (float)(q->beta[r + j] * q->p.J);
         a.beta[j] = q->beta[r + j];
       }
+      q->ran = XY_KERNEL_GRID;
       const cudaError_t e = xyk::launch_grid(q->p.sincos_mode, a, q->sms, q->stream);
       if (e == cudaErrorCooperativeLaunchTooLarge && r == 0) {
         (void)cudaGetLastError();
@@ -608,10 +611,12 @@ xy_status xy_quad_sweep(xy_quad* q, int64_t n) {
       pa.sweep0 = (uint32_t)(q->next_sweep + (uint64_t)done);
       pa.n_sweeps = (int)m;
       pa.rec = q->d_rec + (q->rec_count + done) * kR;
+      q->ran = XY_KERNEL_PERSISTENT;
       cudaError_t e = xyk::launch_quad_persistent(q->p.sincos_mode, q->p.reduce_mode, pa, q->stream);
       if (e == cudaErrorCooperativeLaunchTooLarge && q->auto_persistent) {
         // the grid does not fit beside other work: one fused launch per sweep
         (void)cudaGetLastError();
+        q->ran = XY_KERNEL_FUSED;
         xyk::QuadFusedArgs f = pa.a;
         e = cudaSuccess;
         for (int64_t i = 0; i < m && e == cudaSuccess; ++i) {
@@ -631,6 +636,7 @@ xy_status xy_quad_sweep(xy_quad* q, int64_t n) {
     return XY_OK;
   }
   if (q->fused) {
+    q->ran = XY_KERNEL_FUSED;
     xyk::QuadFusedArgs f;
     f.L = q->p.L;
     f.W = q->p.L / 2;
@@ -698,6 +704,17 @@ xy_status xy_quad_measure(xy_quad* q, int32_t replica, int64_t first, int64_t co
     o.accepted = rec.accepted;
     o.beta = rec.beta;
   }
+  return XY_OK;
+}
+
+xy_status xy_quad_sweep_kernel(const xy_quad* q, int32_t* kernel) {
+  xy_status st = check(q);
+  if (st != XY_OK) return st;
+  if (!kernel) {
+    tmsg("xy_quad_sweep_kernel: NULL output");
+    return XY_EINVAL;
+  }
+  *kernel = q->ran;
   return XY_OK;
 }
 

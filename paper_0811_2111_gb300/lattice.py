@@ -75,6 +75,12 @@ class Lattice:
                 X.XY_ALGO_PERSISTENT: "persistent",
                 X.XY_ALGO_FUSED2: "fused2"}[X.xy_algorithm(self.ctx)]
 
+    @property
+    def kernel(self):
+        """What the last sweeps were launched as: "two_pass", "fused", "fused2", "persistent",
+        "overlap", "cluster" or "grid" (None before the first)."""
+        return X.xy_sweep_kernel(self.ctx)
+
     def observables(self, first=0, count=None):
         n, _ = X.xy_info(self.ctx)
         count = n - first if count is None else count
@@ -301,6 +307,12 @@ class Quad:
         """"persistent" (one launch per call), "fused" (one per sweep) or "two_pass"."""
         return {X.XY_ALGO_FUSED: "fused", X.XY_ALGO_TWO_PASS: "two_pass",
                 X.XY_ALGO_PERSISTENT: "persistent"}[X.xy_quad_algorithm(self.q)]
+
+    @property
+    def kernel(self):
+        """What the last sweeps were launched as: "two_pass", "fused", "persistent" or "grid"
+        (None before the first)."""
+        return X.xy_quad_sweep_kernel(self.q)
 
     def sweep(self, n=1):
         X.xy_quad_sweep(self.q, n)
