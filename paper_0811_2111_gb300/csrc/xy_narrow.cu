@@ -325,9 +325,12 @@ cudaError_t launch_narrow_batch_sweep(int sincos_mode, int reduce_mode, const Fu
 // so every site update -- and each lattice's state -- is bit for bit that of
 // the single-lattice kernels, at one sincos per update instead of two.
 // With L / 2 even a pair's two sites run together on packed FP32 instructions
-// (200 lattices of L = 96: 11.6 -> 11.3 us per sweep of all, compensated sums
-// 13.1 -> 12.5; SFU sincos 9.2 -> 9.4): a dependent chain per pair at 16 warps an
-// SM bounds it.
+// (us per sweep of all, scalar and packed: 200 lattices of L = 96 12.5, 11.9, with
+// compensated sums 13.9, 13.3; 300 of 48 4.30, 4.10): a dependent chain per pair at
+// 16 warps an SM bounds it.  With SFU sincos and exact sums the selects of the packed
+// neighbours cost more than they save (96 10.04, 10.24   64 4.92, 5.12   48 3.49,
+// 3.69; with compensated sums a tie), so there the two sites run by scalar
+// arithmetic, whose same-row neighbours are three loads at computed columns.
 // ---------------------------------------------------------------------------
 namespace xyk {
 
@@ -374,6 +377,9 @@ __global__ void __launch_bounds__(kSThreads, 2) k_batch_small(SmallBatchArgs a) 
   // -- the sites x and x + 2 that share one Philox block -- stepping over the
   // L*W/2 pairs the same way; with W odd (L % 4 == 2) a site at a time
   const bool paired = (W & 1) == 0;
+  // whether a pair's sites run by scalar arithmetic (see above), unit vectors as
+  // (cos, sin) per site, else packed
+  constexpr bool scalar = MODE == 1 && RED == 0;
   const int Wp = paired ? W / 2 : 1;
   const int npairs = half / 2;
   const int py0 = threadIdx.x / Wp, pm0 = threadIdx.x % Wp;
@@ -388,7 +394,7 @@ __global__ void __launch_bounds__(kSThreads, 2) k_batch_small(SmallBatchArgs a) 
   };
 
   float4* vec = reinterpret_cast<float4*>(cs);
-  if (paired) {
+  if (!scalar && paired) {
     for (int i = threadIdx.x; i < half; i += kSThreads) {   // both colours' pairs
       const float2 t = __ldg(reinterpret_cast<const float2*>(src) + i);
       float2 s, c;
@@ -414,7 +420,90 @@ __global__ void __launch_bounds__(kSThreads, 2) k_batch_small(SmallBatchArgs a) 
     xyd::SweepSums<RED> sums;
     sums.init();
     auto add_terms = [&](const float* v) { sums.add(v); };
-    if (paired) {
+    if (scalar && paired) {
+      // ---- red half, a pair per step: sites k = 2m and k + 1 of row y
+      // (flat index o = 2P); left/right neighbours k+q-1, k+q for the first,
+      // k+q, k+q+1 for the second ----
+      for (int P = threadIdx.x, y = py0, m = pm0; P < npairs; P += kSThreads) {
+        // debug build: the carried (y, m) is the pair's position, in range
+        if (!XY_DCHECK(y >= 0 && y < L && m >= 0 && m < Wp && y * Wp + m == P, 0)) {
+          step_pair(y, m);
+          continue;
+        }
+        const int k = 2 * m, o = 2 * P;
+        const int q = y & 1;
+        const int yd = y == 0 ? L - 1 : y - 1, yu = y == L - 1 ? 0 : y + 1;
+        int kl = k + q - 1, kr = k + q + 1;
+        kl += kl < 0 ? W : 0;
+        kr -= kr >= W ? W : 0;
+        const float2* row = cs + half + y * W;
+        const float2 lf = row[kl], md = row[k + q], rg = row[kr];
+        const float4 dn = *reinterpret_cast<const float4*>(cs + half + yd * W + k);
+        const float4 up = *reinterpret_cast<const float4*>(cs + half + yu * W + k);
+        const float Sc0 = xyd::nb_sum(lf.x, md.x, dn.x, up.x);
+        const float Ss0 = xyd::nb_sum(lf.y, md.y, dn.y, up.y);
+        const float Sc1 = xyd::nb_sum(md.x, rg.x, dn.z, up.z);
+        const float Ss1 = xyd::nb_sum(md.y, rg.y, dn.w, up.w);
+        const uint32_t x0 = 2u * (uint32_t)k + (uint32_t)q;          // x0 & 2 == 0
+        const uint4 w =
+            xyd::philox4x32_10(make_uint4((uint32_t)y * uL + x0, sweep, lid, 1u), a.rk);
+        const float2 t = *reinterpret_cast<const float2*>(th + o);
+        const float4 own = *reinterpret_cast<const float4*>(cs + o);
+        const xyd::SiteResult r0 =
+            xyd::metropolis_step<MODE>(t.x, own.x, own.y, Sc0, Ss0, w.x, w.y, K, a.delta);
+        const xyd::SiteResult r1 =
+            xyd::metropolis_step<MODE>(t.y, own.z, own.w, Sc1, Ss1, w.z, w.w, K, a.delta);
+        *reinterpret_cast<float2*>(th + o) = make_float2(r0.th, r1.th);
+        *reinterpret_cast<float4*>(cs + o) = make_float4(r0.c, r0.s, r1.c, r1.s);
+        n_acc += (r0.accept ? 1u : 0u) + (r1.accept ? 1u : 0u);
+        step_pair(y, m);
+      }
+      __syncthreads();
+      // ---- black half, a pair per step, with the sweep sums ----
+      for (int P = threadIdx.x, y = py0, m = pm0; P < npairs; P += kSThreads) {
+        // debug build: the carried (y, m) is the pair's position, in range
+        if (!XY_DCHECK(y >= 0 && y < L && m >= 0 && m < Wp && y * Wp + m == P, 0)) {
+          step_pair(y, m);
+          continue;
+        }
+        const int k = 2 * m, o = half + 2 * P;
+        const int q = (y + 1) & 1;
+        const int yd = y == 0 ? L - 1 : y - 1, yu = y == L - 1 ? 0 : y + 1;
+        int kl = k + q - 1, kr = k + q + 1;
+        kl += kl < 0 ? W : 0;
+        kr -= kr >= W ? W : 0;
+        const float2* row = cs + y * W;
+        const float2 lf = row[kl], md = row[k + q], rg = row[kr];
+        const float4 dn = *reinterpret_cast<const float4*>(cs + yd * W + k);
+        const float4 up = *reinterpret_cast<const float4*>(cs + yu * W + k);
+        const float Sc0 = xyd::nb_sum(lf.x, md.x, dn.x, up.x);
+        const float Ss0 = xyd::nb_sum(lf.y, md.y, dn.y, up.y);
+        const float Sc1 = xyd::nb_sum(md.x, rg.x, dn.z, up.z);
+        const float Ss1 = xyd::nb_sum(md.y, rg.y, dn.w, up.w);
+        const uint32_t x0 = 2u * (uint32_t)k + (uint32_t)q;          // x0 & 2 == 0
+        const uint4 w =
+            xyd::philox4x32_10(make_uint4((uint32_t)y * uL + x0, sweep, lid, 1u), a.rk);
+        const float2 t = *reinterpret_cast<const float2*>(th + o);
+        const float4 own = *reinterpret_cast<const float4*>(cs + o);
+        const xyd::SiteResult r0 =
+            xyd::metropolis_step<MODE>(t.x, own.x, own.y, Sc0, Ss0, w.x, w.y, K, a.delta);
+        const xyd::SiteResult r1 =
+            xyd::metropolis_step<MODE>(t.y, own.z, own.w, Sc1, Ss1, w.z, w.w, K, a.delta);
+        *reinterpret_cast<float2*>(th + o) = make_float2(r0.th, r1.th);
+        *reinterpret_cast<float4*>(cs + o) = make_float4(r0.c, r0.s, r1.c, r1.s);
+        n_acc += (r0.accept ? 1u : 0u) + (r1.accept ? 1u : 0u);
+        // the red sites with the same (y, k) and (y, k + 1) enter M once each
+        const float4 mr = *reinterpret_cast<const float4*>(cs + 2 * P);
+        float v[5];
+        xyd::measure_terms(r0.c, r0.s, lf.x, lf.y, md.x, md.y, dn.x, dn.y, up.x, up.y, Sc0, Ss0,
+                           mr.x, mr.y, v);
+        add_terms(v);
+        xyd::measure_terms(r1.c, r1.s, md.x, md.y, rg.x, rg.y, dn.z, dn.w, up.z, up.w, Sc1, Ss1,
+                           mr.z, mr.w, v);
+        add_terms(v);
+        step_pair(y, m);
+      }
+    } else if (paired) {
       // A pair's unit vectors are one float4 (cos, cos, sin, sin): pair P of
       // colour c is vec[c * npairs + P].
       auto half_sweep = [&](int c) {
