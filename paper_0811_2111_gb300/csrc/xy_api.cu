@@ -295,6 +295,17 @@ cudaError_t timed_persistent(xy_ctx* c, const xyk::FusedPersistArgs& a) {
   return e;
 }
 
+// L*L floats for a state on its way to or from the host.  Between calls the
+// second buffer of the overlapping tiles is free: so it is that one, and such a
+// lattice holds no more memory than the two-pass kernels' with their scratch.
+cudaError_t scratch_of(xy_ctx* c, float** scratch) {
+  cudaError_t e = cudaSuccess;
+  if (!c->ragged && !c->d_scratch)
+    e = xyk::dev_malloc(&c->d_scratch, (size_t)c->p.L * (size_t)c->p.L * sizeof(float));
+  *scratch = c->ragged ? c->d_pong : c->d_scratch;
+  return e;
+}
+
 // At most this many sweeps in one resident launch (a fraction of a second).
 constexpr int64_t kResidentSweeps = 1 << 16;
 
@@ -945,10 +956,11 @@ xy_status xy_get_state(xy_ctx* c, float* host, uint64_t* next_sweep) {
   if (st != XY_OK) return st;
   if (!host) return fail(c, XY_EINVAL, "xy_get_state: NULL output");
   const size_t N = (size_t)c->p.L * (size_t)c->p.L;
-  if (!c->d_scratch) XY_CUDA(c, xyk::dev_malloc(&c->d_scratch, N * sizeof(float)), "xy_get_state: scratch");
-  XY_CUDA(c, xyk::launch_split_to_natural(c->d_theta, c->d_scratch, c->p.L, c->stream),
+  float* scratch = nullptr;
+  XY_CUDA(c, scratch_of(c, &scratch), "xy_get_state: scratch");
+  XY_CUDA(c, xyk::launch_split_to_natural(c->d_theta, scratch, c->p.L, c->stream),
           "xy_get_state: layout kernel");
-  XY_CUDA(c, cudaMemcpyAsync(host, c->d_scratch, N * sizeof(float), cudaMemcpyDeviceToHost,
+  XY_CUDA(c, cudaMemcpyAsync(host, scratch, N * sizeof(float), cudaMemcpyDeviceToHost,
                              c->stream),
           "xy_get_state: copy");
   XY_CUDA(c, cudaStreamSynchronize(c->stream), "xy_get_state: stream");
@@ -964,12 +976,13 @@ xy_status xy_set_state(xy_ctx* c, const float* host, uint64_t next_sweep) {
   if (!host) return fail(c, XY_EINVAL, "xy_set_state: NULL input");
   if (next_sweep > 0xffffffffull) return fail(c, XY_EINVAL, "xy_set_state: sweep >= 2^32");
   const size_t N = (size_t)c->p.L * (size_t)c->p.L;
-  if (!c->d_scratch) XY_CUDA(c, xyk::dev_malloc(&c->d_scratch, N * sizeof(float)), "xy_set_state: scratch");
-  XY_CUDA(c, cudaMemcpyAsync(c->d_scratch, host, N * sizeof(float), cudaMemcpyHostToDevice,
+  float* scratch = nullptr;
+  XY_CUDA(c, scratch_of(c, &scratch), "xy_set_state: scratch");
+  XY_CUDA(c, cudaMemcpyAsync(scratch, host, N * sizeof(float), cudaMemcpyHostToDevice,
                              c->stream),
           "xy_set_state: copy");
   XY_CUDA(c, cudaMemsetAsync(c->d_flag, 0, sizeof(unsigned int), c->stream), "xy_set_state: flag");
-  XY_CUDA(c, xyk::launch_check_finite(c->d_scratch, (int64_t)N, c->d_flag, c->stream),
+  XY_CUDA(c, xyk::launch_check_finite(scratch, (int64_t)N, c->d_flag, c->stream),
           "xy_set_state: check kernel");
   unsigned int flag = 0;
   XY_CUDA(c, cudaMemcpyAsync(&flag, c->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, c->stream),
@@ -979,7 +992,7 @@ xy_status xy_set_state(xy_ctx* c, const float* host, uint64_t next_sweep) {
     set_thread_msg("xy_set_state: non-finite angle rejected; state unchanged");
     return XY_EINVAL;   // not sticky: the context is untouched
   }
-  XY_CUDA(c, xyk::launch_natural_to_split(c->d_scratch, c->d_theta, c->p.L, c->stream),
+  XY_CUDA(c, xyk::launch_natural_to_split(scratch, c->d_theta, c->p.L, c->stream),
           "xy_set_state: layout kernel");
   XY_CUDA(c, cudaStreamSynchronize(c->stream), "xy_set_state: stream");
   c->next_sweep = next_sweep;

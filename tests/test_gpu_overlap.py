@@ -97,3 +97,23 @@ def test_captured_sweeps_replay(L):
             lat.sweep(2)
             ref.sweep(2)
             assert np.array_equal(lat.state()[0], ref.state()[0])
+
+
+def test_the_second_buffer_is_the_scratch_of_a_read_back():
+    """A state goes to the host and back without another L*L floats."""
+    from paper_0811_2111_gb300.lattice import Lattice
+    with Lattice(1300, 1.1, 9, lattice_id=3) as lat:
+        lat.reserve(8)
+        lat.sweep(3)                        # odd: the state moves back to its buffer
+        assert lat.kernel == "overlap"
+        X.lib().xy_debug_fail_alloc(1)
+        try:
+            th, t = lat.state()
+            lat.sweep(2)
+            lat.set_state(th, t)
+            lat.sweep(2)
+            got = lat.state()[0]
+        finally:
+            X.lib().xy_debug_fail_alloc(0)
+    assert np.array_equal(th, _two_pass(1300, 3)[0])
+    assert np.array_equal(got, _two_pass(1300, 5)[0])
