@@ -267,6 +267,14 @@ xy_status xy_debug_checks(uint32_t *failed);
  * for k < 0.  Exists to test the failure path; the paper has no counterpart. */
 xy_status xy_debug_fail_alloc(int32_t k);
 
+/* Test hook of the kernels that take over where a cooperative launch finds no
+ * room beside other work: the next k >= 0 such launches of the library (counted
+ * across every engine and thread of the process) are refused without reaching
+ * the driver.  XY_ALGO_AUTO makes up for them with other kernels, an explicit
+ * XY_ALGO_PERSISTENT reports XY_ECUDA.  Returns XY_EINVAL for k < 0.  The paper
+ * has no counterpart. */
+xy_status xy_debug_fail_cooperative(int32_t k);
+
 /* Host memory whose contents no longer matter, before a large copy into it
  * (xy_get_state and its like): where its pages are not resident, a byte of each
  * is overwritten by eight host threads, which have ended when the call returns

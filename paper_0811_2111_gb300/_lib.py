@@ -188,6 +188,7 @@ def lib():
                                  C.POINTER(C.c_double), C.POINTER(C.c_double)]),
         "xy_peak_last_error": (C.c_char_p, []),
         "xy_debug_fail_alloc": (st, [C.c_int32]),
+        "xy_debug_fail_cooperative": (st, [C.c_int32]),
         "xy_touch_pages": (st, [P, C.c_int64]),
         "xy_debug_build": (C.c_int32, []),
         "xy_debug_checks": (st, [C.POINTER(C.c_uint32)]),

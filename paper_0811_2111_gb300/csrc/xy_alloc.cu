@@ -1,5 +1,5 @@
-// xy_alloc.cu -- the one device-allocation wrapper of the library, with a
-// host-side failure hook for tests.
+// xy_alloc.cu -- the library's device-allocation and cooperative-launch wrappers,
+// with host-side failure hooks for tests.
 //
 // Every cudaMalloc of the library's engines (contexts, batches, HMC, four
 // replicas, record growth) goes through xyk::dev_malloc.  xy_debug_fail_alloc
@@ -7,6 +7,10 @@
 // cudaErrorMemoryAllocation without reaching the driver, so the engines'
 // out-of-memory paths (XY_ENOMEM, nothing leaked, the device still usable) can
 // be exercised on a GPU without exhausting its memory.
+//
+// Every cooperative launch goes through xyk::coop_launch; xy_debug_fail_cooperative
+// makes the next ones fail as a grid does that finds no room beside other work, so
+// that the kernels which then take over can be exercised.
 //
 // Also xy_touch_pages: the first touch of a large array that the caller has just
 // allocated.
@@ -25,6 +29,9 @@ namespace {
 
 // Allocations left before the armed failure (0: disarmed).
 std::atomic<int> g_fail_countdown{0};
+
+// Cooperative launches still to fail.
+std::atomic<int> g_fail_coop{0};
 
 // MADV_POPULATE_WRITE (Linux 5.14; older headers do not name it).
 constexpr int kPopulateWrite = 23;
@@ -47,6 +54,14 @@ cudaError_t dev_malloc_raw(void** p, size_t bytes) {
   return cudaMalloc(p, bytes);
 }
 
+cudaError_t coop_launch(const void* fn, int grid, int threads, void** args, size_t smem,
+                        cudaStream_t stream) {
+  int left = g_fail_coop.load();
+  while (left > 0)
+    if (g_fail_coop.compare_exchange_weak(left, left - 1)) return cudaErrorCooperativeLaunchTooLarge;
+  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), args, smem, stream);
+}
+
 }  // namespace xyk
 
 extern "C" {
@@ -54,6 +69,12 @@ extern "C" {
 xy_status xy_debug_fail_alloc(int32_t k) {
   if (k < 0) return XY_EINVAL;
   g_fail_countdown.store(k);
+  return XY_OK;
+}
+
+xy_status xy_debug_fail_cooperative(int32_t k) {
+  if (k < 0) return XY_EINVAL;
+  g_fail_coop.store(k);
   return XY_OK;
 }
 

@@ -817,9 +817,8 @@ cudaError_t launch_persist_one(const FusedPersistArgs& a, int grid, cudaStream_t
     for (int k = 0; k < 3; ++k) pm.m[b][k] = a.maps->m[i][k];
   }
   void* args[] = {const_cast<FusedPersistArgs*>(&a), &pm};
-  return cudaLaunchCooperativeKernel(
-      reinterpret_cast<const void*>(&k_sweep_fused_persist<MODE, RED, MINB, RAG>), dim3(grid),
-      dim3(kThreads), args, persist_smem<RAG>(), stream);
+  return coop_launch(reinterpret_cast<const void*>(&k_sweep_fused_persist<MODE, RED, MINB, RAG>),
+                     grid, kThreads, args, persist_smem<RAG>(), stream);
 }
 
 template <int MODE, int RED, int MINB, int RAG>

@@ -559,8 +559,9 @@ cudaError_t launch_grid(int sincos_mode, const GridArgs& args, int sms, cudaStre
   a.tile_warps = p.tile_warps;
   return with_kernel(sincos_mode, args.L, p.shape, [&](auto* fn) {
     void* params[] = {&a};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fn), dim3(args.replicas * p.nx * p.ny - args.skip_tiles),
-                                       dim3(p.threads), params, p.smem, stream);
+    return coop_launch(reinterpret_cast<const void*>(fn),
+                       args.replicas * p.nx * p.ny - args.skip_tiles, p.threads, params, p.smem,
+                       stream);
   });
 }
 

@@ -1474,7 +1474,7 @@ cudaError_t launch_hmc_steps_persist(int sincos_mode, const HmcStepsArgs& q, con
   int tx = tiles_x, nt = n_tiles;
   void* args[] = {const_cast<CUtensorMap*>(&m[0]), const_cast<CUtensorMap*>(&m[1]),
                   const_cast<CUtensorMap*>(&m[2]), const_cast<CUtensorMap*>(&m[3]), &qq, &tx, &nt};
-  return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kTileThreads), args, smem, stream);
+  return coop_launch(fn, grid, kTileThreads, args, smem, stream);
 }
 
 int hmc_persist_tiles(int L) {

@@ -43,6 +43,10 @@ inline cudaError_t dev_malloc(T** p, size_t bytes) {
   return dev_malloc_raw(reinterpret_cast<void**>(p), bytes);
 }
 
+// cudaLaunchCooperativeKernel, with a test hook (xy_alloc.cu).
+cudaError_t coop_launch(const void* fn, int grid, int threads, void** args, size_t smem,
+                        cudaStream_t stream);
+
 // The debug build's device-side check words (xy_debug.h) of the instrumented
 // translation units, read and cleared (0 in the release build).
 unsigned int debug_take_sweep();    // xy_sweep.cu: two-pass sweep, layout kernels

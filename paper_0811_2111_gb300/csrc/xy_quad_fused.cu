@@ -636,8 +636,7 @@ cudaError_t launch_persist_plan(const QuadPersistArgs& p, cudaStream_t stream) {
   e = cudaMemsetAsync(p.flags, 0, sizeof(unsigned int) * ((size_t)tiles + 1), stream);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<QuadPersistArgs*>(&p)};
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fn), dim3(grid), dim3(kThreads),
-                                     args, kSmemBytes, stream);
+  return coop_launch(reinterpret_cast<const void*>(fn), grid, kThreads, args, kSmemBytes, stream);
 }
 
 template <int MODE, int RED>
