@@ -25,10 +25,12 @@
 // of two elements, so its same-row neighbours are whole float4s.  Scalar / packed,
 // us per sweep: L = 256 8.1 / 6.8, 512 11.4 / 10.0, 1024 26.9 / 23.1, 4096 371 /
 // 335 (SFU sincos 289 / 281; CUDA's sincosf, which does not pack, 9.9 / 8.9 at
-// 256, 31.1 / 32.0 at 1024 and a tie at 2048).
+// 256, 31.1 / 32.0 at 1024, and beyond see k_quad_fused_libm).
 // Requires L % 32 == 0 (then 4W = 2L is a multiple of 64).
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "xy_device.cuh"
 #include "xy_internal.h"
@@ -59,6 +61,8 @@ typedef float ThArr[kSRows][kSCols];
 // (cos, cos, sin, sin) of stage columns 2j, 2j + 1: the packed instructions'
 // operands
 typedef float4 CsArr[kSRows][kSPairs];
+// (cos, sin) per stage column: the scalar kernel's
+typedef float2 CsScalar[kSRows][kSCols];
 
 __device__ __forceinline__ float2 cosines(const float4& v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 sines(const float4& v) { return make_float2(v.z, v.w); }
@@ -234,8 +238,8 @@ __device__ __forceinline__ float replica_k(const QuadFusedArgs& a, int j) {
 // against a mean of 19.6.  Every load is issued before the first unit vector.
 // Angles are kept only where the tile reads them: the red rows (with their
 // halo sites) and the black tile rows 2..33.
-template <int MODE, bool COHERENT>
-__device__ __forceinline__ void quad_stage(const float* src, ThArr* th, CsArr* cs, int y0, int f0,
+template <int MODE, bool COHERENT, class Cs>
+__device__ __forceinline__ void quad_stage(const float* src, ThArr* th, Cs* cs, int y0, int f0,
                                            int ks0, int L, int W, int F, size_t plane) {
   const int t = threadIdx.x, g = t & 15;
   auto ld = [&](size_t at) {
@@ -269,8 +273,13 @@ __device__ __forceinline__ void quad_stage(const float* src, ThArr* th, CsArr* c
     xyd::unit_vector2<MODE>(make_float2(a.x, a.y), &s01, &c01);
     xyd::unit_vector2<MODE>(make_float2(a.z, a.w), &s23, &c23);
     if (keep_angles) *reinterpret_cast<float4*>(&th[p][r][col]) = a;
-    cs[p][r][col >> 1] = make_float4(c01.x, c01.y, s01.x, s01.y);
-    cs[p][r][(col >> 1) + 1] = make_float4(c23.x, c23.y, s23.x, s23.y);
+    if constexpr (std::is_same<Cs, CsArr>::value) {
+      cs[p][r][col >> 1] = make_float4(c01.x, c01.y, s01.x, s01.y);
+      cs[p][r][(col >> 1) + 1] = make_float4(c23.x, c23.y, s23.x, s23.y);
+    } else {
+      *reinterpret_cast<float4*>(&cs[p][r][col]) = make_float4(c01.x, s01.x, c01.y, s01.y);
+      *reinterpret_cast<float4*>(&cs[p][r][col + 2]) = make_float4(c23.x, s23.x, c23.y, s23.y);
+    }
   };
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -507,6 +516,139 @@ __global__ void __launch_bounds__(kThreads, 3) k_quad_fused(QuadFusedArgs a) {
   quad_sweep_body<MODE, RED, false>(a, blockIdx.x, blockIdx.y);
 }
 
+// The per-sweep kernel with CUDA's sincosf and exact sums beyond four waves of
+// CTAs: scalar arithmetic.  sincosf does not pack, its calls leave no registers
+// for pairs of operands (packed 8 bytes spilled, scalar none), and a large grid
+// shows it; us per sweep, packed and scalar: L = 1376 56.0, 55.7   1600 74.0, 72.0
+// 1856 98.7, 96.8   2048 119.1, 117.2   4096 447, 444, but 1312 (3.7 waves) 49.5,
+// 49.9.  With compensated sums the packed kernel is the faster one (1312 55.6,
+// 57.5; 4096 501, 504).
+__global__ void __launch_bounds__(kThreads, 3) k_quad_fused_libm(QuadFusedArgs a) {
+  constexpr int MODE = 2;
+  extern __shared__ __align__(16) unsigned char smem[];
+  ThArr* th = reinterpret_cast<ThArr*>(smem);
+  CsScalar* cs = reinterpret_cast<CsScalar*>(smem + kThBytes);
+  float(*part)[kR][5][2] = reinterpret_cast<float(*)[kR][5][2]>(smem + kThBytes + kCsBytes);
+  unsigned int(*cnt)[kR] =
+      reinterpret_cast<unsigned int(*)[kR]>(smem + kThBytes + kCsBytes + kPartBytes);
+
+  const int L = a.L, W = a.W;
+  const int F = 4 * W;                                     // elements per plane row
+  const int f0 = blockIdx.x * kTileF;                      // first element of the tile
+  const int ks0 = f0 >> 2;                                 // its first site column
+  const int y0 = blockIdx.y * kTileRows;
+  const size_t plane = (size_t)L * (size_t)F;
+  quad_stage<MODE, false>(a.src, th, cs, y0, f0, ks0, L, W, F, plane);
+  __syncthreads();
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t uL = (uint32_t)L;
+  const int c0 = 2 * lane + 4;                             // stage column of the lane's pair
+  const int fp = f0 + 2 * lane;                            // element of the pair
+  const int j0 = fp & 3;                                   // its replicas j0, j0 + 1
+  const uint32_t kq = (uint32_t)(fp >> 2);                 // its site column
+  const uint32_t id0 = a.lattice_id0 + (uint32_t)j0, id1 = id0 + 1u;
+  const float K0 = (lane & 1) ? a.K[2] : a.K[0];
+  const float K1 = (lane & 1) ? a.K[3] : a.K[1];
+  unsigned int n_acc[2] = {0u, 0u};
+  QuadSums<0> sums;
+
+  // The tile's sites of colour c, written to dst (c = 1: with the sweep sums).
+  auto half = [&](auto colour) {
+    constexpr int c = decltype(colour)::value;
+    const CsScalar& nb = cs[1 - c];
+    float* dst = c ? a.dst + plane : a.dst;
+    float4 D = *reinterpret_cast<const float4*>(&nb[warp * 4 + 1][c0]);
+    float4 P = *reinterpret_cast<const float4*>(&nb[warp * 4 + 2][c0]);
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr) {
+      const int ty = warp * 4 + rr;
+      const int y = y0 + ty;
+      const int r = ty + 2;
+      const int q = (y + c) & 1;                           // x = 2k + q
+      const float4 E = *reinterpret_cast<const float4*>(&nb[r][q ? c0 + 4 : c0 - 4]);
+      const float4 U = *reinterpret_cast<const float4*>(&nb[r + 1][c0]);
+      const float4 l = q ? P : E, rt = q ? E : P, d = D, m = P;
+      D = P;
+      P = U;
+      const float Sc0 = xyd::nb_sum(l.x, rt.x, d.x, U.x), Ss0 = xyd::nb_sum(l.y, rt.y, d.y, U.y);
+      const float Sc1 = xyd::nb_sum(l.z, rt.z, d.z, U.z), Ss1 = xyd::nb_sum(l.w, rt.w, d.w, U.w);
+      const uint32_t x = 2u * kq + (uint32_t)q;
+      const uint32_t ctr = xyd::metropolis_counter((uint32_t)y * uL + x, x);
+      // (lanes l and l ^ 2 pass halves of their blocks across: quad_sweep_body)
+      const bool up = (x & 2u) != 0u;
+      const uint4 wb = xyd::philox4x32_10(make_uint4(ctr, a.sweep, up ? id1 : id0, 1u), a.rk);
+      const uint32_t g0 = __shfl_xor_sync(0xffffffffu, up ? wb.x : wb.z, 2);
+      const uint32_t g1 = __shfl_xor_sync(0xffffffffu, up ? wb.y : wb.w, 2);
+      const uint2 w0 = up ? make_uint2(g0, g1) : make_uint2(wb.x, wb.y);
+      const uint2 w1 = up ? make_uint2(wb.z, wb.w) : make_uint2(g0, g1);
+      const float2 t = *reinterpret_cast<const float2*>(&th[c][r][c0]);
+      const float4 o = *reinterpret_cast<const float4*>(&cs[c][r][c0]);
+      const xyd::SiteResult r0 =
+          xyd::metropolis_step<MODE>(t.x, o.x, o.y, Sc0, Ss0, w0.x, w0.y, K0, a.delta);
+      const xyd::SiteResult r1 =
+          xyd::metropolis_step<MODE>(t.y, o.z, o.w, Sc1, Ss1, w1.x, w1.y, K1, a.delta);
+      n_acc[0] += r0.accept ? 1u : 0u;
+      n_acc[1] += r1.accept ? 1u : 0u;
+      if (c == 0)
+        *reinterpret_cast<float4*>(&cs[0][r][c0]) = make_float4(r0.c, r0.s, r1.c, r1.s);
+      *reinterpret_cast<float2*>(dst + (size_t)y * F + fp) = make_float2(r0.th, r1.th);
+      if (c == 1) {
+        // red elements with the same (y, k, replica): their spins enter M once each
+        float v[5];
+        xyd::measure_terms(r0.c, r0.s, l.x, l.y, rt.x, rt.y, d.x, d.y, U.x, U.y, Sc0, Ss0, m.x,
+                           m.y, v);
+        xyd::fx_add(sums.fx[0], v);
+        xyd::measure_terms(r1.c, r1.s, l.z, l.w, rt.z, rt.w, d.z, d.w, U.z, U.w, Sc1, Ss1, m.z,
+                           m.w, v);
+        xyd::fx_add(sums.fx[1], v);
+      }
+    }
+  };
+  half(std::integral_constant<int, 0>());
+  // the ring at distance one (quad_sweep_body's sites, lane for lane)
+  auto ring_site = [&](int r, int c, int q, uint32_t w0, uint32_t w1, float K) {
+    const float2 l = cs[1][r][c + 4 * q - 4], rt = cs[1][r][c + 4 * q];
+    const float2 d = cs[1][r - 1][c], u = cs[1][r + 1][c], own = cs[0][r][c];
+    const xyd::SiteResult res = xyd::metropolis_step<MODE>(
+        th[0][r][c], own.x, own.y, xyd::nb_sum(l.x, rt.x, d.x, u.x),
+        xyd::nb_sum(l.y, rt.y, d.y, u.y), w0, w1, K, a.delta);
+    cs[0][r][c] = make_float2(res.c, res.s);
+  };
+  if (threadIdx.x < 64) {
+    const int ty = threadIdx.x < 32 ? -1 : kTileRows;
+    const int j = threadIdx.x & 31;
+    const int rep = j & 3;                                 // replica
+    const int sc = 4 + 8 * (j >> 2) + rep;                 // element of site 2 (j >> 2)
+    const int y = wrap_once(y0 + ty, L);
+    const int q = y & 1;
+    const uint32_t x = 2u * (uint32_t)(ks0 + 2 * (j >> 2)) + (uint32_t)q;   // x & 2 == 0
+    const uint4 w = xyd::philox4x32_10(
+        make_uint4((uint32_t)y * uL + x, a.sweep, a.lattice_id0 + (uint32_t)rep, 1u), a.rk);
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      ring_site(ty + 2, sc + 4 * e, q, e ? w.z : w.x, e ? w.w : w.y, replica_k(a, rep));
+  } else if (threadIdx.x < 64 + kTileRows * kR) {
+    const int e = threadIdx.x - 64;
+    const int ty = e >> 2;
+    const int sc = (((y0 + ty) & 1) ? 0 : kTileF + 4) + (e & 3);
+    const int y = y0 + ty;
+    const int q = y & 1;
+    const int ks = wrap_once(ks0 + ((sc - 4) >> 2), W);   // floor: stage columns 0..3 -> ks0 - 1
+    const int j = sc & 3;
+    const uint32_t x = 2u * (uint32_t)ks + (uint32_t)q;
+    const uint32_t site = (uint32_t)y * uL + x;
+    const uint2 uw = xyd::metropolis_words(
+        xyd::philox4x32_10(make_uint4(xyd::metropolis_counter(site, x), a.sweep,
+                                      a.lattice_id0 + (uint32_t)j, 1u), a.rk), x);
+    ring_site(ty + 2, sc, q, uw.x, uw.y, replica_k(a, j));
+  }
+  __syncthreads();
+  sums.init();
+  half(std::integral_constant<int, 1>());
+  quad_commit<0>(sums, n_acc, part, cnt, a.rec, a.beta, blockIdx.x == 0 && blockIdx.y == 0, j0);
+}
+
 // Polls of a tile counter before a wait gives up (with a short sleep between
 // polls: about a second in all).
 constexpr long long kQuadSpinLimit = 1ll << 22;
@@ -653,25 +795,36 @@ cudaError_t launch_persist_one(const QuadPersistArgs& p, cudaStream_t stream) {
                                                  : launch_persist_plan<MODE, RED, 3>(p, stream);
 }
 
-template <int MODE, int RED>
+template <void (*KERNEL)(QuadFusedArgs)>
 cudaError_t launch_one(const QuadFusedArgs& a, cudaStream_t stream) {
-  static bool configured[64] = {};   // attributes set once per instantiation and device
+  static bool configured[64] = {};   // attributes set once per kernel and device
   int dev = 0;
   cudaError_t ge = cudaGetDevice(&dev);
   if (ge != cudaSuccess) return ge;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_quad_fused<MODE, RED>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_quad_fused<MODE, RED>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   const dim3 grid(4 * a.W / kTileF, a.L / kTileRows);
-  k_quad_fused<MODE, RED><<<grid, kThreads, kSmemBytes, stream>>>(a);
+  KERNEL<<<grid, kThreads, kSmemBytes, stream>>>(a);
   return cudaGetLastError();
+}
+
+// CUDA's sincosf: scalar beyond four waves of three CTAs per SM, where the sums
+// are exact.
+cudaError_t launch_libm(bool comp, const QuadFusedArgs& a, cudaStream_t stream) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  if (comp) return launch_one<k_quad_fused<2, 1>>(a, stream);
+  return (4 * a.W / kTileF) * (a.L / kTileRows) > 4 * 3 * sms
+             ? launch_one<k_quad_fused_libm>(a, stream)
+             : launch_one<k_quad_fused<2, 0>>(a, stream);
 }
 
 }  // namespace
@@ -683,9 +836,13 @@ cudaError_t launch_quad_fused(int sincos_mode, int reduce_mode, const QuadFusedA
   if (!quad_fused_supported(a.L) || a.W * 2 != a.L || a.src == a.dst) return cudaErrorInvalidValue;
   const bool comp = reduce_mode != 0;
   switch (sincos_mode) {
-    case 0: return comp ? launch_one<0, 1>(a, stream) : launch_one<0, 0>(a, stream);
-    case 1: return comp ? launch_one<1, 1>(a, stream) : launch_one<1, 0>(a, stream);
-    default: return comp ? launch_one<2, 1>(a, stream) : launch_one<2, 0>(a, stream);
+    case 0:
+      return comp ? launch_one<k_quad_fused<0, 1>>(a, stream)
+                  : launch_one<k_quad_fused<0, 0>>(a, stream);
+    case 1:
+      return comp ? launch_one<k_quad_fused<1, 1>>(a, stream)
+                  : launch_one<k_quad_fused<1, 0>>(a, stream);
+    default: return launch_libm(comp, a, stream);
   }
 }
 
