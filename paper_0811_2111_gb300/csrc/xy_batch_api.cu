@@ -194,6 +194,23 @@ size_t band_bytes(bool fused, int rows, int L) {
                : (size_t)(rows + 2) * W * sizeof(float2);
 }
 
+// Time of a sweep of n lattices of side L by the whole-lattice kernel (304 CTAs at
+// a time), as prepare_resident_batch's estimate compares with it.  With L / 2 even
+// it works on pairs and is the faster for it; us per sweep of all in rounds of ten,
+// exchange included, this kernel and clusters:
+//   16 of L = 44 2.26, 2.46 (SFU 2.05, 2.31; libm 2.46, 2.67), 41 2.26, 2.29 (2.05,
+//   2.26; 2.46, 2.67), 8 of 40 2.26, 2.23 (2.05, 2.23; 2.46, 2.46), but one of 44
+//   2.26, 2.05 (2.05, 2.04; 2.46, 2.34)
+//   100 of 52 2.87, 3.13, but 41 2.88, 2.65
+// and with L / 2 odd 41 of 42 2.87, 2.40, of 46 3.28, 2.49.
+double small_us(int L, int n) {
+  const bool pairs = L % 4 == 0;
+  double us = L <= 32 ? 1.0 : L <= 36 ? 1.4 : L <= 44 ? 1.7 : L <= 48 ? 2.05 : 2.9;
+  if (pairs && L > 36 && L <= 44 && n > 1) us = 1.4;
+  if (pairs && L > 48 && L <= 52) us = 2.25;
+  return us * ((n + 303) / 304);
+}
+
 void make_plan(xy_batch* b, int target_sites) {
   const int CS = xyk::kClusterSize;
   // fused algorithm: sides the single-lattice fused kernel takes (L % 128 ==
@@ -208,9 +225,9 @@ void make_plan(xy_batch* b, int target_sites) {
   // default plan throughout and one side in the whole batch so are the others
   // where that is estimated faster than their own path (measured: tiles 230 G
   // updates/s and no less than 5 us a sweep, narrow tiles 155 and 4.5, whole
-  // lattices 1.0 us up to L = 32, 1.4 to 36, 1.7 to 44, 2.05 to 48, 2.9 above): ten of L = 64 3.0 ->
-  // 1.65, ten of 96 6.25 -> 1.95, four of 128 5.0 -> 1.6, two of 256 5.0 -> 3.3.  Beside lattices of
-  // other sides those paths share the GPU better.
+  // lattices small_us): ten of L = 64 3.0 -> 1.65, ten of 96 6.25 -> 1.95, four of
+  // 128 5.0 -> 1.6, two of 256 5.0 -> 3.3.  Beside lattices of other sides those
+  // paths share the GPU better.
   std::map<int, int> res_ctas;
   if (b->p.algorithm == XY_ALGO_AUTO && b->p.reduce_mode == XY_REDUCE_EXACT &&
       b->p.target_band_sites == 0) {
@@ -220,8 +237,7 @@ void make_plan(xy_batch* b, int target_sites) {
       const int L = kv.first, n = (int)kv.second.size();
       const double sites = (double)n * L * L;
       const double other = xyk::fused_supported(L) ? std::max(5.0, sites / 230e3)
-                           : xyk::small_supported(L)
-                               ? (L <= 32 ? 1.0 : L <= 36 ? 1.4 : L <= 44 ? 1.7 : L <= 48 ? 2.05 : 2.9) * ((n + 303) / 304)
+                           : xyk::small_supported(L) ? small_us(L, n)
                            : xyk::narrow_supported(L) ? std::max(4.5, sites / 155e3) : 1e30;
       if (other < 1e30 && (by_side.size() > 1 || !default_plan)) continue;
       int ctas = 0;
