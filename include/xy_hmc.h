@@ -73,10 +73,7 @@ typedef struct {
  * that streams each tile into double-buffered shared memory with the tensor
  * memory accelerator (needs L % 128 == 0 and the driver's tensor-map encoder;
  * begin and final launches as TILED); TILED2 runs the full steps two per
- * launch (temporal blocking: half the DRAM traffic, a recomputed halo of two;
- * where every resident CTA gets at least four tiles, L >= 4096, two CTAs per
- * SM walk the tiles and bring the next tile's rows in ahead by TMA, which
- * needs the driver's tensor-map encoder: without it one tile per CTA runs);
+ * launch (temporal blocking: half the DRAM traffic, a recomputed halo of two);
  * SITE is one thread per site (any L); CLUSTER runs a whole trajectory in one
  * launch of one thread-block cluster that keeps the lattice in shared memory
  * (L a power of two in [16, 256]; strips of 16 rows per CTA, neighbouring strips
@@ -89,7 +86,7 @@ typedef struct {
  * GB300: 256 against 331 G site-steps/s at L = 4096).  AUTO holds
  * lattices of 4 <= L <= 176 on the chip and runs many trajectories per cluster
  * launch (where the device can run the cluster), takes SITE up to L = 351
- * (419 where L is no multiple of 128, 469 there without accurate sincos), and
+ * (419 to 521 where L is no multiple of 128, by sincos and L % 4), and
  * from there TILED2's two steps per launch, on overlapping tiles where L is no
  * multiple of 128 (the begin, final and odd step then by SITE); the choices
  * measured fastest on GB300 (us per unit trajectory: L = 128 17.6 against 29.6
@@ -99,7 +96,8 @@ typedef struct {
  * give bit-identical angles, momenta and sums. */
 enum { XY_HMC_KERNEL_AUTO = 0, XY_HMC_KERNEL_TILED = 1, XY_HMC_KERNEL_SITE = 2,
        XY_HMC_KERNEL_TILED2 = 3, XY_HMC_KERNEL_TILED_TMA = 4, XY_HMC_KERNEL_CLUSTER = 5,
-       XY_HMC_KERNEL_PERSISTENT = 6 };
+       XY_HMC_KERNEL_PERSISTENT = 6,
+       XY_HMC_KERNEL_RESIDENT = 7 /* an answer of xy_hmc_kernel only: AUTO on the chip */ };
 
 /* One record per trajectory (96 bytes).
  *   sum       C, Ix, Iy, Mx, My of the state after the test (2^-30 units,
@@ -167,6 +165,10 @@ xy_status xy_hmc_measure(xy_hmc *h, int64_t first, int64_t count, xy_obs *host_o
 
 /* Raw device records (xy_hmc_record[count]); stream-ordered. */
 xy_status xy_hmc_records_device(xy_hmc *h, const xy_hmc_record **d_records, int64_t *count);
+
+/* The kernel that trajectories run: the one asked for, or what AUTO resolved to
+ * (XY_HMC_KERNEL_RESIDENT, _SITE or _TILED2). */
+xy_status xy_hmc_kernel(const xy_hmc *h, int32_t *kernel);
 
 /* Number of records, next trajectory number, trajectories accepted so far. */
 xy_status xy_hmc_info(const xy_hmc *h, int64_t *n_records, uint64_t *next_traj,

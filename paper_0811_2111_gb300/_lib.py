@@ -88,6 +88,8 @@ XY_HMC_KERNEL_AUTO, XY_HMC_KERNEL_TILED, XY_HMC_KERNEL_SITE, XY_HMC_KERNEL_TILED
 XY_HMC_KERNEL_TILED_TMA = 4
 XY_HMC_KERNEL_CLUSTER = 5
 XY_HMC_KERNEL_PERSISTENT = 6
+# xy_hmc_kernel's XY_HMC_KERNEL_* by value
+HMC_KERNEL_NAMES = ("auto", "tiled", "site", "tiled2", "tiled_tma", "cluster", "persistent", "resident")
 
 
 class xy_hmc_params(C.Structure):
@@ -164,6 +166,7 @@ def lib():
         "xy_hmc_last_sums": (st, [P, P]),
         "xy_hmc_measure": (st, [P, C.c_int64, C.c_int64, C.POINTER(xy_obs), P]),
         "xy_hmc_records_device": (st, [P, C.POINTER(P), C.POINTER(C.c_int64)]),
+        "xy_hmc_kernel": (st, [P, C.POINTER(C.c_int32)]),
         "xy_hmc_info": (st, [P, C.POINTER(C.c_int64), C.POINTER(C.c_uint64),
                              C.POINTER(C.c_uint64)]),
         "xy_hmc_get_state": (st, [P, P, P, C.POINTER(C.c_uint64)]),
@@ -457,6 +460,12 @@ def xy_hmc_records_device(h):
     n = C.c_int64()
     hmc_check(lib().xy_hmc_records_device(h, C.byref(p), C.byref(n)), h)
     return p.value, n.value
+
+
+def xy_hmc_kernel(h):
+    k = C.c_int32()
+    hmc_check(lib().xy_hmc_kernel(h, C.byref(k)), h)
+    return HMC_KERNEL_NAMES[k.value]
 
 
 def xy_hmc_info(h):

@@ -29,15 +29,24 @@ constexpr uint32_t kMagicDead = 0xDEADBEEFu;
 // (overlapping ones where L is no multiple of 128), below them one launch per
 // step of one thread per site, which fills the GPU with fewer sites.  us per unit
 // trajectory, two per launch / per site: L = 256 57.6 / 45.3, 384 67.9 / 68.7;
-// overlapping 360 69.7 / 67.6, 390 74.2 / 70.0, 420 76.1 / 82.0, 500 82.9 / 103, 1000 171 / 375, by
-// rows 2000 612 / 1768; with SFU or libm sincos, whose unit vectors a thread per
-// site hides better, 400 64.4 / 64.1 and 94.5 / 90.4, 450 75.3 / 77.2 and 107.8 /
-// 107.3, 480 69.9 / 78.2 and 102 / 106.
-constexpr int kAutoPairsMinL = 352, kAutoPairsMinRagged = 420, kAutoPairsMinRaggedOther = 470;
+// overlapping 360 69.7 / 67.6, 390 74.2 / 70.0, 500 82.9 / 103, 1000 171 / 375, by
+// rows 2000 612 / 1768.  On overlapping tiles the line depends on the width that
+// rows allow (16, 8 or 4 bytes for L % 4 = 0, 2, odd) and, as a thread per site
+// hides SFU and libm unit vectors better, on the precision; the per-site time goes
+// up in steps (its last wave), which is where the lines are.  us per trajectory of
+// 30 steps:
+//   accurate   420 86.5 / 92.3   422 89.1 / 92.7   441 94.7 / 91.9   445 96.5 / 100.9
+//   SFU        472 77.1 / 84.4   470 82.4 / 82.5   483 88.6 / 82.4   521 88.6 / 88.6
+//              529 90.0 / 93.6
+//   libm       472 115.4 / 119.2   482 120.7 / 117.9   486 122.5 / 126.5
+//              483 125.5 / 117.2   489 127.5 / 129.0
+constexpr int kAutoPairsMinL = 352;
+constexpr int kAutoPairsMinRagged[3][3] = {   // [sincos mode][L % 4 = 0, 2, odd]
+    {420, 420, 445}, {470, 470, 522}, {470, 484, 486}};
 
 int auto_pairs_min(const xy_hmc_params* p) {
   if (p->L % 128 == 0) return kAutoPairsMinL;
-  return p->sincos_mode == 0 ? kAutoPairsMinRagged : kAutoPairsMinRaggedOther;
+  return kAutoPairsMinRagged[p->sincos_mode][(p->L & 1) ? 2 : (p->L & 2) ? 1 : 0];
 }
 
 thread_local char g_msg[512] = "no error";
@@ -629,6 +638,19 @@ xy_status xy_hmc_records_device(xy_hmc* h, const xy_hmc_record** d_records, int6
   if (st != XY_OK) return st;
   if (d_records) *d_records = h->d_rec;
   if (count) *count = h->rec_count;
+  return XY_OK;
+}
+
+xy_status xy_hmc_kernel(const xy_hmc* h, int32_t* kernel) {
+  xy_status st = check(h);
+  if (st != XY_OK) return st;
+  if (!kernel) {
+    tmsg("xy_hmc_kernel: NULL output");
+    return XY_EINVAL;
+  }
+  *kernel = h->p.kernel != XY_HMC_KERNEL_AUTO ? h->p.kernel
+            : h->use_resident ? XY_HMC_KERNEL_RESIDENT
+            : h->use_pairs ? XY_HMC_KERNEL_TILED2 : XY_HMC_KERNEL_SITE;
   return XY_OK;
 }
 

@@ -51,6 +51,12 @@ class HMC:
             self.h = X.xy_hmc_create(p, C.c_void_p(self.stream.cuda_stream), None)
 
     # -- ABI calls ---------------------------------------------------------
+    @property
+    def kernel(self):
+        """The kernel that trajectories run: the one asked for, or "resident", "site" or "tiled2"
+        (what "auto" resolved to)."""
+        return X.xy_hmc_kernel(self.h)
+
     def run(self, n_traj=1):
         X.xy_hmc_run(self.h, n_traj)
 
