@@ -135,12 +135,14 @@ typedef struct {
                              tile kernel per SM (at most 80 registers a thread), 4 (at
                              most 64: more warps per SM), 2 (at most 128: more
                              independent work in flight per warp, fewer warps), or 0
-                             for the library's default: 2 for the persistent sweep
-                             where that holds all of a sweep's tiles, else 3; 4 for
-                             one fused launch per sweep (the faster plans at L <= 1024,
-                             L = 4096 and L = 8192, 16384).  Results do not
-                             depend on it; tuning callers time the plans
-                             (autotune.py). */
+                             for the library's default: for the persistent sweep 2 up
+                             to six of a sweep's tiles per SM (four with SFU sincos
+                             or on overlapping tiles), beyond that 3; 4 for one fused
+                             launch per sweep.  With XY_ALGO_AUTO any value but 0 also
+                             keeps the lattice off the chip and off the overlapping
+                             tiles: the tile kernels of multiples of 128 and the
+                             two-pass kernels run.  Results do not depend on it;
+                             tuning callers time the plans (autotune.py). */
 } xy_params;
 
 /* Per-sweep record as stored on the device (64 bytes).  The five sums are

@@ -27,11 +27,13 @@
 // written and polled with relaxed GPU-scope accesses.  A word itself says that
 // it has arrived: no fence, no counter, no second round trip.  The tag counts
 // exchanges over the lattice's lifetime (ctl[0], advanced by the last CTA to
-// finish, so that captured launches replay).  A slot is rewritten two exchanges
-// later, when the writer has read the next exchange's words of each of the
-// eight tiles around it, and those, its readers, wrote them after reading the
-// slot.  (All eight are read: even rows make the ring need the corner at the
-// upper right and the one at the lower left.)  The first exchange carries the
+// finish, so that captured launches replay).  A tile reads six of the tiles around
+// it: left, right, above (row y0 - 1), below, and the corners at the upper right
+// and the lower left (y0 and the heights are even: the red sites of the odd row
+// y0 - 1 have a black neighbour right of the tile, those of the even row below it
+// one left of it).  Those are the six that read it.  A slot is rewritten two
+// exchanges later, when the writer has read the next exchange's words of all six,
+// and they wrote those after reading the slot.  The first exchange carries the
 // initial state, so the state buffer itself is touched by its owner only.  Every
 // wait is bounded; one that runs out sets *error and ends the CTA, and those
 // that wait for it see *error and end too.
