@@ -66,9 +66,11 @@ def obs_arrays(obs):
 
 def state_array(n):
     """n float32 to read a state into, their pages made present where they are fresh: the
-    array is new, so nothing of it can be lost."""
+    array is new, so nothing of it can be lost.  (Below 8 MB xy_touch_pages does nothing, and
+    the call would cost a small state's read-back 2 us.)"""
     a = np.empty(n, np.float32)
-    lib().xy_touch_pages(a.ctypes.data_as(C.c_void_p), a.nbytes)
+    if a.nbytes >= 8 << 20:
+        lib().xy_touch_pages(a.ctypes.data_as(C.c_void_p), a.nbytes)
     return a
 
 
