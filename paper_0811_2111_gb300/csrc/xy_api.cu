@@ -80,7 +80,8 @@ struct xy_ctx {
   bool resident;           // XY_ALGO_AUTO: the lattice fits on the chip (xy_resident.cu)
   bool ragged;             // XY_ALGO_AUTO: persistent sweeps on overlapping tiles
   bool grid;               // XY_ALGO_AUTO: every tile stays with its CTA (xy_grid.cu)
-  unsigned long long* d_words;   // its exchange words, then ctl[2] and the wait word
+  unsigned long long* d_words;   // its exchange words, then ctl[2], the wait word and records
+  bool rec_inside;         // d_rec lies in d_words' or the overlapping tiles' allocation
   int skip_tiles;          // xy_selftest_grid_wait: GridArgs::skip_tiles, and
   long long polls;         // its spin_limit (0: the default)
   int32_t ran;             // XY_KERNEL_*: what the last sweeps were launched as
@@ -200,9 +201,17 @@ xy_status validate(const xy_params* p) {
   return XY_OK;
 }
 
+// Capacity of the first record buffer.  A lattice on the chip or on overlapping
+// tiles has it at the end of the one allocation that it needs besides the angles, so
+// that creating it and reserving records makes no more allocations than on the
+// two-pass kernels: us for both, two-pass, records apart and inside, L = 200 62, 70,
+// 58   256 66, 72, 58   1000 64, 199, 189 (the words are 16 MB there: a cudaMalloc
+// beyond a megabyte or so takes 110 us)   1300 64, 178, 168.
+constexpr int64_t kFirstRecords = 1024;
+
 xy_status grow_records(xy_ctx* c, int64_t need) {
   if (need <= c->rec_cap) return XY_OK;
-  int64_t cap = c->rec_cap > 0 ? c->rec_cap : 1024;
+  int64_t cap = c->rec_cap > 0 ? c->rec_cap : kFirstRecords;
   while (cap < need) cap *= 2;
   xy_record* nr = nullptr;
   XY_CUDA(c, xyk::dev_malloc(&nr, (size_t)cap * sizeof(xy_record)), "allocating records");
@@ -215,10 +224,18 @@ xy_status grow_records(xy_ctx* c, int64_t need) {
     cudaFree(nr);
     return cuda_fail(c, e, "growing records");
   }
-  if (c->d_rec) cudaFree(c->d_rec);
+  if (c->d_rec && !c->rec_inside) cudaFree(c->d_rec);
+  c->rec_inside = false;
   c->d_rec = nr;
   c->rec_cap = cap;
   return XY_OK;
+}
+
+// The first records at `at`, inside another allocation.
+void first_records(xy_ctx* c, void* at) {
+  c->d_rec = static_cast<xy_record*>(at);
+  c->rec_cap = kFirstRecords;
+  c->rec_inside = true;
 }
 
 // Event pair for the next timed launch of kernel k (grows the pool).
@@ -362,7 +379,7 @@ void release(xy_ctx* c) {
     c->ev_used[k] = 0;
   }
   if (c->owns_theta && c->d_theta) cudaFree(c->d_theta);
-  if (c->d_rec) cudaFree(c->d_rec);
+  if (c->d_rec && !c->rec_inside) cudaFree(c->d_rec);
   if (c->d_pong) cudaFree(c->d_pong);
   if (c->d_scratch) cudaFree(c->d_scratch);
   if (c->d_flag) cudaFree(c->d_flag);
@@ -461,12 +478,15 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
     if (xyk::prepare_grid(p->sincos_mode, p->L, c->sms, 1, &fits) != cudaSuccess)
       (void)cudaGetLastError();       // the other kernels take the lattice
     if (fits) {
-      // optional, and one allocation: the words, the two of ctl, the wait word
+      // optional, and one allocation: the words, the two of ctl, the wait word (and
+      // one of padding), the first records
       const size_t bytes = xyk::grid_words(p->L) * sizeof(unsigned long long);
-      if (xyk::dev_malloc(&c->d_words, bytes + 4 * sizeof(unsigned int)) == cudaSuccess) {
+      const size_t all = bytes + 4 * sizeof(unsigned int) + kFirstRecords * sizeof(xy_record);
+      if (xyk::dev_malloc(&c->d_words, all) == cudaSuccess) {
         unsigned int* ctl = reinterpret_cast<unsigned int*>(c->d_words) + bytes / sizeof(unsigned int);
         c->d_wait = ctl + 2;
-        e = cudaMemsetAsync(c->d_words, 0, bytes + 4 * sizeof(unsigned int), c->stream);
+        first_records(c, ctl + 4);
+        e = cudaMemsetAsync(c->d_words, 0, all, c->stream);
         // ctl[0] = 1 (the low byte)
         if (e == cudaSuccess) e = cudaMemsetAsync(ctl, 1, 1, c->stream);
       } else {
@@ -494,15 +514,19 @@ xy_status xy_create(const xy_params* p, void* cuda_stream, void* d_angles, xy_ct
   if (e == cudaSuccess && p->algorithm == XY_ALGO_AUTO && p->ctas_per_sm == 0 &&
       p->reduce_mode == XY_REDUCE_EXACT && !c->resident && !c->grid &&
       xyk::ragged_supported(p->L)) {
-    // the second buffer, behind it the counters and the wait word: optional
-    // (without them the two-pass kernels run in place) and one allocation
-    const size_t words = (size_t)xyk::fused_tiles(p->L) + 2;
-    cudaError_t r = xyk::dev_malloc(&c->d_pong, N * sizeof(float) + words * sizeof(unsigned int));
+    // the second buffer, behind it the counters, the wait word and the first
+    // records: optional (without them the two-pass kernels run in place) and one
+    // allocation
+    const size_t words = ((size_t)xyk::fused_tiles(p->L) + 2 + 1) & ~(size_t)1;
+    const size_t records = kFirstRecords * sizeof(xy_record);
+    cudaError_t r =
+        xyk::dev_malloc(&c->d_pong, N * sizeof(float) + words * sizeof(unsigned int) + records);
     if (r == cudaSuccess) {
       c->ragged = true;
       c->d_tiles = reinterpret_cast<unsigned int*>(c->d_pong + N);
       c->d_wait = c->d_tiles + words - 1;
-      e = cudaMemsetAsync(c->d_wait, 0, sizeof(unsigned int), c->stream);
+      first_records(c, c->d_tiles + words);
+      e = cudaMemsetAsync(c->d_wait, 0, sizeof(unsigned int) + records, c->stream);
     } else {
       (void)cudaGetLastError();
       c->d_pong = nullptr;
